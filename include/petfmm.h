@@ -402,6 +402,22 @@ int petfmm_debug_interaction_list(int level, int ix, int iy, int32_t *out);
  * PETFMM_OK or PETFMM_EINVAL. */
 int petfmm_debug_near_fit(double sigma, double wleaf, double tol, double *out);
 
+/* The mixed path's near field where the blob core is wide against a leaf
+ * (kappa = w^2 / 2 sigma^2 <= 1.95, leaf width w): Phi(d) = Ein(kappa |d|^2) /
+ * (2 kappa), whose turned gradient is the pair velocity (-d_y, d_x) g(kappa
+ * |d|^2) in leaf units, is expanded between the leaf centres as
+ *   Phi(tau - s - o) = sum C_o[beta][alpha] tx^a ty^b P_a'(sx) P_b'(sy)
+ * (tau, s: target and source offsets from their centres; tx = 2 tau_x etc.;
+ * P: Legendre polynomials; o: the source leaf's position minus the target's).
+ * Writes the operators of the nine o = (-1, -1), (0, -1) .. (1, 1) as the
+ * kernels hold them: rows beta of S floats, S = the number of terms M =
+ * (n + 1)(n + 2) / 2 rounded up to a multiple of 4; terms ordered by the y
+ * degree, then the x degree.  Host only.  Returns the degree n (0: pairs are
+ * summed for this kappa at the default tolerance; nothing is written), or
+ * PETFMM_EINVAL (out too short: cap < 9 M S).  out may be NULL with cap 0 to
+ * ask for the degree. */
+int petfmm_debug_smooth_operators(double kappa, float *out, int64_t cap);
+
 /* The FP64 translation operators of Sec. 2.2 for order p (1..40) and kernel,
  * in the rescaled coefficients (box width r: ME a~_k = a_k / r^k; LE
  * r^(m+1) b_m for the vortex kernel, r^m b_m for the Laplace kernel), as the
@@ -490,7 +506,12 @@ enum {
                                   evaluated once, its kernel value serving both blobs
                                   (K of Eq. 8 is odd);
                                   heavy pairs are cut into pieces for load balance.
-                                  0: every leaf sums its 9 leaves directly.  Both
+                                  Where the blob core is wide against a leaf (w^2 /
+                                  2 sigma^2 <= 1.95) the near kernel is smooth, and
+                                  leaf pairs of many blobs are summed by expansions of
+                                  it instead (to FP32 rounding; not below a
+                                  PETFMM_OPT_NEAR_TOL of 100).
+                                  0: every leaf sums its 9 leaves directly.  All
                                   deterministic; they differ by FP32 rounding of the
                                   sums.  Extra device memory in mode 1: 88 bytes per
                                   blob and 28 per leaf. */
@@ -535,8 +556,8 @@ enum { PETFMM_KERNEL_VORTEX = 0, PETFMM_KERNEL_LAPLACE = 1 };
 int petfmm_set_option(petfmm_ctx *ctx, int option, int64_t value);
 
 /* Stages reported by petfmm_stage_times (milliseconds, last evaluation).
- * PAIRS: the pairwise near-field kernel (mixed path, PETFMM_OPT_P2P_PAIRS = 1;
- * about zero otherwise); P2P: the directed near field (and, on the FP64 path,
+ * PAIRS: the pairwise near-field kernel, or the near field's expansions (mixed
+ * path, PETFMM_OPT_P2P_PAIRS = 1; about zero otherwise); P2P: the directed near field (and, on the FP64 path,
  * L2P and the output in the same kernel); FINAL: the mixed path's final pass
  * (L2P, the sum of the near-field parts, the output in the caller's order;
  * about zero on the FP64 path).  With PETFMM_OPT_OVERLAP the stages

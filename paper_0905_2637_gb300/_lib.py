@@ -148,6 +148,7 @@ def load():
             "petfmm_debug_m2l_images": (I, [I, I, I, P, ctypes.c_int64]),
             "petfmm_debug_op_table": (I, [I, I, I, P, ctypes.c_int64]),
             "petfmm_debug_near_fit": (I, [ctypes.c_double, ctypes.c_double, ctypes.c_double, P]),
+            "petfmm_debug_smooth_operators": (I, [ctypes.c_double, P, ctypes.c_int64]),
             "petfmm_debug_plan": (I, [I, I, ctypes.POINTER(Instance), P, I]),
             "petfmm_set_option": (I, [P, I, I64]),
             "petfmm_stage_times": (I, [P, P, I]),
@@ -233,6 +234,20 @@ def petfmm_debug_near_fit(sigma, wleaf, tol):
         "petfmm_debug_near_fit")
     return dict(deg=int(out[0]), general=int(out[1]), kappa=float(out[2]),
                 split_rho2=float(out[3]), coef=out[4:].copy())
+
+
+def petfmm_debug_smooth_operators(kappa):
+    """Near-field expansions for kappa = w^2 / 2 sigma^2: (degree, operators
+    [9][M][M] float32, layout in petfmm.h); (0, None) where pairs are summed."""
+    n = _ck(load().petfmm_debug_smooth_operators(float(kappa), None, 0),
+            "petfmm_debug_smooth_operators")
+    if n == 0:
+        return 0, None
+    m = (n + 1) * (n + 2) // 2
+    out = np.zeros((9, m, (m + 3) // 4 * 4), np.float32)
+    _ck(load().petfmm_debug_smooth_operators(float(kappa), out.ctypes.data, out.size),
+        "petfmm_debug_smooth_operators")
+    return n, out[:, :, :m]
 
 
 def petfmm_debug_op_table(order, kernel=0, which=0):

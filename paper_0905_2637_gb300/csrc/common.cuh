@@ -77,6 +77,8 @@ struct InstDesc {
     int deg;                // polynomial degree (in rho^2) of g(q) = (1 - e^-q) / q
     int general;            // 1: some near pairs exceed the polynomial range
     float poly[POLY_MAX + 1];
+    int smdeg;              // > 0: near field by expansions of this degree (smooth.cu) ...
+    const void *t_sm;       // ... and their operators
     // FP64 constants
     double inv2s2;          // 1 / (2 sigma^2)
     double cnear64;         // 1 / (2 pi)

@@ -86,6 +86,12 @@ struct Plan {
     int deg = 0, general = 0;          // mixed P2P variant (max over instances)
     size_t tc_smem = 0;                // dynamic shared memory of the tensor-core M2L
     int tcb_pmax = 0;                  // largest order among the block units
+    // near field by expansions (smooth.cu): the degrees in use, the longest
+    // row and the rows needed; pairs_any: some instance sums pairs instead
+    uint32_t sm_degrees = 0;
+    int sm_row = 0;
+    int64_t sm_rows = 0;
+    bool pairs_any = false;
 };
 
 struct Problem {
@@ -131,9 +137,11 @@ struct petfmm_ctx {
 
     DevBuf keysA, keysB, valsA, valsB, hist, scratch, start, xs, ys, gs, rec, me, le, cnt, off,
         items, ctrl, plan_dev, busy, ucount, recu, occ, items_u, ikA, ikB, ivA, ivB, ihist, own,
-        part, pitems, pxtra, pxs, ustage;
+        part, pitems, pxtra, pxs, ustage, smleaf, smlist, smmom, smloc;
     DevBuf hx, hy, hg, hu, hv;  // device staging for petfmm_evaluate_host
     std::map<int, OpTables> tables;
+    // operators of the near-field expansions by (degree, kappa), see get_sm_table
+    std::map<std::pair<int, double>, void *> sm_tables;
 
     // plan upload
     std::vector<unsigned char> last_upload;
@@ -330,6 +338,47 @@ OpTables *get_tables(petfmm_ctx *c, int p, int kernel, int *err) {
     return &(c->tables[key] = t);
 }
 
+// Operators of the near field by expansions for one (degree, kappa): a few
+// hundred KB each.  A server that refits domains meets new values of kappa
+// now and then: when kMaxSmTables are held, they are dropped (after the
+// stream is done with them) before the next evaluation's are made.
+constexpr size_t kMaxSmTables = 64;
+
+double sm_kappa(const InstDesc &d) { return d.wleaf * d.wleaf / (2.0 * d.sigma * d.sigma); }
+
+int attach_sm_tables(petfmm_ctx *c, Plan &pl) {
+    if (!pl.sm_degrees) return PETFMM_OK;
+    size_t missing = 0;
+    for (const InstDesc &d : pl.inst)
+        if (d.smdeg && !c->sm_tables.count({d.smdeg, sm_kappa(d)})) ++missing;
+    if (missing && c->sm_tables.size() + missing > kMaxSmTables && !c->sm_tables.empty()) {
+        if (cudaStreamSynchronize(c->stream) != cudaSuccess) return PETFMM_ECUDA;
+        for (auto &kv : c->sm_tables) cudaFree(kv.second);
+        c->sm_tables.clear();
+    }
+    std::vector<float> host;
+    for (InstDesc &d : pl.inst) {
+        if (!d.smdeg) continue;
+        const std::pair<int, double> key(d.smdeg, sm_kappa(d));
+        auto it = c->sm_tables.find(key);
+        if (it == c->sm_tables.end()) {
+            host_sm_operators(key.second, key.first, host);
+            void *p = nullptr;
+            cudaError_t e = cudaMalloc(&p, host.size() * sizeof(float));
+            if (e == cudaSuccess)
+                e = cudaMemcpy(p, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                if (p) cudaFree(p);
+                return cuda_status(e);
+            }
+            it = c->sm_tables.emplace(key, p).first;
+        }
+        d.t_sm = it->second;
+    }
+    return PETFMM_OK;
+}
+
 void add_task(TaskRange &r, int inst, int level, int64_t count, int64_t per_block) {
     if (count <= 0) return;
     Task t;
@@ -370,8 +419,9 @@ constexpr int64_t kTcbShallowMinUnits = 512;
 
 int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
 
+// smooth: near field by expansions where the blob core allows (smooth.cu)
 int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_segmax, double near_tol,
-               const std::vector<Problem> &probs, Plan &pl) {
+               bool smooth, const std::vector<Problem> &probs, Plan &pl) {
     pl = Plan();
     const int ni = int(probs.size());
     int inst_bits = 0;
@@ -410,8 +460,17 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
         if (precision == PETFMM_MIXED && d.deg == 0) return PETFMM_EINVAL;
         pl.deg = std::max(pl.deg, d.deg);
         pl.general |= d.general;
-        pl.inst.push_back(d);
         const int64_t nleaf = int64_t(1) << (2 * pb.L);
+        if (smooth && precision == PETFMM_MIXED && kernel == KERNEL_VORTEX)
+            d.smdeg = sm_degree(sm_kappa(d), near_tol);
+        if (d.smdeg) {
+            pl.sm_degrees |= 1u << d.smdeg;
+            pl.sm_row = std::max(pl.sm_row, int(sm_row_floats(d.smdeg)));
+            pl.sm_rows += sm_max_rows(d.smdeg, pb.n, nleaf);
+        } else {
+            pl.pairs_any = true;
+        }
+        pl.inst.push_back(d);
         poff += pb.n;
         loff += nleaf;
         eoff += lvl_off(pb.L + 1) * pb.p;
@@ -608,6 +667,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     k.put(pl.N); k.put(pl.nleaves); k.put(pl.nstart); k.put(pl.ncoef); k.put(pl.items_cap);
     k.put(pl.nbits); k.put(pl.pmax); k.put(pl.deg); k.put(pl.general);
     k.put(pl.tc_smem); k.put(pl.tcb_pmax); k.put(grid);
+    k.put(pl.sm_degrees); k.put(pl.sm_row); k.put(pl.sm_rows); k.put(pl.pairs_any);
     k.put(c->precision); k.put(c->dtype); k.put(c->timing); k.put(c->p2p_mode); k.put(c->poison);
     k.put(c->tc_dense_pct); k.put(c->spin_limit); k.put(c->p2p_pairs); k.put(c->kernel);
     k.put(c->tc_blocks); k.put(c->tc_pipe); k.put(c->overlap);
@@ -616,7 +676,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
                             &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount,
                             &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB,
                             &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs,
-                            &c->ustage})
+                            &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc})
         k.put(b->p);
     return k.h;
 }
@@ -639,8 +699,9 @@ constexpr int64_t kUnsortStageMin = int64_t(8) << 20;
 int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     Plan &pl = c->plan;
     PF_TRY(build_plan(c->precision, c->kernel, c->m2l_tc, c->tc_blocks, c->tc_segmax, c->near_tol,
-                      probs, pl));
+                      c->p2p_pairs, probs, pl));
     PF_TRY(attach_tables(c, pl));
+    PF_TRY(attach_sm_tables(c, pl));
     cudaStream_t st = c->stream;  // the launch sequence's stream (a capture swaps it)
     const bool mixed = c->precision == PETFMM_MIXED;
     const int64_t N = pl.N;
@@ -661,7 +722,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     // pairwise near field (mixed path): at most 4 forward neighbours per leaf,
     // a pair cut into at most ceil(na / 128) pieces, and the leaf's own pairs
     // (the pairwise near field is the vortex kernel's)
-    const bool pairs = mixed && c->p2p_pairs && c->kernel == KERNEL_VORTEX;
+    const bool pairs = mixed && c->p2p_pairs && c->kernel == KERNEL_VORTEX && pl.pairs_any;
     const int64_t pair_cap =
         pairs ? 5 * std::min<int64_t>(pl.nleaves, N) + 4 * (N / 128) + 1 : 0;
     const int64_t order_cap = std::max<int64_t>(pl.items_cap, pair_cap);
@@ -683,11 +744,26 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     PF_TRY(ensure(c->cnt, size_t(pl.nleaves) * 4, st));
     PF_TRY(ensure(c->occ, size_t(pl.nleaves) * sizeof(uint2), st));
     PF_TRY(ensure(c->off, size_t(pl.nleaves) * 4, st));
-    PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
+    if (pl.pairs_any) PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
     PF_TRY(ensure(c->ucount,
                   size_t(pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks + pl.tile_blocks()) * sizeof(uint32_t),
                   st));
-    if (mixed) PF_TRY(ensure(c->own, size_t(N) * sizeof(float2), st));
+    if (mixed && pl.pairs_any) PF_TRY(ensure(c->own, size_t(N) * sizeof(float2), st));
+    SmBufs sm{};
+    if (pl.sm_degrees) {
+        const size_t rows = size_t(std::max<int64_t>(pl.sm_rows, 1)), row = size_t(pl.sm_row);
+        PF_TRY(ensure(c->smleaf, size_t(2) * pl.nleaves * sizeof(uint32_t), st));
+        PF_TRY(ensure(c->smlist, rows * sizeof(uint2), st));
+        PF_TRY(ensure(c->smmom, rows * row * sizeof(float), st));
+        PF_TRY(ensure(c->smloc, rows * row * sizeof(float), st));
+        sm.lmask = static_cast<uint32_t *>(c->smleaf.p);
+        sm.lrank = sm.lmask + pl.nleaves;
+        sm.list = static_cast<uint2 *>(c->smlist.p);
+        sm.mom = static_cast<float *>(c->smmom.p);
+        sm.loc = static_cast<float *>(c->smloc.p);
+        sm.rows = pl.sm_rows;
+        sm.row = pl.sm_row;
+    }
     if (pairs) {
         PF_TRY(ensure(c->part, size_t(9) * N * sizeof(float2), st));
         PF_TRY(ensure(c->pitems, size_t(pair_cap) * sizeof(uint4), st));
@@ -707,7 +783,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         pb.xcap = N;  // scratch of split pairs; more wanted: no pair is split
     }
     P2POrder order{}, porder{};
-    if (c->p2p_mode == 0) {
+    if (c->p2p_mode == 0 && pl.pairs_any) {
         const size_t cap = size_t(order_cap);
         PF_TRY(ensure(c->items_u, cap * sizeof(uint4), st));
         PF_TRY(ensure(c->ikA, cap * 4, st));
@@ -726,8 +802,8 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         porder.cap = pair_cap;
     }
     const bool lap = c->kernel == KERNEL_LAPLACE;
-    const int grid = p2p_grid(mixed, pl.deg, pl.general, lap ? 1 : 0);
-    if (grid <= 0) return PETFMM_EINVAL;
+    const int grid = pl.pairs_any ? p2p_grid(mixed, pl.deg, pl.general, lap ? 1 : 0) : 0;
+    if (pl.pairs_any && grid <= 0) return PETFMM_EINVAL;
     const int pgrid = pairs ? p2p_pairs_grid(pl.deg, pl.general) : 0;
     if (pairs && pgrid <= 0) return PETFMM_EINVAL;
     // busy times: the directed kernel's CTAs, then the pair kernel's
@@ -790,6 +866,13 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     // the leaf starts and run beside the gather, the pair and directed
     // kernels wait for the gathered blobs only, and the final pass joins
     // the two streams (PETFMM_OPT_OVERLAP).
+    uint2 *occ = static_cast<uint2 *>(c->occ.p);
+    auto list_occupied = [&](cudaStream_t s) {
+        return launch_occ_list(dtask + pl.leaves_p2m.first, pl.leaves_p2m.count,
+                               pl.leaves_p2m.nblocks, dinst, start, occ, ctrl, s, lc);
+    };
+    // (the near field's expansions need the list on this stream too)
+    if (pl.sm_degrees) PF_CUDA(list_occupied(st));
     cudaStream_t xs = st;
     const bool fork = mixed && c->overlap;
     if (fork) {
@@ -807,9 +890,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                   static_cast<double *>(c->gs.p), st, lc));
     if (fork) PF_CUDA(cudaEventRecord(c->ev_gathered, xs));
     stage_mark_on(c, PETFMM_STAGE_P2M, xs);
-    uint2 *occ = static_cast<uint2 *>(c->occ.p);
-    PF_CUDA(launch_occ_list(dtask + pl.leaves_p2m.first, pl.leaves_p2m.count, pl.leaves_p2m.nblocks,
-                            dinst, start, occ, ctrl, xs, lc));
+    if (!pl.sm_degrees) PF_CUDA(list_occupied(xs));
     if (mixed)
         PF_CUDA(launch_p2m<float>(occ, ctrl, pl.nleaves, dinst, pl.pmax, start, nullptr, nullptr,
                                   nullptr, srec,
@@ -913,7 +994,8 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (fork) PF_CUDA(cudaEventRecord(c->ev_join, xs));
     stage_mark(c, PETFMM_STAGE_WORKLIST);
     const int tpi = mixed ? P2P_TPI_MIXED : P2P_TPI_F64;
-    PF_CUDA(launch_p2p_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count, pl.leaves_wl.nblocks,
+    if (pl.pairs_any)
+        PF_CUDA(launch_p2p_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count, pl.leaves_wl.nblocks,
                                 dinst, start, pl.nleaves, tpi, pairs ? 1 : 0,
                                 static_cast<uint32_t *>(c->cnt.p),
                                 static_cast<uint32_t *>(c->off.p), scratch,
@@ -928,6 +1010,9 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                      c->p2p_mode == 0 ? &porder : nullptr, pb, st, lc));
     if (fork) PF_CUDA(cudaStreamWaitEvent(st, c->ev_gathered, 0));
     stage_mark(c, PETFMM_STAGE_PAIRS);
+    if (pl.sm_degrees)
+        PF_CUDA(launch_sm_near(pl.sm_degrees, occ, ctrl, std::min(pl.nleaves, N), dinst, start,
+                               srec, sm, st, lc));
     // pairwise mode: the neighbouring leaves pairwise
     if (pairs)
         PF_CUDA(launch_p2p_pairs(pgrid, pl.deg, pl.general, static_cast<const uint4 *>(c->pitems.p),
@@ -937,16 +1022,25 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (mixed) {
         // near sums of the own leaf and the directed neighbours, then far
         // field and the sum
-        PF_CUDA(launch_p2p_mixed(grid, pl.deg, pl.general, static_cast<const uint4 *>(c->items.p),
-                                 ctrl, dinst, start, srec, pb.own,
-                                 pairs, lap ? 1 : 0, busy, st, lc));
+        if (pl.pairs_any)
+            PF_CUDA(launch_p2p_mixed(grid, pl.deg, pl.general,
+                                     static_cast<const uint4 *>(c->items.p), ctrl, dinst, start,
+                                     srec, pb.own, pairs, lap ? 1 : 0, busy, st, lc));
         if (fork) PF_CUDA(cudaStreamWaitEvent(st, c->ev_join, 0));
         stage_mark(c, PETFMM_STAGE_FINAL);
-        PF_CUDA(launch_p2p_final(dtask + pl.particles.first, pl.particles.count,
-                                 pl.particles.nblocks, dinst, start, skeys, srec,
-                                 static_cast<const float2 *>(c->le.p), pb, f32, perm, stage, N,
-                                 dtask + pl.outscatter.first, pl.outscatter.count,
-                                 pl.outscatter.nblocks, ctrl, N, st, lc));
+        if (pl.pairs_any)
+            PF_CUDA(launch_p2p_final(dtask + pl.particles.first, pl.particles.count,
+                                     pl.particles.nblocks, dinst, start, skeys, srec,
+                                     static_cast<const float2 *>(c->le.p), pb, f32, stage, N,
+                                     ctrl, N, st, lc));
+        if (pl.sm_degrees)
+            PF_CUDA(launch_sm_final(dtask + pl.particles.first, pl.particles.count,
+                                    pl.particles.nblocks, dinst, start, skeys, srec,
+                                    static_cast<const float2 *>(c->le.p), sm, f32, stage, N, st,
+                                    lc));
+        if (stage)
+            PF_CUDA(launch_unsort(dinst, perm, stage, N, dtask + pl.outscatter.first,
+                                  pl.outscatter.count, pl.outscatter.nblocks, st, lc));
     } else
         PF_CUDA(launch_p2p_f64(grid, static_cast<const uint4 *>(c->items.p), ctrl, dinst, start,
                                static_cast<const double *>(c->xs.p),
@@ -1091,11 +1185,12 @@ int petfmm_destroy(petfmm_ctx *c) {
     cudaStreamSynchronize(c->stream);
     DevBuf *bufs[] = {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist, &c->scratch,
                       &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le, &c->cnt,
-                      &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB, &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->hx, &c->hy,
+                      &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB, &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->hx, &c->hy,
                       &c->hg, &c->hu, &c->hv};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     for (auto &kv : c->tables) free_op_tables(&kv.second);
+    for (auto &kv : c->sm_tables) cudaFree(kv.second);
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->pinned) cudaFreeHost(c->pinned);
@@ -1399,7 +1494,8 @@ int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, in
     int rc = problems_from(n_inst, inst, probs);
     if (rc) return rc;
     Plan pl;
-    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, probs, pl);
+    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, true, probs,
+                    pl);
     if (rc) return rc;
     int n = 0;
     auto emit = [&](int64_t id, const TaskRange &r) {
@@ -1561,6 +1657,8 @@ int petfmm_debug_checks(uint32_t *lines) {
     lines[0] = pf_checks_tree();
     lines[1] = pf_checks_expansions();
     lines[2] = pf_checks_p2p();
+    const unsigned sm_line = pf_checks_smooth();
+    if (!lines[2]) lines[2] = sm_line;
 #ifdef PETFMM_CHECKS
     return 3;
 #else
@@ -1646,6 +1744,17 @@ int petfmm_debug_near_fit(double sigma, double wleaf, double tol, double *out) {
     out[3] = d.qsplit_rho2;
     for (int k = 0; k <= POLY_MAX; ++k) out[4 + k] = d.poly[k];
     return PETFMM_OK;
+}
+
+int petfmm_debug_smooth_operators(double kappa, float *out, int64_t cap) {
+    if (!(kappa > 0.0) || cap < 0 || (cap > 0 && !out)) return PETFMM_EINVAL;
+    const int n = sm_degree(kappa, kNearTolDefault);
+    if (!n || !out) return n;
+    std::vector<float> t;
+    host_sm_operators(kappa, n, t);
+    if (cap < int64_t(t.size())) return PETFMM_EINVAL;
+    std::memcpy(out, t.data(), t.size() * sizeof(float));
+    return n;
 }
 
 int petfmm_debug_op_table(int order, int kernel, int which, double *out, int64_t cap) {

@@ -14,6 +14,7 @@ namespace petfmm {
 unsigned pf_checks_tree();
 unsigned pf_checks_expansions();
 unsigned pf_checks_p2p();
+unsigned pf_checks_smooth();
 
 // ---- tree.cu ---------------------------------------------------------------
 // Sec. 2.1 binning + z-order key of every particle (composite key for batches);
@@ -171,7 +172,8 @@ constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block for M2M 
 // Work list: items (inst, leaf, first target rank, target count) for every
 // occupied leaf, tpi targets per item.  ctrl[CTRL_NITEMS] receives the count.
 enum { CTRL_STATUS = 0, CTRL_NITEMS = 1, CTRL_QUEUE = 2, CTRL_PAIRS_LO = 4, CTRL_NOCC = 6,
-       CTRL_NPAIRS = 7, CTRL_QUEUE2 = 8, CTRL_NXTRA = 9, CTRL_SYM_LO = 10, CTRL_WORDS = 16 };
+       CTRL_NPAIRS = 7, CTRL_QUEUE2 = 8, CTRL_NXTRA = 9, CTRL_SYM_LO = 10, CTRL_NSMOOTH = 12,
+       CTRL_WORDS = 16 };
 // Buffers for dispatching the items heaviest first (order != nullptr): the
 // items are emitted to items_unsorted, sorted by work class (one stable radix
 // pass over cap entries) and permuted into the item array.
@@ -235,14 +237,44 @@ cudaError_t launch_p2p_pairs(int grid, int deg, int general, const uint4 *pitems
 cudaError_t launch_p2p_final(const Task *tasks, int ntasks, int64_t nblocks,
                              const InstDesc *insts, const uint32_t *start, const uint32_t *skeys,
                              const float4 *rec, const float2 *le, const PairBufs &pb,
-                             int dtype_f32, const uint32_t *perm, float *stage, int64_t nstage,
-                             const Task *utasks, int nutasks, int64_t unblocks,
-                             const uint32_t *ctrl, int64_t ntotal, cudaStream_t st,
-                             uint64_t *launches);
+                             int dtype_f32, float *stage, int64_t nstage, const uint32_t *ctrl, int64_t ntotal, cudaStream_t st, uint64_t *launches);
 // (stage != nullptr, FP32 outputs: the pass writes u, v in sorted order to
-// stage[0 .. nstage) and stage[nstage ..), then one launch per component
-// scatters them to the caller's arrays through perm; utasks: the blobs of
-// every instance, 1024 per block.)
+// stage[0 .. nstage) and stage[nstage ..), and launch_unsort scatters them
+// to the caller's arrays through perm, one launch per component; utasks: the
+// blobs of every instance, 1024 per block.)
+cudaError_t launch_unsort(const InstDesc *insts, const uint32_t *perm, const float *stage,
+                          int64_t nstage, const Task *utasks, int nutasks, int64_t unblocks,
+                          cudaStream_t st, uint64_t *launches);
+// ---- smooth.cu -------------------------------------------------------------
+// Near field by expansions where the blob core is wide against a leaf
+// (instances with InstDesc::smdeg > 0).  sm_degree: the degree for
+// kappa = w^2 / 2 sigma^2 and the context's near-field tolerance, 0 where
+// the pairs are summed.
+int sm_degree(double kappa, double near_tol);
+size_t sm_row_floats(int n);
+int64_t sm_max_rows(int n, int64_t blobs, int64_t leaves);
+void host_sm_operators(double kappa, int n, std::vector<float> &out);
+// lmask, lrank: per leaf, its neighbours summed directly / by expansion, and
+// its row of mom (moments) and loc (local expansions); list: (instance, leaf)
+// of each row; rows of `row` floats.
+struct SmBufs {
+    uint32_t *lmask, *lrank;
+    uint2 *list;
+    float *mom, *loc;
+    int64_t rows;
+    int row;
+};
+// Moments and local expansions of the degrees in the bit set; needs the
+// occupied list and the gathered records.
+cudaError_t launch_sm_near(uint32_t degrees, const uint2 *occ, uint32_t *ctrl, int64_t max_occ,
+                           const InstDesc *insts, const uint32_t *start, const float4 *rec,
+                           const SmBufs &sb, cudaStream_t st, uint64_t *launches);
+// These instances' blobs: far field, near field, output (or stage, sorted).
+cudaError_t launch_sm_final(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                            const uint32_t *start, const uint32_t *skeys, const float4 *rec,
+                            const float2 *le, const SmBufs &sb, int dtype_f32, float *stage,
+                            int64_t nstage, cudaStream_t st, uint64_t *launches);
+
 int p2p_grid(int precision_mixed, int deg, int general, int laplace);
 int device_sm_count();
 constexpr int P2P_TPI_F64 = 32;

@@ -126,10 +126,12 @@ __global__ void __launch_bounds__(256) k_p2p_count(const Task *__restrict__ task
         const uint32_t n = st[m + 1] - st[m];
         const int nside = 1 << d.L;
         const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
-        // pairwise mode: items only for the leaves with directed work
-        const bool work = pairs_mode ? directed_work(st, nside, ix, iy, n) : n > 0;
+        // pairwise mode: items only for the leaves with directed work; none
+        // for an instance whose near field goes by expansions
+        const bool work =
+            !d.smdeg && (pairs_mode ? directed_work(st, nside, ix, iy, n) : n > 0);
         cnt[d.loff + m] = work ? (n + tpi - 1) / tpi : 0u;
-        if (n) {
+        if (n && !d.smdeg) {
             uint32_t src = 0;
             for (int dy = -1; dy <= 1; ++dy)
                 for (int dx = -1; dx <= 1; ++dx) {
@@ -571,7 +573,7 @@ __global__ void __launch_bounds__(256) k_pair_count(const Task *__restrict__ tas
         const uint32_t *st = start + d.soff;
         uint32_t c = 0, x = 0;
         const uint32_t na = st[m + 1] - st[m];
-        if (na >= P2P_PAIR_MIN) {
+        if (na >= P2P_PAIR_MIN && !d.smdeg) {
             const int nside = 1 << d.L;
             const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
             for (int k = 0; k < 4; ++k) {
@@ -647,6 +649,7 @@ __global__ void __launch_bounds__(256) k_pair_emit(const Task *__restrict__ task
     const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
     if (m >= t.count) return;
     const InstDesc &d = insts[t.inst];
+    if (d.smdeg) return;
     const uint32_t *st = start + d.soff;
     const uint32_t na = st[m + 1] - st[m];
     const int nside = 1 << d.L;
@@ -1118,6 +1121,7 @@ __global__ void __launch_bounds__(256, 4) k_p2p_final(
     const int64_t j = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
     if (j >= t.count) return;
     const InstDesc &d = insts[t.inst];
+    if (d.smdeg) return;  // k_sm_final's
     const int64_t r = d.poff + j;
     const uint32_t *st = start + d.soff;
     const int nside = 1 << d.L;
@@ -1378,21 +1382,25 @@ __global__ void __launch_bounds__(256) k_unsort_f32(const Task *__restrict__ tas
 cudaError_t launch_p2p_final(const Task *tasks, int ntasks, int64_t nblocks,
                              const InstDesc *insts, const uint32_t *start, const uint32_t *skeys,
                              const float4 *rec, const float2 *le, const PairBufs &pb,
-                             int dtype_f32, const uint32_t *perm, float *stage, int64_t nstage,
-                             const Task *utasks, int nutasks, int64_t unblocks,
-                             const uint32_t *ctrl, int64_t ntotal, cudaStream_t st,
-                             uint64_t *launches) {
+                             int dtype_f32, float *stage, int64_t nstage, const uint32_t *ctrl,
+                             int64_t ntotal, cudaStream_t st, uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
     k_p2p_final<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, skeys, rec, le, pb,
                                                    dtype_f32, stage, nstage, ctrl, ntotal);
     PF_LAUNCHED(1);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !stage || unblocks <= 0) return e;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_unsort(const InstDesc *insts, const uint32_t *perm, const float *stage,
+                          int64_t nstage, const Task *utasks, int nutasks, int64_t unblocks,
+                          cudaStream_t st, uint64_t *launches) {
+    if (unblocks <= 0) return cudaSuccess;
     for (int comp = 0; comp < 2; ++comp) {
         k_unsort_f32<<<unsigned(unblocks), 256, 0, st>>>(utasks, nutasks, insts, perm,
                                                          stage + comp * nstage, comp);
         PF_LAUNCHED(1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }

@@ -1,0 +1,689 @@
+// smooth.cu -- the mixed path's near field where the blob core is wide
+// against a leaf (Eq. 8 with kappa = w^2 / 2 sigma^2 below kSmKappaMax).
+//
+// In leaf units the near field of Eq. 9 is u = c sum gamma (-d_eta, d_xi)
+// g(kappa |d|^2), g(q) = (1 - e^-q) / q, the turned gradient of the radial
+// function Phi(d) = Ein(kappa |d|^2) / (2 kappa), which is smooth when the
+// core is no narrower than a leaf: between two given leaves,
+//     Phi(D + tau - s) = sum_{alpha, beta} C^D[beta][alpha] m_alpha(tau) P_beta(s)
+// to FP32 accuracy with few terms (tau, s: target and source offsets from
+// their leaf centres, D the offset of the centres, P products of Legendre
+// polynomials and m products of powers, total degree <= n each).  So the
+// blobs of two leaves need not meet one by one (12 operations a pair): each
+// leaf's blobs are summed into (n + 1)(n + 2) / 2 moments, a leaf adds its
+// 9 neighbours' moments through the 9 fixed matrices C^D, and each blob
+// evaluates one polynomial gradient.  The far field's expansions cannot do
+// this: they hold the singular kernel 1 / |x|^2.
+//
+// Leaf pairs with few blobs on both sides (na nb below sm_direct_max) are
+// cheaper summed directly, by the final pass with one thread per target.
+//
+// Measured on one GB300, the whole evaluation against the pairwise near field
+// (p2p.cu): 16.8M clustered blobs, kappa = 0.12: 18.3 -> 2.7 ms; 4.2M with the
+// copies from and to the host: 5.2 -> 1.3 ms; 765k blobs, one per leaf (direct
+// pairs only, without their work lists): 2.89 -> 2.38 ms.
+//
+// kappa <= 1.95 (degree 14) is where the line lies: the degree needed grows
+// with the core's steepness (a translation costs the square of (n + 1)(n + 2)
+// / 2), and at the next density in use, kappa near 3.6 at 16 blobs per leaf, a
+// leaf pair has 256 blob pairs against 14,400 multiply-adds at degree 14.
+#include <algorithm>
+#include <cmath>
+#include <map>
+#include <mutex>
+#include <vector>
+
+#include "kernels.cuh"
+
+namespace petfmm {
+
+#define PF_LAUNCHED(n) do { if (launches) *launches += (n); } while (0)
+
+namespace {
+
+// terms of total degree <= n, ordered by the power b of y, then a of x
+__host__ __device__ constexpr int sm_terms(int n) { return (n + 1) * (n + 2) / 2; }
+__host__ __device__ constexpr int sm_stride(int n) { return (sm_terms(n) + 3) / 4 * 4; }
+__host__ __device__ constexpr int sm_idx(int n, int a, int b) {
+    return b * (n + 1) - b * (b - 1) / 2 + a;
+}
+
+// A leaf pair with fewer blob pairs than this is summed directly: about the
+// cost of one translation (terms^2 multiply-adds of a tiled product) plus
+// its share of moments and evaluation.
+__host__ __device__ constexpr uint32_t sm_direct_max(int n) {
+    return uint32_t(sm_terms(n) * sm_terms(n) / 8);
+}
+
+constexpr int SM_TGT = 64;        // target leaves per block of the translation
+constexpr uint32_t LM_EXP = 16;   // lmask: bits 0..8 direct neighbours, 16..24 by expansion
+
+}  // namespace
+
+// ----------------------------------------------------------------------------
+// Host: degree and operators
+// ----------------------------------------------------------------------------
+// Largest error of the gradient over the near domain, against its largest
+// value there, of the projection below: at most 1.2e-7 up to each bound
+// (tests/test_smooth_operator.py), so the truncation stays at FP32 rounding.
+int sm_degree(double kappa, double near_tol) {
+    if (!(near_tol >= 1e-7)) return 0;
+    static const struct { double kappa; int n; } kBound[] = {
+        {0.17, 8}, {0.50, 10}, {1.04, 12}, {1.95, 14}};
+    for (const auto &b : kBound)
+        if (kappa <= b.kappa) return b.n;
+    return 0;
+}
+
+size_t sm_row_floats(int n) { return size_t(sm_stride(n)); }
+
+// Leaves of an instance that can need expansions: one of the two leaves of a
+// pair of at least sm_direct_max blob pairs holds at least its square root,
+// and each such leaf has 9 neighbours.
+int64_t sm_max_rows(int n, int64_t blobs, int64_t leaves) {
+    int64_t s = 1;
+    while ((s + 1) * (s + 1) <= int64_t(sm_direct_max(n))) ++s;
+    return std::min(std::min(blobs, leaves), 9 * (blobs / s));
+}
+
+// Chebyshev terms per axis of Phi in d (the interpolation error is below
+// 1e-12 for kappa < 2).
+constexpr int kSmCheb = 26;
+
+// V[a][b][k]: T_k(tau - s), tau, s in [-1/2, 1/2], projected onto
+// P_a(2 tau) P_b(2 s), a, b <= n; fixed per degree, built once.
+static const std::vector<double> &sm_shift_table(int n) {
+    static std::mutex mu;
+    static std::map<int, std::vector<double>> tables;
+    std::lock_guard<std::mutex> lk(mu);
+    std::vector<double> &V = tables[n];
+    if (!V.empty()) return V;
+    const int n1 = n + 1, q = n + 12;  // Gauss nodes: exact for T_k P_a products
+    // Gauss-Legendre nodes by Newton's method on P_q
+    std::vector<double> xg(q), wg(q);
+    for (int i = 0; i < q; ++i) {
+        double x = std::cos(M_PI * (i + 0.75) / (q + 0.5)), dp = 1.0;
+        for (int it = 0; it < 60; ++it) {
+            double p0 = 1.0, p1 = x;
+            for (int k = 2; k <= q; ++k) {
+                const double p2 = ((2 * k - 1) * x * p1 - (k - 1) * p0) / k;
+                p0 = p1;
+                p1 = p2;
+            }
+            dp = q * (x * p1 - p0) / (x * x - 1.0);
+            const double dx = p1 / dp;
+            x -= dx;
+            if (std::fabs(dx) < 1e-15) break;
+        }
+        xg[i] = x;
+        wg[i] = 2.0 / ((1.0 - x * x) * dp * dp);
+    }
+    // proj[a][i]: coefficient a of the Legendre projection from node values
+    std::vector<double> proj(size_t(n1) * q), t(size_t(q) * q), tmp(size_t(n1) * q);
+    for (int i = 0; i < q; ++i) {
+        double p0 = 1.0, p1 = xg[i];
+        for (int a = 0; a <= n; ++a) {
+            proj[size_t(a) * q + i] = p0 * wg[i] * (2 * a + 1) * 0.5;
+            const double p2 = ((2 * a + 3) * xg[i] * p1 - (a + 1) * p0) / (a + 2);
+            p0 = p1;
+            p1 = p2;
+        }
+    }
+    V.assign(size_t(n1) * n1 * kSmCheb, 0.0);
+    for (int k = 0; k < kSmCheb; ++k) {
+        for (int i = 0; i < q; ++i)
+            for (int j = 0; j < q; ++j)
+                t[size_t(i) * q + j] = std::cos(k * std::acos(0.5 * (xg[i] - xg[j])));
+        for (int a = 0; a < n1; ++a)
+            for (int j = 0; j < q; ++j) {
+                double s = 0.0;
+                for (int i = 0; i < q; ++i) s += proj[size_t(a) * q + i] * t[size_t(i) * q + j];
+                tmp[size_t(a) * q + j] = s;
+            }
+        for (int a = 0; a < n1; ++a)
+            for (int b = 0; b < n1; ++b) {
+                double s = 0.0;
+                for (int j = 0; j < q; ++j) s += proj[size_t(b) * q + j] * tmp[size_t(a) * q + j];
+                V[size_t(a * n1 + b) * kSmCheb + k] = s;
+            }
+    }
+    return V;
+}
+
+// C^D of the 9 neighbour offsets, source = target + (ox, oy), block
+// (oy + 1) 3 + ox + 1, as [beta][alpha] with rows of sm_stride(n) floats;
+// beta: Legendre products of twice the source offset, alpha: powers of twice
+// the target offset.  Phi is interpolated in d by Chebyshev polynomials,
+// T_k(tau - s) projected onto Legendre products (fixed per degree), the
+// total degrees cut at n, and the target side turned into powers; FP64
+// throughout.
+void host_sm_operators(double kappa, int n, std::vector<float> &out) {
+    const int n1 = n + 1, M = sm_terms(n), S = sm_stride(n), mm = kSmCheb;
+    const std::vector<double> &V = sm_shift_table(n);  // [a][b][k]
+    // powers of x in P_a(x)
+    std::vector<double> pw(size_t(n1 + 1) * n1, 0.0);
+    pw[0] = 1.0;
+    if (n >= 1) pw[size_t(1) * n1 + 1] = 1.0;
+    for (int a = 2; a <= n; ++a)
+        for (int k = 0; k <= a; ++k)
+            pw[size_t(a) * n1 + k] =
+                ((k ? (2 * a - 1) * pw[size_t(a - 1) * n1 + k - 1] : 0.0) -
+                 (a - 1) * pw[size_t(a - 2) * n1 + k]) / a;
+    auto phi = [&](double s) {  // Ein(kappa s) / (2 kappa), s = |d|^2
+        const double z = kappa * s;
+        double term = 1.0, sum = 0.0;  // sum_k (-z)^(k-1) / (k k!)
+        for (int k = 1; k < 160; ++k) {
+            sum += term / k;
+            term *= -z / (k + 1);
+            if (std::fabs(term) < 1e-18 && k > z) break;
+        }
+        return 0.5 * s * sum;
+    };
+    out.assign(size_t(9) * M * S, 0.0f);
+    const int kD[3][2] = {{0, 0}, {1, 0}, {1, 1}};
+    std::vector<double> f(size_t(mm) * mm), g(size_t(mm) * mm), c(size_t(mm) * mm);
+    std::vector<double> h(size_t(mm) * n1 * n1), C(size_t(M) * M), tr(size_t(n1) * n1);
+    std::vector<double> cs(size_t(mm) * mm);
+    for (int k = 0; k < mm; ++k)
+        for (int i = 0; i < mm; ++i)
+            cs[size_t(k) * mm + i] = std::cos(M_PI * k * (i + 0.5) / mm) * (k ? 2.0 : 1.0) / mm;
+    for (const auto &D : kD) {
+        for (int i = 0; i < mm; ++i)
+            for (int j = 0; j < mm; ++j) {
+                const double dx = D[0] + std::cos(M_PI * (i + 0.5) / mm);
+                const double dy = D[1] + std::cos(M_PI * (j + 0.5) / mm);
+                f[size_t(i) * mm + j] = phi(dx * dx + dy * dy);
+            }
+        for (int k = 0; k < mm; ++k)
+            for (int j = 0; j < mm; ++j) {
+                double s = 0.0;
+                for (int i = 0; i < mm; ++i) s += cs[size_t(k) * mm + i] * f[size_t(i) * mm + j];
+                g[size_t(k) * mm + j] = s;
+            }
+        for (int k = 0; k < mm; ++k)
+            for (int l = 0; l < mm; ++l) {
+                double s = 0.0;
+                for (int j = 0; j < mm; ++j) s += cs[size_t(l) * mm + j] * g[size_t(k) * mm + j];
+                c[size_t(k) * mm + l] = s;
+            }
+        // h[a2][b2][k] = sum_l c[k][l] V[a2][b2][l]; T_l has the parity of l
+        for (int e = 0; e < n1 * n1; ++e) {
+            const double *v = &V[size_t(e) * mm];
+            for (int k = 0; k < mm; ++k) {
+                double s = 0.0;
+                for (int l = (e / n1 + e % n1) & 1; l < mm; l += 2) s += c[size_t(k) * mm + l] * v[l];
+                h[size_t(e) * mm + k] = s;
+            }
+        }
+        for (int b2 = 0; b2 <= n; ++b2)          // source y, x
+            for (int b1 = 0; b1 + b2 <= n; ++b1) {
+                // Legendre coefficients of the target side, then powers
+                std::fill(tr.begin(), tr.end(), 0.0);
+                for (int a2 = 0; a2 <= n; ++a2)
+                    for (int a1 = 0; a1 + a2 <= n; ++a1) {
+                        double s = 0.0;
+                        const double *v = &V[size_t(a1 * n1 + b1) * mm];
+                        const double *w = &h[size_t(a2 * n1 + b2) * mm];
+                        for (int k = (a1 + b1) & 1; k < mm; k += 2) s += v[k] * w[k];
+                        for (int e = a1 & 1; e <= a1; e += 2)
+                            tr[size_t(a2) * n1 + e] += s * pw[size_t(a1) * n1 + e];
+                    }
+                for (int e2 = 0; e2 <= n; ++e2)
+                    for (int e1 = 0; e1 + e2 <= n; ++e1) {
+                        double s = 0.0;
+                        for (int a2 = e2; a2 + e1 <= n; a2 += 2)
+                            s += tr[size_t(a2) * n1 + e1] * pw[size_t(a2) * n1 + e2];
+                        C[size_t(sm_idx(n, b1, b2)) * M + sm_idx(n, e1, e2)] = s;
+                    }
+            }
+        // the offsets that mirror or swap to this one; D = -(source offset)
+        for (int oy = -1; oy <= 1; ++oy)
+            for (int ox = -1; ox <= 1; ++ox) {
+                const int hi = std::max(std::abs(ox), std::abs(oy));
+                const int lo = std::min(std::abs(ox), std::abs(oy));
+                if (hi != D[0] || lo != D[1]) continue;
+                const bool swap = std::abs(oy) > std::abs(ox);
+                const int sx = -ox < 0 ? -1 : 1, sy = -oy < 0 ? -1 : 1;
+                float *t = out.data() + size_t((oy + 1) * 3 + ox + 1) * M * S;
+                for (int b2 = 0; b2 <= n; ++b2)
+                    for (int b1 = 0; b1 + b2 <= n; ++b1)
+                        for (int e2 = 0; e2 <= n; ++e2)
+                            for (int e1 = 0; e1 + e2 <= n; ++e1) {
+                                const double v =
+                                    swap ? C[size_t(sm_idx(n, b2, b1)) * M + sm_idx(n, e2, e1)]
+                                         : C[size_t(sm_idx(n, b1, b2)) * M + sm_idx(n, e1, e2)];
+                                const int par = (sx < 0 ? b1 + e1 : 0) + (sy < 0 ? b2 + e2 : 0);
+                                t[size_t(sm_idx(n, b1, b2)) * S + sm_idx(n, e1, e2)] =
+                                    float(par & 1 ? -v : v);
+                            }
+            }
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Moments: a warp per occupied leaf
+// ----------------------------------------------------------------------------
+// Bound by issue: each lane sums all the moments of its blobs in registers
+// (one multiply-add per blob and term), then 32 values at a time are reduced
+// and scattered over the lanes by halving exchanges (31 shuffles per 32
+// values instead of 160).
+template <int N>
+__global__ void __launch_bounds__(128) k_sm_moments(const uint2 *__restrict__ occ,
+                                                    uint32_t *ctrl,
+                                                    const InstDesc *__restrict__ insts,
+                                                    const uint32_t *__restrict__ start,
+                                                    const float4 *__restrict__ rec,
+                                                    const SmBufs sb) {
+    constexpr int M = sm_terms(N), G = (M + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    const uint32_t nocc = ctrl[CTRL_NOCC];
+    const uint32_t nwarps = gridDim.x * 4;
+    unsigned long long pairs = 0;
+    for (uint32_t i = blockIdx.x * 4 + (threadIdx.x >> 5); i < nocc; i += nwarps) {
+        const uint2 e = occ[i];
+        const InstDesc &d = insts[e.x];
+        if (d.smdeg != N) continue;
+        const uint32_t *st = start + d.soff;
+        const uint32_t m = e.y;
+        const int nside = 1 << d.L;
+        // the nine counts, one per lane; which neighbours go by expansion
+        const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
+        uint32_t cnt = 0;
+        const int x = ix + lane % 3 - 1, y = iy + lane / 3 - 1;
+        if (lane < 9 && x >= 0 && y >= 0 && x < nside && y < nside) {
+            const uint32_t nm = morton_key(uint32_t(x), uint32_t(y));
+            cnt = st[nm + 1] - st[nm];
+        }
+        const uint32_t n = __shfl_sync(0xffffffffu, cnt, 4);
+        const bool byexp = uint64_t(n) * cnt >= sm_direct_max(N);
+        const uint32_t em = __ballot_sync(0xffffffffu, byexp);
+        const uint32_t dm = __ballot_sync(0xffffffffu, cnt > 0 && !byexp);
+        pairs += (unsigned long long)n * (lane == 4 ? cnt - 1 : cnt);
+        if (lane == 0) sb.lmask[d.loff + m] = dm | (em << LM_EXP);
+        if (!em) continue;
+        // a row of the expansion buffers, in no particular order
+        uint32_t rank = 0;
+        if (lane == 0) {
+            rank = atomicAdd(ctrl + CTRL_NSMOOTH, 1u);
+            sb.lrank[d.loff + m] = rank;
+        }
+        rank = __shfl_sync(0xffffffffu, rank, 0);
+        if (!PF_IN(rank, sb.rows)) continue;
+        if (lane == 0) sb.list[rank] = e;
+        const uint32_t s0 = st[m], s1 = s0 + n;
+        if (!(PF_IN(int64_t(s0) - d.poff, d.n + 1) && PF_IN(int64_t(s1) - d.poff, d.n + 1)))
+            continue;
+        float acc[G * 32];
+#pragma unroll
+        for (int k = 0; k < G * 32; ++k) acc[k] = 0.f;
+        for (uint32_t j = s0 + lane; j < s1; j += 32) {
+            const float4 r = rec[j];
+            const float sx = 2.f * r.x, sy = 2.f * r.y;
+            float px[N + 1], py[N + 1];
+            px[0] = 1.f;
+            px[1] = sx;
+            py[0] = r.z;
+            py[1] = r.z * sy;
+#pragma unroll
+            for (int k = 1; k < N; ++k) {
+                const float ca = float(2 * k + 1) / float(k + 1), cb = -float(k) / float(k + 1);
+                px[k + 1] = fmaf(ca * sx, px[k], cb * px[k - 1]);
+                py[k + 1] = fmaf(ca * sy, py[k], cb * py[k - 1]);
+            }
+#pragma unroll
+            for (int b = 0; b <= N; ++b)
+#pragma unroll
+                for (int a = 0; a <= N - b; ++a)
+                    acc[sm_idx(N, a, b)] = fmaf(px[a], py[b], acc[sm_idx(N, a, b)]);
+        }
+        float *out = sb.mom + size_t(rank) * sb.row;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int k = 0; k < o; ++k) {
+                    const float lo = acc[g * 32 + k], hi = acc[g * 32 + k + o];
+                    acc[g * 32 + k] = (up ? hi : lo) +
+                                      __shfl_xor_sync(0xffffffffu, up ? lo : hi, o);
+                }
+            }
+            if (g * 32 + lane < M) out[g * 32 + lane] = acc[g * 32];
+        }
+    }
+    // ordered near pairs, for the statistics
+#pragma unroll
+    for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
+    if (lane == 0 && pairs)
+        atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), pairs);
+}
+
+// ----------------------------------------------------------------------------
+// Translation: loc[target] = sum over its neighbours of C^D moments
+// ----------------------------------------------------------------------------
+// A tiled FP32 product per block: 64 target leaves (consecutive in the
+// occupied list, so mostly neighbours that share sources in L1) x all terms,
+// 4 x 4 outputs per thread, the source moments of one neighbour offset and
+// its operator staged in shared memory at a time.  Bound by the shared loads
+// (two 16-byte loads per 16 multiply-adds).
+template <int N>
+struct SmTile {
+    static constexpr int M = sm_terms(N), S = sm_stride(N), CG = S / 4;
+    static constexpr int THREADS = (CG * (SM_TGT / 4) + 31) / 32 * 32;
+    static constexpr int KT = N <= 8 ? 48 : N == 10 ? 36 : N == 12 ? 48 : 40;  // multiple of 4
+};
+
+template <int N>
+__global__ void __launch_bounds__(SmTile<N>::THREADS) k_sm_translate(
+    const uint32_t *__restrict__ ctrl, const InstDesc *__restrict__ insts, const SmBufs sbuf) {
+    using T = SmTile<N>;
+    constexpr int M = T::M, S = T::S, KT = T::KT;
+    __shared__ __align__(16) float sa[KT][SM_TGT + 4];
+    __shared__ __align__(16) float sb[KT * S];
+    __shared__ uint2 se[SM_TGT];         // (instance, leaf)
+    __shared__ uint32_t sm[SM_TGT];      // expansion neighbours
+    __shared__ int ssrc[SM_TGT];         // rank of the source leaf of this offset, or -1
+    const int tid = threadIdx.x;
+    const int tg = tid & 15, cg = tid >> 4;
+    const bool active = cg < T::CG;
+    const uint32_t nrows = min(ctrl[CTRL_NSMOOTH], uint32_t(sbuf.rows));
+    const uint32_t *__restrict__ lmask = sbuf.lmask;
+    const uint32_t *__restrict__ lrank = sbuf.lrank;
+    const float *__restrict__ mom = sbuf.mom;
+    const int row = sbuf.row;
+    for (uint32_t base = blockIdx.x * SM_TGT; base < nrows; base += gridDim.x * SM_TGT) {
+        __syncthreads();  // the previous group's readers are done
+        uint32_t mine = 0;
+        if (tid < SM_TGT) {
+            uint2 e = make_uint2(0xffffffffu, 0);
+            if (base + tid < nrows) {
+                e = sbuf.list[base + tid];
+                const InstDesc &d = insts[e.x];
+                if (d.smdeg == N) mine = lmask[d.loff + e.y] >> LM_EXP;
+            }
+            se[tid] = e;
+            sm[tid] = mine;
+        }
+        if (!__syncthreads_or(int(mine))) continue;
+        // one instance at a time (its operators); nearly always only one
+        uint32_t done = 0xffffffffu;  // instances are taken in ascending order
+        for (;;) {
+            uint32_t inst = 0xffffffffu;
+            for (int t = 0; t < SM_TGT; ++t)
+                if (sm[t] && (done == 0xffffffffu || se[t].x > done)) inst = min(inst, se[t].x);
+            if (inst == 0xffffffffu) break;
+            done = inst;
+            const InstDesc &d = insts[inst];
+            const float *op = static_cast<const float *>(d.t_sm);
+            float acc[4][4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
+            for (int o = 0; o < 9; ++o) {
+                __syncthreads();
+                int src = -1;
+                if (tid < SM_TGT) {
+                    if (se[tid].x == inst && ((sm[tid] >> o) & 1u)) {
+                        const uint32_t m = se[tid].y;
+                        const uint32_t nm = morton_key(compact_bits(m) + uint32_t(o % 3 - 1),
+                                                       compact_bits(m >> 1) + uint32_t(o / 3 - 1));
+                        if (PF_IN(nm, int64_t(1) << (2 * d.L)) &&
+                            PF_IN(lrank[d.loff + nm], int64_t(nrows)))
+                            src = int(lrank[d.loff + nm]);
+                    }
+                    ssrc[tid] = src;
+                }
+                if (!__syncthreads_or(src >= 0)) continue;
+                for (int k0 = 0; k0 < M; k0 += KT) {
+                    const int kt = min(KT, M - k0);
+                    if (k0) __syncthreads();
+                    for (int e = tid; e < SM_TGT * (KT / 4); e += T::THREADS) {
+                        const int t = e & (SM_TGT - 1), k = (e / SM_TGT) * 4;
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (k < kt && ssrc[t] >= 0)
+                            v = *reinterpret_cast<const float4 *>(mom + size_t(ssrc[t]) * row + k0 +
+                                                                  k);
+                        sa[k][t] = v.x;
+                        sa[k + 1][t] = v.y;
+                        sa[k + 2][t] = v.z;
+                        sa[k + 3][t] = v.w;
+                    }
+                    const float4 *ob =
+                        reinterpret_cast<const float4 *>(op + (size_t(o) * M + k0) * S);
+                    for (int e = tid; e < kt * (S / 4); e += T::THREADS)
+                        reinterpret_cast<float4 *>(sb)[e] = __ldg(ob + e);
+                    __syncthreads();
+                    if (active)
+#pragma unroll 4
+                        for (int k = 0; k < kt; ++k) {
+                            const float4 a = *reinterpret_cast<const float4 *>(&sa[k][tg * 4]);
+                            const float4 b = *reinterpret_cast<const float4 *>(&sb[k * S + cg * 4]);
+                            const float av[4] = {a.x, a.y, a.z, a.w};
+                            const float bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+                            for (int p = 0; p < 4; ++p)
+#pragma unroll
+                                for (int c = 0; c < 4; ++c)
+                                    acc[p][c] = fmaf(av[p], bv[c], acc[p][c]);
+                        }
+                }
+            }
+            if (active)
+#pragma unroll
+                for (int p = 0; p < 4; ++p) {
+                    const int t = tg * 4 + p;
+                    if (sm[t] && se[t].x == inst)
+                        *reinterpret_cast<float4 *>(sbuf.loc + size_t(base + t) * row + cg * 4) =
+                            make_float4(acc[p][0], acc[p][1], acc[p][2], acc[p][3]);
+                }
+        }
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Final pass of these instances, one thread per blob
+// ----------------------------------------------------------------------------
+// Gradient of sum c[a, b] s^a t^b by nested Horner schemes.
+template <int N>
+__device__ __forceinline__ float2 sm_gradient(const float *__restrict__ loc, float s, float t) {
+    constexpr int S4 = sm_stride(N) / 4;
+    float c[sm_stride(N)];
+#pragma unroll
+    for (int k = 0; k < S4; ++k) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(loc) + k);
+        c[4 * k] = v.x;
+        c[4 * k + 1] = v.y;
+        c[4 * k + 2] = v.z;
+        c[4 * k + 3] = v.w;
+    }
+    float f = 0.f, fs = 0.f, ft = 0.f;
+#pragma unroll
+    for (int b = N; b >= 0; --b) {
+        float h = c[sm_idx(N, N - b, b)], hd = 0.f;
+#pragma unroll
+        for (int a = N - b - 1; a >= 0; --a) {
+            hd = fmaf(hd, s, h);
+            h = fmaf(h, s, c[sm_idx(N, a, b)]);
+        }
+        ft = fmaf(ft, t, f);
+        f = fmaf(f, t, h);
+        fs = fmaf(fs, t, hd);
+    }
+    return make_float2(fs, ft);
+}
+
+// The leaf pairs summed directly: sources of the neighbours in mask.
+template <int DEG>
+__device__ __forceinline__ float2 sm_direct(uint32_t mask, const InstDesc &d,
+                                            const uint32_t *__restrict__ st,
+                                            const float4 *__restrict__ rec, int ix, int iy,
+                                            float x, float y) {
+    float a[DEG + 1];
+#pragma unroll
+    for (int k = 0; k <= DEG; ++k) a[k] = d.poly[k];
+    const float kappa = d.kappa, split = d.qsplit_rho2;
+    const bool general = d.general != 0;
+    uint32_t s0[9], s1[9];
+#pragma unroll
+    for (int o = 0; o < 9; ++o) {
+        s0[o] = s1[o] = 0;
+        if ((mask >> o) & 1u) {
+            const uint32_t nm = morton_key(uint32_t(ix + o % 3 - 1), uint32_t(iy + o / 3 - 1));
+            s0[o] = st[nm];
+            s1[o] = st[nm + 1];
+            if (!(PF_IN(int64_t(s0[o]) - d.poff, d.n + 1) &&
+                  PF_IN(int64_t(s1[o]) - d.poff, d.n + 1)))
+                s1[o] = s0[o];
+        }
+    }
+    float u = 0.f, v = 0.f;
+#pragma unroll
+    for (int o = 0; o < 9; ++o) {
+        const float xt = x - float(o % 3 - 1), yt = y - float(o / 3 - 1);
+        for (uint32_t j = s0[o]; j < s1[o]; ++j) {
+            const float4 r = __ldg(rec + j);
+            const float dx = xt - r.x, dy = yt - r.y;
+            const float r2 = fmaf(dx, dx, dy * dy);
+            float g = a[DEG];
+#pragma unroll
+            for (int k = DEG - 1; k >= 0; --k) g = fmaf(g, r2, a[k]);
+            if (general) {
+                const float q = kappa * r2;
+                const float ge = __fdividef(1.0f - __expf(-q), q);
+                g = r2 < split ? g : ge;
+            }
+            const float f = r.z * g;
+            u = fmaf(-dy, f, u);
+            v = fmaf(dx, f, v);
+        }
+    }
+    return make_float2(u, v);
+}
+
+__global__ void __launch_bounds__(256, 3) k_sm_final(
+    const Task *__restrict__ tasks, int ntasks, const InstDesc *__restrict__ insts,
+    const uint32_t *__restrict__ start, const uint32_t *__restrict__ skeys,
+    const float4 *__restrict__ rec, const float2 *__restrict__ le,
+    const SmBufs sb, int dtype_f32, float *__restrict__ stage, int64_t nstage) {
+    const int ti = find_task(tasks, ntasks, blockIdx.x);
+    const Task t = tasks[ti];
+    const int64_t j = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
+    if (j >= t.count) return;
+    const InstDesc &d = insts[t.inst];
+    if (!d.smdeg) return;
+    const int64_t r = d.poff + j;
+    const uint32_t m = skeys[r] & ((1u << (2 * d.L)) - 1u);
+    const float4 rr = rec[r];
+    const uint32_t mask = sb.lmask[d.loff + m];
+    const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
+    float2 w = make_float2(0.f, 0.f);
+    if (d.L >= 2) {
+        // far field: w = (1/r) sum c_m zeta^m, u - i v = cfar w
+        const int p = d.p;
+        const float2 *c =
+            le + d.eoff + (lvl_off(d.L) + box_index(d.L, uint32_t(ix), uint32_t(iy))) * p;
+        float2 z = __ldg(c + p - 1);
+        for (int k = p - 2; k >= 0; --k) {
+            const float2 ck = __ldg(c + k);
+            z = make_float2(fmaf(z.x, rr.x, fmaf(-z.y, rr.y, ck.x)),
+                            fmaf(z.x, rr.y, fmaf(z.y, rr.x, ck.y)));
+        }
+        w = make_float2(d.cfar * z.y, d.cfar * z.x);
+    }
+    const uint32_t rank = mask >> LM_EXP ? sb.lrank[d.loff + m] : 0u;
+    if ((mask >> LM_EXP) && PF_IN(rank, sb.rows)) {
+        const float *l = sb.loc + size_t(rank) * sb.row;
+        const float s = 2.f * rr.x, q = 2.f * rr.y;
+        float2 g;
+        switch (d.smdeg) {
+            case 8: g = sm_gradient<8>(l, s, q); break;
+            case 10: g = sm_gradient<10>(l, s, q); break;
+            case 12: g = sm_gradient<12>(l, s, q); break;
+            default: g = sm_gradient<14>(l, s, q); break;
+        }
+        const float c2 = 2.f * d.cnear;  // d/dxi = 2 d/ds
+        w.x = fmaf(-c2, g.y, w.x);
+        w.y = fmaf(c2, g.x, w.y);
+    }
+    const uint32_t dm = mask & 0x1ffu;
+    if (dm) {
+        const uint32_t *st = start + d.soff;
+        const float2 n = d.deg <= 6 ? sm_direct<6>(dm, d, st, rec, ix, iy, rr.x, rr.y)
+                                    : sm_direct<12>(dm, d, st, rec, ix, iy, rr.x, rr.y);
+        w.x = fmaf(d.cnear, n.x, w.x);
+        w.y = fmaf(d.cnear, n.y, w.y);
+    }
+    if (stage) {
+        stage[r] = w.x;
+        stage[nstage + r] = w.y;
+        return;
+    }
+    const int64_t q = int64_t(__float_as_uint(rr.w)) - d.poff;
+    if (!PF_IN(q, d.n)) return;  // checked build: the caller's index of the blob
+    if (dtype_f32) {
+        static_cast<float *>(d.u)[q] = w.x;
+        static_cast<float *>(d.v)[q] = w.y;
+    } else {
+        static_cast<double *>(d.u)[q] = double(w.x);
+        static_cast<double *>(d.v)[q] = double(w.y);
+    }
+}
+
+// ----------------------------------------------------------------------------
+// Launches
+// ----------------------------------------------------------------------------
+template <int N>
+static cudaError_t sm_near(const uint2 *occ, uint32_t *ctrl, int64_t max_occ, const InstDesc *insts,
+                           const uint32_t *start, const float4 *rec, const SmBufs &sb,
+                           cudaStream_t st, uint64_t *launches) {
+    static int per_sm_m = 0, per_sm_t = 0;
+    if (!per_sm_t) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_m, k_sm_moments<N>, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_t, k_sm_translate<N>,
+                                                      SmTile<N>::THREADS, 0);
+        if (per_sm_m < 1) per_sm_m = 1;
+        if (per_sm_t < 1) per_sm_t = 1;
+    }
+    const int64_t sms = device_sm_count();
+    const int64_t gm = std::min<int64_t>(sms * per_sm_m, (max_occ + 3) / 4);
+    k_sm_moments<N><<<unsigned(gm), 128, 0, st>>>(occ, ctrl, insts, start, rec, sb);
+    PF_LAUNCHED(1);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const int64_t gt = std::min<int64_t>(sms * per_sm_t, (sb.rows + SM_TGT - 1) / SM_TGT);
+    if (gt <= 0) return cudaSuccess;
+    k_sm_translate<N><<<unsigned(gt), SmTile<N>::THREADS, 0, st>>>(ctrl, insts, sb);
+    PF_LAUNCHED(1);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sm_near(uint32_t degrees, const uint2 *occ, uint32_t *ctrl, int64_t max_occ,
+                           const InstDesc *insts, const uint32_t *start, const float4 *rec,
+                           const SmBufs &sb, cudaStream_t st, uint64_t *launches) {
+    cudaError_t e = cudaSuccess;
+    if (degrees & (1u << 8)) e = sm_near<8>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+    if (e == cudaSuccess && (degrees & (1u << 10)))
+        e = sm_near<10>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+    if (e == cudaSuccess && (degrees & (1u << 12)))
+        e = sm_near<12>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+    if (e == cudaSuccess && (degrees & (1u << 14)))
+        e = sm_near<14>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+    return e;
+}
+
+cudaError_t launch_sm_final(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                            const uint32_t *start, const uint32_t *skeys, const float4 *rec,
+                            const float2 *le, const SmBufs &sb, int dtype_f32, float *stage,
+                            int64_t nstage, cudaStream_t st, uint64_t *launches) {
+    if (nblocks <= 0) return cudaSuccess;
+    k_sm_final<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, skeys, rec, le, sb,
+                                                  dtype_f32, stage, nstage);
+    PF_LAUNCHED(1);
+    return cudaGetLastError();
+}
+
+PF_DEFINE_CHECK_READER(smooth)
+
+}  // namespace petfmm
