@@ -527,78 +527,163 @@ __global__ void __launch_bounds__(W3 * 32) k3_m2m(int l, int L, int p, const uin
 }
 
 // ---------------------------------------------------------------------------
-// M2L (level l >= 2): L~_k^l = (-1)^k sum_{n,m} M~_n^m I_{n+k}^{m+l}(delta),
-// delta = target - source in box widths, over the interaction list: the
-// children of the parent's neighbours that are not neighbours of the box,
-// in a fixed order.  A warp per target box; the source's expansion is staged
-// in shared memory for the warp, lanes over output coefficients.  The result
-// is written (the L2L that follows adds the parent's part).
+// M2L of the FP64 path (all levels in one launch).  The coefficients of a
+// real potential with degrees < p are p^2 real numbers (host_m2l_real); in
+// that basis a reflection of an axis is a diagonal of signs, so the operator
+// of delta = (+-a, +-b, +-c) is S T S with the one of (a, b, c) and S the
+// signs of the reflected axes.  The up to eight sources of an orbit are
+// therefore added first, with signs, and translated by one product:
+//   c_r += sum_k T[k][r] H[q(r) ^ q(k)][k],
+//   H[q][k] = sum_s (-1)^popc(q & s) a_s[k]
+// (q: a coefficient's parity along x, y, z; s: the reflected axes), 56 real
+// p^2 x p^2 products for the up to 189 boxes of the interaction list and
+// three butterfly stages for H.  Bound by the FP64 pipe (two lanes a cycle
+// and SM on this part), so the work is laid out to leave no lane idle: a
+// block takes M2L64_ITEMS (target box, coefficient) pairs flat over its
+// threads, four each; operators come through L1, H from shared memory.
+// Measured (one GB300, 262,144 uniform charges, L = 4, p = 8): M2L 76.6 ms with
+// a warp per target box and the complex sums of every source -> 2.45 ms.
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(W3 * 32) k3_m2l(int l, int L, int p, const uint32_t *__restrict__ start,
-                                                  const typename C3<T>::V *__restrict__ itab,
-                                                  const typename C3<T>::V *__restrict__ me,
-                                                  typename C3<T>::V *__restrict__ le) {
-    using V = typename C3<T>::V;
-    __shared__ V sme[W3][NC3_MAX];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t b = int64_t(blockIdx.x) * W3 + wid;
-    if (b >= (int64_t(1) << (3 * l))) return;
-    if (box_count3(start, L, l, uint32_t(b)) == 0) return;
-    const int nc = nc3(p), nci = nci3(p);
-    const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
-              iz = int(compact3(uint32_t(b) >> 2));
-    const int pside = 1 << (l - 1);
-    V acc[OUT3];
-    int on[OUT3], om[OUT3];
-#pragma unroll
-    for (int u = 0; u < OUT3; ++u) {
-        acc[u] = mk<V>(T(0), T(0));
-        const int j = lane + 32 * u;
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= j) ++n;
-        on[u] = n;
-        om[u] = j - n * (n + 1) / 2;
+constexpr int M2L64_THREADS = 256, M2L64_NI = 4, M2L64_ITEMS = M2L64_THREADS * M2L64_NI;
+
+// the largest dynamic shared memory of any order (p = 1: 1,024 targets)
+constexpr size_t M2L64_SMEM_MAX = size_t(8) * (M2L64_ITEMS + 2) * 8 + size_t(8) * M2L64_ITEMS * 4;
+
+__host__ __device__ __forceinline__ int m2l64_rows(int p) { return M2L64_ITEMS / (p * p); }
+// blocks of level l: ceil(8^(l-1) / rows) x 8 child classes
+__host__ __device__ __forceinline__ int64_t m2l64_blocks(int l, int rows) {
+    return ((int64_t(1) << (3 * (l - 1))) + rows - 1) / rows * 8;
+}
+// doubles between the H of two parity classes (two of padding keep the eight
+// classes on different banks)
+__host__ __device__ __forceinline__ int m2l64_stride(int p) { return m2l64_rows(p) * p * p + 2; }
+
+__global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
+    int L, int p, const uint32_t *__restrict__ start, const double *__restrict__ atab,
+    const short2 *__restrict__ rmap, const uint8_t *__restrict__ parity,
+    const double2 *__restrict__ me, double2 *__restrict__ le) {
+    extern __shared__ __align__(16) double m64_h[];
+    int *srow = reinterpret_cast<int *>(m64_h + 8 * m2l64_stride(p));  // source box of
+                                                                       // (target, member), -1: none
+    __shared__ uint8_t sq[P3_MAX * P3_MAX];    // parity class of each real index
+    __shared__ uint16_t soff[P3_MAX * P3_MAX]; // its place in a box's stored doubles
+    const int tid = threadIdx.x, nr = p * p, nc = nc3(p);
+    const int rows = m2l64_rows(p), qs = m2l64_stride(p);
+    int l = 2;
+    int64_t bid = blockIdx.x;
+    while (l < L && bid >= m2l64_blocks(l, rows)) bid -= m2l64_blocks(l++, rows);
+    const int c = int(bid & 7);
+    const int64_t np = int64_t(1) << (3 * (l - 1)), p0 = (bid >> 3) * rows;
+    const int side = 1 << l;
+    bool mine = false;
+    for (int t = tid; t < rows; t += M2L64_THREADS)
+        if (p0 + t < np) mine |= box_count3(start, L, l, uint32_t((p0 + t) * 8 + c)) != 0;
+    if (!__syncthreads_or(mine)) return;  // no target holds particles
+    for (int r = tid; r < nr; r += M2L64_THREADS) {
+        sq[r] = parity[r];
+        const short2 mp = rmap[r];
+        soff[r] = uint16_t(2 * mp.x + (mp.y == 1));
     }
-    const V *lev = me + lvl_off3(l) * nc;
-    for (int qz = (iz >> 1) - 1; qz <= (iz >> 1) + 1; ++qz)
-        for (int qy = (iy >> 1) - 1; qy <= (iy >> 1) + 1; ++qy)
-            for (int qx = (ix >> 1) - 1; qx <= (ix >> 1) + 1; ++qx) {
-                if (qx < 0 || qy < 0 || qz < 0 || qx >= pside || qy >= pside || qz >= pside)
-                    continue;
-                for (int c = 0; c < 8; ++c) {
-                    const int sx = 2 * qx + (c & 1), sy = 2 * qy + ((c >> 1) & 1),
-                              sz = 2 * qz + (c >> 2);
-                    const int dx = ix - sx, dy = iy - sy, dz = iz - sz;
-                    if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1 && dz >= -1 && dz <= 1) continue;
-                    const uint32_t sb = morton3(uint32_t(sx), uint32_t(sy), uint32_t(sz));
-                    if (box_count3(start, L, l, sb) == 0) continue;
-                    __syncwarp();
-                    for (int i = lane; i < nc; i += 32) sme[wid][i] = lev[int64_t(sb) * nc + i];
-                    __syncwarp();
-                    const V *tab = itab + ((dx + 3) + 7 * (dy + 3) + 49 * (dz + 3)) * nci;
+    // this thread's (target, coefficient) pairs
+    int it_r[M2L64_NI], it_t[M2L64_NI], it_q[M2L64_NI];
+    double acc[M2L64_NI];
 #pragma unroll
-                    for (int u = 0; u < OUT3; ++u) {
-                        if (lane + 32 * u >= nc) continue;
-                        const int k = on[u], lo = om[u];
-                        V s = mk<V>(T(0), T(0));
-                        for (int n = 0; n < p; ++n)
-                            for (int m = -n; m <= n; ++m)
-                                cmac(s, coef3(sme[wid], n, m), coef3(tab, n + k, m + lo));
-                        if (k & 1) {
-                            acc[u].x -= s.x;
-                            acc[u].y -= s.y;
-                        } else {
-                            acc[u].x += s.x;
-                            acc[u].y += s.y;
-                        }
-                    }
-                }
+    for (int i = 0; i < M2L64_NI; ++i) {
+        const int e = tid + i * M2L64_THREADS;
+        const bool in = e < rows * nr;
+        it_t[i] = in ? e / nr : 0;
+        it_r[i] = in ? e % nr : 0;
+        it_q[i] = parity[it_r[i]];
+        acc[i] = 0.0;
+    }
+    const double *lev = reinterpret_cast<const double *>(me + lvl_off3(l) * nc);
+    for (int o = 1; o < 64; ++o) {
+        const int a[3] = {o & 3, (o >> 2) & 3, o >> 4};
+        if (a[0] < 2 && a[1] < 2 && a[2] < 2) continue;  // near field
+        // axis d: both signs of the offset, or one (0; 3 reaches out of the
+        // parent's neighbours on one side); delta = target - source
+        bool both[3], neg[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            both[d] = a[d] == 1 || a[d] == 2;
+            neg[d] = a[d] == 3 && !((c >> d) & 1);
+        }
+        __syncthreads();  // the previous orbit's products are done
+        bool have = false;
+        for (int e = tid; e < 8 * rows; e += M2L64_THREADS) {
+            const int s = e & 7, t = e >> 3;
+            int src = -1;
+            bool member = p0 + t < np;
+            int x[3];
+            const uint32_t tb = uint32_t((p0 + t) * 8 + c);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const bool up = (s >> d) & 1;  // reflected
+                member = member && (both[d] || !up);
+                x[d] = int(compact3(tb >> d)) + (up || neg[d] ? a[d] : -a[d]);
+                member = member && x[d] >= 0 && x[d] < side;
             }
-    V *dst = le + (lvl_off3(l) + b) * nc;
+            if (member) {
+                const uint32_t sb = morton3(uint32_t(x[0]), uint32_t(x[1]), uint32_t(x[2]));
+                if (box_count3(start, L, l, sb)) src = int(sb);
+            }
+            srow[e] = src;
+            have |= src >= 0;
+        }
+        if (!__syncthreads_or(have)) continue;
+        for (int e = tid; e < rows * nr; e += M2L64_THREADS) {
+            const int t = e / nr, k = e - t * nr;
+            double v[8];
 #pragma unroll
-    for (int u = 0; u < OUT3; ++u)
-        if (lane + 32 * u < nc) dst[lane + 32 * u] = acc[u];
+            for (int s = 0; s < 8; ++s) {
+                const int sb = srow[8 * t + s];
+                v[s] = sb >= 0 ? lev[int64_t(sb) * (2 * nc) + soff[k]] : 0.0;
+            }
+            // butterflies along the axes with both signs (entries reflected
+            // along another axis are not there yet), then copies
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                if (both[d])
+#pragma unroll
+                    for (int s = 0; s < 8; ++s) {
+                        if ((s >> d) & 1) continue;
+                        bool there = true;
+#pragma unroll
+                        for (int f = 0; f < 3; ++f) there = there && (both[f] || !((s >> f) & 1));
+                        if (!there) continue;
+                        const double x = v[s], y = v[s | (1 << d)];
+                        v[s] = x + y;
+                        v[s | (1 << d)] = x - y;
+                    }
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                if (!both[d])
+#pragma unroll
+                    for (int s = 0; s < 8; ++s)
+                        if (!((s >> d) & 1)) v[s | (1 << d)] = neg[d] ? -v[s] : v[s];
+#pragma unroll
+            for (int s = 0; s < 8; ++s) m64_h[s * qs + e] = v[s];
+        }
+        __syncthreads();
+        const double *at = atab + size_t(o) * nr * nr;
+#pragma unroll 2
+        for (int k = 0; k < nr; ++k) {
+            const int qk = sq[k];
+#pragma unroll
+            for (int i = 0; i < M2L64_NI; ++i)
+                acc[i] = fma(__ldg(at + size_t(k) * nr + it_r[i]),
+                             m64_h[(it_q[i] ^ qk) * qs + it_t[i] * nr + k], acc[i]);
+        }
+    }
+    double *lef = reinterpret_cast<double *>(le + lvl_off3(l) * nc);
+#pragma unroll
+    for (int i = 0; i < M2L64_NI; ++i) {
+        if (tid + i * M2L64_THREADS >= rows * nr || p0 + it_t[i] >= np) continue;
+        const short2 mp = rmap[it_r[i]];
+        double *dst = lef + ((p0 + it_t[i]) * 8 + c) * (2 * nc) + 2 * mp.x;
+        dst[mp.y == 1] = acc[i];
+        if (mp.y == 2) dst[1] = 0.0;  // Im of m = 0
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1827,25 +1912,54 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_mixed(int L, int p, double
     }
 }
 
-// The FP64 path: global coordinates, 1/r by division and sqrt.
+// 1/sqrt(x): the hardware's approximation y and one step of Householder's
+// third-order iteration, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y^2
+// (|e| < 2^-18 leaves |e|^3 below 2^-54): five FP64 operations, where a
+// division by sqrt took about thirty.  Subnormal, infinite and NaN x (the
+// approximation flushes or saturates there) by division.
+__device__ __forceinline__ double rsqrt_f64(double x) {
+    const uint32_t h = uint32_t(__double2hiint(x));
+    if (h - 0x00100000u >= 0x7fe00000u) return 1.0 / sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+// The FP64 path: global coordinates; a warp per work item, its lanes shared
+// out over an item's few targets as in the mixed kernel.  Bound by the FP64
+// pipe (two lanes a cycle and SM): 18 operations a pair.  Measured (one
+// GB300, 262,144 uniform charges, L = 4): 32.9 ms with a division and a square
+// root per pair and a warp per leaf -> 16.6 ms.
 template <typename TOut>
 __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
                                                        const uint32_t *__restrict__ start,
                                                        const Dbl4 *__restrict__ xs,
                                                        const double2 *__restrict__ le,
                                                        const uint32_t *__restrict__ perm,
+                                                       const uint2 *__restrict__ items,
+                                                       const uint32_t *__restrict__ nitems,
                                                        int64_t n, void *phi, void *ex, void *ey,
                                                        void *ez) {
     __shared__ double2 sle[W3][NC3_MAX];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t b = int64_t(blockIdx.x) * W3 + wid;
-    if (b >= (int64_t(1) << (3 * L))) return;
-    const uint32_t s0 = start[b], s1 = start[b + 1];
-    if (s0 == s1) return;
+    const int64_t it = int64_t(blockIdx.x) * W3 + wid;
+    if (it >= int64_t(*nitems)) return;
+    // one item: the targets s0 .. s1 - 1 of leaf b, rep lanes each
+    const uint2 item = items[it];
+    const int64_t b = item.x;
+    if (!PF_IN(b, int64_t(1) << (3 * L))) return;
+    const uint32_t s0 = item.y, s1 = min(start[b + 1], s0 + 32u);
+    const int k = int(s1 - s0);
+    int lg = 0;
+    while (lg < 5 && (k << (lg + 1)) <= 32) ++lg;
+    const uint32_t rep = 1u << lg, c = uint32_t(lane) & (rep - 1u);
+    const uint32_t i = s0 + uint32_t(lane >> lg);
+    const bool live = i < s1;
     const int nc = nc3(p);
     const bool far = L >= 2;
     if (far)
-        for (int i = lane; i < nc; i += 32) sle[wid][i] = le[(lvl_off3(L) + b) * nc + i];
+        for (int t = lane; t < nc; t += 32) sle[wid][t] = le[(lvl_off3(L) + b) * nc + t];
     __syncwarp();
     const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
               iz = int(compact3(uint32_t(b) >> 2));
@@ -1853,40 +1967,44 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
     const double w = d.width / double(side);
     const double cx = d.x0 + (ix + 0.5) * w, cy = d.y0 + (iy + 0.5) * w,
                  cz = d.z0 + (iz + 0.5) * w;
-    for (uint32_t t0 = s0; t0 < s1; t0 += 32) {
-        const uint32_t i = t0 + uint32_t(lane);
-        const bool valid = i < s1;
-        const Dbl4 tg = valid ? xs[i] : Dbl4{cx, cy, cz, 0.0};
-        double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int nx = ix + dx, ny = iy + dy, nz = iz + dz;
-                    if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side)
-                        continue;
-                    const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
-                    const uint32_t a = start[nb], e = start[nb + 1];
-                    for (uint32_t j = a; j < e; ++j) {
-                        const Dbl4 s = xs[j];
-                        const double ddx = tg.x - s.x, ddy = tg.y - s.y, ddz = tg.z - s.z;
-                        const double r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-                        if (r2 == 0.0) continue;
-                        const double ri = 1.0 / sqrt(r2);
-                        const double qr = s.w * ri;
-                        const double qr3 = qr * ri * ri;
-                        f += qr;
-                        gx += qr3 * ddx;
-                        gy += qr3 * ddy;
-                        gz += qr3 * ddz;
-                    }
+    const Dbl4 tg = live ? xs[i] : Dbl4{cx, cy, cz, 0.0};
+    double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+            for (int dx = -1; dx <= 1; ++dx) {
+                const int nx = ix + dx, ny = iy + dy, nz = iz + dz;
+                if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side)
+                    continue;
+                const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
+                const uint32_t e = start[nb + 1];
+#pragma unroll 2
+                for (uint32_t j = start[nb] + c; j < e; j += rep) {
+                    const Dbl4 s = xs[j];
+                    const double ddx = tg.x - s.x, ddy = tg.y - s.y, ddz = tg.z - s.z;
+                    const double r2 = fma(ddx, ddx, fma(ddy, ddy, ddz * ddz));
+                    // self and coincident pairs (r2 = 0, tested on the bits)
+                    const bool pair = (__double2hiint(r2) | __double2loint(r2)) != 0;
+                    const double ri = pair ? rsqrt_f64(r2) : 0.0;
+                    const double qr = s.w * ri, qr3 = qr * (ri * ri);
+                    f = fma(s.w, ri, f);
+                    gx = fma(qr3, ddx, gx);
+                    gy = fma(qr3, ddy, gy);
+                    gz = fma(qr3, ddz, gz);
                 }
+            }
+    for (uint32_t o = 1; o < rep; o <<= 1) {
+        f += __shfl_xor_sync(0xffffffffu, f, int(o));
+        gx += __shfl_xor_sync(0xffffffffu, gx, int(o));
+        gy += __shfl_xor_sync(0xffffffffu, gy, int(o));
+        gz += __shfl_xor_sync(0xffffffffu, gz, int(o));
+    }
+    if (c == 0 && live) {
         double ff = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
         if (far)
             l2p3<double, double2>(sle[wid], p, (tg.x - cx) / w, (tg.y - cy) / w, (tg.z - cz) / w,
                                   ff, fx, fy, fz);
-        if (valid) {
-            const int64_t o = perm[i];
-            if (!PF_IN(o, n)) continue;
+        const int64_t o = perm[i];
+        if (PF_IN(o, n)) {
             store3<TOut>(phi, o, f + ff / w);
             store3<TOut>(ex, o, gx - fx / (w * w));
             store3<TOut>(ey, o, gy - fy / (w * w));
@@ -2106,7 +2224,8 @@ struct petfmm3d_ctx {
     cudaStream_t stream = nullptr;
     DevBuf3 keysA, keysB, valsA, valsB, sortw, start, recu, rec, xs, me, le, status;
     DevBuf3 ncnt, noff, nscan, nitems;  // the mixed near field's work items
-    DevBuf3 rtab32, itab32, rtab64, itab64, atab32, rmap;
+    // operator tables of the context's precision only
+    DevBuf3 rtab32, rtab64, atab32, atab64, rmap, parity;
     DevBuf3 m2m32, l2l32;  // p <= 8: the real M2M / L2L operators of the 8 octants
     DevBuf3 tcimg;  // p <= 8: TF32 hi / lo images of the M2L operators (tensor-core M2L)
     bool m2l_tc = true;  // PETFMM3D_OPT_M2L_TC
@@ -2125,97 +2244,95 @@ namespace {
 
 int upload_tables(petfmm3d_ctx *c) {
     const int p = c->p, nc = nc3(p), nci = nci3(p);
-    std::vector<cd> rt(size_t(8) * nc), it(size_t(NSLOT3) * nci, cd(0.0, 0.0));
+    std::vector<cd> rt(size_t(8) * nc);
     for (int o = 0; o < 8; ++o)
         host_rec_r((o & 1) ? 0.25 : -0.25, (o & 2) ? 0.25 : -0.25, (o & 4) ? 0.25 : -0.25, p,
                    rt.data() + size_t(o) * nc);
-    for (int dz = -3; dz <= 3; ++dz)
-        for (int dy = -3; dy <= 3; ++dy)
-            for (int dx = -3; dx <= 3; ++dx) {
-                if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
-                host_rec_i(dx, dy, dz, 2 * p - 1,
-                           it.data() + size_t((dx + 3) + 7 * (dy + 3) + 49 * (dz + 3)) * nci);
-            }
-    // the mixed path's M2L matrices: real index r < nc is Re of coefficient
-    // r, r >= nc Im of the coefficients with m > 0 in order
+    // the real basis of the M2L matrices: real index r < nc is Re of
+    // coefficient r, r >= nc Im of the coefficients with m > 0 in order;
+    // parity: bit d set if the solid harmonic changes sign with axis d
     const int nr = p * p, nrp = mg_nrp(p);
     std::vector<short2> rm(static_cast<size_t>(nr));
-    std::vector<int> imidx(size_t(nc), -1);
+    std::vector<uint8_t> par(static_cast<size_t>(nr));
     for (int n = 0, r = nc; n < p; ++n)
         for (int m = 0; m <= n; ++m) {
             const int j = n * (n + 1) / 2 + m;
             rm[size_t(j)] = make_short2(short(j), short(m == 0 ? 2 : 0));
+            par[size_t(j)] = uint8_t((m & 1) | (((n + m) & 1) << 2));
             if (m > 0) {
-                imidx[size_t(j)] = r;
+                par[size_t(r)] = uint8_t(((m + 1) & 1) | 2 | (((n + m) & 1) << 2));
                 rm[size_t(r++)] = make_short2(short(j), 1);
             }
         }
-    std::vector<float> at(size_t(NSLOT3) * nrp * nrp, 0.f);
+    P3_TRY(ensure3(c->rmap, rm.size() * sizeof(short2), c->stream));
+    P3_CUDA(cudaMemcpy(c->rmap.p, rm.data(), rm.size() * sizeof(short2), cudaMemcpyHostToDevice));
     std::vector<double> a64(size_t(nr) * nr);
+    std::vector<cd> iv(static_cast<size_t>(nci));
+    if (c->precision == PETFMM_FP64) {
+        // [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
+        std::vector<double> at(size_t(64) * nr * nr, 0.0);
+        for (int o = 0; o < 64; ++o) {
+            const int dx = o & 3, dy = (o >> 2) & 3, dz = o >> 4;
+            if (dx < 2 && dy < 2 && dz < 2) continue;
+            host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
+            host_m2l_real(p, iv.data(), at.data() + size_t(o) * nr * nr);
+        }
+        std::vector<double2> r64(rt.size());
+        for (size_t i = 0; i < rt.size(); ++i) r64[i] = make_double2(rt[i].real(), rt[i].imag());
+        P3_TRY(ensure3(c->atab64, at.size() * sizeof(double), c->stream));
+        P3_TRY(ensure3(c->parity, par.size(), c->stream));
+        P3_TRY(ensure3(c->rtab64, r64.size() * sizeof(double2), c->stream));
+        P3_CUDA(cudaMemcpy(c->atab64.p, at.data(), at.size() * sizeof(double), cudaMemcpyHostToDevice));
+        P3_CUDA(cudaMemcpy(c->parity.p, par.data(), par.size(), cudaMemcpyHostToDevice));
+        P3_CUDA(cudaMemcpy(c->rtab64.p, r64.data(), r64.size() * sizeof(double2), cudaMemcpyHostToDevice));
+        return PETFMM_OK;
+    }
+    // The mixed path's M2L matrices, FP32: ap[k_in * nrp + r_out]; for p <= 8
+    // also their TF32 hi / lo images for the tensor cores:
+    // [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero padding), K in the
+    // input basis of the tensor-core M2L (coefficient by coefficient: Re, then
+    // Im if m > 0), N in the M2L matrices' basis.
+    const bool tc = p <= TT_MAXP;
+    std::vector<float> at(size_t(NSLOT3) * nrp * nrp, 0.f);
+    std::vector<float> img(tc ? size_t(NSLOT3) * 2 * nrp * nrp : 0, 0.f);
+    std::vector<int> tc3_kin(static_cast<size_t>(nr));
+    for (int n = 0, k = 0, t = 0; n < p; ++n)
+        for (int m = 0; m <= n; ++m) {
+            const int j = n * (n + 1) / 2 + m;
+            tc3_kin[size_t(k++)] = j;
+            if (m > 0) tc3_kin[size_t(k++)] = nc + t++;
+        }
     for (int slot = 0; slot < NSLOT3; ++slot) {
         const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
         if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
-        host_m2l_real(p, it.data() + size_t(slot) * nci, a64.data());
-        float *ap = at.data() + size_t(slot) * nrp * nrp;  // ap[k_in * nrp + r_out]
+        host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
+        host_m2l_real(p, iv.data(), a64.data());
+        float *ap = at.data() + size_t(slot) * nrp * nrp;
         for (int k = 0; k < nr; ++k)
             for (int r = 0; r < nr; ++r) ap[size_t(k) * nrp + r] = float(a64[size_t(k) * nr + r]);
-    }
-    if (p <= TT_MAXP) {
-        // TF32 hi / lo images of every operator for the tensor-core M2L:
-        // [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero padding)
-        std::vector<float> img(size_t(NSLOT3) * 2 * nrp * nrp, 0.f);
-        // input-basis position k -> row of the M2L matrix (Re of j: j; Im of
-        // j: NC + its rank among the m > 0 coefficients)
-        std::vector<int> tc3_kin(static_cast<size_t>(nr));
-        for (int n = 0, k = 0, t = 0; n < p; ++n)
-            for (int m = 0; m <= n; ++m) {
-                const int j = n * (n + 1) / 2 + m;
-                tc3_kin[size_t(k++)] = j;
-                if (m > 0) tc3_kin[size_t(k++)] = nc + t++;
-            }
-        for (int slot = 0; slot < NSLOT3; ++slot) {
-            const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
-            if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
-            host_m2l_real(p, it.data() + size_t(slot) * nci, a64.data());
-            float *hi = img.data() + size_t(slot) * 2 * nrp * nrp, *lo = hi + size_t(nrp) * nrp;
-            // K in the input basis of the tensor-core M2L (coefficient by
-            // coefficient: Re, then Im if m > 0); N in the M2L matrices' basis
-            for (int k = 0; k < nr; ++k) {
-                const int kin = tc3_kin[size_t(k)];
-                for (int n = 0; n < nr; ++n) {
-                    const double a = a64[size_t(kin) * nr + n];
-                    const float h = host_tf32_rna(float(a));
-                    const size_t o = (size_t(k / 4) * nrp + n) * 4 + size_t(k % 4);
-                    hi[o] = h;
-                    lo[o] = host_tf32_rna(float(a - double(h)));
-                }
+        if (!tc) continue;
+        float *hi = img.data() + size_t(slot) * 2 * nrp * nrp, *lo = hi + size_t(nrp) * nrp;
+        for (int k = 0; k < nr; ++k) {
+            const int kin = tc3_kin[size_t(k)];
+            for (int n = 0; n < nr; ++n) {
+                const double a = a64[size_t(kin) * nr + n];
+                const float h = host_tf32_rna(float(a));
+                const size_t o = (size_t(k / 4) * nrp + n) * 4 + size_t(k % 4);
+                hi[o] = h;
+                lo[o] = host_tf32_rna(float(a - double(h)));
             }
         }
+    }
+    if (tc) {
         P3_TRY(ensure3(c->tcimg, img.size() * sizeof(float), c->stream));
         P3_CUDA(cudaMemcpy(c->tcimg.p, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
     }
     P3_TRY(ensure3(c->atab32, at.size() * sizeof(float), c->stream));
-    P3_TRY(ensure3(c->rmap, rm.size() * sizeof(short2), c->stream));
     P3_CUDA(cudaMemcpy(c->atab32.p, at.data(), at.size() * sizeof(float), cudaMemcpyHostToDevice));
-    P3_CUDA(cudaMemcpy(c->rmap.p, rm.data(), rm.size() * sizeof(short2), cudaMemcpyHostToDevice));
-    std::vector<double2> r64(rt.size()), i64(it.size());
-    std::vector<float2> r32(rt.size()), i32(it.size());
-    for (size_t i = 0; i < rt.size(); ++i) {
-        r64[i] = make_double2(rt[i].real(), rt[i].imag());
-        r32[i] = make_float2(float(rt[i].real()), float(rt[i].imag()));
-    }
-    for (size_t i = 0; i < it.size(); ++i) {
-        i64[i] = make_double2(it[i].real(), it[i].imag());
-        i32[i] = make_float2(float(it[i].real()), float(it[i].imag()));
-    }
-    P3_TRY(ensure3(c->rtab64, r64.size() * sizeof(double2), c->stream));
-    P3_TRY(ensure3(c->itab64, i64.size() * sizeof(double2), c->stream));
+    std::vector<float2> r32(rt.size());
+    for (size_t i = 0; i < rt.size(); ++i) r32[i] = make_float2(float(rt[i].real()), float(rt[i].imag()));
     P3_TRY(ensure3(c->rtab32, r32.size() * sizeof(float2), c->stream));
-    P3_TRY(ensure3(c->itab32, i32.size() * sizeof(float2), c->stream));
-    P3_CUDA(cudaMemcpy(c->rtab64.p, r64.data(), r64.size() * sizeof(double2), cudaMemcpyHostToDevice));
-    P3_CUDA(cudaMemcpy(c->itab64.p, i64.data(), i64.size() * sizeof(double2), cudaMemcpyHostToDevice));
     P3_CUDA(cudaMemcpy(c->rtab32.p, r32.data(), r32.size() * sizeof(float2), cudaMemcpyHostToDevice));
-    P3_CUDA(cudaMemcpy(c->itab32.p, i32.data(), i32.size() * sizeof(float2), cudaMemcpyHostToDevice));
     if (p <= TT_MAXP) {
         // op[(octant * p^2 + k_in) * p^2 + r_out]
         std::vector<float> mm(size_t(8) * nr * nr), ll(size_t(8) * nr * nr);
@@ -2345,7 +2462,6 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
     V *me = static_cast<V *>(c->me.p), *le = static_cast<V *>(c->le.p);
     const bool f32 = sizeof(T) == 4;
     const V *rtab = static_cast<const V *>(f32 ? c->rtab32.p : c->rtab64.p);
-    const V *itab = static_cast<const V *>(f32 ? c->itab32.p : c->itab64.p);
     const Dom3 d = make_dom3(c->dom, L);
     mark3(c, PETFMM3D_STAGE_P2M);
     if constexpr (sizeof(T) == 4) {
@@ -2376,9 +2492,9 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
         c->launches++;
     }
     mark3(c, PETFMM3D_STAGE_M2L);
-    // mixed path with p <= 8: one launch for all levels (launch_m2l_gemm
-    // launches at l = L)
-    const bool one = sizeof(T) == 4 && mg_nrp(p) <= 64;
+    // one launch for all levels: the FP64 path, and the mixed path with
+    // p <= 8 (launch_m2l_gemm launches at l = L)
+    const bool one = sizeof(T) == 8 || mg_nrp(p) <= 64;
     // mixed path, p <= 8, PETFMM3D_OPT_M2L_TC: all levels on the tensor cores
     const bool tc = sizeof(T) == 4 && c->m2l_tc && p <= TT_MAXP;
     if constexpr (sizeof(T) == 4) {
@@ -2393,8 +2509,16 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
             P3_CUDA(launch_m2l_gemm(p, l, L, start, static_cast<const float *>(c->atab32.p),
                                     static_cast<const short2 *>(c->rmap.p), me, le, st));
         } else {
-            k3_m2l<T><<<grid_w(int64_t(1) << (3 * l)), W3 * 32, 0, st>>>(l, L, p, start, itab,
-                                                                          me, le);
+            const size_t smem = size_t(8) * m2l64_stride(p) * sizeof(double) +
+                                size_t(8) * m2l64_rows(p) * sizeof(int);
+            P3_CUDA(cudaFuncSetAttribute(k3_m2l_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         int(M2L64_SMEM_MAX)));
+            int64_t grid = 0;
+            for (int k = 2; k <= L; ++k) grid += m2l64_blocks(k, m2l64_rows(p));
+            k3_m2l_f64<<<unsigned(grid), M2L64_THREADS, smem, st>>>(
+                L, p, start, static_cast<const double *>(c->atab64.p),
+                static_cast<const short2 *>(c->rmap.p), static_cast<const uint8_t *>(c->parity.p),
+                me, le);
         }
         P3_CUDA(cudaGetLastError());
         c->launches++;
@@ -2499,29 +2623,28 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
         for (int s = PETFMM3D_STAGE_P2M; s <= PETFMM3D_STAGE_L2L; ++s) mark3(c, s);
     }
     mark3(c, PETFMM3D_STAGE_NEAR);
-    const unsigned gl = grid_w(nleaf);
     const double w = c->dom.width / double(int64_t(1) << L);
+    // work items: ceil(n_b / 32) per leaf, at most min(8^L, n) + n / 32
+    const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
+    P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
+    P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
+    P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
+    P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
+    uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
+    uint32_t *nit = off + nleaf;  // the item count, after the offsets
+    uint2 *items = static_cast<uint2 *>(c->nitems.p);
+    const unsigned gb = unsigned((nleaf + 255) / 256);
+    k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
+    P3_CUDA(cudaGetLastError());
+    P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
+                           &c->launches));
+    k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
+    P3_CUDA(cudaGetLastError());
+    c->launches += 2;
+    const unsigned gi = grid_w(cap);
     if (mixed) {
-        // work items: ceil(n_b / 32) per leaf, at most min(8^L, n) + n / 32
-        const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
-        P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
-        P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
-        P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
-        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-        uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
-        uint32_t *nit = off + nleaf;  // the item count, after the offsets
-        uint2 *items = static_cast<uint2 *>(c->nitems.p);
-        const unsigned gb = unsigned((nleaf + 255) / 256);
-        k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
-        P3_CUDA(cudaGetLastError());
-        P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
-                               &c->launches));
-        k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
-        P3_CUDA(cudaGetLastError());
-        c->launches += 2;
         const float4 *rec = static_cast<const float4 *>(c->rec.p);
         const float2 *le = static_cast<const float2 *>(c->le.p);
-        const unsigned gi = grid_w(cap);
         if (f32)
             k3_near_mixed<float><<<gi, W3 * 32, 0, st>>>(L, p, w, start, rec, le, perm, items,
                                                          nit, n, phi, ex, ey, ez);
@@ -2532,9 +2655,11 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
         const Dbl4 *xs = static_cast<const Dbl4 *>(c->xs.p);
         const double2 *le = static_cast<const double2 *>(c->le.p);
         if (f32)
-            k3_near_f64<float><<<gl, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, n, phi, ex, ey, ez);
+            k3_near_f64<float><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
+                                                       phi, ex, ey, ez);
         else
-            k3_near_f64<double><<<gl, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, n, phi, ex, ey, ez);
+            k3_near_f64<double><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
+                                                        phi, ex, ey, ez);
     }
     P3_CUDA(cudaGetLastError());
     c->launches++;
@@ -2675,7 +2800,7 @@ int petfmm3d_destroy(petfmm3d_ctx *c) {
     DevBuf3 *bufs[] = {&c->ncnt, &c->noff, &c->nscan, &c->nitems,
                        &c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->sortw, &c->start,
                        &c->recu,  &c->rec,   &c->xs,    &c->me,    &c->le,    &c->status,
-                       &c->rtab32, &c->itab32, &c->rtab64, &c->itab64, &c->atab32, &c->rmap,
+                       &c->rtab32, &c->rtab64, &c->atab32, &c->atab64, &c->parity, &c->rmap,
                        &c->m2m32, &c->l2l32, &c->tcimg};
     for (DevBuf3 *b : bufs)
         if (b->p) cudaFree(b->p);
