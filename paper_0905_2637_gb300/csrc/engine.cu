@@ -70,6 +70,10 @@ struct Plan {
     std::vector<InstDesc> inst;
     std::vector<Task> tasks;
     TaskRange outscatter, start, particles, leaves_p2m, leaves_wl, m2l, m2l_tc, m2l_tcb, m2l_log;
+    // FP64 vortex M2L by orbits: (box, coefficient) pairs per thread, shared memory
+    TaskRange m2l64;
+    int m2l64_ni = 0;
+    size_t m2l64_smem = 0;
     // tiled SIMT M2L, one launch per order class (p <= 8, 12, 18, 24): each
     // launch's kernel is specialised for its class's largest order
     static constexpr int kTileClasses = 4;
@@ -137,7 +141,7 @@ struct petfmm_ctx {
 
     DevBuf keysA, keysB, valsA, valsB, hist, scratch, start, xs, ys, gs, rec, me, le, cnt, off,
         items, ctrl, plan_dev, busy, ucount, recu, occ, items_u, ikA, ikB, ivA, ivB, ihist, own,
-        part, pitems, pxtra, pxs, ustage, smleaf, smlist, smmom, smloc;
+        part, pitems, pxtra, pxs, ustage, smleaf, smlist, smmom, smloc, gtab;
     DevBuf hx, hy, hg, hu, hv;  // device staging for petfmm_evaluate_host
     std::map<int, OpTables> tables;
     // operators of the near-field expansions by (degree, kappa), see get_sm_table
@@ -407,6 +411,7 @@ void flatten_tasks(Plan &pl) {
     put(pl.m2l_tcb);
     for (TaskRange &r : pl.m2l_tile) put(r);
     put(pl.m2l_log);
+    put(pl.m2l64);
     for (TaskRange &r : pl.m2m) put(r);
     for (TaskRange &r : pl.l2l) put(r);
 }
@@ -416,6 +421,10 @@ void flatten_tasks(Plan &pl) {
 // rather than on the tiled SIMT kernel (a batch of 512 trees has 3,260; one
 // tree, at most 42).
 constexpr int64_t kTcbShallowMinUnits = 512;
+
+// Units of 512 (box, coefficient) pairs from which the FP64 M2L uses them: two
+// for each of 152 SMs.
+constexpr int64_t kM2L64LargeUnits = 304;
 
 int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
 
@@ -557,6 +566,20 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
             base += tr.nblocks;
         }
     }
+    // FP64 vortex M2L: large units where they still give every SM two blocks
+    // (an orbit's set-up is shared by more boxes), small ones otherwise
+    if (precision == PETFMM_FP64 && kernel == KERNEL_VORTEX) {
+        int64_t units = 0;
+        for (const InstDesc &d : pl.inst)
+            for (int l = 2; l <= d.L; ++l) units += m2l64_units(d.p, l, M2L64_NI_MAX);
+        pl.m2l64_ni = units >= kM2L64LargeUnits ? M2L64_NI_MAX : 1;
+        for (int i = 0; i < ni; ++i) {
+            const InstDesc &d = pl.inst[i];
+            for (int l = 2; l <= d.L; ++l)
+                add_task(pl.m2l64, i, l, m2l64_units(d.p, l, pl.m2l64_ni), 1);
+            pl.m2l64_smem = std::max(pl.m2l64_smem, m2l64_smem(d.p, pl.m2l64_ni));
+        }
+    }
     // M2M rounds: round r computes level L_i - 1 - r (>= 2) of every instance.
     for (int r = 0; r + 3 <= Lmax; ++r) {
         TaskRange tr;
@@ -588,7 +611,10 @@ int attach_tables(petfmm_ctx *c, Plan &pl) {
         OpTables *t = get_tables(c, d.p, c->kernel, &err);
         if (!t) return err;
         if (c->precision == PETFMM_FP64) {
-            d.t_m2m = t->m2m64; d.t_l2l = t->l2l64; d.t_m2l = t->m2l64;
+            d.t_m2m = t->m2m64;
+            d.t_l2l = t->l2l64;
+            if (c->kernel == KERNEL_VORTEX) d.t_m2l = t->m2l64r;
+            else d.t_m2l = t->m2l64;
         } else {
             d.t_m2m = t->m2m32; d.t_l2l = t->l2l32; d.t_m2l = t->m2l32;
             d.t_m2l_tc = t->m2l_tc;
@@ -657,7 +683,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     if (!pl.tasks.empty()) k.add(pl.tasks.data(), pl.tasks.size() * sizeof(Task));
     auto range = [&](const TaskRange &r) { k.put(r.first); k.put(r.count); k.put(r.nblocks); };
     for (const TaskRange *r : {&pl.outscatter, &pl.start, &pl.particles, &pl.leaves_p2m, &pl.leaves_wl,
-                               &pl.m2l, &pl.m2l_tc, &pl.m2l_tcb, &pl.m2l_log})
+                               &pl.m2l, &pl.m2l_tc, &pl.m2l_tcb, &pl.m2l_log, &pl.m2l64})
         range(*r);
     for (const TaskRange &r : pl.m2l_tile) range(r);
     for (int cls = 0; cls < Plan::kTileClasses; ++cls) k.put(pl.tile_pmax[cls]);
@@ -667,6 +693,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     k.put(pl.N); k.put(pl.nleaves); k.put(pl.nstart); k.put(pl.ncoef); k.put(pl.items_cap);
     k.put(pl.nbits); k.put(pl.pmax); k.put(pl.deg); k.put(pl.general);
     k.put(pl.tc_smem); k.put(pl.tcb_pmax); k.put(grid);
+    k.put(pl.m2l64_ni); k.put(pl.m2l64_smem);
     k.put(pl.sm_degrees); k.put(pl.sm_row); k.put(pl.sm_rows); k.put(pl.pairs_any);
     k.put(c->precision); k.put(c->dtype); k.put(c->timing); k.put(c->p2p_mode); k.put(c->poison);
     k.put(c->tc_dense_pct); k.put(c->spin_limit); k.put(c->p2p_pairs); k.put(c->kernel);
@@ -935,6 +962,11 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                       start, static_cast<const float2 *>(c->me.p),
                                       static_cast<float2 *>(c->le.p), ucount, c->tc_dense_pct,
                                       xs, lc));
+        else if (pl.m2l64.count)
+            PF_CUDA(launch_m2l64(dtask + pl.m2l64.first, pl.m2l64.count, pl.m2l64.nblocks,
+                                 pl.m2l64_ni, pl.m2l64_smem, dinst, start,
+                                 static_cast<const double2 *>(c->me.p),
+                                 static_cast<double2 *>(c->le.p), xs, lc));
         else
             PF_CUDA(launch_m2l<double>(dtask + pl.m2l.first, pl.m2l.count, pl.m2l.nblocks, dinst,
                                        start, static_cast<const double2 *>(c->me.p),
@@ -1046,7 +1078,9 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                static_cast<const double *>(c->xs.p),
                                static_cast<const double *>(c->ys.p),
                                static_cast<const double *>(c->gs.p), perm,
-                               static_cast<const double2 *>(c->le.p), f32, busy, st, lc));
+                               static_cast<const double2 *>(c->le.p),
+                               static_cast<const double *>(c->gtab.p), lap ? 1 : 0, f32, busy, st,
+                               lc));
     if (!mixed) stage_mark(c, PETFMM_STAGE_FINAL);
     stage_mark(c, PETFMM_STAGE_COUNT);
     return PETFMM_OK;
@@ -1171,6 +1205,17 @@ int petfmm_create(const petfmm_domain *dom, int levels, int order, double sigma,
         petfmm_destroy(c);
         return PETFMM_ECUDA;
     }
+    if (precision == PETFMM_FP64) {
+        const size_t bytes = G64_WORDS * sizeof(double);
+        rc = ensure(c->gtab, bytes, c->stream);
+        if (rc == PETFMM_OK)
+            rc = cuda_status(cudaMemcpy(c->gtab.p, host_g64_table(), bytes, cudaMemcpyHostToDevice));
+        if (rc != PETFMM_OK) {
+            cudaGetLastError();
+            petfmm_destroy(c);
+            return rc;
+        }
+    }
     int err = PETFMM_OK;
     if (!get_tables(c, order, KERNEL_VORTEX, &err)) {
         petfmm_destroy(c);
@@ -1185,7 +1230,7 @@ int petfmm_destroy(petfmm_ctx *c) {
     cudaStreamSynchronize(c->stream);
     DevBuf *bufs[] = {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist, &c->scratch,
                       &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le, &c->cnt,
-                      &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB, &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->hx, &c->hy,
+                      &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB, &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->gtab, &c->hx, &c->hy,
                       &c->hg, &c->hu, &c->hv};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);

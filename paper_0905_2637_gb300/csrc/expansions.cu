@@ -295,6 +295,11 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
     if ((e = up((void **)&t->m2m64, m2m.data(), m2m.size() * 8)) != cudaSuccess) return e;
     if ((e = up((void **)&t->l2l64, l2l.data(), l2l.size() * 8)) != cudaSuccess) return e;
     if ((e = up((void **)&t->m2l64, m2l.data(), m2l.size() * 8)) != cudaSuccess) return e;
+    if (kernel == KERNEL_VORTEX) {
+        std::vector<double> r;
+        host_m2l64_table(p, r);
+        if ((e = up((void **)&t->m2l64r, r.data(), r.size() * 8)) != cudaSuccess) return e;
+    }
     if ((e = up((void **)&t->m2m32, m2m32.data(), m2m32.size() * 4)) != cudaSuccess) return e;
     if ((e = up((void **)&t->l2l32, l2l32.data(), l2l32.size() * 4)) != cudaSuccess) return e;
     if ((e = up((void **)&t->m2l32, m2l32.data(), m2l32.size() * 4)) != cudaSuccess) return e;
@@ -310,6 +315,7 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
 
 void free_op_tables(OpTables *t) {
     cudaFree(t->m2m64); cudaFree(t->l2l64); cudaFree(t->m2l64);
+    cudaFree(t->m2l64r);
     cudaFree(t->m2m32); cudaFree(t->l2l32); cudaFree(t->m2l32);
     cudaFree(t->m2l_tc);
     cudaFree(t->m2l_tcb);

@@ -64,6 +64,7 @@ struct OpTables {
     int p = 0;
     double2 *m2m64 = nullptr, *l2l64 = nullptr, *m2l64 = nullptr;
     float2 *m2m32 = nullptr, *l2l32 = nullptr, *m2l32 = nullptr;
+    double *m2l64r = nullptr; // FP64 M2L by orbits (vortex kernel, m2l64.cu)
     float *m2l_tc = nullptr;  // hi/lo B images for the tensor-core M2L (p <= 24)
     float *m2l_tcb = nullptr; // ... the four target classes side by side (block units)
 };
@@ -157,6 +158,19 @@ cudaError_t launch_m2l_tile(const Task *tasks, int ntasks, int64_t nblocks, int 
                             float2 *le, const uint32_t *ucount, int dense_pct, cudaStream_t st,
                             uint64_t *launches);
 
+// ---- m2l64.cu --------------------------------------------------------------
+// FP64 M2L of the vortex kernel by orbits of quarter turns (InstDesc::t_m2l =
+// the host_m2l64_table of its order).  A unit (one block) is a run of target
+// boxes of one class holding ni 128 (box, coefficient) pairs; ni is 1 or
+// M2L64_NI_MAX, the same results either way.
+constexpr int M2L64_NI_MAX = 4;
+void host_m2l64_table(int p, std::vector<double> &out);
+int64_t m2l64_units(int p, int level, int ni);
+size_t m2l64_smem(int p, int ni);
+cudaError_t launch_m2l64(const Task *tasks, int ntasks, int64_t nblocks, int ni, size_t smem,
+                         const InstDesc *insts, const uint32_t *start, const double2 *me,
+                         double2 *le, cudaStream_t st, uint64_t *launches);
+
 // units of work per block of each expansion kernel (the host plans with them)
 constexpr int P2M_WARPS = 4;      // warps per block
 constexpr int M2L_WARPS = 4;      // warps per block
@@ -192,8 +206,11 @@ cudaError_t launch_p2p_worklist(const Task *tasks, int ntasks, int64_t nblocks,
 cudaError_t launch_p2p_f64(int grid, const uint4 *items, uint32_t *ctrl, const InstDesc *insts,
                            const uint32_t *start, const double *xs, const double *ys,
                            const double *gs, const uint32_t *perm, const double2 *le,
-                           int dtype_f32, unsigned long long *busy, cudaStream_t st,
-                           uint64_t *launches);
+                           const double *gtab, int laplace, int dtype_f32,
+                           unsigned long long *busy, cudaStream_t st, uint64_t *launches);
+// The table behind its kernel factor (vortex), G64_WORDS doubles.
+constexpr int G64_CELLS = 640, G64_TERMS = 7, G64_WORDS = G64_CELLS * (G64_TERMS + 1);
+const double *host_g64_table();
 // Mixed near field, every leaf against all 9 leaves (pairs: not the
 // neighbours the pair kernel covers): own[r] = the near sum of sorted blob r
 // (launch_p2p_final then adds the far field).
@@ -277,7 +294,7 @@ cudaError_t launch_sm_final(const Task *tasks, int ntasks, int64_t nblocks, cons
 
 int p2p_grid(int precision_mixed, int deg, int general, int laplace);
 int device_sm_count();
-constexpr int P2P_TPI_F64 = 32;
+constexpr int P2P_TPI_F64 = 16;
 constexpr int P2P_TPI_MIXED = 64;
 
 }  // namespace petfmm
