@@ -473,7 +473,8 @@ enum {
                                   < 0: no iterations, so the first wait of the tensor-core
                                   M2L reports PETFMM_ETIMEOUT -- for testing the report;
                                   that evaluation's u, v are then unspecified) */
-    PETFMM_OPT_P2P_MODE = 3,   /* order in which the persistent P2P warps take the work
+    PETFMM_OPT_P2P_MODE = 3,   /* order in which persistent P2P warps (FP64 path, and mixed
+                                  path with PETFMM_OPT_P2P_PAIRS 0 or 1) take the work
                                   items from their queue: 0 (default) heaviest first by
                                   the targets x sources cost of Eq. 14, 1 leaf (Morton)
                                   order; the results are identical */
@@ -501,20 +502,21 @@ enum {
                                   arrays may change) and replayed while it repeats;
                                   0 (default) plain launches.  Results are identical.
                                   The context's stream must not be capturing. */
-    PETFMM_OPT_P2P_PAIRS = 11, /* mixed path: 1 (default) each pair of blobs in the same
-                                  or neighbouring leaves that both hold >= 32 blobs is
-                                  evaluated once, its kernel value serving both blobs
-                                  (K of Eq. 8 is odd);
-                                  heavy pairs are cut into pieces for load balance.
-                                  Where the blob core is wide against a leaf (w^2 /
-                                  2 sigma^2 <= 1.95) the near kernel is smooth, and
-                                  leaf pairs of many blobs are summed by expansions of
-                                  it instead (to FP32 rounding; not below a
-                                  PETFMM_OPT_NEAR_TOL of 100).
-                                  0: every leaf sums its 9 leaves directly.  All
-                                  deterministic; they differ by FP32 rounding of the
-                                  sums.  Extra device memory in mode 1: 88 bytes per
-                                  blob and 28 per leaf. */
+    PETFMM_OPT_P2P_PAIRS = 11, /* mixed path's near field: 2 (default) automatic: where the
+                                  blob core is wide against a leaf (w^2 / 2 sigma^2 <= 1.95)
+                                  the near kernel is smooth, and leaf pairs of many blobs
+                                  are summed by expansions of it (to FP32 rounding; not
+                                  below a PETFMM_OPT_NEAR_TOL of 100); elsewhere one
+                                  thread per target sums its 9 leaves.  1: each pair of
+                                  blobs in the same or neighbouring leaves that both hold
+                                  >= 32 blobs is evaluated once, its kernel value serving
+                                  both blobs (K of Eq. 8 is odd), heavy pairs cut into
+                                  pieces for load balance, the others by one thread per
+                                  target.  0: every leaf sums its 9 leaves from work
+                                  items.  All deterministic; they differ by FP32 rounding
+                                  of the sums.  Extra device memory: mode 1, 88 bytes per
+                                  blob and 20 per leaf; the expansions, 8 bytes per leaf
+                                  and at most about 220 per blob. */
     PETFMM_OPT_TC_BLOCKS = 13, /* mixed path, with PETFMM_OPT_M2L_TC = 1: the shape of
                                   the tensor-core M2L.  0 (default): blocks of 8 x 16
                                   parent cells (all four child classes) at levels >= 8,
@@ -556,8 +558,8 @@ enum { PETFMM_KERNEL_VORTEX = 0, PETFMM_KERNEL_LAPLACE = 1 };
 int petfmm_set_option(petfmm_ctx *ctx, int option, int64_t value);
 
 /* Stages reported by petfmm_stage_times (milliseconds, last evaluation).
- * PAIRS: the pairwise near-field kernel, or the near field's expansions (mixed
- * path, PETFMM_OPT_P2P_PAIRS = 1; about zero otherwise); P2P: the directed near field (and, on the FP64 path,
+ * PAIRS: the pairwise near-field kernel (mixed path, PETFMM_OPT_P2P_PAIRS = 1) or
+ * the near field's expansions (2), about zero otherwise; P2P: the directed near field (and, on the FP64 path,
  * L2P and the output in the same kernel); FINAL: the mixed path's final pass
  * (L2P, the sum of the near-field parts, the output in the caller's order;
  * about zero on the FP64 path).  With PETFMM_OPT_OVERLAP the stages
@@ -577,7 +579,8 @@ typedef struct {
     int64_t p2p_pairs;         /* ordered near-field pairs of the last evaluation */
     int64_t m2l_pairs;         /* (target, source) M2L translations of the last evaluation */
     int64_t p2p_items;         /* P2P work items of the last evaluation */
-    float p2p_load_balance;    /* min / max CTA busy time of the last P2P (Eq. 20) */
+    float p2p_load_balance;    /* min / max CTA busy time of the last P2P (Eq. 20); of the
+                                  SMs, for the near field by one thread per target */
     int64_t p2p_pair_items;    /* pairwise mode: (leaf pair, piece) items of the last evaluation */
     int64_t p2p_split_entries; /* pairwise mode: scratch entries the split pairs wanted (pairs
                                   are split only when these fit in one entry per blob) */

@@ -74,9 +74,11 @@ struct InstDesc {
     float cnear;            // w / (4 pi sigma^2)
     float cfar;             // 1 / (2 pi w)
     float qsplit_rho2;      // general path: polynomial below this rho^2
+    float direct_rho2;      // one thread per target: polynomial below this rho^2
     int deg;                // polynomial degree (in rho^2) of g(q) = (1 - e^-q) / q
     int general;            // 1: some near pairs exceed the polynomial range
     float poly[POLY_MAX + 1];
+    uint32_t pair_min;      // pairwise near field: leaf pairs of at least this many blobs each
     int smdeg;              // > 0: near field by expansions of this degree (smooth.cu) ...
     const void *t_sm;       // ... and their operators
     // FP64 constants

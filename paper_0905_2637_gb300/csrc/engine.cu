@@ -95,7 +95,9 @@ struct Plan {
     uint32_t sm_degrees = 0;
     int sm_row = 0;
     int64_t sm_rows = 0;
-    bool pairs_any = false;
+    // the others: pairs_any sums pairs of leaves pairwise (pair kernel),
+    // direct sums by one thread per target, else by work items
+    bool pairs_any = false, direct = false, items_any = false;
 };
 
 struct Problem {
@@ -125,7 +127,8 @@ struct petfmm_ctx {
     int device = 0;
     bool timing = false;
     int p2p_mode = 0;  // 0: work items heaviest first (Eq. 14 weights), 1: Morton order
-    bool p2p_pairs = true;  // mixed path: neighbouring leaves pairwise (PETFMM_OPT_P2P_PAIRS)
+    int p2p_pairs = 2;  // mixed path's near field (PETFMM_OPT_P2P_PAIRS): 0 work items, every
+                        // leaf against 9; 1 pairs from 32 blobs; 2 automatic
     int kernel = KERNEL_VORTEX;  // PETFMM_OPT_KERNEL
     int tc_blocks = 0;           // PETFMM_OPT_TC_BLOCKS: 0 automatic, 1 always, 2 never
     int tc_pipe = 0;             // PETFMM_OPT_TC_PIPE: 0 automatic, 1 single A, 2 double A
@@ -158,6 +161,7 @@ struct petfmm_ctx {
     Plan plan;
     bool sorted_in_first = true;
     int p2p_grid = 0, pairs_grid = 0;  // CTAs of the persistent near-field launches
+    int direct_sms = 0;                // SMs of the one-thread-per-target kernel, if it ran
     // CUDA-graph replay of the launch sequence (PETFMM_OPT_GRAPH)
     bool use_graph = false;
     bool capturing = false;
@@ -285,6 +289,10 @@ void fill_p2p_constants(InstDesc &d, double tol) {
     d.inv2s2 = 1.0 / (2.0 * d.sigma * d.sigma);
     d.cnear64 = 1.0 / (2.0 * M_PI);
     d.cfar64 = 1.0 / (2.0 * M_PI * w);
+    // (1 - e^-q) / q loses about 2^-22.5 / q to the subtraction: the direct sums
+    // take it from the q where that is within the tolerance (and at most 1, the
+    // fit's range)
+    d.direct_rho2 = float(std::min(1.0, 1.7e-7 / tol) / kappa);
     // The fit depends on kappa alone; evaluations of the same problem shape
     // (a served request's every round, a repeated batch) reuse it.
     struct Fit {
@@ -428,9 +436,14 @@ constexpr int64_t kM2L64LargeUnits = 304;
 
 int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
 
-// smooth: near field by expansions where the blob core allows (smooth.cu)
+// Laplace kernel, mixed path: blobs per leaf (empty ones included) up to which
+// one thread per target sums its near field; denser trees take work items of
+// 64 targets, two per lane, which share each source load.
+constexpr int64_t kLaplaceDirectMax = 64;
+
+// near: PETFMM_OPT_P2P_PAIRS
 int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_segmax, double near_tol,
-               bool smooth, const std::vector<Problem> &probs, Plan &pl) {
+               int near, const std::vector<Problem> &probs, Plan &pl) {
     pl = Plan();
     const int ni = int(probs.size());
     int inst_bits = 0;
@@ -470,20 +483,26 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
         pl.deg = std::max(pl.deg, d.deg);
         pl.general |= d.general;
         const int64_t nleaf = int64_t(1) << (2 * pb.L);
-        if (smooth && precision == PETFMM_MIXED && kernel == KERNEL_VORTEX)
+        if (near == 2 && precision == PETFMM_MIXED && kernel == KERNEL_VORTEX)
             d.smdeg = sm_degree(sm_kappa(d), near_tol);
+        d.pair_min = kernel == KERNEL_VORTEX && near == 1 ? P2P_PAIR_MIN : ~0u;
         if (d.smdeg) {
             pl.sm_degrees |= 1u << d.smdeg;
             pl.sm_row = std::max(pl.sm_row, int(sm_row_floats(d.smdeg)));
             pl.sm_rows += sm_max_rows(d.smdeg, pb.n, nleaf);
-        } else {
-            pl.pairs_any = true;
         }
         pl.inst.push_back(d);
         poff += pb.n;
         loff += nleaf;
         eoff += lvl_off(pb.L + 1) * pb.p;
     }
+    bool others = false;  // instances without expansions of the near field
+    for (const InstDesc &d : pl.inst) others |= d.smdeg == 0;
+    if (precision == PETFMM_MIXED && near != 0 && others) {
+        pl.direct = kernel == KERNEL_VORTEX || poff <= kLaplaceDirectMax * loff;
+        pl.pairs_any = kernel == KERNEL_VORTEX && near == 1;
+    }
+    pl.items_any = others && !pl.direct;
     pl.N = poff;
     pl.nleaves = loff;
     pl.nstart = loff + ni;
@@ -695,6 +714,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     k.put(pl.tc_smem); k.put(pl.tcb_pmax); k.put(grid);
     k.put(pl.m2l64_ni); k.put(pl.m2l64_smem);
     k.put(pl.sm_degrees); k.put(pl.sm_row); k.put(pl.sm_rows); k.put(pl.pairs_any);
+    k.put(pl.direct); k.put(pl.items_any); k.put(c->p2p_mode);
     k.put(c->precision); k.put(c->dtype); k.put(c->timing); k.put(c->p2p_mode); k.put(c->poison);
     k.put(c->tc_dense_pct); k.put(c->spin_limit); k.put(c->p2p_pairs); k.put(c->kernel);
     k.put(c->tc_blocks); k.put(c->tc_pipe); k.put(c->overlap);
@@ -746,15 +766,12 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     PF_TRY(ensure(c->valsA, N * 4, st));
     PF_TRY(ensure(c->valsB, N * 4, st));
     PF_TRY(ensure(c->hist, size_t(radix_scratch_words(N)) * 4, st));
-    // pairwise near field (mixed path): at most 4 forward neighbours per leaf,
-    // a pair cut into at most ceil(na / 128) pieces, and the leaf's own pairs
-    // (the pairwise near field is the vortex kernel's)
-    const bool pairs = mixed && c->p2p_pairs && c->kernel == KERNEL_VORTEX && pl.pairs_any;
+    // pairwise near field (mixed path, vortex kernel): at most 4 forward
+    // neighbours per leaf, a pair cut into at most ceil(na / 128) pieces, and
+    // the leaf's own pairs; a leaf with items holds at least pair_min blobs
+    const bool pairs = pl.pairs_any;
     const int64_t pair_cap =
-        pairs ? 5 * std::min<int64_t>(pl.nleaves, N) + 4 * (N / 128) + 1 : 0;
-    const int64_t order_cap = std::max<int64_t>(pl.items_cap, pair_cap);
-    const int64_t scan_n = pl.nleaves;
-    PF_TRY(ensure(c->scratch, size_t(scan_scratch_words(scan_n)) * 4, st));
+        pairs ? 5 * std::min<int64_t>(pl.nleaves, N / P2P_PAIR_MIN) + 4 * (N / 128) + 1 : 0;
     PF_TRY(ensure(c->start, size_t(pl.nstart) * 4, st));
     if (mixed) {
         PF_TRY(ensure(c->rec, size_t(N) * sizeof(float4), st));
@@ -768,14 +785,17 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         PF_TRY(ensure(c->me, size_t(pl.ncoef) * sizeof(double2), st));
         PF_TRY(ensure(c->le, size_t(pl.ncoef) * sizeof(double2), st));
     }
-    PF_TRY(ensure(c->cnt, size_t(pl.nleaves) * 4, st));
+    if (pl.items_any) {
+        PF_TRY(ensure(c->cnt, size_t(pl.nleaves) * 4, st));
+        PF_TRY(ensure(c->off, size_t(pl.nleaves) * 4, st));
+        PF_TRY(ensure(c->scratch, size_t(scan_scratch_words(pl.nleaves)) * 4, st));
+    }
     PF_TRY(ensure(c->occ, size_t(pl.nleaves) * sizeof(uint2), st));
-    PF_TRY(ensure(c->off, size_t(pl.nleaves) * 4, st));
-    if (pl.pairs_any) PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
+    if (pl.items_any) PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
     PF_TRY(ensure(c->ucount,
                   size_t(pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks + pl.tile_blocks()) * sizeof(uint32_t),
                   st));
-    if (mixed && pl.pairs_any) PF_TRY(ensure(c->own, size_t(N) * sizeof(float2), st));
+    if (mixed && (pl.direct || pl.items_any)) PF_TRY(ensure(c->own, size_t(N) * sizeof(float2), st));
     SmBufs sm{};
     if (pl.sm_degrees) {
         const size_t rows = size_t(std::max<int64_t>(pl.sm_rows, 1)), row = size_t(pl.sm_row);
@@ -794,7 +814,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (pairs) {
         PF_TRY(ensure(c->part, size_t(9) * N * sizeof(float2), st));
         PF_TRY(ensure(c->pitems, size_t(pair_cap) * sizeof(uint4), st));
-        PF_TRY(ensure(c->pxtra, size_t(7) * pl.nleaves * sizeof(uint32_t), st));
+        PF_TRY(ensure(c->pxtra, size_t(5) * pl.nleaves * sizeof(uint32_t), st));
         PF_TRY(ensure(c->pxs, size_t(N) * sizeof(float2), st));
     }
     PairBufs pb{};
@@ -802,22 +822,20 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (pairs) {
         pb.part = static_cast<float2 *>(c->part.p);
         pb.nslot = N;
-        pb.xcnt = static_cast<uint32_t *>(c->pxtra.p);
-        pb.xoff = pb.xcnt + pl.nleaves;
-        pb.xtab = pb.xoff + pl.nleaves;
+        pb.xtab = static_cast<uint32_t *>(c->pxtra.p);
         pb.lflags = pb.xtab + 4 * pl.nleaves;
         pb.xs = static_cast<float2 *>(c->pxs.p);
         pb.xcap = N;  // scratch of split pairs; more wanted: no pair is split
     }
-    P2POrder order{}, porder{};
-    if (c->p2p_mode == 0 && pl.pairs_any) {
-        const size_t cap = size_t(order_cap);
+    P2POrder order{};
+    if (c->p2p_mode == 0 && pl.items_any) {
+        const size_t cap = size_t(pl.items_cap);
         PF_TRY(ensure(c->items_u, cap * sizeof(uint4), st));
         PF_TRY(ensure(c->ikA, cap * 4, st));
         PF_TRY(ensure(c->ikB, cap * 4, st));
         PF_TRY(ensure(c->ivA, cap * 4, st));
         PF_TRY(ensure(c->ivB, cap * 4, st));
-        PF_TRY(ensure(c->ihist, size_t(radix_scratch_words(order_cap)) * 4, st));
+        PF_TRY(ensure(c->ihist, size_t(radix_scratch_words(pl.items_cap)) * 4, st));
         order.cap = pl.items_cap;
         order.items_unsorted = static_cast<uint4 *>(c->items_u.p);
         order.kA = static_cast<uint32_t *>(c->ikA.p);
@@ -825,22 +843,24 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         order.vA = static_cast<uint32_t *>(c->ivA.p);
         order.vB = static_cast<uint32_t *>(c->ivB.p);
         order.hist = static_cast<uint32_t *>(c->ihist.p);
-        porder = order;
-        porder.cap = pair_cap;
     }
     const bool lap = c->kernel == KERNEL_LAPLACE;
-    const int grid = pl.pairs_any ? p2p_grid(mixed, pl.deg, pl.general, lap ? 1 : 0) : 0;
-    if (pl.pairs_any && grid <= 0) return PETFMM_EINVAL;
+    const int grid = pl.items_any ? p2p_grid(mixed, pl.deg, pl.general, lap ? 1 : 0) : 0;
+    if (pl.items_any && grid <= 0) return PETFMM_EINVAL;
     const int pgrid = pairs ? p2p_pairs_grid(pl.deg, pl.general) : 0;
     if (pairs && pgrid <= 0) return PETFMM_EINVAL;
-    // busy times: the directed kernel's CTAs, then the pair kernel's
+    // busy times: the work items' CTAs, then the pair kernel's, then the SMs of
+    // the one-thread-per-target kernel
     c->p2p_grid = grid;
     c->pairs_grid = pgrid;
-    unsigned long long *busy = nullptr, *pbusy = nullptr;
+    c->direct_sms = pl.direct ? device_sm_count() : 0;
+    unsigned long long *busy = nullptr, *pbusy = nullptr, *dbusy = nullptr;
+    const size_t busy_words = size_t(grid + pgrid) * 8 * 2;
     if (c->timing) {
-        PF_TRY(ensure(c->busy, size_t(grid + pgrid) * 8 * 2 * sizeof(unsigned long long), st));
+        PF_TRY(ensure(c->busy, (busy_words + 2 * size_t(c->direct_sms)) * sizeof(unsigned long long), st));
         busy = static_cast<unsigned long long *>(c->busy.p);
         if (pairs) pbusy = busy + size_t(grid) * 8 * 2;
+        if (pl.direct) dbusy = busy + busy_words;
     }
 
     const InstDesc *dinst = static_cast<const InstDesc *>(c->plan_dev.p);
@@ -872,6 +892,10 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     }
     // per-evaluation control words (the status word survives until sync)
     PF_CUDA(cudaMemsetAsync(ctrl + 1, 0, (CTRL_WORDS - 1) * 4, st));
+    if (dbusy) {  // {all ones, 0} per SM
+        PF_CUDA(cudaMemsetAsync(dbusy, 0, size_t(c->direct_sms) * 16, st));
+        PF_CUDA(cudaMemset2DAsync(dbusy, 16, 0xff, 8, size_t(c->direct_sms), st));
+    }
 
     stage_mark(c, PETFMM_STAGE_MORTON);
     float4 *recu = mixed ? static_cast<float4 *>(c->recu.p) : nullptr;
@@ -1026,20 +1050,17 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (fork) PF_CUDA(cudaEventRecord(c->ev_join, xs));
     stage_mark(c, PETFMM_STAGE_WORKLIST);
     const int tpi = mixed ? P2P_TPI_MIXED : P2P_TPI_F64;
-    if (pl.pairs_any)
-        PF_CUDA(launch_p2p_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count, pl.leaves_wl.nblocks,
-                                dinst, start, pl.nleaves, tpi, pairs ? 1 : 0,
-                                static_cast<uint32_t *>(c->cnt.p),
-                                static_cast<uint32_t *>(c->off.p), scratch,
-                                static_cast<uint4 *>(c->items.p), ctrl,
-                                c->p2p_mode == 0 ? &order : nullptr, st, lc));
+    if (pl.items_any)
+        PF_CUDA(launch_p2p_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count,
+                                    pl.leaves_wl.nblocks, dinst, start, pl.nleaves, tpi,
+                                    static_cast<uint32_t *>(c->cnt.p),
+                                    static_cast<uint32_t *>(c->off.p), scratch,
+                                    static_cast<uint4 *>(c->items.p), ctrl,
+                                    c->p2p_mode == 0 ? &order : nullptr, st, lc));
     if (pairs)
         PF_CUDA(launch_pair_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count,
-                                     pl.leaves_wl.nblocks, dinst, start, pl.nleaves,
-                                     static_cast<uint32_t *>(c->cnt.p),
-                                     static_cast<uint32_t *>(c->off.p), scratch,
-                                     static_cast<uint4 *>(c->pitems.p), ctrl,
-                                     c->p2p_mode == 0 ? &porder : nullptr, pb, st, lc));
+                                     pl.leaves_wl.nblocks, dinst, start, c->p2p_mode == 0,
+                                     static_cast<uint4 *>(c->pitems.p), pair_cap, ctrl, pb, st, lc));
     if (fork) PF_CUDA(cudaStreamWaitEvent(st, c->ev_gathered, 0));
     stage_mark(c, PETFMM_STAGE_PAIRS);
     if (pl.sm_degrees)
@@ -1052,15 +1073,18 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                  pbusy, st, lc));
     stage_mark(c, PETFMM_STAGE_P2P);
     if (mixed) {
-        // near sums of the own leaf and the directed neighbours, then far
-        // field and the sum
-        if (pl.pairs_any)
+        // near sums outside the pair kernel, then far field and the sum
+        if (pl.direct)
+            PF_CUDA(launch_near_direct(dtask + pl.particles.first, pl.particles.count,
+                                       pl.particles.nblocks, dinst, start, skeys, srec, pb.own,
+                                       ctrl, dbusy, st, lc));
+        else if (pl.items_any)
             PF_CUDA(launch_p2p_mixed(grid, pl.deg, pl.general,
                                      static_cast<const uint4 *>(c->items.p), ctrl, dinst, start,
-                                     srec, pb.own, pairs, lap ? 1 : 0, busy, st, lc));
+                                     srec, pb.own, lap ? 1 : 0, busy, st, lc));
         if (fork) PF_CUDA(cudaStreamWaitEvent(st, c->ev_join, 0));
         stage_mark(c, PETFMM_STAGE_FINAL);
-        if (pl.pairs_any)
+        if (pl.direct || pl.items_any)
             PF_CUDA(launch_p2p_final(dtask + pl.particles.first, pl.particles.count,
                                      pl.particles.nblocks, dinst, start, skeys, srec,
                                      static_cast<const float2 *>(c->le.p), pb, f32, stage, N,
@@ -1539,8 +1563,7 @@ int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, in
     int rc = problems_from(n_inst, inst, probs);
     if (rc) return rc;
     Plan pl;
-    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, true, probs,
-                    pl);
+    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, 2, probs, pl);
     if (rc) return rc;
     int n = 0;
     auto emit = [&](int64_t id, const TaskRange &r) {
@@ -1606,7 +1629,7 @@ int petfmm_set_option(petfmm_ctx *c, int option, int64_t value) {
             c->tc_segmax = int(value);
             return PETFMM_OK;
         case PETFMM_OPT_GRAPH: c->use_graph = value != 0; return PETFMM_OK;
-        case PETFMM_OPT_P2P_PAIRS: c->p2p_pairs = value != 0; return PETFMM_OK;
+        case PETFMM_OPT_P2P_PAIRS: c->p2p_pairs = value == 0 ? 0 : value == 2 ? 2 : 1; return PETFMM_OK;
         case PETFMM_OPT_TC_BLOCKS:
             if (value < 0 || value > 2) return PETFMM_EINVAL;
             c->tc_blocks = int(value);
@@ -1668,11 +1691,12 @@ int petfmm_get_stats(petfmm_ctx *c, petfmm_stats *out) {
             out->p2p_sym_pairs = int64_t(sym);
         }
     }
-    if (c->timing && c->busy.p && c->p2p_grid > 0 && c->ev_recorded) {
+    if (c->timing && c->busy.p && c->p2p_grid + c->pairs_grid + c->direct_sms > 0 &&
+        c->ev_recorded) {
         const int warps = 8;
-        const bool pairs = c->p2p_pairs && c->precision != PETFMM_FP64 && c->pairs_grid > 0;
+        const bool pairs = c->pairs_grid > 0;
         const size_t nblk = size_t(c->p2p_grid) + (pairs ? size_t(c->pairs_grid) : 0);
-        std::vector<unsigned long long> b(nblk * warps * 2);
+        std::vector<unsigned long long> b(nblk * warps * 2 + 2 * size_t(c->direct_sms));
         if (cudaMemcpy(b.data(), c->busy.p, b.size() * 8, cudaMemcpyDeviceToHost) != cudaSuccess)
             return PETFMM_ECUDA;
         // Eq. 20 over the CTAs of one persistent launch: min / max busy span
@@ -1691,8 +1715,20 @@ int petfmm_get_stats(petfmm_ctx *c, petfmm_stats *out) {
             }
             return hi > 0 ? float(lo / hi) : 1.0f;
         };
-        out->p2p_load_balance = lb(0, size_t(c->p2p_grid));
         if (pairs) out->pairs_load_balance = lb(size_t(c->p2p_grid), size_t(c->pairs_grid));
+        if (c->p2p_grid > 0) {
+            out->p2p_load_balance = lb(0, size_t(c->p2p_grid));
+        } else if (c->direct_sms > 0) {  // over the SMs that had blocks of the launch
+            double lo = 0, hi = 0;
+            for (int s = 0; s < c->direct_sms; ++s) {
+                const unsigned long long *q = b.data() + nblk * warps * 2 + 2 * size_t(s);
+                if (q[1] == 0) continue;
+                const double span = double(q[1] - q[0]);
+                lo = hi == 0 ? span : std::min(lo, span);
+                hi = std::max(hi, span);
+            }
+            out->p2p_load_balance = hi > 0 ? float(lo / hi) : 1.0f;
+        }
     }
     return PETFMM_OK;
 }

@@ -187,7 +187,7 @@ constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block for M2M 
 // occupied leaf, tpi targets per item.  ctrl[CTRL_NITEMS] receives the count.
 enum { CTRL_STATUS = 0, CTRL_NITEMS = 1, CTRL_QUEUE = 2, CTRL_PAIRS_LO = 4, CTRL_NOCC = 6,
        CTRL_NPAIRS = 7, CTRL_QUEUE2 = 8, CTRL_NXTRA = 9, CTRL_SYM_LO = 10, CTRL_NSMOOTH = 12,
-       CTRL_WORDS = 16 };
+       CTRL_CLASSES = 16, CTRL_WORDS = 288 };  // from CTRL_CLASSES: the pair items' classes
 // Buffers for dispatching the items heaviest first (order != nullptr): the
 // items are emitted to items_unsorted, sorted by work class (one stable radix
 // pass over cap entries) and permuted into the item array.
@@ -196,11 +196,9 @@ struct P2POrder {
     uint4 *items_unsorted;
     uint32_t *kA, *kB, *vA, *vB, *hist;  // hist: radix_scratch_words(cap) words
 };
-// pairs_mode: only the leaves with directed work (leaves under 32 blobs, or
-// with a neighbour the pair kernel does not cover) get items.
 cudaError_t launch_p2p_worklist(const Task *tasks, int ntasks, int64_t nblocks,
                                 const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                int tpi, int pairs_mode, uint32_t *cnt, uint32_t *off,
+                                int tpi, uint32_t *cnt, uint32_t *off,
                                 uint32_t *scan_scratch, uint4 *items, uint32_t *ctrl,
                                 const P2POrder *order, cudaStream_t st, uint64_t *launches);
 cudaError_t launch_p2p_f64(int grid, const uint4 *items, uint32_t *ctrl, const InstDesc *insts,
@@ -211,39 +209,45 @@ cudaError_t launch_p2p_f64(int grid, const uint4 *items, uint32_t *ctrl, const I
 // The table behind its kernel factor (vortex), G64_WORDS doubles.
 constexpr int G64_CELLS = 640, G64_TERMS = 7, G64_WORDS = G64_CELLS * (G64_TERMS + 1);
 const double *host_g64_table();
-// Mixed near field, every leaf against all 9 leaves (pairs: not the
-// neighbours the pair kernel covers): own[r] = the near sum of sorted blob r
-// (launch_p2p_final then adds the far field).
+// Mixed near field from work items, every leaf against all 9 leaves: own[r] =
+// the near sum of sorted blob r (launch_p2p_final then adds the far field).
 cudaError_t launch_p2p_mixed(int grid, int deg, int general, const uint4 *items, uint32_t *ctrl,
                              const InstDesc *insts, const uint32_t *start, const float4 *rec,
-                             float2 *own, int pairs, int laplace, unsigned long long *busy,
-                             cudaStream_t st, uint64_t *launches);
+                             float2 *own, int laplace, unsigned long long *busy, cudaStream_t st,
+                             uint64_t *launches);
+// Mixed near field, one thread per target: own[r] = blob r's sum over the
+// leaves not summed pairwise with its own (tasks over blobs).
+cudaError_t launch_near_direct(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                               const uint32_t *start, const uint32_t *skeys, const float4 *rec,
+                               float2 *own, uint32_t *ctrl, unsigned long long *busy,
+                               cudaStream_t st, uint64_t *launches);
+// (busy: per SM the first start, preset to all ones, and the last end.)
+// Fewest blobs in both leaves of a pair for the pair kernel.
+constexpr uint32_t P2P_PAIR_MIN = 32;
 // Pairwise near field between neighbouring leaves (mixed path).  Buffers:
 // own[N]: each blob's directly summed part (sorted order; the only one used
-// by the directed mode, part == nullptr there); part: 9 slots of
+// by the modes without pairs, part == nullptr there); part: 9 slots of
 // nslot float2 (slot d: A's blobs from forward neighbour d, slot 4 + d: B's
-// blobs from A, slot 8: each blob from the other blobs of its leaf); xcnt, xoff: per leaf, the scratch entries of its split pairs
-// and their exclusive scan; xtab[4 nleaves]: per (leaf, direction) of a split
+// blobs from A, slot 8: each blob from the other blobs of its leaf); xtab[4 nleaves]: per (leaf, direction) of a split
 // pair its scratch base (all ones: not split); lflags[nleaves]: per leaf,
 // which of these hold its blobs' sums; xs[xcap]: the scratch runs of pieces
 // 1 .. of split pairs.
 struct PairBufs {
     float2 *own, *part;
     int64_t nslot;
-    uint32_t *xcnt, *xoff, *xtab, *lflags;
+    uint32_t *xtab, *lflags;
     float2 *xs;
     int64_t xcap;
 };
 // ... the item list (inst, leaf A, direction | swap << 3 | piece << 4,
-// scratch base; direction 4: the leaf's own pairs),
+// scratch base; direction 4: the leaf's own pairs), at most cap of them,
+// heaviest first (ordered),
 // ctrl[CTRL_NPAIRS] its count, ctrl[CTRL_NXTRA] the scratch entries wanted ...
 cudaError_t launch_pair_worklist(const Task *tasks, int ntasks, int64_t nblocks,
-                                 const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                 uint32_t *cnt, uint32_t *off, uint32_t *scan_scratch,
-                                 uint4 *items, uint32_t *ctrl, const P2POrder *order,
-                                 const PairBufs &pb, cudaStream_t st, uint64_t *launches);
-// ... the pair items, one persistent launch (the directed items follow in
-// launch_p2p_mixed with pairs = 1) ...
+                                 const InstDesc *insts, const uint32_t *start, int ordered,
+                                 uint4 *items, int64_t cap, uint32_t *ctrl, const PairBufs &pb,
+                                 cudaStream_t st, uint64_t *launches);
+// ... the pair items, one persistent launch ...
 int p2p_pairs_grid(int deg, int general);
 cudaError_t launch_p2p_pairs(int grid, int deg, int general, const uint4 *pitems, uint32_t *ctrl,
                              const InstDesc *insts, const uint32_t *start, const float4 *rec,

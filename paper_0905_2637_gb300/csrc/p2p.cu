@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "near_direct.cuh"
 
 namespace petfmm {
 
@@ -58,12 +59,16 @@ __host__ __device__ __forceinline__ int p2p_group_log2(uint32_t nt, int r) {
 __constant__ int8_t c_fwd[4][2] = {{1, 0}, {-1, 1}, {0, 1}, {1, 1}};
 
 // A pair of neighbouring leaves is evaluated pairwise when both hold at least
-// a warp's worth of blobs; with fewer, most lanes of the 64 x 32 tile would
-// idle, and the leaves' own warps sum that neighbour directly instead.  Both
-// leaves of a pair decide from the same two counts.
-constexpr uint32_t P2P_PAIR_MIN = 32;
-__host__ __device__ __forceinline__ bool pairwise(uint32_t na, uint32_t nb) {
-    return na >= P2P_PAIR_MIN && nb >= P2P_PAIR_MIN;
+// pmin (InstDesc::pair_min) blobs; the others are summed directly, one thread
+// per target (k_near_direct).  Both leaves of a pair decide from the same two
+// counts.  PETFMM_OPT_P2P_PAIRS = 1 sets pmin to a warp's worth, 32.  The
+// automatic choice never does: wide cores (kappa <= 1.95) go by expansions,
+// and beyond the polynomial's range the pair kernel ran at 0.2 to 1.06 of the
+// direct kernel's rate (349,185 clustered blobs, 530 per leaf, kappa = 7.6:
+// 3.2 ms, its few heavy items unbalanced, against 1.2; 4,000,000 blobs, 560 per
+// leaf, kappa = 3.9, its best case: 7.5 against 8.0).
+__host__ __device__ __forceinline__ bool pairwise(uint32_t na, uint32_t nb, uint32_t pmin) {
+    return na >= pmin && nb >= pmin;
 }
 
 // A heavy pair is cut into pieces along A, each piece a run of whole
@@ -90,35 +95,19 @@ __device__ __forceinline__ uint32_t leaf_count(const uint32_t *st, int nside, in
     return st[m + 1] - st[m];
 }
 
-// Whether a leaf (n blobs, at ix, iy) has directed near-field work in the
-// pairwise mode: its own blobs when it is too small for the pair kernel, or
-// an occupied neighbour the pair kernel does not cover.
-__device__ __forceinline__ bool directed_work(const uint32_t *st, int nside, int ix, int iy,
-                                              uint32_t n) {
-    if (!pairwise(n, n)) return n > 0;
-    for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-            const uint32_t nb = leaf_count(st, nside, ix + dx, iy + dy);
-            if (nb && !pairwise(n, nb)) return true;
-        }
-    return false;
-}
-
 // Per-leaf flags of the pairwise mode, read by the final pass: which result
 // slots hold this leaf's blobs' sums.
 enum : uint32_t {
     LF_FWD = 1u,        // << k: pairs with forward neighbour k (slot k)
     LF_BWD = 16u,       // << k: pairs with backward neighbour k (slot 4 + k)
     LF_SPLIT = 256u,    // << k: ... cut into pieces, partial sums in the scratch
-    LF_SELF = 4096u,    // the leaf's own pairs (slot 8)
-    LF_DIRECTED = 8192u // directed items (own[])
+    LF_SELF = 4096u     // the leaf's own pairs (slot 8)
 };
 
 __global__ void __launch_bounds__(256) k_p2p_count(const Task *__restrict__ tasks, int ntasks,
                                                    const InstDesc *__restrict__ insts,
                                                    const uint32_t *__restrict__ start, int tpi,
-                                                   int pairs_mode, uint32_t *__restrict__ cnt,
-                                                   uint32_t *ctrl) {
+                                                   uint32_t *__restrict__ cnt, uint32_t *ctrl) {
     const int ti = find_task(tasks, ntasks, blockIdx.x);
     const Task t = tasks[ti];
     const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
@@ -129,12 +118,8 @@ __global__ void __launch_bounds__(256) k_p2p_count(const Task *__restrict__ task
         const uint32_t n = st[m + 1] - st[m];
         const int nside = 1 << d.L;
         const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
-        // pairwise mode: items only for the leaves with directed work; none
-        // for an instance whose near field goes by expansions
-        const bool work =
-            !d.smdeg && (pairs_mode ? directed_work(st, nside, ix, iy, n) : n > 0);
-        cnt[d.loff + m] = work ? (n + tpi - 1) / tpi : 0u;
-        if (n && !d.smdeg) {
+        cnt[d.loff + m] = (n + tpi - 1) / tpi;
+        if (n) {
             uint32_t src = 0;
             for (int dy = -1; dy <= 1; ++dy)
                 for (int dx = -1; dx <= 1; ++dx) {
@@ -235,12 +220,11 @@ static cudaError_t order_items(const P2POrder *order, uint4 *items, const uint32
 
 cudaError_t launch_p2p_worklist(const Task *tasks, int ntasks, int64_t nblocks,
                                 const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                int tpi, int pairs_mode, uint32_t *cnt, uint32_t *off,
+                                int tpi, uint32_t *cnt, uint32_t *off,
                                 uint32_t *scan_scratch, uint4 *items, uint32_t *ctrl,
                                 const P2POrder *order, cudaStream_t st, uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
-    k_p2p_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, tpi, pairs_mode,
-                                                   cnt, ctrl);
+    k_p2p_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, tpi, cnt, ctrl);
     PF_LAUNCHED(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -298,8 +282,8 @@ __device__ __forceinline__ void pair2(const float4 s, float xa, float ya, float 
 }
 
 // One work item of the directed near field: up to 64 targets of a leaf
-// against the leaf and its neighbours (PAIRS: not the neighbours the pair
-// kernel covers); the near sum goes to own[] in sorted order, the final pass
+// against the leaf and its neighbours; the near sum goes to own[] in sorted
+// order, the final pass
 // adds the far field.  No L2P here: with few targets per item the lanes of
 // all source groups would repeat it.
 // Laplace kernel: one source against the lane's two targets, both in the
@@ -317,7 +301,7 @@ __device__ __forceinline__ void pair2_lap(const float4 s, float xa, float ya, fl
     ub = fmaf(s.z, lb, ub);
 }
 
-template <int DEG, bool GENERAL, bool PAIRS, bool LAP>
+template <int DEG, bool GENERAL, bool LAP>
 __device__ __forceinline__ void directed_item(const uint4 item, const InstDesc *__restrict__ insts,
                                               const uint32_t *__restrict__ start,
                                               const float4 *__restrict__ rec,
@@ -346,12 +330,11 @@ __device__ __forceinline__ void directed_item(const uint4 item, const InstDesc *
     const uint32_t *st = start + d.soff;
     const int nside = 1 << L;
     const float logw = LAP ? float(d.logw0 - double(L) * 0.69314718055994530942) : 0.f;
-    // The pairwise mode's directed items (small leaves, leftover neighbours)
-    // and the Laplace kernel's are mostly short: lanes 0..8 fetch the 9
-    // leaves' source ranges at once (lane q: offset (q % 3 - 1, q / 3 - 1)),
-    // so an item pays one load latency, not nine.  The directed-only vortex
-    // mode (long items) keeps the plain loop, which measured faster there.
-    constexpr bool FETCH9 = PAIRS || LAP;
+    // The Laplace kernel's lanes 0..8 fetch the 9 leaves' source ranges at
+    // once (lane q: offset (q % 3 - 1, q / 3 - 1)), so an item pays one load
+    // latency, not nine; the vortex kernel keeps the plain loop, which
+    // measured faster there.
+    constexpr bool FETCH9 = LAP;
     uint32_t lj0 = 0, lj1 = 0;
     if (FETCH9 && lane < 9) {
         const int sx = ix + lane % 3 - 1, sy = iy + lane / 3 - 1;
@@ -361,7 +344,6 @@ __device__ __forceinline__ void directed_item(const uint4 item, const InstDesc *
             lj1 = st[nm + 1];
         }
     }
-    const uint32_t nme = PAIRS ? st[m + 1] - st[m] : 0u;
     for (int q = 0; q < 9; ++q) {
         const int dx = q % 3 - 1, dy = q / 3 - 1;
         uint32_t j0, j1;
@@ -377,9 +359,6 @@ __device__ __forceinline__ void directed_item(const uint4 item, const InstDesc *
         }
         if (j0 == j1) continue;
         {
-            // pairwise mode: the leaves the pair kernel covers (the leaf itself
-            // included) are skipped
-            if (PAIRS && pairwise(nme, j1 - j0)) continue;
             const float xa = ra.x - float(dx), ya = ra.y - float(dy);
             const float xb = rb.x - float(dx), yb = rb.y - float(dy);
             // the stride-1 loop keeps constant load offsets after unrolling
@@ -416,7 +395,7 @@ __device__ __forceinline__ void directed_item(const uint4 item, const InstDesc *
     if (has_b && grp == 0) own[tb] = make_float2(cn * ub, cn * vb);
 }
 
-template <int DEG, bool GENERAL, bool PAIRS, bool LAP>
+template <int DEG, bool GENERAL, bool LAP>
 __global__ void __launch_bounds__(P2P_THREADS, 5) k_p2p_mixed(
     const uint4 *__restrict__ items, uint32_t *ctrl, const InstDesc *__restrict__ insts,
     const uint32_t *__restrict__ start, const float4 *__restrict__ rec,
@@ -429,7 +408,7 @@ __global__ void __launch_bounds__(P2P_THREADS, 5) k_p2p_mixed(
         if (lane == 0) it = atomicAdd(ctrl + CTRL_QUEUE, 1u);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= nitems) break;
-        directed_item<DEG, GENERAL, PAIRS, LAP>(items[it], insts, start, rec, own, lane);
+        directed_item<DEG, GENERAL, LAP>(items[it], insts, start, rec, own, lane);
     }
     if (busy && lane == 0) {
         const uint64_t t_end = global_ns();
@@ -657,56 +636,6 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_f64(
 // warp ran which item.
 // ----------------------------------------------------------------------------
 
-// cnt[leaf] = forward neighbours of an occupied leaf that hold particles
-__global__ void __launch_bounds__(256) k_pair_count(const Task *__restrict__ tasks, int ntasks,
-                                                    const InstDesc *__restrict__ insts,
-                                                    const uint32_t *__restrict__ start,
-                                                    uint32_t *__restrict__ cnt,
-                                                    uint32_t *__restrict__ xcnt,
-                                                    uint32_t *ctrl) {
-    const int ti = find_task(tasks, ntasks, blockIdx.x);
-    const Task t = tasks[ti];
-    const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
-    unsigned long long sym = 0;
-    if (m < t.count) {
-        const InstDesc &d = insts[t.inst];
-        const uint32_t *st = start + d.soff;
-        uint32_t c = 0, x = 0;
-        const uint32_t na = st[m + 1] - st[m];
-        if (na >= P2P_PAIR_MIN && !d.smdeg) {
-            const int nside = 1 << d.L;
-            const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t nb = leaf_count(st, nside, ix + c_fwd[k][0], iy + c_fwd[k][1]);
-                if (!pairwise(na, nb)) continue;
-                uint32_t pc;
-                const uint32_t np = pair_pieces(na, nb, &pc);
-                c += np;
-                x += (np - 1) * nb;
-                sym += (unsigned long long)na * nb;
-            }
-            // the leaf's own pairs: one item
-            c += 1;
-            sym += (unsigned long long)na * (na - 1) / 2;
-        }
-        cnt[d.loff + m] = c;
-        xcnt[d.loff + m] = x;
-    }
-    // block reduction of the unordered pair count (for the statistics)
-#pragma unroll
-    for (int o = 16; o; o >>= 1) sym += __shfl_down_sync(0xffffffffu, sym, o);
-    __shared__ unsigned long long ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = sym;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long s = 0;
-        for (int w = 0; w < 8; ++w) s += ws[w];
-        if (s) atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_SYM_LO), s);
-    }
-}
-
-// items (inst, leaf A, direction d, 0) and their work class (targets x
-// sources, log2 in quarter steps, stored as 127 - class: heaviest first)
 // Estimated time of nt targets against ns sources in the pair kernel: the
 // target chunks it cuts (320/256/128/64/32, see pair_leaves) weighted by
 // their measured time per source step (10 and 8 packed, 4 packed, 2 and 1
@@ -733,73 +662,178 @@ __device__ __forceinline__ uint32_t pair_wclass(uint32_t cost) {
     const uint32_t frac = e >= 2 ? (cost >> (e - 2)) & 3u : (cost << (2 - e)) & 3u;
     return 127u - (uint32_t(e) * 4u + frac);
 }
+constexpr int PAIR_CLASSES = 128;
 
-__global__ void __launch_bounds__(256) k_pair_emit(const Task *__restrict__ tasks, int ntasks,
-                                                   const InstDesc *__restrict__ insts,
-                                                   const uint32_t *__restrict__ start,
-                                                   const uint32_t *__restrict__ off,
-                                                   const uint32_t *__restrict__ xoff,
-                                                   const uint32_t *__restrict__ ctrl,
-                                                   int64_t xcap, uint32_t *__restrict__ xtab,
-                                                   uint32_t *__restrict__ lflags,
-                                                   uint4 *__restrict__ items,
-                                                   uint32_t *__restrict__ wclass) {
+// The work list takes two launches, both walking every leaf's items in the
+// same way: the first counts the items of each work class (and the scratch
+// entries and blob pairs), the second puts the items down class after class,
+// heaviest first, their places within a class by atomics (the order of items
+// changes no result).  ordered = 0 (PETFMM_OPT_P2P_MODE = 1): one class.
+//
+// Calls emit(class, item, scratch entries) for every item of leaf m.
+template <typename F>
+__device__ __forceinline__ void leaf_pair_items(const InstDesc &d, const uint32_t *st, uint32_t m,
+                                                uint32_t inst, int ordered, F &&emit) {
+    const uint32_t na = st[m + 1] - st[m];
+    if (d.smdeg || na < d.pair_min) return;
+    const int nside = 1 << d.L;
+    const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t nb = leaf_count(st, nside, ix + c_fwd[k][0], iy + c_fwd[k][1]);
+        if (!pairwise(na, nb, d.pair_min)) continue;
+        uint32_t pc;
+        const uint32_t np = pair_pieces(na, nb, &pc);
+        // a pair in one piece runs with the leaf that pads less as targets
+        const uint32_t swap = np == 1 && pair_cost(nb, na) < pair_cost(na, nb) ? 1u : 0u;
+        for (uint32_t i = 0; i < np; ++i) {
+            // a warp spends 32 steps per (64-target chunk, 32-source chunk)
+            const uint32_t nt = min(pc, na - i * pc);
+            const uint32_t cls =
+                ordered ? pair_wclass(((nt + 63) / 64) * ((nb + 31) / 32)) : 0u;
+            emit(cls, make_uint4(inst, m, uint32_t(k) | (swap << 3) | (i << 4), 0u),
+                 i ? 0u : (np - 1) * nb, (unsigned long long)(i ? 0u : na) * nb);
+        }
+    }
+    // the leaf's own pairs (direction 4): half the tiles of the leaf with itself
+    const uint32_t cls = ordered ? pair_wclass(((na + 63) / 64) * ((na + 31) / 32) / 2) : 0u;
+    emit(cls, make_uint4(inst, m, 4u, 0u), 0u, (unsigned long long)na * (na - 1) / 2);
+}
+
+__global__ void __launch_bounds__(256) k_pair_count(const Task *__restrict__ tasks, int ntasks,
+                                                    const InstDesc *__restrict__ insts,
+                                                    const uint32_t *__restrict__ start,
+                                                    int ordered, uint32_t *ctrl,
+                                                    uint32_t *__restrict__ ccount) {
+    __shared__ uint32_t hist[PAIR_CLASSES];
+    __shared__ unsigned long long sums;
+    __shared__ uint32_t extra;
+    for (int i = threadIdx.x; i < PAIR_CLASSES; i += 256) hist[i] = 0;
+    if (threadIdx.x == 0) {
+        sums = 0;
+        extra = 0;
+    }
+    __syncthreads();
     const int ti = find_task(tasks, ntasks, blockIdx.x);
     const Task t = tasks[ti];
     const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
-    if (m >= t.count) return;
+    unsigned long long sym = 0;
+    uint32_t x = 0;
+    if (m < t.count) {
+        const InstDesc &d = insts[t.inst];
+        const uint32_t *st = start + d.soff;
+        const uint32_t n = st[m + 1] - st[m];
+        if (n && !d.smdeg)
+            leaf_pair_items(d, st, uint32_t(m), uint32_t(t.inst), ordered,
+                            [&](uint32_t cls, const uint4 &, uint32_t xtra, unsigned long long bp) {
+                                atomicAdd(&hist[cls], 1u);
+                                x += xtra;
+                                sym += bp;
+                            });
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        sym += __shfl_down_sync(0xffffffffu, sym, o);
+        x += __shfl_down_sync(0xffffffffu, x, o);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (sym) atomicAdd(&sums, sym);
+        if (x) atomicAdd(&extra, x);
+    }
+    __syncthreads();
+    uint32_t items = 0;
+    for (int i = threadIdx.x; i < PAIR_CLASSES; i += 256)
+        if (hist[i]) {
+            atomicAdd(ccount + i, hist[i]);
+            items += hist[i];
+        }
+    if (items) atomicAdd(ctrl + CTRL_NPAIRS, items);
+    if (threadIdx.x == 0) {
+        if (sums) atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_SYM_LO), sums);
+        if (extra) atomicAdd(ctrl + CTRL_NXTRA, extra);
+    }
+}
+
+// ccount: the class counts; cplace: the items placed so far in each class
+// (zeroed before), and one more word for the scratch entries handed out.
+__global__ void __launch_bounds__(256) k_pair_emit(const Task *__restrict__ tasks, int ntasks,
+                                                   const InstDesc *__restrict__ insts,
+                                                   const uint32_t *__restrict__ start, int ordered,
+                                                   const uint32_t *__restrict__ ctrl,
+                                                   const uint32_t *__restrict__ ccount,
+                                                   uint32_t *__restrict__ cplace, int64_t xcap,
+                                                   int64_t cap, uint32_t *__restrict__ xtab,
+                                                   uint32_t *__restrict__ lflags,
+                                                   uint4 *__restrict__ items) {
+    __shared__ uint32_t hist[PAIR_CLASSES], base[PAIR_CLASSES];
+    const int ti = find_task(tasks, ntasks, blockIdx.x);
+    const Task t = tasks[ti];
+    const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
     const InstDesc &d = insts[t.inst];
-    if (d.smdeg) return;
     const uint32_t *st = start + d.soff;
-    const uint32_t na = st[m + 1] - st[m];
-    const int nside = 1 << d.L;
-    const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
+    for (int i = threadIdx.x; i < PAIR_CLASSES; i += 256) hist[i] = 0;
+    const bool live = m < t.count && !d.smdeg;
+    const uint32_t na = live ? st[m + 1] - st[m] : 0u;
     // the pieces' scratch runs exist only if all of them fit; else every pair
     // is one piece (decided alike for all pairs, so the result does not depend
     // on which fit)
     const bool split = int64_t(ctrl[CTRL_NXTRA]) <= xcap;
-    // this leaf's flags for the final pass
-    uint32_t fl = directed_work(st, nside, ix, iy, na) ? LF_DIRECTED : 0u;
-    if (na >= P2P_PAIR_MIN) {
-        fl |= LF_SELF;
-        for (int k = 0; k < 4; ++k) {
-            if (pairwise(na, leaf_count(st, nside, ix + c_fwd[k][0], iy + c_fwd[k][1])))
-                fl |= LF_FWD << k;
-            const uint32_t nbk = leaf_count(st, nside, ix - c_fwd[k][0], iy - c_fwd[k][1]);
-            if (pairwise(nbk, na)) {
-                fl |= LF_BWD << k;
-                uint32_t pc;
-                if (split && pair_pieces(nbk, na, &pc) > 1) fl |= LF_SPLIT << k;
+    if (live) {
+        // this leaf's flags for the final pass
+        const int nside = 1 << d.L;
+        const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
+        uint32_t fl = 0;
+        if (na >= d.pair_min) {
+            fl |= LF_SELF;
+            for (int k = 0; k < 4; ++k) {
+                if (pairwise(na, leaf_count(st, nside, ix + c_fwd[k][0], iy + c_fwd[k][1]),
+                             d.pair_min))
+                    fl |= LF_FWD << k;
+                const uint32_t nbk = leaf_count(st, nside, ix - c_fwd[k][0], iy - c_fwd[k][1]);
+                if (pairwise(nbk, na, d.pair_min)) {
+                    fl |= LF_BWD << k;
+                    uint32_t pc;
+                    if (split && pair_pieces(nbk, na, &pc) > 1) fl |= LF_SPLIT << k;
+                }
             }
         }
+        lflags[d.loff + m] = fl;
     }
-    lflags[d.loff + m] = fl;
-    if (na < P2P_PAIR_MIN) return;
-    uint32_t o = off[d.loff + m], xb = xoff[d.loff + m];
-    for (int k = 0; k < 4; ++k) {
-        const uint32_t nb = leaf_count(st, nside, ix + c_fwd[k][0], iy + c_fwd[k][1]);
-        if (!pairwise(na, nb)) continue;
-        uint32_t pc;
-        const uint32_t np = pair_pieces(na, nb, &pc);
-        const uint32_t base = split ? xb : 0xffffffffu;
-        if (np > 1) xtab[(d.loff + m) * 4 + k] = base;
-        // a pair in one piece runs with the leaf that pads less as targets
-        const uint32_t swap = np == 1 && pair_cost(nb, na) < pair_cost(na, nb) ? 1u : 0u;
-        for (uint32_t i = 0; i < np; ++i) {
-            items[o] = make_uint4(uint32_t(t.inst), uint32_t(m),
-                                  uint32_t(k) | (swap << 3) | (i << 4), base);
-            if (wclass) {
-                // a warp spends 32 steps per (64-target chunk, 32-source chunk)
-                const uint32_t nt = split ? min(pc, na - i * pc) : (i ? 0u : na);
-                wclass[o] = pair_wclass(((nt + 63) / 64) * ((nb + 31) / 32));
-            }
-            ++o;
-        }
-        xb += (np - 1) * nb;
+    if (!__syncthreads_or(na >= d.pair_min)) return;
+    if (live)
+        leaf_pair_items(d, st, uint32_t(m), uint32_t(t.inst), ordered,
+                        [&](uint32_t cls, const uint4 &, uint32_t, unsigned long long) {
+                            atomicAdd(&hist[cls], 1u);
+                        });
+    __syncthreads();
+    // this block's run within each class
+    if (threadIdx.x < PAIR_CLASSES) {
+        uint32_t first = 0;
+        for (int i = 0; i < int(threadIdx.x); ++i) first += ccount[i];
+        const uint32_t n = hist[threadIdx.x];
+        base[threadIdx.x] = first + (n ? atomicAdd(cplace + threadIdx.x, n) : 0u);
+        hist[threadIdx.x] = 0;
     }
-    // the leaf's own pairs (direction 4): half the tiles of the leaf with itself
-    items[o] = make_uint4(uint32_t(t.inst), uint32_t(m), 4u, 0u);
-    if (wclass) wclass[o] = pair_wclass(((na + 63) / 64) * ((na + 31) / 32) / 2);
+    __syncthreads();
+    if (live)
+        leaf_pair_items(
+            d, st, uint32_t(m), uint32_t(t.inst), ordered,
+            [&](uint32_t cls, uint4 item, uint32_t xtra, unsigned long long) {
+                const uint32_t o = base[cls] + atomicAdd(&hist[cls], 1u);
+                const int k = int(item.z & 7u);
+                if (k < 4 && (item.z >> 4) == 0 && xtra)  // a pair in pieces: its scratch runs
+                    xtab[(d.loff + m) * 4 + k] =
+                        split ? atomicAdd(cplace + PAIR_CLASSES, xtra) : 0xffffffffu;
+                // (the pieces of a pair follow one another in this thread)
+                if (k < 4) {
+                    uint32_t pc;
+                    const uint32_t nb = leaf_count(st, 1 << d.L,
+                                                   int(compact_bits(item.y)) + c_fwd[k][0],
+                                                   int(compact_bits(item.y >> 1)) + c_fwd[k][1]);
+                    item.w = pair_pieces(na, nb, &pc) > 1 ? xtab[(d.loff + m) * 4 + k]
+                                                          : (split ? 0u : 0xffffffffu);
+                }
+                if (PF_IN(o, cap)) items[o] = item;
+            });
 }
 
 // One target (in A's frame) against the travelling source (already in A's
@@ -1260,13 +1294,12 @@ __global__ void __launch_bounds__(256, 4) k_p2p_final(
         w = d.kernel == KERNEL_LAPLACE ? make_float2(z.x, 0.f)
                                        : make_float2(d.cfar * z.y, d.cfar * z.x);
     }
-    // then the near-field parts this leaf has, in a fixed order
-    const uint32_t fl = pb.part ? pb.lflags[d.loff + m] : LF_DIRECTED;
-    if (fl & LF_DIRECTED) {
-        const float2 o = eager ? e_own : pb.own[r];
-        w.x += o.x;
-        w.y += o.y;
-    }
+    // then the directly summed part and the slots this leaf has, in a fixed
+    // order
+    const uint32_t fl = pb.part ? pb.lflags[d.loff + m] : 0u;
+    const float2 o = eager ? e_own : pb.own[r];
+    w.x += o.x;
+    w.y += o.y;
     if (fl & LF_SELF) {
         const float2 sp = eager ? e_self : pb.part[8 * pb.nslot + r];
         w.x += sp.x;
@@ -1317,27 +1350,115 @@ __global__ void __launch_bounds__(256, 4) k_p2p_final(
 }
 
 cudaError_t launch_pair_worklist(const Task *tasks, int ntasks, int64_t nblocks,
-                                 const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                 uint32_t *cnt, uint32_t *off, uint32_t *scan_scratch,
-                                 uint4 *items, uint32_t *ctrl, const P2POrder *order,
-                                 const PairBufs &pb, cudaStream_t st, uint64_t *launches) {
+                                 const InstDesc *insts, const uint32_t *start, int ordered,
+                                 uint4 *items, int64_t cap, uint32_t *ctrl, const PairBufs &pb,
+                                 cudaStream_t st, uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
-    k_pair_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, cnt, pb.xcnt,
-                                                    ctrl);
+    uint32_t *ccount = ctrl + CTRL_CLASSES, *cplace = ccount + PAIR_CLASSES;
+    static_assert(CTRL_CLASSES + 2 * PAIR_CLASSES + 1 <= CTRL_WORDS, "class counters");
+    k_pair_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, ordered, ctrl,
+                                                    ccount);
     PF_LAUNCHED(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = exclusive_scan(cnt, off, nleaves, scan_scratch, ctrl + CTRL_NPAIRS, st, launches);
-    if (e != cudaSuccess) return e;
-    e = exclusive_scan(pb.xcnt, pb.xoff, nleaves, scan_scratch, ctrl + CTRL_NXTRA, st, launches);
-    if (e != cudaSuccess) return e;
-    uint4 *emit_to = order ? order->items_unsorted : items;
-    k_pair_emit<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, off, pb.xoff, ctrl,
-                                                   pb.xcap, pb.xtab, pb.lflags, emit_to,
-                                                   order ? order->kA : nullptr);
+    k_pair_emit<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, ordered, ctrl,
+                                                   ccount, cplace, pb.xcap, cap, pb.xtab,
+                                                   pb.lflags, items);
     PF_LAUNCHED(1);
-    if ((e = cudaGetLastError()) != cudaSuccess || !order) return e;
-    return order_items(order, items, ctrl + CTRL_NPAIRS, scan_scratch, st, launches);
+    return cudaGetLastError();
+}
+
+// The near field outside the pair kernel, one thread per target blob: own[r]
+// = its sum over the leaves of its neighbourhood that are not summed pairwise
+// with its own (Laplace kernel, and vortex cores narrow against a leaf: all
+// nine).  Bound by issue (about 16 instructions a pair, two of them special
+// functions, 12 of the special-function pipe's cycles): every lane has a
+// target of its own, so leaves of any count fill the warps, where a warp per
+// leaf of 17 blobs kept 17 of 32 lanes busy; the lanes of a leaf read the
+// same source (one request), and no work list is needed.
+// Measured on one GB300 (this kernel alone, against work items and the pair
+// kernel with their lists): 512 uneven trees, 3.9e9 pairs: 9.0 -> 3.6 ms;
+// 1,048,576 blobs, 16 per leaf: 0.29 -> 0.12 ms; 349,185 clustered blobs, 530
+// per leaf, kappa = 7.6: 3.3 -> 1.2 ms.
+constexpr int NEAR_THREADS = 128;  // half a particle task block: more blocks, better balance
+
+__global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
+    const Task *__restrict__ tasks, int ntasks, const InstDesc *__restrict__ insts,
+    const uint32_t *__restrict__ start, const uint32_t *__restrict__ skeys,
+    const float4 *__restrict__ rec, float2 *__restrict__ own, uint32_t *ctrl,
+    unsigned long long *busy) {
+    __shared__ unsigned long long spairs;
+    // busy: first start and last end of this kernel's blocks on each SM
+    uint32_t sm = 0;
+    if (threadIdx.x == 0) {
+        spairs = 0;
+        if (busy) {
+            asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
+            atomicMin(busy + 2 * sm, (unsigned long long)global_ns());
+        }
+    }
+    __syncthreads();
+    const int64_t blk = blockIdx.x / (256 / NEAR_THREADS);
+    const int ti = find_task(tasks, ntasks, blk);
+    const Task t = tasks[ti];
+    const int64_t j = (blk - t.block0) * 256 + (blockIdx.x % (256 / NEAR_THREADS)) * NEAR_THREADS +
+                      threadIdx.x;
+    const InstDesc &d = insts[t.inst];
+    unsigned long long pairs = 0;
+    if (j < t.count && !d.smdeg) {
+        const int64_t r = d.poff + j;
+        const uint32_t *st = start + d.soff;
+        const uint32_t m = skeys[r] & ((1u << (2 * d.L)) - 1u);
+        const int nside = 1 << d.L;
+        const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
+        uint32_t mask = 0;
+#pragma unroll
+        for (int o = 0; o < 9; ++o) {
+            const int x = ix + o % 3 - 1, y = iy + o / 3 - 1;
+            if (x >= 0 && y >= 0 && x < nside && y < nside) mask |= 1u << o;
+        }
+        uint32_t s0[9], s1[9];
+        near_ranges(mask, d, st, ix, iy, s0, s1);
+        const uint32_t n = s1[4] - s0[4];
+#pragma unroll
+        for (int o = 0; o < 9; ++o) {
+            pairs += s1[o] - s0[o];
+            if (pairwise(n, s1[o] - s0[o], d.pair_min)) s1[o] = s0[o];
+        }
+        --pairs;  // not with itself
+        const float4 rr = rec[r];
+        float2 w;
+        if (d.kernel == KERNEL_LAPLACE) {
+            const float logw = float(d.logw0 - double(d.L) * 0.69314718055994530942);
+            w = make_float2(near_laplace(s0, s1, rec, rr.x, rr.y, logw), 0.f);
+        } else {
+            w = near_vortex_of(s0, s1, d, rec, rr.x, rr.y);
+            w.x *= d.cfar;  // cnear / kappa = cfar
+            w.y *= d.cfar;
+        }
+        own[r] = w;
+    }
+    // ordered near pairs, for the statistics
+#pragma unroll
+    for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
+    if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&spairs, pairs);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (spairs)
+            atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), spairs);
+        if (busy) atomicMax(busy + 2 * sm + 1, (unsigned long long)global_ns());
+    }
+}
+
+cudaError_t launch_near_direct(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                               const uint32_t *start, const uint32_t *skeys, const float4 *rec,
+                               float2 *own, uint32_t *ctrl, unsigned long long *busy,
+                               cudaStream_t st, uint64_t *launches) {
+    if (nblocks <= 0) return cudaSuccess;
+    k_near_direct<<<unsigned(nblocks * (256 / NEAR_THREADS)), NEAR_THREADS, 0, st>>>(
+        tasks, ntasks, insts, start, skeys, rec, own, ctrl, busy);
+    PF_LAUNCHED(1);
+    return cudaGetLastError();
 }
 
 // ----------------------------------------------------------------------------
@@ -1346,24 +1467,22 @@ cudaError_t launch_pair_worklist(const Task *tasks, int ntasks, int64_t nblocks,
 typedef void (*MixedKernel)(const uint4 *, uint32_t *, const InstDesc *, const uint32_t *,
                             const float4 *, float2 *, unsigned long long *);
 template <int D>
-static MixedKernel pick2(int general, bool pairs) {
-    if (pairs)
-        return general ? k_p2p_mixed<D, true, true, false> : k_p2p_mixed<D, false, true, false>;
-    return general ? k_p2p_mixed<D, true, false, false> : k_p2p_mixed<D, false, false, false>;
+static MixedKernel pick2(int general) {
+    return general ? k_p2p_mixed<D, true, false> : k_p2p_mixed<D, false, false>;
 }
 
-static MixedKernel pick_mixed(int deg, int general, bool pairs = false, bool lap = false) {
-    if (lap) return k_p2p_mixed<4, false, false, true>;  // no polynomial, no pairs
+static MixedKernel pick_mixed(int deg, int general, bool lap = false) {
+    if (lap) return k_p2p_mixed<4, false, true>;  // no polynomial
     switch (deg) {
-        case 4: return pick2<4>(general, pairs);
-        case 5: return pick2<5>(general, pairs);
-        case 6: return pick2<6>(general, pairs);
-        case 7: return pick2<7>(general, pairs);
-        case 8: return pick2<8>(general, pairs);
-        case 9: return pick2<9>(general, pairs);
-        case 10: return pick2<10>(general, pairs);
-        case 11: return pick2<11>(general, pairs);
-        case 12: return pick2<12>(general, pairs);
+        case 4: return pick2<4>(general);
+        case 5: return pick2<5>(general);
+        case 6: return pick2<6>(general);
+        case 7: return pick2<7>(general);
+        case 8: return pick2<8>(general);
+        case 9: return pick2<9>(general);
+        case 10: return pick2<10>(general);
+        case 11: return pick2<11>(general);
+        case 12: return pick2<12>(general);
         default: return nullptr;
     }
 }
@@ -1383,7 +1502,7 @@ int device_sm_count() {
 int p2p_grid(int precision_mixed, int deg, int general, int laplace) {
     int per_sm = 1;
     if (precision_mixed) {
-        MixedKernel k = pick_mixed(deg, general, false, laplace != 0);
+        MixedKernel k = pick_mixed(deg, general, laplace != 0);
         if (!k) return 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, P2P_THREADS, 0);
     } else {
@@ -1398,9 +1517,9 @@ int p2p_grid(int precision_mixed, int deg, int general, int laplace) {
 
 cudaError_t launch_p2p_mixed(int grid, int deg, int general, const uint4 *items, uint32_t *ctrl,
                              const InstDesc *insts, const uint32_t *start, const float4 *rec,
-                             float2 *own, int pairs, int laplace, unsigned long long *busy,
-                             cudaStream_t st, uint64_t *launches) {
-    MixedKernel k = pick_mixed(deg, general, pairs != 0, laplace != 0);
+                             float2 *own, int laplace, unsigned long long *busy, cudaStream_t st,
+                             uint64_t *launches) {
+    MixedKernel k = pick_mixed(deg, general, laplace != 0);
     if (!k) return cudaErrorInvalidValue;
     k<<<grid, P2P_THREADS, 0, st>>>(items, ctrl, insts, start, rec, own, busy);
     PF_LAUNCHED(1);

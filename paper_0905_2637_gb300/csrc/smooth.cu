@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "near_direct.cuh"
 
 namespace petfmm {
 
@@ -514,54 +515,6 @@ __device__ __forceinline__ float2 sm_gradient(const float *__restrict__ loc, flo
     return make_float2(fs, ft);
 }
 
-// The leaf pairs summed directly: sources of the neighbours in mask.
-template <int DEG>
-__device__ __forceinline__ float2 sm_direct(uint32_t mask, const InstDesc &d,
-                                            const uint32_t *__restrict__ st,
-                                            const float4 *__restrict__ rec, int ix, int iy,
-                                            float x, float y) {
-    float a[DEG + 1];
-#pragma unroll
-    for (int k = 0; k <= DEG; ++k) a[k] = d.poly[k];
-    const float kappa = d.kappa, split = d.qsplit_rho2;
-    const bool general = d.general != 0;
-    uint32_t s0[9], s1[9];
-#pragma unroll
-    for (int o = 0; o < 9; ++o) {
-        s0[o] = s1[o] = 0;
-        if ((mask >> o) & 1u) {
-            const uint32_t nm = morton_key(uint32_t(ix + o % 3 - 1), uint32_t(iy + o / 3 - 1));
-            s0[o] = st[nm];
-            s1[o] = st[nm + 1];
-            if (!(PF_IN(int64_t(s0[o]) - d.poff, d.n + 1) &&
-                  PF_IN(int64_t(s1[o]) - d.poff, d.n + 1)))
-                s1[o] = s0[o];
-        }
-    }
-    float u = 0.f, v = 0.f;
-#pragma unroll
-    for (int o = 0; o < 9; ++o) {
-        const float xt = x - float(o % 3 - 1), yt = y - float(o / 3 - 1);
-        for (uint32_t j = s0[o]; j < s1[o]; ++j) {
-            const float4 r = __ldg(rec + j);
-            const float dx = xt - r.x, dy = yt - r.y;
-            const float r2 = fmaf(dx, dx, dy * dy);
-            float g = a[DEG];
-#pragma unroll
-            for (int k = DEG - 1; k >= 0; --k) g = fmaf(g, r2, a[k]);
-            if (general) {
-                const float q = kappa * r2;
-                const float ge = __fdividef(1.0f - __expf(-q), q);
-                g = r2 < split ? g : ge;
-            }
-            const float f = r.z * g;
-            u = fmaf(-dy, f, u);
-            v = fmaf(dx, f, v);
-        }
-    }
-    return make_float2(u, v);
-}
-
 __global__ void __launch_bounds__(256, 3) k_sm_final(
     const Task *__restrict__ tasks, int ntasks, const InstDesc *__restrict__ insts,
     const uint32_t *__restrict__ start, const uint32_t *__restrict__ skeys,
@@ -609,11 +562,11 @@ __global__ void __launch_bounds__(256, 3) k_sm_final(
     }
     const uint32_t dm = mask & 0x1ffu;
     if (dm) {
-        const uint32_t *st = start + d.soff;
-        const float2 n = d.deg <= 6 ? sm_direct<6>(dm, d, st, rec, ix, iy, rr.x, rr.y)
-                                    : sm_direct<12>(dm, d, st, rec, ix, iy, rr.x, rr.y);
-        w.x = fmaf(d.cnear, n.x, w.x);
-        w.y = fmaf(d.cnear, n.y, w.y);
+        uint32_t s0[9], s1[9];
+        near_ranges(dm, d, start + d.soff, ix, iy, s0, s1);
+        const float2 n = near_vortex_of(s0, s1, d, rec, rr.x, rr.y);
+        w.x = fmaf(d.cfar, n.x, w.x);  // cnear / kappa = cfar
+        w.y = fmaf(d.cfar, n.y, w.y);
     }
     if (stage) {
         stage[r] = w.x;
