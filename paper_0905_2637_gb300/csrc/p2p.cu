@@ -1409,33 +1409,20 @@ __global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
         const int64_t r = d.poff + j;
         const uint32_t *st = start + d.soff;
         const uint32_t m = skeys[r] & ((1u << (2 * d.L)) - 1u);
-        const int nside = 1 << d.L;
-        const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
-        uint32_t mask = 0;
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-            const int x = ix + o % 3 - 1, y = iy + o / 3 - 1;
-            if (x >= 0 && y >= 0 && x < nside && y < nside) mask |= 1u << o;
-        }
-        uint32_t s0[9], s1[9];
-        near_ranges(mask, d, st, ix, iy, s0, s1);
-        const uint32_t n = s1[4] - s0[4];
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-            pairs += s1[o] - s0[o];
-            if (pairwise(n, s1[o] - s0[o], d.pair_min)) s1[o] = s0[o];
-        }
-        --pairs;  // not with itself
+        const NearLeaves q{&d, st, int(compact_bits(m)), int(compact_bits(m >> 1)), 0x1ffu,
+                           st[m + 1] - st[m], d.pair_min};
         const float4 rr = rec[r];
+        uint32_t total;
         float2 w;
         if (d.kernel == KERNEL_LAPLACE) {
             const float logw = float(d.logw0 - double(d.L) * 0.69314718055994530942);
-            w = make_float2(near_laplace(s0, s1, rec, rr.x, rr.y, logw), 0.f);
+            w = make_float2(near_laplace(q, rec, rr.x, rr.y, logw, total), 0.f);
         } else {
-            w = near_vortex_of(s0, s1, d, rec, rr.x, rr.y);
+            w = near_vortex_of(q, rec, rr.x, rr.y, total);
             w.x *= d.cfar;  // cnear / kappa = cfar
             w.y *= d.cfar;
         }
+        pairs = total - 1u;  // not with itself
         own[r] = w;
     }
     // ordered near pairs, for the statistics

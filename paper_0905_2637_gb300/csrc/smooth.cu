@@ -562,9 +562,9 @@ __global__ void __launch_bounds__(256, 3) k_sm_final(
     }
     const uint32_t dm = mask & 0x1ffu;
     if (dm) {
-        uint32_t s0[9], s1[9];
-        near_ranges(dm, d, start + d.soff, ix, iy, s0, s1);
-        const float2 n = near_vortex_of(s0, s1, d, rec, rr.x, rr.y);
+        uint32_t total;
+        const NearLeaves q{&d, start + d.soff, ix, iy, dm, 0u, ~0u};
+        const float2 n = near_vortex_of(q, rec, rr.x, rr.y, total);
         w.x = fmaf(d.cfar, n.x, w.x);  // cnear / kappa = cfar
         w.y = fmaf(d.cfar, n.y, w.y);
     }
