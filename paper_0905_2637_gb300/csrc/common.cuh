@@ -58,7 +58,7 @@ struct InstDesc {
     int kernel;             // KERNEL_VORTEX or KERNEL_LAPLACE
     const void *x, *y, *g;  // caller's arrays (storage type of the context)
     void *u, *v;
-    const void *t_m2m, *t_l2l, *t_m2l;  // operator tables for this p (path's real type)
+    const void *t_shift, *t_m2l;  // operator tables for this p (path's real type)
     const void *t_m2l_tc;               // tensor-core M2L operator images (mixed path)
     const void *t_m2l_tcb;              // ... side by side for the block units
     int64_t tc_unit0[MAX_L + 1];        // per level: first unit of this (instance, level)

@@ -84,7 +84,12 @@ struct Plan {
         for (const TaskRange &r : m2l_tile) b += r.nblocks;
         return b;
     }
-    std::vector<TaskRange> m2m, l2l;  // in launch order
+    // M2M and L2L, in launch order: a task's units are runs of parents (on the
+    // mixed path the top levels run apart, shift_top)
+    std::vector<TaskRange> up, down;
+    size_t shift_smem = 0, shift_top_smem = 0;
+    bool shift_top = false;
+    std::vector<TaskRange> m2m, l2l;  // the plan dump's (box, coefficient) pairs
     int64_t N = 0, nleaves = 0, nstart = 0, ncoef = 0, items_cap = 0;
     int nbits = 0, pmax = 1, Lmax = 0;
     int deg = 0, general = 0;          // mixed P2P variant (max over instances)
@@ -420,6 +425,8 @@ void flatten_tasks(Plan &pl) {
     for (TaskRange &r : pl.m2l_tile) put(r);
     put(pl.m2l_log);
     put(pl.m2l64);
+    for (TaskRange &r : pl.up) put(r);
+    for (TaskRange &r : pl.down) put(r);
     for (TaskRange &r : pl.m2m) put(r);
     for (TaskRange &r : pl.l2l) put(r);
 }
@@ -443,7 +450,7 @@ constexpr int64_t kLaplaceDirectMax = 64;
 
 // near: PETFMM_OPT_P2P_PAIRS
 int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_segmax, double near_tol,
-               int near, const std::vector<Problem> &probs, Plan &pl) {
+               int near, const std::vector<Problem> &probs, Plan &pl, bool dump = false) {
     pl = Plan();
     const int ni = int(probs.size());
     int inst_bits = 0;
@@ -599,24 +606,46 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
             pl.m2l64_smem = std::max(pl.m2l64_smem, m2l64_smem(d.p, pl.m2l64_ni));
         }
     }
-    // M2M rounds: round r computes level L_i - 1 - r (>= 2) of every instance.
-    for (int r = 0; r + 3 <= Lmax; ++r) {
-        TaskRange tr;
+    // M2M rounds: round r computes level L_i - 1 - r of every instance, down to
+    // the first level the top launch does not take; L2L rounds start there
+    const int bottom = precision == PETFMM_FP64 ? 2 : kShiftTop + 1;
+    for (int r = 0; Lmax - 1 - r >= bottom; ++r) {
+        TaskRange u, w;
         for (int i = 0; i < ni; ++i) {
-            const int l = pl.inst[i].L - 1 - r;
-            if (l >= 2) add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
+            const InstDesc &d = pl.inst[i];
+            if (d.L - 1 - r >= bottom) add_task(u, i, d.L - 1 - r, shift_units(d.p, d.L - 1 - r), 1);
+            if (bottom + r <= d.L - 1) add_task(w, i, bottom + r, shift_units(d.p, bottom + r), 1);
         }
-        if (tr.count) pl.m2m.push_back(tr);
+        pl.up.push_back(u);
+        pl.down.push_back(w);
     }
-    // L2L rounds: round r translates level 2 + r into level 3 + r.
-    for (int r = 0; r + 3 <= Lmax; ++r) {
-        TaskRange tr;
-        for (int i = 0; i < ni; ++i) {
-            const int l = 3 + r;
-            if (l <= pl.inst[i].L)
-                add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
+    for (const InstDesc &d : pl.inst) {
+        pl.shift_smem = std::max(pl.shift_smem, shift_smem(d.p, precision == PETFMM_FP64, false));
+        if (precision == PETFMM_MIXED && d.L >= 3) {
+            pl.shift_top = true;
+            pl.shift_top_smem = std::max(pl.shift_top_smem, shift_smem(d.p, false, true));
         }
-        if (tr.count) pl.l2l.push_back(tr);
+    }
+    if (dump) {
+        // M2M rounds: round r computes level L_i - 1 - r (>= 2) of every instance.
+        for (int r = 0; r + 3 <= Lmax; ++r) {
+            TaskRange tr;
+            for (int i = 0; i < ni; ++i) {
+                const int l = pl.inst[i].L - 1 - r;
+                if (l >= 2) add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
+            }
+            if (tr.count) pl.m2m.push_back(tr);
+        }
+        // L2L rounds: round r translates level 2 + r into level 3 + r.
+        for (int r = 0; r + 3 <= Lmax; ++r) {
+            TaskRange tr;
+            for (int i = 0; i < ni; ++i) {
+                const int l = 3 + r;
+                if (l <= pl.inst[i].L)
+                    add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
+            }
+            if (tr.count) pl.l2l.push_back(tr);
+        }
     }
     pl.items_cap = items_cap;
     flatten_tasks(pl);
@@ -630,12 +659,12 @@ int attach_tables(petfmm_ctx *c, Plan &pl) {
         OpTables *t = get_tables(c, d.p, c->kernel, &err);
         if (!t) return err;
         if (c->precision == PETFMM_FP64) {
-            d.t_m2m = t->m2m64;
-            d.t_l2l = t->l2l64;
+            d.t_shift = t->shift64;
             if (c->kernel == KERNEL_VORTEX) d.t_m2l = t->m2l64r;
             else d.t_m2l = t->m2l64;
         } else {
-            d.t_m2m = t->m2m32; d.t_l2l = t->l2l32; d.t_m2l = t->m2l32;
+            d.t_shift = t->shift32;
+            d.t_m2l = t->m2l32;
             d.t_m2l_tc = t->m2l_tc;
             d.t_m2l_tcb = t->m2l_tcb;
         }
@@ -706,9 +735,10 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
         range(*r);
     for (const TaskRange &r : pl.m2l_tile) range(r);
     for (int cls = 0; cls < Plan::kTileClasses; ++cls) k.put(pl.tile_pmax[cls]);
-    for (const TaskRange &r : pl.m2m) range(r);
-    for (const TaskRange &r : pl.l2l) range(r);
-    k.put(pl.m2m.size()); k.put(pl.l2l.size());
+    for (const TaskRange &r : pl.up) range(r);
+    for (const TaskRange &r : pl.down) range(r);
+    k.put(pl.up.size()); k.put(pl.shift_smem); k.put(pl.shift_top); k.put(pl.shift_top_smem);
+    k.put(pl.inst.size());
     k.put(pl.N); k.put(pl.nleaves); k.put(pl.nstart); k.put(pl.ncoef); k.put(pl.items_cap);
     k.put(pl.nbits); k.put(pl.pmax); k.put(pl.deg); k.put(pl.general);
     k.put(pl.tc_smem); k.put(pl.tcb_pmax); k.put(grid);
@@ -953,14 +983,19 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                    static_cast<const double *>(c->gs.p), nullptr,
                                    static_cast<double2 *>(c->me.p), xs, lc));
     stage_mark_on(c, PETFMM_STAGE_M2M, xs);
-    for (const TaskRange &tr : pl.m2m) {
+    for (const TaskRange &tr : pl.up) {
         if (mixed)
-            PF_CUDA(launch_m2m<float>(dtask + tr.first, tr.count, tr.nblocks, dinst, start,
-                                      static_cast<float2 *>(c->me.p), xs, lc));
+            PF_CUDA(launch_shift<float>(false, dtask + tr.first, tr.count, tr.nblocks,
+                                        pl.shift_smem, dinst, start,
+                                        static_cast<float2 *>(c->me.p), xs, lc));
         else
-            PF_CUDA(launch_m2m<double>(dtask + tr.first, tr.count, tr.nblocks, dinst, start,
-                                       static_cast<double2 *>(c->me.p), xs, lc));
+            PF_CUDA(launch_shift<double>(false, dtask + tr.first, tr.count, tr.nblocks,
+                                         pl.shift_smem, dinst, start,
+                                         static_cast<double2 *>(c->me.p), xs, lc));
     }
+    if (pl.shift_top)
+        PF_CUDA(launch_shift_top(false, int(pl.inst.size()), pl.shift_top_smem, dinst, start,
+                                 static_cast<float2 *>(c->me.p), xs, lc));
     stage_mark_on(c, PETFMM_STAGE_M2L, xs);
     uint32_t *ucount = nullptr;
     if (pl.m2l_tc.count || pl.m2l_tcb.count || pl.tile_blocks()) {
@@ -1038,13 +1073,18 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                                static_cast<double2 *>(c->le.p), xs, lc));
     }
     stage_mark_on(c, PETFMM_STAGE_L2L, xs);
-    for (const TaskRange &tr : pl.l2l) {
+    if (pl.shift_top)
+        PF_CUDA(launch_shift_top(true, int(pl.inst.size()), pl.shift_top_smem, dinst, start,
+                                 static_cast<float2 *>(c->le.p), xs, lc));
+    for (const TaskRange &tr : pl.down) {
         if (mixed)
-            PF_CUDA(launch_l2l<float>(dtask + tr.first, tr.count, tr.nblocks, dinst, start,
-                                      static_cast<float2 *>(c->le.p), xs, lc));
+            PF_CUDA(launch_shift<float>(true, dtask + tr.first, tr.count, tr.nblocks,
+                                        pl.shift_smem, dinst, start,
+                                        static_cast<float2 *>(c->le.p), xs, lc));
         else
-            PF_CUDA(launch_l2l<double>(dtask + tr.first, tr.count, tr.nblocks, dinst, start,
-                                       static_cast<double2 *>(c->le.p), xs, lc));
+            PF_CUDA(launch_shift<double>(true, dtask + tr.first, tr.count, tr.nblocks,
+                                         pl.shift_smem, dinst, start,
+                                         static_cast<double2 *>(c->le.p), xs, lc));
     }
     stage_mark_on(c, PETFMM_STAGE_COUNT + 1, xs);  // end of the L2L stage
     if (fork) PF_CUDA(cudaEventRecord(c->ev_join, xs));
@@ -1563,7 +1603,8 @@ int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, in
     int rc = problems_from(n_inst, inst, probs);
     if (rc) return rc;
     Plan pl;
-    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, 2, probs, pl);
+    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, 2, probs, pl,
+                    true);
     if (rc) return rc;
     int n = 0;
     auto emit = [&](int64_t id, const TaskRange &r) {

@@ -274,34 +274,23 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
     cudaError_t e = upload_il();
     if (e != cudaSuccess) return e;
     t->p = p;
-    const size_t n_m2m = size_t(4) * p * p, n_m2l = size_t(40) * p * p;
-    std::vector<double> m2m(2 * n_m2m), l2l(2 * n_m2m), m2l(2 * n_m2l);
-    if (kernel == KERNEL_LAPLACE) {
-        host_lap_m2m_table(p, m2m.data());
-        host_lap_l2l_table(p, l2l.data());
-        host_lap_m2l_table(p, m2l.data());
-    } else {
-        host_m2m_table(p, m2m.data());
-        host_l2l_table(p, l2l.data());
-        host_m2l_table(p, m2l.data());
-    }
-    std::vector<float> m2m32(m2m.begin(), m2m.end()), l2l32(l2l.begin(), l2l.end()),
-        m2l32(m2l.begin(), m2l.end());
+    std::vector<double> m2l(size_t(2) * 40 * p * p), shift;
+    (kernel == KERNEL_LAPLACE ? host_lap_m2l_table : host_m2l_table)(p, m2l.data());
+    host_shift_table(p, kernel, shift);
+    std::vector<float> m2l32(m2l.begin(), m2l.end()), shift32(shift.begin(), shift.end());
     auto up = [&](void **dst, const void *src, size_t bytes) -> cudaError_t {
         cudaError_t r = cudaMalloc(dst, bytes);
         if (r != cudaSuccess) return r;
         return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
     };
-    if ((e = up((void **)&t->m2m64, m2m.data(), m2m.size() * 8)) != cudaSuccess) return e;
-    if ((e = up((void **)&t->l2l64, l2l.data(), l2l.size() * 8)) != cudaSuccess) return e;
+    if ((e = up((void **)&t->shift64, shift.data(), shift.size() * 8)) != cudaSuccess) return e;
+    if ((e = up((void **)&t->shift32, shift32.data(), shift32.size() * 4)) != cudaSuccess) return e;
     if ((e = up((void **)&t->m2l64, m2l.data(), m2l.size() * 8)) != cudaSuccess) return e;
     if (kernel == KERNEL_VORTEX) {
         std::vector<double> r;
         host_m2l64_table(p, r);
         if ((e = up((void **)&t->m2l64r, r.data(), r.size() * 8)) != cudaSuccess) return e;
     }
-    if ((e = up((void **)&t->m2m32, m2m32.data(), m2m32.size() * 4)) != cudaSuccess) return e;
-    if ((e = up((void **)&t->l2l32, l2l32.data(), l2l32.size() * 4)) != cudaSuccess) return e;
     if ((e = up((void **)&t->m2l32, m2l32.data(), m2l32.size() * 4)) != cudaSuccess) return e;
     if (((2 * p + 15) & ~15) <= 48) {
         std::vector<float> img;
@@ -314,9 +303,9 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
 }
 
 void free_op_tables(OpTables *t) {
-    cudaFree(t->m2m64); cudaFree(t->l2l64); cudaFree(t->m2l64);
+    cudaFree(t->shift64); cudaFree(t->shift32); cudaFree(t->m2l64);
     cudaFree(t->m2l64r);
-    cudaFree(t->m2m32); cudaFree(t->l2l32); cudaFree(t->m2l32);
+    cudaFree(t->m2l32);
     cudaFree(t->m2l_tc);
     cudaFree(t->m2l_tcb);
     *t = OpTables();
@@ -646,96 +635,6 @@ cudaError_t launch_p2m(const uint2 *occ, const uint32_t *ctrl, int64_t max_occ,
 }
 
 // ----------------------------------------------------------------------------
-// M2M: one thread per (parent box, output coefficient).  Task = (instance,
-// parent level l); units = 4^l * p in row-major box order.
-// ----------------------------------------------------------------------------
-template <typename R>
-__global__ void __launch_bounds__(EXP_THREADS) k_m2m(const Task *__restrict__ tasks, int ntasks,
-                                                     const InstDesc *__restrict__ insts,
-                                                     const uint32_t *__restrict__ start,
-                                                     typename Cplx<R>::T *__restrict__ me) {
-    using C2 = typename Cplx<R>::T;
-    const int ti = find_task(tasks, ntasks, blockIdx.x);
-    const Task t = tasks[ti];
-    const int64_t u = (int64_t(blockIdx.x) - t.block0) * EXP_THREADS + threadIdx.x;
-    if (u >= t.count) return;
-    const InstDesc &d = insts[t.inst];
-    const int p = d.p, l = t.level;
-    const int64_t box = u / p;
-    const int lp = int(u - box * p);
-    const uint32_t ix = uint32_t(box & ((int64_t(1) << l) - 1)), iy = uint32_t(box >> l);
-    const uint32_t *st = start + d.soff;
-    const uint32_t pm = morton_key(ix, iy);
-    if (!box_count(st, d.L, l, pm)) return;
-    const C2 *tab = static_cast<const C2 *>(d.t_m2m);
-    const int64_t quarter = int64_t(1) << (2 * l);
-    const C2 *child = me + d.eoff + (lvl_off(l + 1) + int64_t(iy) * (int64_t(1) << l) + ix) * p;
-    C2 s = mk2<R>(R(0), R(0));
-    for (int c = 0; c < 4; ++c) {
-        // child c of the parent has Morton index 4 pm + c; an empty child has
-        // no expansion (it would be zero)
-        if (!box_count(st, d.L, l + 1, 4 * pm + uint32_t(c))) continue;
-        const C2 *a = child + c * quarter * p;
-        const C2 *row = tab + (size_t(c) * p + lp) * p;
-        for (int k = 0; k <= lp; ++k) s = cfma(row[k], a[k], s);
-    }
-    me[d.eoff + (lvl_off(l) + box_index(l, ix, iy)) * p + lp] = s;
-}
-
-template <typename R>
-cudaError_t launch_m2m(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, typename Cplx<R>::T *me, cudaStream_t st,
-                       uint64_t *launches) {
-    if (nblocks <= 0) return cudaSuccess;
-    k_m2m<R><<<unsigned(nblocks), EXP_THREADS, 0, st>>>(tasks, ntasks, insts, start, me);
-    PF_LAUNCHED(1);
-    return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
-// L2L: one thread per (child box, output coefficient); adds the parent's
-// local expansion, translated, to the child's.  Task = (instance, child
-// level l); units = 4^l * p, row-major.
-// ----------------------------------------------------------------------------
-template <typename R>
-__global__ void __launch_bounds__(EXP_THREADS) k_l2l(const Task *__restrict__ tasks, int ntasks,
-                                                     const InstDesc *__restrict__ insts,
-                                                     const uint32_t *__restrict__ start,
-                                                     typename Cplx<R>::T *__restrict__ le) {
-    using C2 = typename Cplx<R>::T;
-    const int ti = find_task(tasks, ntasks, blockIdx.x);
-    const Task t = tasks[ti];
-    const int64_t u = (int64_t(blockIdx.x) - t.block0) * EXP_THREADS + threadIdx.x;
-    if (u >= t.count) return;
-    const InstDesc &d = insts[t.inst];
-    const int p = d.p, l = t.level;
-    const int64_t box = u / p;
-    const int n = int(u - box * p);
-    const uint32_t ix = uint32_t(box & ((int64_t(1) << l) - 1)), iy = uint32_t(box >> l);
-    if (!box_count(start + d.soff, d.L, l, morton_key(ix, iy))) return;
-    const int c = int((ix & 1u) | ((iy & 1u) << 1));
-    const C2 *tab = static_cast<const C2 *>(d.t_l2l) + (size_t(c) * p + n) * p;
-    const C2 *par = le + d.eoff + (lvl_off(l - 1) + box_index(l - 1, ix >> 1, iy >> 1)) * p;
-    C2 s = mk2<R>(R(0), R(0));
-    for (int m = n; m < p; ++m) s = cfma(tab[m], par[m], s);
-    C2 *dst = le + d.eoff + (lvl_off(l) + box_index(l, ix, iy)) * p + n;
-    C2 o = *dst;
-    o.x += s.x;
-    o.y += s.y;
-    *dst = o;
-}
-
-template <typename R>
-cudaError_t launch_l2l(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, typename Cplx<R>::T *le, cudaStream_t st,
-                       uint64_t *launches) {
-    if (nblocks <= 0) return cudaSuccess;
-    k_l2l<R><<<unsigned(nblocks), EXP_THREADS, 0, st>>>(tasks, ntasks, insts, start, le);
-    PF_LAUNCHED(1);
-    return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
 // M2L (SIMT): one warp per target box; lane m owns output coefficient m (and
 // m + 32).  The source ME is staged in per-warp shared memory and read as a
 // broadcast; operator rows come through L1.  Task = (instance, level l),
@@ -888,14 +787,6 @@ template cudaError_t launch_p2m<float>(const uint2 *, const uint32_t *, int64_t,
                                        int, const uint32_t *, const double *, const double *,
                                        const double *, const float4 *, float2 *, cudaStream_t,
                                        uint64_t *);
-template cudaError_t launch_m2m<double>(const Task *, int, int64_t, const InstDesc *,
-                                        const uint32_t *, double2 *, cudaStream_t, uint64_t *);
-template cudaError_t launch_m2m<float>(const Task *, int, int64_t, const InstDesc *,
-                                       const uint32_t *, float2 *, cudaStream_t, uint64_t *);
-template cudaError_t launch_l2l<double>(const Task *, int, int64_t, const InstDesc *,
-                                        const uint32_t *, double2 *, cudaStream_t, uint64_t *);
-template cudaError_t launch_l2l<float>(const Task *, int, int64_t, const InstDesc *,
-                                       const uint32_t *, float2 *, cudaStream_t, uint64_t *);
 template cudaError_t launch_m2l<double>(const Task *, int, int64_t, const InstDesc *,
                                         const uint32_t *, const double2 *, double2 *,
                                         const uint32_t *, int, cudaStream_t, uint64_t *);

@@ -62,8 +62,10 @@ cudaError_t launch_gather_mixed(const float4 *recu, const uint32_t *perm, float4
 // Operator tables for p (FP64 build, also rounded to FP32), device-resident.
 struct OpTables {
     int p = 0;
-    double2 *m2m64 = nullptr, *l2l64 = nullptr, *m2l64 = nullptr;
-    float2 *m2m32 = nullptr, *l2l32 = nullptr, *m2l32 = nullptr;
+    double *shift64 = nullptr;  // M2M and L2L (shifts.cu)
+    float *shift32 = nullptr;
+    double2 *m2l64 = nullptr;
+    float2 *m2l32 = nullptr;
     double *m2l64r = nullptr; // FP64 M2L by orbits (vortex kernel, m2l64.cu)
     float *m2l_tc = nullptr;  // hi/lo B images for the tensor-core M2L (p <= 24)
     float *m2l_tcb = nullptr; // ... the four target classes side by side (block units)
@@ -93,10 +95,7 @@ cudaError_t launch_p2m(const uint2 *occ, const uint32_t *ctrl, int64_t max_occ,
 // M2M, M2L and L2L skip boxes with no particles in their subtree (and M2L
 // skips empty sources): their coefficients would be exactly zero and are
 // never read.  start = the batch's leaf-start array.
-template <typename R>
-cudaError_t launch_m2m(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, typename Cplx<R>::T *me, cudaStream_t st,
-                       uint64_t *launches);
+//
 // For levels that also have tensor-core units (InstDesc::tc_unit0 >= 0) the
 // SIMT M2L skips the boxes of dense units (ucount, dense_pct).
 template <typename R>
@@ -104,10 +103,25 @@ cudaError_t launch_m2l(const Task *tasks, int ntasks, int64_t nblocks, const Ins
                        const uint32_t *start, const typename Cplx<R>::T *me,
                        typename Cplx<R>::T *le, const uint32_t *ucount, int dense_pct,
                        cudaStream_t st, uint64_t *launches);
+// ---- shifts.cu -------------------------------------------------------------
+// M2M (into the tasks' parents) and L2L (from them) of one level per instance;
+// ex: ME or LE.  A task: instance, the parents' level; units: shift_units
+// blocks.  smem: the largest shift_smem of the orders in the plan.
+// InstDesc::t_shift = host_shift_table of its order and kernel.
+void host_shift_table(int p, int kernel, std::vector<double> &out);
+int64_t shift_units(int p, int level);
+size_t shift_smem(int p, bool fp64, bool top);
 template <typename R>
-cudaError_t launch_l2l(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, typename Cplx<R>::T *le, cudaStream_t st,
-                       uint64_t *launches);
+cudaError_t launch_shift(bool l2l, const Task *tasks, int ntasks, int64_t nblocks, size_t smem,
+                         const InstDesc *insts, const uint32_t *start, typename Cplx<R>::T *ex,
+                         cudaStream_t st, uint64_t *launches);
+// Mixed path: the parents' levels 2 .. kShiftTop of every instance in one
+// launch, a block each.  (64 + 16 parents take about a launch's time there;
+// the FP64 path spreads them over the SMs.)
+constexpr int kShiftTop = 3;
+cudaError_t launch_shift_top(bool l2l, int ninst, size_t smem, const InstDesc *insts,
+                             const uint32_t *start, float2 *ex, cudaStream_t st,
+                             uint64_t *launches);
 
 // ---- m2l_tc.cu -------------------------------------------------------------
 // Tensor-core M2L (mixed path) for levels with at least 128 parent cells per
@@ -180,7 +194,7 @@ constexpr int M2L_WARPS = 4;      // warps per block
 // scheduling.
 constexpr int BOX_RUN = 8;
 constexpr int M2L_BOXES = M2L_WARPS * BOX_RUN;   // target boxes per block
-constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block for M2M / L2L
+constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block in the plan dump's M2M / L2L
 
 // ---- p2p.cu ----------------------------------------------------------------
 // Work list: items (inst, leaf, first target rank, target count) for every
