@@ -459,11 +459,14 @@ int petfmm_debug_m2l_images(int order, int kernel, int blocks, float *out, int64
  * (pointers in inst are not dereferenced).  Each task is written as five
  * int64 {range, instance, level, units, first block}; range 0 the scatter of
  * staged FP32 outputs to the caller's order (1024 blobs per block),
- * 1 leaf starts, 2 gather, 3 P2M, 4 P2P work list, 5 M2L (SIMT, units =
- * target boxes), 6 M2L on the tensor cores (units = CTAs), 7 tiled SIMT M2L
- * (units = CTAs), 100 + r the r-th M2M launch, 200 + r the r-th L2L launch,
- * as a context with default options would launch them.  Writes at most cap
- * tasks and returns the total count, or PETFMM_EINVAL. */
+ * 1 leaf starts, 2 gather, 3 P2M, 4 P2P work list, 5 M2L target boxes (every
+ * level), 6 M2L on the tensor cores (units = CTAs, row units), 7 the same in
+ * blocks, 70 + c the mixed path's levels without tensor-core units for orders
+ * up to 8, 12, 18 and 24 (units of 128 boxes of a class, or whole rows of 64),
+ * 100 + r the r-th M2M level, 200 + r the r-th L2L level (units = (box,
+ * coefficient) pairs), with default options.  Ranges 5 and 70 .. describe the
+ * work; its launches group M2L's and M2M / L2L's boxes their own way.  Writes
+ * at most cap tasks and returns the total count, or PETFMM_EINVAL. */
 int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, int64_t *out, int cap);
 
 /* Options. */
@@ -484,10 +487,9 @@ enum {
     PETFMM_OPT_M2L_TC = 5,     /* mixed path: 1 (default) M2L of levels >= 8 on the tensor
                                   cores (3xTF32; see PETFMM_OPT_TC_BLOCKS), 0 all levels
                                   on the FP32 SIMT kernels */
-    PETFMM_OPT_TC_DENSE = 6,   /* percent (0..100, default 1) of a tensor-core (or
-                                  tiled) unit's targets that must hold particles for the
-                                  unit to run there; sparser units use the per-box SIMT
-                                  kernel */
+    PETFMM_OPT_TC_DENSE = 6,   /* percent (0..100, default 1) of a tensor-core unit's
+                                  targets that must hold particles for the unit to run
+                                  there; sparser units use the per-box SIMT kernel */
     PETFMM_OPT_TC_SEG = 8,     /* widest tensor-core M2L unit in parent cells: 128
                                   (default), 256 or 512 */
     PETFMM_OPT_NEAR_TOL = 9,   /* mixed path: relative tolerance of the polynomial that
@@ -522,7 +524,7 @@ enum {
                                   parent cells (all four child classes) at levels >= 8,
                                   and at levels 5 to 7 when the evaluation has at least
                                   512 blocks there (a batch; a single tree runs those
-                                  levels on the tiled SIMT kernel in FP32); 1: blocks at every
+                                  levels on the SIMT orbit kernel, FP32); 1: blocks at every
                                   level >= 5; 2: row units (one child class, a segment
                                   of a parent row) at levels >= 8 and no blocks.
                                   Results differ by FP32 rounding only. */

@@ -59,16 +59,16 @@ struct InstDesc {
     const void *x, *y, *g;  // caller's arrays (storage type of the context)
     void *u, *v;
     const void *t_shift, *t_m2l;  // operator tables for this p (path's real type)
+    const void *t_m2l_box;        // mixed path: complex M2L operators of the per-box kernel
     const void *t_m2l_tc;               // tensor-core M2L operator images (mixed path)
     const void *t_m2l_tcb;              // ... side by side for the block units
     int64_t tc_unit0[MAX_L + 1];        // per level: first unit of this (instance, level)
                                         // in the tensor-core M2L launch, or -1
     int tc_segmax;                      // widest tensor-core unit (parent cells)
     uint32_t tc_levels;                 // bit l: level l's dense units run on the tensor
-                                        // cores (else, if tc_unit0[l] >= 0, on the
-                                        // tiled SIMT kernel)
-    uint32_t tcb_levels;                // bit l: ... on the tensor cores in 8 x 16 blocks
-                                        // (all four classes per block)
+                                        // cores as row units
+    uint32_t tcb_levels;                // bit l: ... in 8 x 16 blocks (all four classes
+                                        // per block); the other levels go by orbits
     // mixed-precision P2P constants (leaf units)
     float kappa;            // w^2 / (2 sigma^2): q = kappa * rho^2
     float cnear;            // w / (4 pi sigma^2)
@@ -283,59 +283,19 @@ __host__ __device__ __forceinline__ void tcb_unit_decode(int l, int64_t unit, in
     *Px0 = int(unit - (unit / nbx) * nbx) * TCB_BX;
 }
 
-// Units of the tiled SIMT M2L: a segment of M2L_TILE_SEG parent cells of one
-// parent row, or, where rows are shorter, R whole rows of together at most
-// M2L_TILE_ROWS_BOXES target boxes (half a full unit: a shallow level has few
-// boxes, and smaller units keep more CTAs in flight).
-constexpr int M2L_TILE_SEG = 128;
-constexpr int M2L_TILE_ROWS_BOXES = 64;
-
-__host__ __device__ __forceinline__ void tile_geom(int l, int *R, int *seg) {
-    const int W = 1 << (l - 1);
-    *seg = W < M2L_TILE_SEG ? W : M2L_TILE_SEG;
-    const int r = W < M2L_TILE_SEG ? M2L_TILE_ROWS_BOXES / *seg : 1;
-    *R = r < 1 ? 1 : r < W ? r : W;
-}
-
-__host__ __device__ __forceinline__ int64_t tile_units(int l) {
-    const int W = 1 << (l - 1);
-    int R, s;
-    tile_geom(l, &R, &s);
-    return int64_t(4) * (W / R) * (W / s);
-}
-
-__host__ __device__ __forceinline__ void tile_unit_decode(int l, int64_t unit, int *c, int *Py0,
-                                                          int *R, int *Px0, int *seg) {
-    const int W = 1 << (l - 1);
-    tile_geom(l, R, seg);
-    const int nseg = W / *seg, nrow = W / *R;
-    *c = int(unit / (int64_t(nrow) * nseg));
-    const int64_t rem = unit - int64_t(*c) * nrow * nseg;
-    *Py0 = int(rem / nseg) * *R;
-    *Px0 = int(rem - (rem / nseg) * nseg) * *seg;
-}
-
-// Unit of box (c, Py, Px) of level l (tensor-core or tiled units) and the
-// number of its targets.
+// Unit of box (c, Py, Px) of a level with tensor-core units, and the number
+// of its targets.
 __host__ __device__ __forceinline__ int64_t unit_of(const InstDesc &d, int l, int c, int Py,
                                                     int Px, int *nbox) {
     if ((d.tc_levels >> l) & 1u) {
         *nbox = tc_seg(l, d.tc_segmax);
         return tc_unit_of(l, d.tc_segmax, c, Py, Px);
     }
-    const int W = 1 << (l - 1);
-    if ((d.tcb_levels >> l) & 1u) {
-        (void)c;
-        *nbox = 4 * TCB_BX * TCB_BY;
-        return int64_t(Py / TCB_BY) * (W / TCB_BX) + Px / TCB_BX;
-    }
-    int R, s;
-    tile_geom(l, &R, &s);
-    *nbox = R * s;
-    return (int64_t(c) * (W / R) + Py / R) * (W / s) + Px / s;
+    *nbox = 4 * TCB_BX * TCB_BY;
+    return int64_t(Py / TCB_BY) * ((1 << (l - 1)) / TCB_BX) + Px / TCB_BX;
 }
 
-// A unit goes to the tensor cores (or the tiled SIMT kernel) when at least
+// A unit goes to the tensor cores when at least
 // dense_pct percent of its targets hold particles; the per-box SIMT kernel
 // takes the boxes of the others.
 __host__ __device__ __forceinline__ bool tc_unit_dense(uint32_t count, int seg, int dense_pct) {

@@ -70,20 +70,15 @@ struct Plan {
     std::vector<InstDesc> inst;
     std::vector<Task> tasks;
     TaskRange outscatter, start, particles, leaves_p2m, leaves_wl, m2l, m2l_tc, m2l_tcb, m2l_log;
-    // FP64 vortex M2L by orbits: (box, coefficient) pairs per thread, shared memory
-    TaskRange m2l64;
-    int m2l64_ni = 0;
-    size_t m2l64_smem = 0;
-    // tiled SIMT M2L, one launch per order class (p <= 8, 12, 18, 24): each
-    // launch's kernel is specialised for its class's largest order
+    // M2L by orbits (FP64 path; mixed path, levels without tensor-core units):
+    // (box, coefficient) pairs per thread, shared memory
+    TaskRange orbits;
+    int orbit_ni = 0;
+    size_t orbit_smem = 0;
+    // the plan dump's units of 128 (or whole rows of 64) target boxes of those
+    // levels, by order class (p <= 8, 12, 18, 24)
     static constexpr int kTileClasses = 4;
     TaskRange m2l_tile[kTileClasses];
-    int tile_pmax[kTileClasses] = {};
-    int64_t tile_blocks() const {
-        int64_t b = 0;
-        for (const TaskRange &r : m2l_tile) b += r.nblocks;
-        return b;
-    }
     // M2M and L2L, in launch order: a task's units are runs of parents (on the
     // mixed path the top levels run apart, shift_top)
     std::vector<TaskRange> up, down;
@@ -424,23 +419,29 @@ void flatten_tasks(Plan &pl) {
     put(pl.m2l_tcb);
     for (TaskRange &r : pl.m2l_tile) put(r);
     put(pl.m2l_log);
-    put(pl.m2l64);
+    put(pl.orbits);
     for (TaskRange &r : pl.up) put(r);
     for (TaskRange &r : pl.down) put(r);
     for (TaskRange &r : pl.m2m) put(r);
     for (TaskRange &r : pl.l2l) put(r);
 }
 
-// order class of the tiled M2L launches: p <= 8, 12, 18, 24
 // Fewest block units at levels 5 to 7 for which those levels run as blocks
-// rather than on the tiled SIMT kernel (a batch of 512 trees has 3,260; one
-// tree, at most 42).
+// rather than by orbits (a batch of 512 trees has 3,260; one tree, at most 42).
 constexpr int64_t kTcbShallowMinUnits = 512;
 
-// Units of 512 (box, coefficient) pairs from which the FP64 M2L uses them: two
-// for each of 152 SMs.
-constexpr int64_t kM2L64LargeUnits = 304;
+// Units of 256 (box, coefficient) pairs from which the FP64 path's M2L by
+// orbits uses them, four for each of 152 SMs: at 1,048,576 blobs, L = 8, they
+// take 1.97 ms against 2.09 for units of 128, at 10,000, L = 4, 0.064 against
+// 0.036.  On the mixed path units of 128 were as fast or faster everywhere.
+constexpr int64_t kOrbitLargeUnits = 608;
 
+// The plan dump's units of a level without tensor-core units.
+int64_t dump_tile_units(int l) {
+    const int W = 1 << (l - 1), seg = std::min(W, 128);
+    const int rows = W < 128 ? std::max(1, std::min(64 / seg, W)) : 1;
+    return int64_t(4) * (W / rows) * (W / seg);
+}
 int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
 
 // Laplace kernel, mixed path: blobs per leaf (empty ones included) up to which
@@ -542,21 +543,19 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
                 add_task(pl.m2l_tc, i, l, m2l_tc_units(l, tc_segmax), 1);
                 pl.tc_smem = std::max(pl.tc_smem, m2l_tc_smem_bytes(d.p, m2l_tc_seg(l, tc_segmax)));
             }
-            add_task(pl.m2l, i, l, int64_t(1) << (2 * l), M2L_BOXES);
             if (kernel == KERNEL_LAPLACE) add_task(pl.m2l_log, i, l, int64_t(1) << (2 * l), 256);
         }
         items_cap += d.n / tpi + std::min<int64_t>(d.n, nleaf) + 1;
     }
     // the other levels of the mixed path: dense units on the tensor cores in
     // blocks of 8 x 16 parent cells (levels >= 8; levels 5 to 7 too when the
-    // plan has many blocks), the rest on the tiled SIMT kernel (their units
-    // follow the row units in the unit-count array: blocks, then the tile
-    // classes one by one)
+    // plan has many blocks; their units follow the row units in the unit-count
+    // array), the rest by orbits
     if (precision == PETFMM_MIXED) {
         int64_t base = pl.m2l_tc.nblocks;
         // levels 5 to 7: a batch fills the GPU with blocks; a single tree has
-        // few, and runs them on the tiled SIMT kernel (also in FP32, where
-        // the blocks' 3xTF32 adds about 1e-6 to the rel-L2 error)
+        // few, and runs them by orbits (also in FP32, where the blocks' 3xTF32
+        // adds about 1e-6 to the rel-L2 error)
         int64_t blocks = 0;
         for (int i = 0; i < ni; ++i)
             for (int l = 2; l <= std::min(pl.inst[i].L, 7); ++l)
@@ -576,36 +575,37 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
                 }
             }
         }
-        base += pl.m2l_tcb.nblocks;
-        for (int cls = 0; cls < Plan::kTileClasses; ++cls) {
-            TaskRange &tr = pl.m2l_tile[cls];
+    }
+    // per box: the sparse units of the tensor cores' levels (the dump lists
+    // every level); by orbits: the levels without tensor-core units
+    int64_t large = 0;
+    for (int i = 0; i < ni; ++i) {
+        const InstDesc &d = pl.inst[i];
+        for (int l = 2; l <= d.L; ++l) {
+            const bool tc = ((d.tc_levels | d.tcb_levels) >> l) & 1u;
+            if (tc || dump) add_task(pl.m2l, i, l, int64_t(1) << (2 * l), M2L_BOXES);
+            if (!tc) large += m2l_orbit_units(d.p, l, M2L_ORBIT_NI_MAX);
+        }
+    }
+    pl.orbit_ni = precision == PETFMM_FP64 && large >= kOrbitLargeUnits ? M2L_ORBIT_NI_MAX : 1;
+    for (int i = 0; i < ni; ++i) {
+        const InstDesc &d = pl.inst[i];
+        for (int l = 2; l <= d.L; ++l) {
+            if (((d.tc_levels | d.tcb_levels) >> l) & 1u) continue;
+            add_task(pl.orbits, i, l, m2l_orbit_units(d.p, l, pl.orbit_ni), 1);
+            pl.orbit_smem = std::max(pl.orbit_smem,
+                                     m2l_orbit_smem(d.p, pl.orbit_ni, precision == PETFMM_FP64));
+        }
+    }
+    if (dump && precision == PETFMM_MIXED)
+        for (int cls = 0; cls < Plan::kTileClasses; ++cls)
             for (int i = 0; i < ni; ++i) {
-                InstDesc &d = pl.inst[i];
-                if (!m2l_tile_supported(d.p) || tile_class(d.p) != cls) continue;
-                for (int l = 2; l <= d.L; ++l) {
-                    if (((d.tc_levels | d.tcb_levels) >> l) & 1u) continue;
-                    d.tc_unit0[l] = base + tr.nblocks;
-                    add_task(tr, i, l, m2l_tile_units(l), 1);
-                    pl.tile_pmax[cls] = std::max(pl.tile_pmax[cls], d.p);
-                }
+                const InstDesc &d = pl.inst[i];
+                if (d.p > 24 || tile_class(d.p) != cls) continue;
+                for (int l = 2; l <= d.L; ++l)
+                    if (!(((d.tc_levels | d.tcb_levels) >> l) & 1u))
+                        add_task(pl.m2l_tile[cls], i, l, dump_tile_units(l), 1);
             }
-            base += tr.nblocks;
-        }
-    }
-    // FP64 vortex M2L: large units where they still give every SM two blocks
-    // (an orbit's set-up is shared by more boxes), small ones otherwise
-    if (precision == PETFMM_FP64 && kernel == KERNEL_VORTEX) {
-        int64_t units = 0;
-        for (const InstDesc &d : pl.inst)
-            for (int l = 2; l <= d.L; ++l) units += m2l64_units(d.p, l, M2L64_NI_MAX);
-        pl.m2l64_ni = units >= kM2L64LargeUnits ? M2L64_NI_MAX : 1;
-        for (int i = 0; i < ni; ++i) {
-            const InstDesc &d = pl.inst[i];
-            for (int l = 2; l <= d.L; ++l)
-                add_task(pl.m2l64, i, l, m2l64_units(d.p, l, pl.m2l64_ni), 1);
-            pl.m2l64_smem = std::max(pl.m2l64_smem, m2l64_smem(d.p, pl.m2l64_ni));
-        }
-    }
     // M2M rounds: round r computes level L_i - 1 - r of every instance, down to
     // the first level the top launch does not take; L2L rounds start there
     const int bottom = precision == PETFMM_FP64 ? 2 : kShiftTop + 1;
@@ -660,11 +660,11 @@ int attach_tables(petfmm_ctx *c, Plan &pl) {
         if (!t) return err;
         if (c->precision == PETFMM_FP64) {
             d.t_shift = t->shift64;
-            if (c->kernel == KERNEL_VORTEX) d.t_m2l = t->m2l64r;
-            else d.t_m2l = t->m2l64;
+            d.t_m2l = t->orbit64;
         } else {
             d.t_shift = t->shift32;
-            d.t_m2l = t->m2l32;
+            d.t_m2l = t->orbit32;
+            d.t_m2l_box = t->m2l32;
             d.t_m2l_tc = t->m2l_tc;
             d.t_m2l_tcb = t->m2l_tcb;
         }
@@ -731,10 +731,8 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     if (!pl.tasks.empty()) k.add(pl.tasks.data(), pl.tasks.size() * sizeof(Task));
     auto range = [&](const TaskRange &r) { k.put(r.first); k.put(r.count); k.put(r.nblocks); };
     for (const TaskRange *r : {&pl.outscatter, &pl.start, &pl.particles, &pl.leaves_p2m, &pl.leaves_wl,
-                               &pl.m2l, &pl.m2l_tc, &pl.m2l_tcb, &pl.m2l_log, &pl.m2l64})
+                               &pl.m2l, &pl.m2l_tc, &pl.m2l_tcb, &pl.m2l_log, &pl.orbits})
         range(*r);
-    for (const TaskRange &r : pl.m2l_tile) range(r);
-    for (int cls = 0; cls < Plan::kTileClasses; ++cls) k.put(pl.tile_pmax[cls]);
     for (const TaskRange &r : pl.up) range(r);
     for (const TaskRange &r : pl.down) range(r);
     k.put(pl.up.size()); k.put(pl.shift_smem); k.put(pl.shift_top); k.put(pl.shift_top_smem);
@@ -742,7 +740,7 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     k.put(pl.N); k.put(pl.nleaves); k.put(pl.nstart); k.put(pl.ncoef); k.put(pl.items_cap);
     k.put(pl.nbits); k.put(pl.pmax); k.put(pl.deg); k.put(pl.general);
     k.put(pl.tc_smem); k.put(pl.tcb_pmax); k.put(grid);
-    k.put(pl.m2l64_ni); k.put(pl.m2l64_smem);
+    k.put(pl.orbit_ni); k.put(pl.orbit_smem);
     k.put(pl.sm_degrees); k.put(pl.sm_row); k.put(pl.sm_rows); k.put(pl.pairs_any);
     k.put(pl.direct); k.put(pl.items_any); k.put(c->p2p_mode);
     k.put(c->precision); k.put(c->dtype); k.put(c->timing); k.put(c->p2p_mode); k.put(c->poison);
@@ -823,7 +821,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     PF_TRY(ensure(c->occ, size_t(pl.nleaves) * sizeof(uint2), st));
     if (pl.items_any) PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
     PF_TRY(ensure(c->ucount,
-                  size_t(pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks + pl.tile_blocks()) * sizeof(uint32_t),
+                  size_t(pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks) * sizeof(uint32_t),
                   st));
     if (mixed && (pl.direct || pl.items_any)) PF_TRY(ensure(c->own, size_t(N) * sizeof(float2), st));
     SmBufs sm{};
@@ -998,7 +996,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                  static_cast<float2 *>(c->me.p), xs, lc));
     stage_mark_on(c, PETFMM_STAGE_M2L, xs);
     uint32_t *ucount = nullptr;
-    if (pl.m2l_tc.count || pl.m2l_tcb.count || pl.tile_blocks()) {
+    if (pl.m2l_tc.count || pl.m2l_tcb.count) {
         ucount = static_cast<uint32_t *>(c->ucount.p);
         if (pl.m2l_tc.count)
             PF_CUDA(launch_tc_unit_count(dtask + pl.m2l_tc.first, pl.m2l_tc.count,
@@ -1007,30 +1005,23 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
             PF_CUDA(launch_tc_unit_count(dtask + pl.m2l_tcb.first, pl.m2l_tcb.count,
                                          pl.m2l_tcb.nblocks, dinst, start,
                                          ucount + pl.m2l_tc.nblocks, xs, lc));
-        int64_t base = pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks;
-        for (const TaskRange &tr : pl.m2l_tile) {
-            if (tr.count)
-                PF_CUDA(launch_tc_unit_count(dtask + tr.first, tr.count, tr.nblocks, dinst, start,
-                                             ucount + base, xs, lc));
-            base += tr.nblocks;
-        }
     }
-    if (pl.m2l.count) {
+    if (pl.orbits.count) {
         if (mixed)
-            PF_CUDA(launch_m2l<float>(dtask + pl.m2l.first, pl.m2l.count, pl.m2l.nblocks, dinst,
-                                      start, static_cast<const float2 *>(c->me.p),
-                                      static_cast<float2 *>(c->le.p), ucount, c->tc_dense_pct,
-                                      xs, lc));
-        else if (pl.m2l64.count)
-            PF_CUDA(launch_m2l64(dtask + pl.m2l64.first, pl.m2l64.count, pl.m2l64.nblocks,
-                                 pl.m2l64_ni, pl.m2l64_smem, dinst, start,
-                                 static_cast<const double2 *>(c->me.p),
-                                 static_cast<double2 *>(c->le.p), xs, lc));
+            PF_CUDA(launch_m2l_orbits<float>(dtask + pl.orbits.first, pl.orbits.count,
+                                             pl.orbits.nblocks, pl.orbit_ni, pl.orbit_smem, dinst,
+                                             start, static_cast<const float2 *>(c->me.p),
+                                             static_cast<float2 *>(c->le.p), xs, lc));
         else
-            PF_CUDA(launch_m2l<double>(dtask + pl.m2l.first, pl.m2l.count, pl.m2l.nblocks, dinst,
-                                       start, static_cast<const double2 *>(c->me.p),
-                                       static_cast<double2 *>(c->le.p), nullptr, 0, xs, lc));
+            PF_CUDA(launch_m2l_orbits<double>(dtask + pl.orbits.first, pl.orbits.count,
+                                              pl.orbits.nblocks, pl.orbit_ni, pl.orbit_smem, dinst,
+                                              start, static_cast<const double2 *>(c->me.p),
+                                              static_cast<double2 *>(c->le.p), xs, lc));
     }
+    if (pl.m2l.count)
+        PF_CUDA(launch_m2l(dtask + pl.m2l.first, pl.m2l.count, pl.m2l.nblocks, dinst, start,
+                           static_cast<const float2 *>(c->me.p), static_cast<float2 *>(c->le.p),
+                           ucount, c->tc_dense_pct, xs, lc));
     if (pl.m2l_tc.count) {
         // spin_limit < 0: zero-iteration budget (tests the timeout report)
         const long long spin = c->spin_limit > 0 ? c->spin_limit : c->spin_limit < 0 ? 0 : (1LL << 26);
@@ -1047,18 +1038,6 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                static_cast<float2 *>(c->le.p), ucount + pl.m2l_tc.nblocks,
                                c->tc_dense_pct, pl.tcb_pmax, spin, c->tc_pipe,
                                reinterpret_cast<int *>(ctrl + CTRL_STATUS), xs, lc));
-    }
-    {
-        int64_t base = pl.m2l_tc.nblocks + pl.m2l_tcb.nblocks;
-        for (int cls = 0; cls < Plan::kTileClasses; ++cls) {
-            const TaskRange &tr = pl.m2l_tile[cls];
-            if (tr.count)
-                PF_CUDA(launch_m2l_tile(dtask + tr.first, tr.count, tr.nblocks, pl.tile_pmax[cls],
-                                        dinst, start, static_cast<const float2 *>(c->me.p),
-                                        static_cast<float2 *>(c->le.p), ucount + base,
-                                        c->tc_dense_pct, xs, lc));
-            base += tr.nblocks;
-        }
     }
     if (pl.m2l_log.count) {
         if (mixed)

@@ -20,6 +20,7 @@
 #include <cmath>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "kernels.cuh"
@@ -274,40 +275,40 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
     cudaError_t e = upload_il();
     if (e != cudaSuccess) return e;
     t->p = p;
-    std::vector<double> m2l(size_t(2) * 40 * p * p), shift;
+    std::vector<double> m2l(size_t(2) * 40 * p * p), shift, orbit;
     (kernel == KERNEL_LAPLACE ? host_lap_m2l_table : host_m2l_table)(p, m2l.data());
     host_shift_table(p, kernel, shift);
-    std::vector<float> m2l32(m2l.begin(), m2l.end()), shift32(shift.begin(), shift.end());
-    auto up = [&](void **dst, const void *src, size_t bytes) -> cudaError_t {
-        cudaError_t r = cudaMalloc(dst, bytes);
-        if (r != cudaSuccess) return r;
-        return cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
+    host_m2l_orbit_table(p, kernel, orbit);
+    std::vector<float> m2l32(m2l.begin(), m2l.end()), shift32(shift.begin(), shift.end()),
+        orbit32(orbit.begin(), orbit.end());
+    // one allocation and one copy for all of them
+    std::vector<unsigned char> blob;
+    std::vector<std::pair<void **, size_t>> at;
+    auto put = [&](void **dst, const void *src, size_t bytes) {
+        at.push_back({dst, blob.size()});
+        const unsigned char *b = static_cast<const unsigned char *>(src);
+        blob.insert(blob.end(), b, b + bytes);
+        blob.resize((blob.size() + 255) / 256 * 256);
     };
-    if ((e = up((void **)&t->shift64, shift.data(), shift.size() * 8)) != cudaSuccess) return e;
-    if ((e = up((void **)&t->shift32, shift32.data(), shift32.size() * 4)) != cudaSuccess) return e;
-    if ((e = up((void **)&t->m2l64, m2l.data(), m2l.size() * 8)) != cudaSuccess) return e;
-    if (kernel == KERNEL_VORTEX) {
-        std::vector<double> r;
-        host_m2l64_table(p, r);
-        if ((e = up((void **)&t->m2l64r, r.data(), r.size() * 8)) != cudaSuccess) return e;
-    }
-    if ((e = up((void **)&t->m2l32, m2l32.data(), m2l32.size() * 4)) != cudaSuccess) return e;
+    put((void **)&t->shift64, shift.data(), shift.size() * 8);
+    put((void **)&t->shift32, shift32.data(), shift32.size() * 4);
+    put((void **)&t->orbit64, orbit.data(), orbit.size() * 8);
+    put((void **)&t->orbit32, orbit32.data(), orbit32.size() * 4);
+    put((void **)&t->m2l32, m2l32.data(), m2l32.size() * 4);
     if (((2 * p + 15) & ~15) <= 48) {
         std::vector<float> img;
         host_m2l_tc_images(p, kernel, img);
-        if ((e = up((void **)&t->m2l_tc, img.data(), img.size() * 4)) != cudaSuccess) return e;
+        put((void **)&t->m2l_tc, img.data(), img.size() * 4);
         host_m2l_tcb_images(p, kernel, img);
-        if ((e = up((void **)&t->m2l_tcb, img.data(), img.size() * 4)) != cudaSuccess) return e;
+        put((void **)&t->m2l_tcb, img.data(), img.size() * 4);
     }
-    return cudaSuccess;
+    if ((e = cudaMalloc(&t->blob, blob.size())) != cudaSuccess) return e;
+    for (const auto &x : at) *x.first = static_cast<unsigned char *>(t->blob) + x.second;
+    return cudaMemcpy(t->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice);
 }
 
 void free_op_tables(OpTables *t) {
-    cudaFree(t->shift64); cudaFree(t->shift32); cudaFree(t->m2l64);
-    cudaFree(t->m2l64r);
-    cudaFree(t->m2l32);
-    cudaFree(t->m2l_tc);
-    cudaFree(t->m2l_tcb);
+    cudaFree(t->blob);
     *t = OpTables();
 }
 
@@ -640,16 +641,16 @@ cudaError_t launch_p2m(const uint2 *occ, const uint32_t *ctrl, int64_t max_occ,
 // broadcast; operator rows come through L1.  Task = (instance, level l),
 // units = 4^l target boxes, row-major.
 // ----------------------------------------------------------------------------
-template <typename R>
 __global__ void __launch_bounds__(M2L_WARPS * 32) k_m2l(const Task *__restrict__ tasks,
                                                         int ntasks,
                                                         const InstDesc *__restrict__ insts,
                                                         const uint32_t *__restrict__ start,
-                                                        const typename Cplx<R>::T *__restrict__ me,
-                                                        typename Cplx<R>::T *__restrict__ le,
+                                                        const float2 *__restrict__ me,
+                                                        float2 *__restrict__ le,
                                                         const uint32_t *__restrict__ ucount,
                                                         int dense_pct) {
-    using C2 = typename Cplx<R>::T;
+    using R = float;
+    using C2 = float2;
     __shared__ C2 sa[M2L_WARPS][MAX_P];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int ti = find_task(tasks, ntasks, blockIdx.x);
@@ -680,7 +681,7 @@ __global__ void __launch_bounds__(M2L_WARPS * 32) k_m2l(const Task *__restrict__
         todo &= todo - 1;
         const int ix = int(box & (nside - 1)), iy = int(box >> l);
         const int c = (ix & 1) | ((iy & 1) << 1);
-        const C2 *tab = static_cast<const C2 *>(d.t_m2l);
+        const C2 *tab = static_cast<const C2 *>(d.t_m2l_box);
         const C2 *lev = me + d.eoff + lvl_off(l) * p;
         C2 acc0 = mk2<R>(R(0), R(0)), acc1 = mk2<R>(R(0), R(0));
         for (int e = 0; e < 27; ++e) {
@@ -707,14 +708,12 @@ __global__ void __launch_bounds__(M2L_WARPS * 32) k_m2l(const Task *__restrict__
     }
 }
 
-template <typename R>
 cudaError_t launch_m2l(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, const typename Cplx<R>::T *me,
-                       typename Cplx<R>::T *le, const uint32_t *ucount, int dense_pct,
-                       cudaStream_t st, uint64_t *launches) {
+                       const uint32_t *start, const float2 *me, float2 *le, const uint32_t *ucount,
+                       int dense_pct, cudaStream_t st, uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
-    k_m2l<R><<<unsigned(nblocks), M2L_WARPS * 32, 0, st>>>(tasks, ntasks, insts, start, me, le,
-                                                          ucount, dense_pct);
+    k_m2l<<<unsigned(nblocks), M2L_WARPS * 32, 0, st>>>(tasks, ntasks, insts, start, me, le, ucount,
+                                                       dense_pct);
     PF_LAUNCHED(1);
     return cudaGetLastError();
 }
@@ -787,12 +786,6 @@ template cudaError_t launch_p2m<float>(const uint2 *, const uint32_t *, int64_t,
                                        int, const uint32_t *, const double *, const double *,
                                        const double *, const float4 *, float2 *, cudaStream_t,
                                        uint64_t *);
-template cudaError_t launch_m2l<double>(const Task *, int, int64_t, const InstDesc *,
-                                        const uint32_t *, const double2 *, double2 *,
-                                        const uint32_t *, int, cudaStream_t, uint64_t *);
-template cudaError_t launch_m2l<float>(const Task *, int, int64_t, const InstDesc *,
-                                       const uint32_t *, const float2 *, float2 *,
-                                       const uint32_t *, int, cudaStream_t, uint64_t *);
 
 PF_DEFINE_CHECK_READER(expansions)
 

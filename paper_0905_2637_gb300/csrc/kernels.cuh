@@ -62,11 +62,12 @@ cudaError_t launch_gather_mixed(const float4 *recu, const uint32_t *perm, float4
 // Operator tables for p (FP64 build, also rounded to FP32), device-resident.
 struct OpTables {
     int p = 0;
+    void *blob = nullptr;       // the allocation behind the tables
     double *shift64 = nullptr;  // M2M and L2L (shifts.cu)
     float *shift32 = nullptr;
-    double2 *m2l64 = nullptr;
-    float2 *m2l32 = nullptr;
-    double *m2l64r = nullptr; // FP64 M2L by orbits (vortex kernel, m2l64.cu)
+    float2 *m2l32 = nullptr;    // per-box M2L of the tensor cores' sparse units
+    double *orbit64 = nullptr;  // M2L by orbits (m2l_orbits.cu)
+    float *orbit32 = nullptr;
     float *m2l_tc = nullptr;  // hi/lo B images for the tensor-core M2L (p <= 24)
     float *m2l_tcb = nullptr; // ... the four target classes side by side (block units)
 };
@@ -96,13 +97,12 @@ cudaError_t launch_p2m(const uint2 *occ, const uint32_t *ctrl, int64_t max_occ,
 // skips empty sources): their coefficients would be exactly zero and are
 // never read.  start = the batch's leaf-start array.
 //
-// For levels that also have tensor-core units (InstDesc::tc_unit0 >= 0) the
-// SIMT M2L skips the boxes of dense units (ucount, dense_pct).
-template <typename R>
+// Per-box M2L (mixed path) of the boxes that the tensor-core units of the
+// tasks' levels leave: those of sparse units (ucount, dense_pct).
 cudaError_t launch_m2l(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
-                       const uint32_t *start, const typename Cplx<R>::T *me,
-                       typename Cplx<R>::T *le, const uint32_t *ucount, int dense_pct,
-                       cudaStream_t st, uint64_t *launches);
+                       const uint32_t *start, const float2 *me, float2 *le, const uint32_t *ucount,
+                       int dense_pct, cudaStream_t st, uint64_t *launches);
+
 // ---- shifts.cu -------------------------------------------------------------
 // M2M (into the tasks' parents) and L2L (from them) of one level per instance;
 // ex: ME or LE.  A task: instance, the parents' level; units: shift_units
@@ -149,8 +149,7 @@ cudaError_t launch_m2l_logterm(const Task *tasks, int ntasks, int64_t nblocks,
                                const InstDesc *insts, const uint32_t *start,
                                const typename Cplx<R>::T *me, typename Cplx<R>::T *le,
                                cudaStream_t st, uint64_t *launches);
-// ucount[u] = targets holding particles in unit u of the launch (tensor-core
-// or tiled SIMT units; block index = unit).
+// ucount[u] = targets holding particles in unit u of the launch.
 cudaError_t launch_tc_unit_count(const Task *tasks, int ntasks, int64_t nunits,
                                  const InstDesc *insts, const uint32_t *start, uint32_t *ucount,
                                  cudaStream_t st, uint64_t *launches);
@@ -161,29 +160,21 @@ cudaError_t launch_m2l_tc(const Task *tasks, int ntasks, int64_t nblocks, const 
                           const uint32_t *ucount, int dense_pct, size_t smem_bytes,
                           long long spin_limit, int *status, cudaStream_t st, uint64_t *launches);
 
-// ---- m2l_tile.cu -----------------------------------------------------------
-// Tiled SIMT M2L (mixed path, p <= 24) for the dense units of the levels the
-// tensor cores do not take; units as above with M2L_TILE_SEG parent cells.
-bool m2l_tile_supported(int p);
-int64_t m2l_tile_units(int level);
-size_t m2l_tile_smem_bytes(int p, int level);
-cudaError_t launch_m2l_tile(const Task *tasks, int ntasks, int64_t nblocks, int pmax,
-                            const InstDesc *insts, const uint32_t *start, const float2 *me,
-                            float2 *le, const uint32_t *ucount, int dense_pct, cudaStream_t st,
-                            uint64_t *launches);
-
-// ---- m2l64.cu --------------------------------------------------------------
-// FP64 M2L of the vortex kernel by orbits of quarter turns (InstDesc::t_m2l =
-// the host_m2l64_table of its order).  A unit (one block) is a run of target
-// boxes of one class holding ni 128 (box, coefficient) pairs; ni is 1 or
-// M2L64_NI_MAX, the same results either way.
-constexpr int M2L64_NI_MAX = 4;
-void host_m2l64_table(int p, std::vector<double> &out);
-int64_t m2l64_units(int p, int level, int ni);
-size_t m2l64_smem(int p, int ni);
-cudaError_t launch_m2l64(const Task *tasks, int ntasks, int64_t nblocks, int ni, size_t smem,
-                         const InstDesc *insts, const uint32_t *start, const double2 *me,
-                         double2 *le, cudaStream_t st, uint64_t *launches);
+// ---- m2l_orbits.cu ---------------------------------------------------------
+// M2L by orbits of quarter turns: the FP64 path, and the mixed path's levels
+// that the tensor cores do not take (InstDesc::t_m2l = the
+// host_m2l_orbit_table of its order and kernel).  A unit (one block) is a run
+// of target boxes of one class holding about ni 128 (box, coefficient) pairs;
+// ni is 1 or M2L_ORBIT_NI_MAX, the same results either way.
+constexpr int M2L_ORBIT_NI_MAX = 2;  // (FP64 path only)
+void host_m2l_orbit_table(int p, int kernel, std::vector<double> &out);
+int64_t m2l_orbit_units(int p, int level, int ni);
+size_t m2l_orbit_smem(int p, int ni, bool fp64);
+template <typename R>
+cudaError_t launch_m2l_orbits(const Task *tasks, int ntasks, int64_t nblocks, int ni, size_t smem,
+                              const InstDesc *insts, const uint32_t *start,
+                              const typename Cplx<R>::T *me, typename Cplx<R>::T *le,
+                              cudaStream_t st, uint64_t *launches);
 
 // units of work per block of each expansion kernel (the host plans with them)
 constexpr int P2M_WARPS = 4;      // warps per block
