@@ -34,7 +34,10 @@
 // keys), 8^L + 1 leaf starts, the sorted particles (FP64 path: SoA x, y, z, q
 // in double; mixed path: float4 (xi, eta, zeta, q), the position relative to
 // the leaf centre in leaf widths), ME and LE of every level (8^l boxes in
-// Morton order, level l at box offset (8^l - 1) / 7), the operator tables.
+// Morton order, level l at box offset (8^l - 1) / 7), the operator tables, and
+// on the mixed path the parts of the pairwise near field, 26 + 1 float4 planes
+// of one entry per charge (432 B a charge; without room for them, or above
+// 2^26 charges, every leaf pair is summed one-sided).
 // Every sum runs in a fixed order: results are bitwise reproducible.
 #include <algorithm>
 #include <cmath>
@@ -1771,26 +1774,154 @@ __device__ __forceinline__ void store3(void *o, int64_t i, double v) {
 }
 
 // ---------------------------------------------------------------------------
-// The near field's work items: leaf b with n_b particles gives ceil(n_b / 32)
-// items (b, first sorted rank of the chunk), in leaf order (a hot leaf's
-// chunks go to consecutive warps, so they spread over the SMs).
-__global__ void __launch_bounds__(256) k3_near_count(const uint32_t *__restrict__ start,
-                                                     int64_t nleaf, uint32_t *__restrict__ cnt) {
-    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    cnt[b] = (start[b + 1] - start[b] + 31u) / 32u;
+// Near field of the mixed path.  Leaf pairs of at least P3_PAIR_MIN charges
+// each are evaluated pairwise (k3_pairs): 1/r and 1/r^3 of a pair of charges
+// serve both, 18 FP32 operations where two one-sided sums take 26 and two
+// rsqrt.  The other leaf pairs are summed one-sided (k3_near_directed), and a
+// last pass (k3_near_final) adds the parts and L2P.  Every part has one writer
+// and the parts are added in a fixed order.
+//
+// A pair item is (leaf A, group of the 13 forward directions); a heavier leaf
+// has more groups, so that no item outlasts the launch.  Parts: fwd[g] of A's
+// charges (from group g's neighbours; group 0 also the leaf itself), bwd[d] of
+// a leaf's charges from the leaf behind it in direction d, own (one-sided).
+// ---------------------------------------------------------------------------
+constexpr uint32_t P3_PAIR_MIN = 24;
+constexpr int P3_DIRS = 13;
+constexpr int P3_SLOTS = 2 * P3_DIRS;  // fwd[13], bwd[13]: planes of one float4 per charge
+
+// forward direction k of 13: (dx, dy, dz) with (dz, dy, dx) above zero
+__host__ __device__ __forceinline__ void fwd3(int k, int *dx, int *dy, int *dz) {
+    const int o = 14 + k;  // of 27, 13 the leaf itself
+    *dx = o % 3 - 1;
+    *dy = (o / 3) % 3 - 1;
+    *dz = o / 9 - 1;
 }
-__global__ void __launch_bounds__(256) k3_near_emit(const uint32_t *__restrict__ start,
-                                                    int64_t nleaf, const uint32_t *__restrict__ off,
-                                                    const uint32_t *__restrict__ nitems,
-                                                    int64_t cap, uint2 *__restrict__ items) {
-    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    const uint32_t s0 = start[b], k = (start[b + 1] - s0 + 31u) / 32u;
-    for (uint32_t c = 0; c < k; ++c) {
-        const int64_t o = int64_t(off[b]) + c;
-        if (o < cap && o < int64_t(*nitems)) items[o] = make_uint2(uint32_t(b), s0 + 32u * c);
+// groups of a leaf of n charges, and group g's directions [first, last)
+__host__ __device__ __forceinline__ int groups3(uint32_t n) {
+    return n <= 96 ? 2 : n <= 384 ? 4 : P3_DIRS;
+}
+__host__ __device__ __forceinline__ int group_first3(int g, int groups) {
+    return g * P3_DIRS / groups;
+}
+// leaf flags of the final pass: bit d: bwd[d] holds a part; bit 13: own does;
+// bit 14: fwd of the leaf's groups do
+constexpr uint32_t LF3_OWN = 1u << 13, LF3_FWD = 1u << 14;
+// counters: directed items, pair items, then per work class the pair items
+// counted and placed
+constexpr int C3_DIRECTED = 0, C3_PAIRS = 1, C3_COUNT = 2, C3_CLASSES = 64,
+              C3_PLACED = C3_COUNT + C3_CLASSES, C3_WORDS = C3_PLACED + C3_CLASSES;
+
+struct Near3 {
+    float4 *own, *slots;  // slots[P3_SLOTS][n], or no pairs
+    uint32_t *flags;      // per leaf
+    uint32_t *ctrl;       // C3_WORDS counters
+    uint2 *directed;      // (leaf, first charge): up to 32 targets
+    uint2 *items;         // (leaf, group)
+    int64_t n;
+    uint32_t pmin;        // P3_PAIR_MIN, or all ones: no pairs
+};
+
+__device__ __forceinline__ uint32_t leaf_count3(const uint32_t *start, int side, int x, int y,
+                                                int z) {
+    if (x < 0 || y < 0 || z < 0 || x >= side || y >= side || z >= side) return 0;
+    const uint32_t b = morton3(uint32_t(x), uint32_t(y), uint32_t(z));
+    return start[b + 1] - start[b];
+}
+
+// Work class of group g of a leaf of n charges: log2 of targets x sources in
+// half steps, heaviest = class 0.
+__device__ __forceinline__ int class3(uint32_t n, uint64_t src) {
+    const uint64_t cost = uint64_t(n) * src + 1;
+    const int e = 63 - __clzll((long long)cost);
+    const int c = 2 * e + int(e ? (cost >> (e - 1)) & 1u : 0u);
+    return c >= C3_CLASSES ? 0 : C3_CLASSES - 1 - c;
+}
+
+// Calls f(class, group) for the pair items of leaf b (n charges).
+template <typename F>
+__device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, int L, uint32_t b,
+                                            uint32_t n, uint32_t pmin, F &&f) {
+    const int side = 1 << L;
+    const int ix = int(compact3(b)), iy = int(compact3(b >> 1)), iz = int(compact3(b >> 2));
+    const int groups = groups3(n);
+    for (int g = 0; g < groups; ++g) {
+        uint64_t src = g ? 0 : n;
+        for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
+            int dx, dy, dz;
+            fwd3(k, &dx, &dy, &dz);
+            const uint32_t c = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
+            if (c >= pmin) src += c;
+        }
+        f(class3(n, src), g);
     }
+}
+
+// Two launches over the leaves: EMIT = false counts the pair items of each
+// class, EMIT = true writes them, heaviest class first, the directed items and
+// the leaf flags.  A block counts in shared memory and takes its run of each
+// list by one atomic (the order of items changes no result).
+template <bool EMIT>
+__global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__restrict__ start,
+                                                     Near3 w) {
+    __shared__ uint32_t hist[C3_CLASSES], base[C3_CLASSES], ndir, dbase;
+    const int64_t nleaf = int64_t(1) << (3 * L);
+    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (threadIdx.x < C3_CLASSES) hist[threadIdx.x] = 0;
+    if (threadIdx.x == 0) ndir = 0;
+    __syncthreads();
+    const uint32_t s0 = b < nleaf ? start[b] : 0u, n = b < nleaf ? start[b + 1] - s0 : 0u;
+    const bool big = n >= w.pmin;
+    if (big)
+        leaf_items3(start, L, uint32_t(b), n, w.pmin,
+                    [&](int c, int) { atomicAdd(&hist[c], 1u); });
+    if (!EMIT) {
+        __syncthreads();
+        if (threadIdx.x < C3_CLASSES && hist[threadIdx.x]) {
+            atomicAdd(w.ctrl + C3_COUNT + threadIdx.x, hist[threadIdx.x]);
+            atomicAdd(w.ctrl + C3_PAIRS, hist[threadIdx.x]);
+        }
+        return;
+    }
+    uint32_t mine = 0, at = 0;  // directed items and their place in the block's run
+    if (n) {
+        const int side = 1 << L;
+        const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
+                  iz = int(compact3(uint32_t(b) >> 2));
+        uint32_t flags = big ? LF3_FWD : 0u;
+        bool directed = !big;
+        for (int k = 0; big && k < P3_DIRS; ++k) {
+            int dx, dy, dz;
+            fwd3(k, &dx, &dy, &dz);
+            const uint32_t f = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
+            const uint32_t r = leaf_count3(start, side, ix - dx, iy - dy, iz - dz);
+            if (r >= w.pmin) flags |= 1u << k;
+            directed |= (f && f < w.pmin) || (r && r < w.pmin);
+        }
+        if (directed) {
+            flags |= LF3_OWN;
+            mine = (n + 31) / 32;
+            at = atomicAdd(&ndir, mine);
+        }
+        w.flags[b] = flags;
+    }
+    __syncthreads();
+    if (threadIdx.x < C3_CLASSES) {
+        uint32_t first = 0;
+        for (int i = 0; i < int(threadIdx.x); ++i) first += w.ctrl[C3_COUNT + i];
+        const uint32_t h = hist[threadIdx.x];
+        base[threadIdx.x] = first + (h ? atomicAdd(w.ctrl + C3_PLACED + threadIdx.x, h) : 0u);
+        hist[threadIdx.x] = 0;
+    } else if (threadIdx.x == C3_CLASSES && ndir) {
+        dbase = atomicAdd(w.ctrl + C3_DIRECTED, ndir);
+    }
+    __syncthreads();
+    for (uint32_t i = 0; i < mine; ++i)
+        w.directed[dbase + at + i] = make_uint2(uint32_t(b), s0 + 32 * i);
+    if (big)
+        leaf_items3(start, L, uint32_t(b), n, w.pmin, [&](int c, int g) {
+            w.items[base[c] + atomicAdd(&hist[c], 1u)] = make_uint2(uint32_t(b), uint32_t(g));
+        });
 }
 
 // 1/sqrt(x) for a normal x > 0: the PTX approximate reciprocal square root
@@ -1802,35 +1933,317 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
     return y;
 }
 
-// Near field + L2P, mixed path: a warp per work item (up to 32 targets of
-// one leaf).  An item of k targets gives each target a group of rep lanes,
-// rep the largest power of two with k rep <= 32, lane c of a group taking
-// sources c, c + rep, ... of every range (a leaf's last, partly filled item
-// keeps most lanes busy), the group's partial sums added by shuffles.
+// A lane's 2 TP targets, two to a float2 (packed FP32 instructions).
+template <int TP> struct Tgt3 {
+    float2 x[TP], y[TP], z[TP], q[TP];      // places, charges
+    float2 f[TP], gx[TP], gy[TP], gz[TP];   // sums
+};
+struct Src3 {
+    float nx, ny, nz, q;      // minus the place (in the targets' frame), charge
+    float f, gx, gy, gz;      // sums of the reactions (field: of its negative)
+};
+
+template <int TP> __device__ __forceinline__ void clear3(Tgt3<TP> &t) {
+#pragma unroll
+    for (int i = 0; i < TP; ++i) t.f[i] = t.gx[i] = t.gy[i] = t.gz[i] = make_float2(0.f, 0.f);
+}
+
+// One source against the lane's targets, both ways.  The differences are
+// scalar: packed ones would need the source's coordinates twice in a register
+// pair each, as many instructions again.
+template <int TP> __device__ __forceinline__ void pair3(Tgt3<TP> &t, Src3 &s) {
+    const float2 q = make_float2(s.q, s.q);
+#pragma unroll
+    for (int i = 0; i < TP; ++i) {
+        const float2 dx = make_float2(t.x[i].x + s.nx, t.x[i].y + s.nx);
+        const float2 dy = make_float2(t.y[i].x + s.ny, t.y[i].y + s.ny);
+        const float2 dz = make_float2(t.z[i].x + s.nz, t.z[i].y + s.nz);
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        const float2 ri = make_float2(rsqrt_normal(r2.x), rsqrt_normal(r2.y));
+        const float2 r3 = __fmul2_rn(__fmul2_rn(ri, ri), ri);
+        t.f[i] = __ffma2_rn(q, ri, t.f[i]);
+        s.f = fmaf(t.q[i].x, ri.x, s.f);
+        s.f = fmaf(t.q[i].y, ri.y, s.f);
+        const float2 a = __fmul2_rn(q, r3), c = __fmul2_rn(t.q[i], r3);
+        t.gx[i] = __ffma2_rn(a, dx, t.gx[i]);
+        t.gy[i] = __ffma2_rn(a, dy, t.gy[i]);
+        t.gz[i] = __ffma2_rn(a, dz, t.gz[i]);
+        s.gx = fmaf(c.x, dx.x, s.gx);
+        s.gx = fmaf(c.y, dx.y, s.gx);
+        s.gy = fmaf(c.x, dy.x, s.gy);
+        s.gy = fmaf(c.y, dy.y, s.gy);
+        s.gz = fmaf(c.x, dz.x, s.gz);
+        s.gz = fmaf(c.y, dz.y, s.gz);
+    }
+}
+
+// One source of the targets' own leaf, one way; self and coincident charges
+// (|d| = 0) add nothing.
+template <int TP> __device__ __forceinline__ void own3(Tgt3<TP> &t, const float4 s) {
+    const float2 nx = make_float2(-s.x, -s.x), ny = make_float2(-s.y, -s.y),
+                 nz = make_float2(-s.z, -s.z), q = make_float2(s.w, s.w);
+#pragma unroll
+    for (int i = 0; i < TP; ++i) {
+        const float2 dx = __fadd2_rn(t.x[i], nx), dy = __fadd2_rn(t.y[i], ny),
+                     dz = __fadd2_rn(t.z[i], nz);
+        const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+        const float2 ri = make_float2(r2.x > 0.f ? rsqrtf(r2.x) : 0.f, r2.y > 0.f ? rsqrtf(r2.y) : 0.f);
+        const float2 a = __fmul2_rn(q, ri), a3 = __fmul2_rn(a, __fmul2_rn(ri, ri));
+        t.f[i] = __fadd2_rn(t.f[i], a);
+        t.gx[i] = __ffma2_rn(a3, dx, t.gx[i]);
+        t.gy[i] = __ffma2_rn(a3, dy, t.gy[i]);
+        t.gz[i] = __ffma2_rn(a3, dz, t.gz[i]);
+    }
+}
+
+// Sums v[0..3] over the lane's group of W = 16 or 32 lanes: every lane gets
+// sum (lane mod W) / (W / 4).
+template <int W>
+__device__ __forceinline__ float sum4_3(float v0, float v1, float v2, float v3, int lane) {
+    const bool h = lane & (W / 2);
+    float a = (h ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h ? v0 : v2, W / 2);
+    const float b = (h ? v3 : v1) + __shfl_xor_sync(0xffffffffu, h ? v1 : v3, W / 2);
+    const bool k = lane & (W / 4);
+    a = (k ? b : a) + __shfl_xor_sync(0xffffffffu, k ? a : b, W / 4);
+#pragma unroll
+    for (int o = W / 8; o; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+}
+
+constexpr float FAR3 = 64.f;   // a place no charge is near (leaf widths)
+// sources left over after whole chunks of 32: up to this many one by one
+constexpr int P3_REST = 16;
+
+// A run of up to 64 targets of leaf A (t0 .. t1 of its sorted charges from
+// a0) against the group's forward neighbours.  Both half-warps hold all the
+// targets, four a lane, and 16 of the neighbour's charges each, which travel
+// around the half by shuffles, the reaction on each accumulating as it
+// travels: after 16 steps each has met every target and is home.  (With two
+// targets a lane and whole-warp rings the eight shuffles of a step were a
+// quarter of its instructions.)  first: the reactions are stored, else added
+// to those of A's earlier runs (the same warp's).
+__device__ __forceinline__ void pairs_run3(const Near3 &w, int L, const uint32_t *__restrict__ start,
+                                           const float4 *__restrict__ rec, uint32_t leaf, int g,
+                                           uint32_t t0, uint32_t t1, bool first, int lane) {
+    const int side = 1 << L;
+    const int ix = int(compact3(leaf)), iy = int(compact3(leaf >> 1)), iz = int(compact3(leaf >> 2));
+    const uint32_t a0 = start[leaf], a1 = start[leaf + 1];
+    const uint32_t half = uint32_t(lane) >> 4, l = uint32_t(lane) & 15u;
+    Tgt3<2> t;
+    clear3(t);
+    float4 r[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t u = t0 + 16 * i + l;
+        r[i] = u < t1 ? rec[u] : make_float4(FAR3, FAR3, FAR3, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        t.x[i] = make_float2(r[2 * i].x, r[2 * i + 1].x);
+        t.y[i] = make_float2(r[2 * i].y, r[2 * i + 1].y);
+        t.z[i] = make_float2(r[2 * i].z, r[2 * i + 1].z);
+        t.q[i] = make_float2(r[2 * i].w, r[2 * i + 1].w);
+    }
+    if (g == 0)
+#pragma unroll 2
+        for (uint32_t j = a0 + half; j < a1; j += 2) own3(t, rec[j]);
+    const int groups = groups3(a1 - a0);
+    for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
+        int dx, dy, dz;
+        fwd3(k, &dx, &dy, &dz);
+        const int nx = ix + dx, ny = iy + dy, nz = iz + dz;
+        if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side) continue;
+        const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
+        const uint32_t b0 = start[nb], b1 = start[nb + 1];
+        if (b1 - b0 < w.pmin) continue;
+        float4 *out = w.slots + int64_t(P3_DIRS + k) * w.n;
+        const float ox = float(dx), oy = float(dy), oz = float(dz);
+        uint32_t c = b0;
+        Src3 s;
+        auto load = [&](uint32_t j) {
+            const float4 u = j < b1 ? rec[j] : make_float4(-FAR3, -FAR3, -FAR3, 0.f);
+            s.nx = -(u.x + ox);
+            s.ny = -(u.y + oy);
+            s.nz = -(u.z + oz);
+            s.q = u.w;
+            s.f = s.gx = s.gy = s.gz = 0.f;
+        };
+        for (; c + uint32_t(P3_REST) < b1; c += 32) {
+            const uint32_t j = c + uint32_t(lane);
+            load(j);
+            const int from = (lane & 16) | ((lane + 1) & 15);
+#pragma unroll
+            for (int step = 0; step < 16; ++step) {
+                // the next step's source on its way while this one computes
+                const float nx2 = __shfl_sync(0xffffffffu, s.nx, from);
+                const float ny2 = __shfl_sync(0xffffffffu, s.ny, from);
+                const float nz2 = __shfl_sync(0xffffffffu, s.nz, from);
+                const float q2 = __shfl_sync(0xffffffffu, s.q, from);
+                pair3(t, s);
+                s.f = __shfl_sync(0xffffffffu, s.f, from);
+                s.gx = __shfl_sync(0xffffffffu, s.gx, from);
+                s.gy = __shfl_sync(0xffffffffu, s.gy, from);
+                s.gz = __shfl_sync(0xffffffffu, s.gz, from);
+                s.nx = nx2;
+                s.ny = ny2;
+                s.nz = nz2;
+                s.q = q2;
+            }
+            if (j < b1) {
+                float4 o = make_float4(s.f, -s.gx, -s.gy, -s.gz);
+                if (!first) {
+                    const float4 p = out[j];
+                    o = make_float4(p.x + o.x, p.y + o.y, p.z + o.z, p.w + o.w);
+                }
+                out[j] = o;
+            }
+        }
+        for (; c < b1; c += 2) {  // the rest one by one, a half-warp each
+            const uint32_t j = c + half;
+            load(j);
+            pair3(t, s);
+            const float v = sum4_3<16>(s.f, -s.gx, -s.gy, -s.gz, lane);
+            if ((lane & 3) == 0 && j < b1) {
+                float *o = reinterpret_cast<float *>(out + j) + (l >> 2);
+                *o = first ? v : *o + v;
+            }
+        }
+        __syncwarp();  // a later run of this warp reads what other lanes wrote
+    }
+    // the halves' sums; half h writes targets 32 h ..
+    float4 *own = w.slots + int64_t(g) * w.n;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        t.f[i].x += __shfl_xor_sync(0xffffffffu, t.f[i].x, 16);
+        t.f[i].y += __shfl_xor_sync(0xffffffffu, t.f[i].y, 16);
+        t.gx[i].x += __shfl_xor_sync(0xffffffffu, t.gx[i].x, 16);
+        t.gx[i].y += __shfl_xor_sync(0xffffffffu, t.gx[i].y, 16);
+        t.gy[i].x += __shfl_xor_sync(0xffffffffu, t.gy[i].x, 16);
+        t.gy[i].y += __shfl_xor_sync(0xffffffffu, t.gy[i].y, 16);
+        t.gz[i].x += __shfl_xor_sync(0xffffffffu, t.gz[i].x, 16);
+        t.gz[i].y += __shfl_xor_sync(0xffffffffu, t.gz[i].y, 16);
+        if (int(half) != i) continue;
+        const uint32_t u = t0 + 32 * i + l, v = u + 16;
+        if (u < t1) own[u] = make_float4(t.f[i].x, t.gx[i].x, t.gy[i].x, t.gz[i].x);
+        if (v < t1) own[v] = make_float4(t.f[i].y, t.gx[i].y, t.gy[i].y, t.gz[i].y);
+    }
+}
+
+// The targets left over after whole runs (up to 16), four at a time: the
+// lanes hold the neighbours' charges, so that no lane idles for want of
+// targets; the reactions are added to those of the leaf's first run.
+__device__ __forceinline__ void pairs_rest3(const Near3 &w, int L, const uint32_t *__restrict__ start,
+                                            const float4 *__restrict__ rec, uint32_t leaf, int g,
+                                            uint32_t t0, uint32_t t1, int lane) {
+    const int side = 1 << L;
+    const int ix = int(compact3(leaf)), iy = int(compact3(leaf >> 1)), iz = int(compact3(leaf >> 2));
+    const uint32_t a0 = start[leaf], a1 = start[leaf + 1];
+    const int groups = groups3(a1 - a0);
+    for (uint32_t c = t0; c < t1; c += 4) {
+        Tgt3<2> t;
+        clear3(t);
+        float4 r[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            r[i] = c + i < t1 ? rec[c + i] : make_float4(FAR3, FAR3, FAR3, 0.f);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            t.x[i] = make_float2(r[2 * i].x, r[2 * i + 1].x);
+            t.y[i] = make_float2(r[2 * i].y, r[2 * i + 1].y);
+            t.z[i] = make_float2(r[2 * i].z, r[2 * i + 1].z);
+            t.q[i] = make_float2(r[2 * i].w, r[2 * i + 1].w);
+        }
+        if (g == 0)
+            for (uint32_t j = a0 + uint32_t(lane); j < a1; j += 32) own3(t, rec[j]);
+        for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
+            int dx, dy, dz;
+            fwd3(k, &dx, &dy, &dz);
+            const int nx = ix + dx, ny = iy + dy, nz = iz + dz;
+            if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side) continue;
+            const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
+            const uint32_t b0 = start[nb], b1 = start[nb + 1];
+            if (b1 - b0 < w.pmin) continue;
+            float4 *out = w.slots + int64_t(P3_DIRS + k) * w.n;
+            for (uint32_t j = b0 + uint32_t(lane); j < b1; j += 32) {
+                const float4 u = rec[j], p = out[j];
+                Src3 s;
+                s.nx = -(u.x + float(dx));
+                s.ny = -(u.y + float(dy));
+                s.nz = -(u.z + float(dz));
+                s.q = u.w;
+                s.f = s.gx = s.gy = s.gz = 0.f;
+                pair3(t, s);
+                out[j] = make_float4(p.x + s.f, p.y - s.gx, p.z - s.gy, p.w - s.gz);
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = t.f[i / 2], x = t.gx[i / 2], y = t.gy[i / 2], z = t.gz[i / 2];
+            const float v = i & 1 ? sum4_3<32>(f.y, x.y, y.y, z.y, lane)
+                                  : sum4_3<32>(f.x, x.x, y.x, z.x, lane);
+            if ((lane & 7) == 0 && c + i < t1)
+                reinterpret_cast<float *>(w.slots + int64_t(g) * w.n + c + i)[lane >> 3] = v;
+        }
+    }
+}
+
+// Bound by the FP32 pipe (65 % busy, issue slots 64 %; a packed instruction
+// holds the pipe two cycles): per target 18 operations, of which 11 packed, and
+// 2 of a step's 8 shuffles; 23.3 instructions a pair in all.  Both near fields
+// whole, on one GB300 (one-sided before / now):
+//   2 M uniform charges (61 a leaf)           2.19 / 1.77 ms
+//   2 M clustered charges (up to 600 a leaf)  11.2 / 8.6 ms
+// Sweeps on the same two: 16 steps unrolled 1.77 / 8.56, by two 1.80 / 8.78;
+// registers for 5, 6, 7 and 8 blocks an SM (steps by two) 1.80 / 8.71,
+// 1.81 / 8.85, 1.80 / 8.77, 1.86 / 9.14; all scalar 1.83 / 8.76 at best; the
+// reactions summed apart from the travelling sums 1.79 / 8.76.
+__global__ void __launch_bounds__(128, 6) k3_pairs(int L, const uint32_t *__restrict__ start,
+                                                const float4 *__restrict__ rec, const Near3 w) {
+    const int lane = threadIdx.x & 31;
+    const uint32_t it = blockIdx.x * 4 + (threadIdx.x >> 5);
+    if (it >= w.ctrl[C3_PAIRS]) return;
+    const uint2 item = w.items[it];
+    const uint32_t leaf = item.x;
+    if (!PF_IN(leaf, int64_t(1) << (3 * L))) return;
+    const int g = int(item.y);
+    const uint32_t a0 = start[leaf], a1 = start[leaf + 1];
+    bool first = true;
+    for (uint32_t t = a0; t < a1;) {
+        const uint32_t left = a1 - t;
+        if (left <= 16 && !first) {
+            pairs_rest3(w, L, start, rec, leaf, g, t, a1, lane);
+            break;
+        }
+        pairs_run3(w, L, start, rec, leaf, g, t, min(a1, t + 64), first, lane);
+        t += 64;
+        first = false;
+    }
+}
+
+// The leaf pairs not evaluated pairwise, one way: a warp per work item (up to
+// 32 targets of one leaf).  An item of k targets gives each target a group of
+// rep lanes, rep the largest power of two with k rep <= 32, lane c of a group
+// taking sources c, c + rep, ... of every range (a leaf's last, partly filled
+// item keeps most lanes busy), the group's partial sums added by shuffles.
 // Sources of the leaf and its neighbours in a fixed order (dz, dy, dx, then
 // sorted rank), each read once per lane group (one address per group) in
 // FP32 leaf units: d = xi_t - (xi_s + offset), 1/|d| from rsqrt, self and
 // coincident pairs (|d| = 0, own leaf only: the records are capped below
-// 0.5 - 2^-24) skipped.  Output in the caller's order.
-template <typename TOut>
-__global__ void __launch_bounds__(W3 * 32, 4) k3_near_mixed(int L, int p, double w,
-                                                            const uint32_t *__restrict__ start,
-                                                            const float4 *__restrict__ rec,
-                                                            const float2 *__restrict__ le,
-                                                            const uint32_t *__restrict__ perm,
-                                                            const uint2 *__restrict__ items,
-                                                            const uint32_t *__restrict__ nitems,
-                                                            int64_t n, void *phi, void *ex,
-                                                            void *ey, void *ez) {
-    __shared__ float2 sle[W3][NC3_MAX];
+// 0.5 - 2^-24) skipped.
+__global__ void __launch_bounds__(W3 * 32, 4) k3_near_directed(int L,
+                                                               const uint32_t *__restrict__ start,
+                                                               const float4 *__restrict__ rec,
+                                                               const Near3 w) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t it = int64_t(blockIdx.x) * W3 + wid;
-    if (it >= int64_t(*nitems)) return;
+    if (it >= int64_t(w.ctrl[C3_DIRECTED])) return;
     // one item: the targets s0 .. s1 - 1 of leaf b
-    const uint2 item = items[it];
+    const uint2 item = w.directed[it];
     const int64_t b = item.x;
     if (!PF_IN(b, int64_t(1) << (3 * L))) return;
     const uint32_t s0 = item.y;
+    const uint32_t nme = start[b + 1] - start[b];
     const uint32_t s1 = min(start[b + 1], s0 + 32u);
     const int k = int(s1 - s0);  // 1..32 (an item holds at least one target)
     int lg = 0;
@@ -1838,15 +2251,9 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_mixed(int L, int p, double
     const uint32_t rep = 1u << lg, c = uint32_t(lane) & (rep - 1u);
     const uint32_t i = s0 + uint32_t(lane >> lg);
     const bool live = i < s1;
-    const int nc = nc3(p);
-    const bool far = L >= 2;
-    if (far)
-        for (int t = lane; t < nc; t += 32) sle[wid][t] = le[(lvl_off3(L) + b) * nc + t];
-    __syncwarp();
     const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
               iz = int(compact3(uint32_t(b) >> 2));
     const int side = 1 << L;
-    const float inv_w = float(1.0 / w), inv_w2 = float(1.0 / (w * w));
     const float4 tg = live ? rec[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     float f = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
     for (int dz = -1; dz <= 1; ++dz)
@@ -1857,6 +2264,7 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_mixed(int L, int p, double
                     continue;
                 const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
                 const uint32_t a = start[nb], e = start[nb + 1];
+                if (nme >= w.pmin && e - a >= w.pmin) continue;  // pairwise
                 const float ox = tg.x - float(dx), oy = tg.y - float(dy), oz = tg.z - float(dz);
                 // |d| = 0 only within the target's own leaf (self, and
                 // coincident particles, which bin to the same leaf); the
@@ -1899,16 +2307,73 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_mixed(int L, int p, double
         gy += __shfl_xor_sync(0xffffffffu, gy, int(o));
         gz += __shfl_xor_sync(0xffffffffu, gz, int(o));
     }
-    if (c == 0 && live) {
-        float ff = 0.f, fx = 0.f, fy = 0.f, fz = 0.f;
-        if (far) l2p3<float, float2>(sle[wid], p, tg.x, tg.y, tg.z, ff, fx, fy, fz);
-        const int64_t o = perm[i];
-        if (PF_IN(o, n)) {
-            store3<TOut>(phi, o, double((f + ff) * inv_w));
-            store3<TOut>(ex, o, double((gx - fx) * inv_w2));
-            store3<TOut>(ey, o, double((gy - fy) * inv_w2));
-            store3<TOut>(ez, o, double((gz - fz) * inv_w2));
-        }
+    if (c == 0 && live) w.own[i] = make_float4(f, gx, gy, gz);
+}
+
+// The parts of each charge and L2P, in the caller's order.
+template <typename TOut>
+__global__ void __launch_bounds__(256) k3_near_final(int L, int p, double w,
+                                                     const uint32_t *__restrict__ skeys,
+                                                     const uint32_t *__restrict__ start,
+                                                     const float4 *__restrict__ rec,
+                                                     const float2 *__restrict__ le,
+                                                     const uint32_t *__restrict__ perm,
+                                                     const Near3 nr, void *phi, void *ex, void *ey,
+                                                     void *ez) {
+    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+    if (i >= nr.n) return;
+    const uint32_t b = skeys[i];
+    if (!PF_IN(b, int64_t(1) << (3 * L))) return;
+    const uint32_t flags = nr.flags[b];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    auto add = [&](const float4 v) {
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    };
+    if (flags & LF3_OWN) add(nr.own[i]);
+    if (flags & LF3_FWD) {
+        const int groups = groups3(start[b + 1] - start[b]);
+        for (int g = 0; g < groups; ++g) add(nr.slots[int64_t(g) * nr.n + i]);
+    }
+#pragma unroll
+    for (int k = 0; k < P3_DIRS; ++k)
+        if ((flags >> k) & 1u) add(nr.slots[int64_t(P3_DIRS + k) * nr.n + i]);
+    float ff = 0.f, fx = 0.f, fy = 0.f, fz = 0.f;
+    if (L >= 2) {
+        const float4 r = rec[i];
+        l2p3<float, float2>(le + (lvl_off3(L) + int64_t(b)) * nc3(p), p, r.x, r.y, r.z, ff, fx, fy, fz);
+    }
+    const float inv_w = float(1.0 / w), inv_w2 = float(1.0 / (w * w));
+    const int64_t o = perm[i];
+    if (!PF_IN(o, nr.n)) return;
+    store3<TOut>(phi, o, double((s.x + ff) * inv_w));
+    store3<TOut>(ex, o, double((s.y - fx) * inv_w2));
+    store3<TOut>(ey, o, double((s.z - fy) * inv_w2));
+    store3<TOut>(ez, o, double((s.w - fz) * inv_w2));
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 near field's work items: leaf b with n_b particles gives ceil(n_b /
+// 32) items (b, first sorted rank of the chunk), in leaf order (a hot leaf's
+// chunks go to consecutive warps, so they spread over the SMs).
+__global__ void __launch_bounds__(256) k3_near_count(const uint32_t *__restrict__ start,
+                                                     int64_t nleaf, uint32_t *__restrict__ cnt) {
+    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (b >= nleaf) return;
+    cnt[b] = (start[b + 1] - start[b] + 31u) / 32u;
+}
+__global__ void __launch_bounds__(256) k3_near_emit(const uint32_t *__restrict__ start,
+                                                    int64_t nleaf, const uint32_t *__restrict__ off,
+                                                    const uint32_t *__restrict__ nitems,
+                                                    int64_t cap, uint2 *__restrict__ items) {
+    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (b >= nleaf) return;
+    const uint32_t s0 = start[b], k = (start[b + 1] - s0 + 31u) / 32u;
+    for (uint32_t c = 0; c < k; ++c) {
+        const int64_t o = int64_t(off[b]) + c;
+        if (o < cap && o < int64_t(*nitems)) items[o] = make_uint2(uint32_t(b), s0 + 32u * c);
     }
 }
 
@@ -2223,7 +2688,10 @@ struct petfmm3d_ctx {
     int L = 0, p = 0, precision = 0, dtype = 0;
     cudaStream_t stream = nullptr;
     DevBuf3 keysA, keysB, valsA, valsB, sortw, start, recu, rec, xs, me, le, status;
-    DevBuf3 ncnt, noff, nscan, nitems;  // the mixed near field's work items
+    DevBuf3 ncnt, noff, nscan, nitems;  // the near field's work items
+    // mixed near field: pair items, parts of the charges' sums, flags, counters
+    DevBuf3 pitems, slots, nown, nflags, nctrl;
+    bool no_pairs = false;  // no room for the parts of pairwise sums
     // operator tables of the context's precision only
     DevBuf3 rtab32, rtab64, atab32, atab64, rmap, parity;
     DevBuf3 m2m32, l2l32;  // p <= 8: the real M2M / L2L operators of the 8 octants
@@ -2237,6 +2705,10 @@ struct petfmm3d_ctx {
 };
 
 namespace {
+
+// Most charges summed pairwise (416 bytes of parts each); more are summed
+// one-sided, as they are where that memory cannot be had.
+constexpr int64_t kPairs3MaxN = int64_t(1) << 26;
 
 #define P3_TRY(x) do { int rc_ = (x); if (rc_) return rc_; } while (0)
 #define P3_CUDA(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { cudaGetLastError(); \
@@ -2624,34 +3096,75 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
     }
     mark3(c, PETFMM3D_STAGE_NEAR);
     const double w = c->dom.width / double(int64_t(1) << L);
-    // work items: ceil(n_b / 32) per leaf, at most min(8^L, n) + n / 32
-    const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
-    P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
-    P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
-    P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
-    P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-    uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
-    uint32_t *nit = off + nleaf;  // the item count, after the offsets
-    uint2 *items = static_cast<uint2 *>(c->nitems.p);
     const unsigned gb = unsigned((nleaf + 255) / 256);
-    k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
-    P3_CUDA(cudaGetLastError());
-    P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
-                           &c->launches));
-    k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
-    P3_CUDA(cudaGetLastError());
-    c->launches += 2;
+    // work items of up to 32 targets: at most min(8^L, n) + n / 32
+    const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
     const unsigned gi = grid_w(cap);
     if (mixed) {
+        // pair items: 2 groups of a leaf of at least P3_PAIR_MIN, 4 above 96
+        // charges, 13 above 384
+        Near3 nr{};
+        nr.n = n;
+        nr.pmin = ~0u;
+        int64_t icap = 0;
+        if (n >= 2 * int64_t(P3_PAIR_MIN) && n <= kPairs3MaxN && !c->no_pairs) {
+            icap = 2 * std::min<int64_t>(nleaf, n / P3_PAIR_MIN) + 2 * (n / 97) + 9 * (n / 385) + 1;
+            int rc = ensure3(c->slots, size_t(P3_SLOTS) * n * sizeof(float4), st);
+            if (rc == PETFMM_OK) rc = ensure3(c->pitems, size_t(icap) * sizeof(uint2), st);
+            if (rc == PETFMM_OK) nr.pmin = P3_PAIR_MIN;
+            else if (rc == PETFMM_ENOMEM) c->no_pairs = true;  // one-sided sums need no slots
+            else return rc;
+        }
+        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
+        P3_TRY(ensure3(c->nown, size_t(n) * sizeof(float4), st));
+        P3_TRY(ensure3(c->nflags, size_t(nleaf) * 4, st));
+        P3_TRY(ensure3(c->nctrl, C3_WORDS * 4, st));
+        nr.own = static_cast<float4 *>(c->nown.p);
+        nr.slots = static_cast<float4 *>(c->slots.p);
+        nr.flags = static_cast<uint32_t *>(c->nflags.p);
+        nr.ctrl = static_cast<uint32_t *>(c->nctrl.p);
+        nr.directed = static_cast<uint2 *>(c->nitems.p);
+        nr.items = static_cast<uint2 *>(c->pitems.p);
         const float4 *rec = static_cast<const float4 *>(c->rec.p);
         const float2 *le = static_cast<const float2 *>(c->le.p);
+        const bool pairs = nr.pmin != ~0u;
+        P3_CUDA(cudaMemsetAsync(nr.ctrl, 0, C3_WORDS * 4, st));
+        if (pairs) {
+            k3_near_items<false><<<gb, 256, 0, st>>>(L, start, nr);
+            P3_CUDA(cudaGetLastError());
+            c->launches++;
+        }
+        k3_near_items<true><<<gb, 256, 0, st>>>(L, start, nr);
+        P3_CUDA(cudaGetLastError());
+        if (pairs) {
+            k3_pairs<<<unsigned((icap + 3) / 4), 128, 0, st>>>(L, start, rec, nr);
+            P3_CUDA(cudaGetLastError());
+            c->launches++;
+        }
+        k3_near_directed<<<gi, W3 * 32, 0, st>>>(L, start, rec, nr);
+        P3_CUDA(cudaGetLastError());
+        c->launches += 2;
         if (f32)
-            k3_near_mixed<float><<<gi, W3 * 32, 0, st>>>(L, p, w, start, rec, le, perm, items,
-                                                         nit, n, phi, ex, ey, ez);
+            k3_near_final<float><<<gp, 256, 0, st>>>(L, p, w, skeys, start, rec, le, perm, nr, phi,
+                                                     ex, ey, ez);
         else
-            k3_near_mixed<double><<<gi, W3 * 32, 0, st>>>(L, p, w, start, rec, le, perm, items,
-                                                          nit, n, phi, ex, ey, ez);
+            k3_near_final<double><<<gp, 256, 0, st>>>(L, p, w, skeys, start, rec, le, perm, nr, phi,
+                                                      ex, ey, ez);
     } else {
+        P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
+        P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
+        P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
+        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
+        uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
+        uint32_t *nit = off + nleaf;  // the item count, after the offsets
+        uint2 *items = static_cast<uint2 *>(c->nitems.p);
+        k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
+        P3_CUDA(cudaGetLastError());
+        P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
+                               &c->launches));
+        k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
+        P3_CUDA(cudaGetLastError());
+        c->launches += 2;
         const Dbl4 *xs = static_cast<const Dbl4 *>(c->xs.p);
         const double2 *le = static_cast<const double2 *>(c->le.p);
         if (f32)
@@ -2797,7 +3310,8 @@ int petfmm3d_debug_shift_operator(int order, int kind, int octant, double *out, 
 int petfmm3d_destroy(petfmm3d_ctx *c) {
     if (!c) return PETFMM_EINVAL;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    DevBuf3 *bufs[] = {&c->ncnt, &c->noff, &c->nscan, &c->nitems,
+    DevBuf3 *bufs[] = {&c->ncnt, &c->noff, &c->nscan, &c->nitems, &c->pitems, &c->slots,
+                       &c->nown, &c->nflags, &c->nctrl,
                        &c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->sortw, &c->start,
                        &c->recu,  &c->rec,   &c->xs,    &c->me,    &c->le,    &c->status,
                        &c->rtab32, &c->rtab64, &c->atab32, &c->atab64, &c->parity, &c->rmap,

@@ -1,0 +1,56 @@
+"""The 3D mixed near field: leaf pairs summed pairwise (both leaves of at least
+24 charges), the others one-sided, at the leaf counts where the work changes
+form; against the FP64 path, and reproducible."""
+import numpy as np
+import pytest
+
+import gpu_util as G
+import test_gpu_fmm3d as T
+from paper_0905_2637_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# around the pairwise limit, whole runs of 32, 64 and 128 targets with few left
+# over, chunks of 32 sources with few left over, 2, 4 and 13 groups a leaf
+COUNTS = [0, 0, 1, 5, 23, 24, 25, 31, 32, 33, 44, 52, 53, 63, 64, 65, 80, 81, 96, 97, 128, 129, 145,
+          208, 385, 700]
+
+
+def by_counts(counts, seed, dtype="f32"):
+    rng = np.random.default_rng(seed)
+    n = counts.shape[0]
+    pts = [(np.array([ix, iy, iz]) + rng.uniform(0, 1, (int(counts[iz, iy, ix]), 3))) / n
+           for iz in range(n) for iy in range(n) for ix in range(n)]
+    pts = np.clip(np.concatenate(pts), 0.0, 1.0)
+    t = np.float32 if dtype == "f32" else np.float64
+    q = rng.uniform(-1, 1, len(pts))
+    return W.Workload3D("counts", *(np.ascontiguousarray(pts[:, k], t) for k in range(3)),
+                        q.astype(t), W.UNIT_CUBE, int(np.log2(n)), 8, dtype)
+
+
+# The mixed path's bar: 1e-5 of the FP64 path (a dropped or doubled leaf pair
+# shows at 1e-3 or more).
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_leaf_counts(seed, dtype):
+    w = by_counts(np.random.default_rng(seed).choice(COUNTS, size=(4, 4, 4)), seed, dtype)
+    rc, mixed = T._run(w, "mixed")
+    assert rc == 0 and all(np.all(np.isfinite(a)) for a in mixed)
+    rc, again = T._run(w, "mixed")
+    assert all(np.array_equal(a, b) for a, b in zip(mixed, again))
+    rc, ref = T._run(w, "fp64")
+    assert T._rel(mixed[0], ref[0]) <= 1e-5 and T._field_rel(mixed, ref) <= 1e-5
+
+
+def test_coincident_and_face_to_face():
+    # coincident charges in a pairwise leaf, and charges on both sides of a
+    # leaf face closer than FP32 resolves
+    w = by_counts(np.full((2, 2, 2), 40), 7, "f64")
+    w.x[:3], w.y[:3], w.z[:3] = w.x[3], w.y[3], w.z[3]
+    w.x[10], w.y[10], w.z[10] = 0.5 - 1e-13, 0.25, 0.25
+    w.x[11], w.y[11], w.z[11] = 0.5 + 1e-13, 0.25, 0.25
+    rc, mixed = T._run(w, "mixed")
+    assert rc == 0 and all(np.all(np.isfinite(a)) for a in mixed)
+    rc, ref = T._run(w, "fp64")
+    rest = np.setdiff1d(np.arange(w.n), [10, 11])
+    assert T._rel(mixed[0][rest], ref[0][rest]) <= 1e-5
