@@ -951,7 +951,9 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
                                pl.leaves_p2m.nblocks, dinst, start, occ, ctrl, s, lc);
     };
     // (the near field's expansions need the list on this stream too)
-    if (pl.sm_degrees) PF_CUDA(list_occupied(st));
+    if (pl.sm_degrees)
+        PF_CUDA(launch_sm_lists(dtask + pl.leaves_p2m.first, pl.leaves_p2m.count,
+                                pl.leaves_p2m.nblocks, dinst, start, occ, ctrl, sm, st, lc));
     cudaStream_t xs = st;
     const bool fork = mixed && c->overlap;
     if (fork) {
@@ -1083,8 +1085,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     if (fork) PF_CUDA(cudaStreamWaitEvent(st, c->ev_gathered, 0));
     stage_mark(c, PETFMM_STAGE_PAIRS);
     if (pl.sm_degrees)
-        PF_CUDA(launch_sm_near(pl.sm_degrees, occ, ctrl, std::min(pl.nleaves, N), dinst, start,
-                               srec, sm, st, lc));
+        PF_CUDA(launch_sm_near(pl.sm_degrees, ctrl, dinst, start, srec, sm, st, lc));
     // pairwise mode: the neighbouring leaves pairwise
     if (pairs)
         PF_CUDA(launch_p2p_pairs(pgrid, pl.deg, pl.general, static_cast<const uint4 *>(c->pitems.p),

@@ -441,6 +441,9 @@ constexpr uint32_t P2M_LANE_MAX = 16;
 // the 32 lanes' sums once per leaf (transposed through shared memory, lane k
 // adding column k: even rows and odd rows separately, then the two).  About a
 // third of the instructions of the per-chunk transpose above.
+// Bound by latency.  765k leaves of one blob, p = 17: 41 us; 200 us when each
+// lane wrote its leaf's coefficients by itself (32 rows a store instruction,
+// 60 us of it) and each warp looked its larger leaves up one by one (100 us).
 template <int PM>
 __global__ void __launch_bounds__(P2M_WARPS * 32) k_p2m_reg(
     const uint2 *__restrict__ occ, const uint32_t *ctrl, const InstDesc *__restrict__ insts,
@@ -465,120 +468,141 @@ __global__ void __launch_bounds__(P2M_WARPS * 32) k_p2m_reg(
     };
     // 1. Leaves of at most P2M_LANE_MAX blobs, one per lane, 32 entries per
     //    warp at a time: the lane sums its few blobs' series by itself and
-    //    writes the p coefficients (a warp and a 32-row reduction per leaf
-    //    of one or a few blobs would be mostly idle).
+    //    the warp writes the 32 leaves' coefficients (a warp and a 32-row
+    //    reduction per leaf of one or a few blobs would be mostly idle).
     for (uint32_t base = gw * 32; base < nocc; base += nwarps * 32) {
         const uint32_t i = base + lane;
-        if (i >= nocc) continue;
-        const InstDesc *dp;
-        uint32_t m, s0, s1;
-        range(i, dp, m, s0, s1);
-        if (s1 - s0 > P2M_LANE_MAX) continue;
-        const InstDesc &d = *dp;
-        const int p = d.p;
-        float2 acc[PM];
+        const InstDesc *dp = nullptr;
+        uint32_t m = 0, s0 = 0, s1 = 0;
+        if (i < nocc) range(i, dp, m, s0, s1);
+        const bool mine = s1 > s0 && s1 - s0 <= P2M_LANE_MAX;
+        int p = 0;
+        float2 *dst = nullptr;
+        if (mine) {
+            const InstDesc &d = *dp;
+            p = d.p;
+            float2 acc[PM];
 #pragma unroll
-        for (int k = 0; k < PM; ++k) acc[k] = make_float2(0.f, 0.f);
-        for (uint32_t j = s0; j < s1; ++j) {
-            const float4 r = rec[j];
-            float2 w = make_float2(r.z, 0.f);
-            const float2 z = make_float2(r.x, r.y);
+            for (int k = 0; k < PM; ++k) acc[k] = make_float2(0.f, 0.f);
+            for (uint32_t j = s0; j < s1; ++j) {
+                const float4 r = rec[j];
+                float2 w = make_float2(r.z, 0.f);
+                const float2 z = make_float2(r.x, r.y);
 #pragma unroll
-            for (int k = 0; k < PM; ++k) {
-                if (k < p) {
-                    acc[k].x += w.x;
-                    acc[k].y += w.y;
-                    w = cmul(w, z);
+                for (int k = 0; k < PM; ++k) {
+                    if (k < p) {
+                        acc[k].x += w.x;
+                        acc[k].y += w.y;
+                        w = cmul(w, z);
+                    }
                 }
-            }
-        }
-        const uint32_t ix = compact_bits(m), iy = compact_bits(m >> 1);
-        float2 *dst = me + d.eoff + (lvl_off(d.L) + box_index(d.L, ix, iy)) * p;
-        const bool lap = d.kernel == KERNEL_LAPLACE;
-#pragma unroll
-        for (int k = 0; k < PM; ++k) {
-            if (k < p) {
-                // Laplace kernel: a_k = -(1/k) sum q zeta^k for k >= 1
-                const float sc = (lap && k) ? -1.0f / float(k) : 1.0f;
-                dst[k] = make_float2(sc * acc[k].x, sc * acc[k].y);
-            }
-        }
-    }
-    // 2. Larger leaves, one per warp (striding over the entries)
-    for (uint32_t i = gw; i < nocc; i += nwarps) {
-        const InstDesc *dp;
-        uint32_t m, s0, s1;
-        range(i, dp, m, s0, s1);
-        if (s1 - s0 <= P2M_LANE_MAX) continue;
-        const InstDesc &d = *dp;
-        const int p = d.p, L = d.L;
-        float2 acc[PM];
-#pragma unroll
-        for (int k = 0; k < PM; ++k) acc[k] = make_float2(0.f, 0.f);
-        // Leaves of more than 32 blobs: two blobs per lane per step (two
-        // independent power chains), and the next step's two records
-        // requested before this step's arithmetic: up to four 16-byte loads
-        // in flight per lane.  Smaller leaves take one step of one blob per
-        // lane (a second chain would only add padding).
-        if (s1 - s0 <= 32) {
-            const float4 r = s0 + lane < s1 ? rec[s0 + lane] : z4;
-            float2 w = make_float2(r.z, 0.f);
-            const float2 z = make_float2(r.x, r.y);
-#pragma unroll
-            for (int k = 0; k < PM; ++k) {
-                if (k < p) {
-                    acc[k].x += w.x;
-                    acc[k].y += w.y;
-                    w = cmul(w, z);
-                }
-            }
-        }
-        float4 na = z4, nb = z4;
-        if (s1 - s0 > 32) {
-            na = rec[s0 + lane];
-            nb = s0 + 32 + lane < s1 ? rec[s0 + 32 + lane] : z4;
-        }
-        for (uint32_t c0 = s0; s1 - s0 > 32 && c0 < s1; c0 += 64) {
-            const float4 ra = na, rb = nb;
-            const uint32_t jn = c0 + 64 + lane;
-            na = jn < s1 ? rec[jn] : z4;
-            nb = jn + 32 < s1 ? rec[jn + 32] : z4;
-            float2 wa = make_float2(ra.z, 0.f), wb = make_float2(rb.z, 0.f);
-            const float2 za = make_float2(ra.x, ra.y), zb = make_float2(rb.x, rb.y);
-#pragma unroll
-            for (int k = 0; k < PM; ++k) {
-                if (k < p) {
-                    acc[k].x += wa.x;
-                    acc[k].y += wa.y;
-                    acc[k].x += wb.x;
-                    acc[k].y += wb.y;
-                    wa = cmul(wa, za);
-                    wb = cmul(wb, zb);
-                }
-            }
-        }
-        float2 *row = buf[wid] + lane * SP;
-#pragma unroll
-        for (int k = 0; k < PM; ++k)
-            if (k < p) row[k] = acc[k];
-        __syncwarp();
-        if (lane < p) {
-            float2 se = make_float2(0.f, 0.f), so = make_float2(0.f, 0.f);
-#pragma unroll 4
-            for (int q = 0; q < 32; q += 2) {
-                const float2 a = buf[wid][q * SP + lane], b = buf[wid][(q + 1) * SP + lane];
-                se.x += a.x;
-                se.y += a.y;
-                so.x += b.x;
-                so.y += b.y;
             }
             const uint32_t ix = compact_bits(m), iy = compact_bits(m >> 1);
-            // Laplace kernel: a_k = -(1/k) sum q zeta^k for k >= 1
-            const float s = (d.kernel == KERNEL_LAPLACE && lane) ? -1.0f / float(lane) : 1.0f;
-            me[d.eoff + (lvl_off(L) + box_index(L, ix, iy)) * p + lane] =
-                make_float2(s * (se.x + so.x), s * (se.y + so.y));
+            dst = me + d.eoff + (lvl_off(d.L) + box_index(d.L, ix, iy)) * p;
+            const bool lap = d.kernel == KERNEL_LAPLACE;
+#pragma unroll
+            for (int k = 0; k < PM; ++k) {
+                if (k < p) {
+                    // Laplace kernel: a_k = -(1/k) sum q zeta^k for k >= 1
+                    const float sc = (lap && k) ? -1.0f / float(k) : 1.0f;
+                    buf[wid][lane * SP + k] = make_float2(sc * acc[k].x, sc * acc[k].y);
+                }
+            }
         }
         __syncwarp();
+        // the 32 leaves' coefficients as one run: consecutive lanes write
+        // consecutive coefficients of a leaf
+        const int pw = __reduce_max_sync(0xffffffffu, p);
+        const uint64_t dst64 = reinterpret_cast<uint64_t>(dst);
+        for (int q = 0, e = lane; q < pw; ++q, e += 32) {
+            const int leaf = e / pw, k = e - leaf * pw;
+            const uint64_t to = __shfl_sync(0xffffffffu, dst64, leaf);
+            const int pl = __shfl_sync(0xffffffffu, p, leaf);
+            if (k < pl) reinterpret_cast<float2 *>(to)[k] = buf[wid][leaf * SP + k];
+        }
+        __syncwarp();
+    }
+    // 2. Larger leaves, one per warp, entry i by warp i mod nwarps so that a
+    //    cluster's leaves spread over all of them; the lanes look up 32 of the
+    //    warp's entries at a time.
+    for (uint64_t base = gw; base < nocc; base += uint64_t(nwarps) * 32) {
+        const uint64_t mine = base + uint64_t(nwarps) * lane;
+        const InstDesc *dp = nullptr;
+        uint32_t m = 0, s0 = 0, s1 = 0;
+        if (mine < nocc) range(uint32_t(mine), dp, m, s0, s1);
+        uint32_t todo = __ballot_sync(0xffffffffu, s1 > s0 && s1 - s0 > P2M_LANE_MAX);
+        for (; todo; todo &= todo - 1) {
+            range(uint32_t(base + uint64_t(nwarps) * (__ffs(todo) - 1)), dp, m, s0, s1);
+            const InstDesc &d = *dp;
+            const int p = d.p, L = d.L;
+            float2 acc[PM];
+#pragma unroll
+            for (int k = 0; k < PM; ++k) acc[k] = make_float2(0.f, 0.f);
+            // Leaves of more than 32 blobs: two blobs per lane per step (two
+            // independent power chains), and the next step's two records
+            // requested before this step's arithmetic: up to four 16-byte loads
+            // in flight per lane.  Smaller leaves take one step of one blob per
+            // lane (a second chain would only add padding).
+            if (s1 - s0 <= 32) {
+                const float4 r = s0 + lane < s1 ? rec[s0 + lane] : z4;
+                float2 w = make_float2(r.z, 0.f);
+                const float2 z = make_float2(r.x, r.y);
+#pragma unroll
+                for (int k = 0; k < PM; ++k) {
+                    if (k < p) {
+                        acc[k].x += w.x;
+                        acc[k].y += w.y;
+                        w = cmul(w, z);
+                    }
+                }
+            }
+            float4 na = z4, nb = z4;
+            if (s1 - s0 > 32) {
+                na = rec[s0 + lane];
+                nb = s0 + 32 + lane < s1 ? rec[s0 + 32 + lane] : z4;
+            }
+            for (uint32_t c0 = s0; s1 - s0 > 32 && c0 < s1; c0 += 64) {
+                const float4 ra = na, rb = nb;
+                const uint32_t jn = c0 + 64 + lane;
+                na = jn < s1 ? rec[jn] : z4;
+                nb = jn + 32 < s1 ? rec[jn + 32] : z4;
+                float2 wa = make_float2(ra.z, 0.f), wb = make_float2(rb.z, 0.f);
+                const float2 za = make_float2(ra.x, ra.y), zb = make_float2(rb.x, rb.y);
+#pragma unroll
+                for (int k = 0; k < PM; ++k) {
+                    if (k < p) {
+                        acc[k].x += wa.x;
+                        acc[k].y += wa.y;
+                        acc[k].x += wb.x;
+                        acc[k].y += wb.y;
+                        wa = cmul(wa, za);
+                        wb = cmul(wb, zb);
+                    }
+                }
+            }
+            float2 *row = buf[wid] + lane * SP;
+#pragma unroll
+            for (int k = 0; k < PM; ++k)
+                if (k < p) row[k] = acc[k];
+            __syncwarp();
+            if (lane < p) {
+                float2 se = make_float2(0.f, 0.f), so = make_float2(0.f, 0.f);
+#pragma unroll 4
+                for (int q = 0; q < 32; q += 2) {
+                    const float2 a = buf[wid][q * SP + lane], b = buf[wid][(q + 1) * SP + lane];
+                    se.x += a.x;
+                    se.y += a.y;
+                    so.x += b.x;
+                    so.y += b.y;
+                }
+                const uint32_t ix = compact_bits(m), iy = compact_bits(m >> 1);
+                // Laplace kernel: a_k = -(1/k) sum q zeta^k for k >= 1
+                const float s = (d.kernel == KERNEL_LAPLACE && lane) ? -1.0f / float(lane) : 1.0f;
+                me[d.eoff + (lvl_off(L) + box_index(L, ix, iy)) * p + lane] =
+                    make_float2(s * (se.x + so.x), s * (se.y + so.y));
+            }
+            __syncwarp();
+        }
     }
 }
 

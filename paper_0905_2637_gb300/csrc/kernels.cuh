@@ -290,11 +290,15 @@ struct SmBufs {
     int64_t rows;
     int row;
 };
+// The occupied list (in place of launch_occ_list) and the lists of sb.
+cudaError_t launch_sm_lists(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                            const uint32_t *start, uint2 *occ, uint32_t *ctrl, const SmBufs &sb,
+                            cudaStream_t st, uint64_t *launches);
 // Moments and local expansions of the degrees in the bit set; needs the
-// occupied list and the gathered records.
-cudaError_t launch_sm_near(uint32_t degrees, const uint2 *occ, uint32_t *ctrl, int64_t max_occ,
-                           const InstDesc *insts, const uint32_t *start, const float4 *rec,
-                           const SmBufs &sb, cudaStream_t st, uint64_t *launches);
+// lists and the gathered records.
+cudaError_t launch_sm_near(uint32_t degrees, const uint32_t *ctrl, const InstDesc *insts,
+                           const uint32_t *start, const float4 *rec, const SmBufs &sb,
+                           cudaStream_t st, uint64_t *launches);
 // These instances' blobs: far field, near field, output (or stage, sorted).
 cudaError_t launch_sm_final(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
                             const uint32_t *start, const uint32_t *skeys, const float4 *rec,

@@ -21,7 +21,7 @@
 // Measured on one GB300, the whole evaluation against the pairwise near field
 // (p2p.cu): 16.8M clustered blobs, kappa = 0.12: 18.3 -> 2.7 ms; 4.2M with the
 // copies from and to the host: 5.2 -> 1.3 ms; 765k blobs, one per leaf (direct
-// pairs only, without their work lists): 2.89 -> 2.38 ms.
+// pairs only, without their work lists): 2.89 -> 2.38 ms then, 1.57 ms now.
 //
 // kappa <= 1.95 (degree 14) is where the line lies: the degree needed grows
 // with the core's steepness (a translation costs the square of (n + 1)(n + 2)
@@ -262,56 +262,115 @@ void host_sm_operators(double kappa, int n, std::vector<float> &out) {
 }
 
 // ----------------------------------------------------------------------------
-// Moments: a warp per occupied leaf
+// Lists: a thread per leaf
+// ----------------------------------------------------------------------------
+// The occupied leaves (as k_occ_list of expansions.cu, which this replaces in
+// plans with smooth instances) and, for those of a smooth instance, which of
+// the nine neighbours are summed directly and which by expansions, the leaves
+// that need a row of the expansion buffers, and the ordered near pairs for the
+// statistics.  One atomic per block and list: a block's leaves, neighbours on
+// the Morton curve, get consecutive rows.  With the classification in
+// k_sm_moments (a warp per occupied leaf) 765k blobs, one per leaf, spent
+// 234 us there, now 25 us here with the occupied list.
+__global__ void __launch_bounds__(256) k_sm_lists(const Task *__restrict__ tasks, int ntasks,
+                                                  const InstDesc *__restrict__ insts,
+                                                  const uint32_t *__restrict__ start,
+                                                  uint2 *__restrict__ occ, uint32_t *ctrl,
+                                                  const SmBufs sb) {
+    __shared__ uint32_t wcnt[2][8], base[2];
+    __shared__ unsigned long long wpairs[8];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int ti = find_task(tasks, ntasks, blockIdx.x);
+    const Task t = tasks[ti];
+    const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
+    const InstDesc &d = insts[t.inst];
+    const uint32_t *st = start + d.soff;
+    const uint32_t n = m < t.count ? st[m + 1] - st[m] : 0u;
+    unsigned long long pairs = 0;
+    uint32_t em = 0;
+    if (n && d.smdeg) {
+        const int nside = 1 << d.L;
+        const uint32_t least = sm_direct_max(d.smdeg);
+        const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
+        uint32_t dm = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            const int x = ix + k % 3 - 1, y = iy + k / 3 - 1;
+            if (x < 0 || y < 0 || x >= nside || y >= nside) continue;
+            const uint32_t nm = morton_key(uint32_t(x), uint32_t(y));
+            const uint32_t cnt = st[nm + 1] - st[nm];
+            const bool byexp = uint64_t(n) * cnt >= least;
+            em |= uint32_t(byexp) << k;
+            dm |= uint32_t(cnt > 0 && !byexp) << k;
+            pairs += (unsigned long long)n * (k == 4 ? cnt - 1 : cnt);
+        }
+        sb.lmask[d.loff + m] = dm | (em << LM_EXP);
+    }
+    const uint32_t bo = __ballot_sync(0xffffffffu, n > 0), be = __ballot_sync(0xffffffffu, em != 0);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
+    if (lane == 0) {
+        wcnt[0][wid] = __popc(bo);
+        wcnt[1][wid] = __popc(be);
+        wpairs[wid] = pairs;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        uint32_t s = 0;
+        for (int w = 0; w < 8; ++w) {
+            const uint32_t v = wcnt[threadIdx.x][w];
+            wcnt[threadIdx.x][w] = s;
+            s += v;
+        }
+        base[threadIdx.x] = s ? atomicAdd(ctrl + (threadIdx.x ? CTRL_NSMOOTH : CTRL_NOCC), s) : 0u;
+    } else if (threadIdx.x == 32) {
+        unsigned long long s = 0;
+        for (int w = 0; w < 8; ++w) s += wpairs[w];
+        if (s) atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), s);
+    }
+    __syncthreads();
+    const uint32_t below = (1u << lane) - 1u;
+    const uint2 e = make_uint2(uint32_t(t.inst), uint32_t(m));
+    if (n) occ[base[0] + wcnt[0][wid] + __popc(bo & below)] = e;
+    if (em) {
+        const uint32_t rank = base[1] + wcnt[1][wid] + __popc(be & below);
+        sb.lrank[d.loff + m] = rank;
+        if (PF_IN(rank, sb.rows)) sb.list[rank] = e;
+    }
+}
+
+cudaError_t launch_sm_lists(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
+                            const uint32_t *start, uint2 *occ, uint32_t *ctrl, const SmBufs &sb,
+                            cudaStream_t st, uint64_t *launches) {
+    if (nblocks <= 0) return cudaSuccess;
+    k_sm_lists<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, occ, ctrl, sb);
+    PF_LAUNCHED(1);
+    return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------
+// Moments: a warp per leaf of the list
 // ----------------------------------------------------------------------------
 // Bound by issue: each lane sums all the moments of its blobs in registers
 // (one multiply-add per blob and term), then 32 values at a time are reduced
 // and scattered over the lanes by halving exchanges (31 shuffles per 32
 // values instead of 160).
 template <int N>
-__global__ void __launch_bounds__(128) k_sm_moments(const uint2 *__restrict__ occ,
-                                                    uint32_t *ctrl,
+__global__ void __launch_bounds__(128) k_sm_moments(const uint32_t *ctrl,
                                                     const InstDesc *__restrict__ insts,
                                                     const uint32_t *__restrict__ start,
                                                     const float4 *__restrict__ rec,
                                                     const SmBufs sb) {
     constexpr int M = sm_terms(N), G = (M + 31) / 32;
     const int lane = threadIdx.x & 31;
-    const uint32_t nocc = ctrl[CTRL_NOCC];
+    const uint32_t nlist = ctrl[CTRL_NSMOOTH];
     const uint32_t nwarps = gridDim.x * 4;
-    unsigned long long pairs = 0;
-    for (uint32_t i = blockIdx.x * 4 + (threadIdx.x >> 5); i < nocc; i += nwarps) {
-        const uint2 e = occ[i];
+    for (uint32_t i = blockIdx.x * 4 + (threadIdx.x >> 5); i < nlist; i += nwarps) {
+        if (!PF_IN(i, sb.rows)) break;
+        const uint2 e = sb.list[i];
         const InstDesc &d = insts[e.x];
         if (d.smdeg != N) continue;
-        const uint32_t *st = start + d.soff;
-        const uint32_t m = e.y;
-        const int nside = 1 << d.L;
-        // the nine counts, one per lane; which neighbours go by expansion
-        const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
-        uint32_t cnt = 0;
-        const int x = ix + lane % 3 - 1, y = iy + lane / 3 - 1;
-        if (lane < 9 && x >= 0 && y >= 0 && x < nside && y < nside) {
-            const uint32_t nm = morton_key(uint32_t(x), uint32_t(y));
-            cnt = st[nm + 1] - st[nm];
-        }
-        const uint32_t n = __shfl_sync(0xffffffffu, cnt, 4);
-        const bool byexp = uint64_t(n) * cnt >= sm_direct_max(N);
-        const uint32_t em = __ballot_sync(0xffffffffu, byexp);
-        const uint32_t dm = __ballot_sync(0xffffffffu, cnt > 0 && !byexp);
-        pairs += (unsigned long long)n * (lane == 4 ? cnt - 1 : cnt);
-        if (lane == 0) sb.lmask[d.loff + m] = dm | (em << LM_EXP);
-        if (!em) continue;
-        // a row of the expansion buffers, in no particular order
-        uint32_t rank = 0;
-        if (lane == 0) {
-            rank = atomicAdd(ctrl + CTRL_NSMOOTH, 1u);
-            sb.lrank[d.loff + m] = rank;
-        }
-        rank = __shfl_sync(0xffffffffu, rank, 0);
-        if (!PF_IN(rank, sb.rows)) continue;
-        if (lane == 0) sb.list[rank] = e;
-        const uint32_t s0 = st[m], s1 = s0 + n;
+        const uint32_t s0 = start[d.soff + e.y], s1 = start[d.soff + e.y + 1];
         if (!(PF_IN(int64_t(s0) - d.poff, d.n + 1) && PF_IN(int64_t(s1) - d.poff, d.n + 1)))
             continue;
         float acc[G * 32];
@@ -337,7 +396,7 @@ __global__ void __launch_bounds__(128) k_sm_moments(const uint2 *__restrict__ oc
                 for (int a = 0; a <= N - b; ++a)
                     acc[sm_idx(N, a, b)] = fmaf(px[a], py[b], acc[sm_idx(N, a, b)]);
         }
-        float *out = sb.mom + size_t(rank) * sb.row;
+        float *out = sb.mom + size_t(i) * sb.row;
 #pragma unroll
         for (int g = 0; g < G; ++g) {
 #pragma unroll
@@ -353,11 +412,6 @@ __global__ void __launch_bounds__(128) k_sm_moments(const uint2 *__restrict__ oc
             if (g * 32 + lane < M) out[g * 32 + lane] = acc[g * 32];
         }
     }
-    // ordered near pairs, for the statistics
-#pragma unroll
-    for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
-    if (lane == 0 && pairs)
-        atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), pairs);
 }
 
 // ----------------------------------------------------------------------------
@@ -588,9 +642,9 @@ __global__ void __launch_bounds__(256, 3) k_sm_final(
 // Launches
 // ----------------------------------------------------------------------------
 template <int N>
-static cudaError_t sm_near(const uint2 *occ, uint32_t *ctrl, int64_t max_occ, const InstDesc *insts,
-                           const uint32_t *start, const float4 *rec, const SmBufs &sb,
-                           cudaStream_t st, uint64_t *launches) {
+static cudaError_t sm_near(const uint32_t *ctrl, const InstDesc *insts, const uint32_t *start,
+                           const float4 *rec, const SmBufs &sb, cudaStream_t st,
+                           uint64_t *launches) {
     static int per_sm_m = 0, per_sm_t = 0;
     if (!per_sm_t) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_m, k_sm_moments<N>, 128, 0);
@@ -600,29 +654,29 @@ static cudaError_t sm_near(const uint2 *occ, uint32_t *ctrl, int64_t max_occ, co
         if (per_sm_t < 1) per_sm_t = 1;
     }
     const int64_t sms = device_sm_count();
-    const int64_t gm = std::min<int64_t>(sms * per_sm_m, (max_occ + 3) / 4);
-    k_sm_moments<N><<<unsigned(gm), 128, 0, st>>>(occ, ctrl, insts, start, rec, sb);
+    if (sb.rows <= 0) return cudaSuccess;
+    const int64_t gm = std::min<int64_t>(sms * per_sm_m, (sb.rows + 3) / 4);
+    k_sm_moments<N><<<unsigned(gm), 128, 0, st>>>(ctrl, insts, start, rec, sb);
     PF_LAUNCHED(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t gt = std::min<int64_t>(sms * per_sm_t, (sb.rows + SM_TGT - 1) / SM_TGT);
-    if (gt <= 0) return cudaSuccess;
     k_sm_translate<N><<<unsigned(gt), SmTile<N>::THREADS, 0, st>>>(ctrl, insts, sb);
     PF_LAUNCHED(1);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sm_near(uint32_t degrees, const uint2 *occ, uint32_t *ctrl, int64_t max_occ,
-                           const InstDesc *insts, const uint32_t *start, const float4 *rec,
-                           const SmBufs &sb, cudaStream_t st, uint64_t *launches) {
+cudaError_t launch_sm_near(uint32_t degrees, const uint32_t *ctrl, const InstDesc *insts,
+                           const uint32_t *start, const float4 *rec, const SmBufs &sb,
+                           cudaStream_t st, uint64_t *launches) {
     cudaError_t e = cudaSuccess;
-    if (degrees & (1u << 8)) e = sm_near<8>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+    if (degrees & (1u << 8)) e = sm_near<8>(ctrl, insts, start, rec, sb, st, launches);
     if (e == cudaSuccess && (degrees & (1u << 10)))
-        e = sm_near<10>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+        e = sm_near<10>(ctrl, insts, start, rec, sb, st, launches);
     if (e == cudaSuccess && (degrees & (1u << 12)))
-        e = sm_near<12>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+        e = sm_near<12>(ctrl, insts, start, rec, sb, st, launches);
     if (e == cudaSuccess && (degrees & (1u << 14)))
-        e = sm_near<14>(occ, ctrl, max_occ, insts, start, rec, sb, st, launches);
+        e = sm_near<14>(ctrl, insts, start, rec, sb, st, launches);
     return e;
 }
 
