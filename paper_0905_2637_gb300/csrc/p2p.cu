@@ -1284,12 +1284,7 @@ __global__ void __launch_bounds__(256, 4) k_p2p_final(
         const int p = d.p;
         const float2 *c =
             le + d.eoff + (lvl_off(d.L) + box_index(d.L, uint32_t(ix), uint32_t(iy))) * p;
-        float2 z = __ldg(c + p - 1);
-        for (int k = p - 2; k >= 0; --k) {
-            const float2 ck = __ldg(c + k);
-            z = make_float2(fmaf(z.x, rr.x, fmaf(-z.y, rr.y, ck.x)),
-                            fmaf(z.x, rr.y, fmaf(z.y, rr.x, ck.y)));
-        }
+        const float2 z = far_series(c, p, rr.x, rr.y);
         // vortex: u - i v = cfar w; Laplace: the potential is Re of the LE
         w = d.kernel == KERNEL_LAPLACE ? make_float2(z.x, 0.f)
                                        : make_float2(d.cfar * z.y, d.cfar * z.x);

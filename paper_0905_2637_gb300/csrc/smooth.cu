@@ -569,7 +569,12 @@ __device__ __forceinline__ float2 sm_gradient(const float *__restrict__ loc, flo
     return make_float2(fs, ft);
 }
 
-__global__ void __launch_bounds__(256, 3) k_sm_final(
+// Bound by load latency: the coefficients are mostly one address per warp, the
+// row number is looked up before the far field, and registers are capped for
+// four blocks an SM.  16.8M clustered blobs, with the two scatters: 806 ->
+// 688 us (three blocks 738; five 658, but 216 bytes of spills and the small
+// cases a little slower).
+__global__ void __launch_bounds__(256, 4) k_sm_final(
     const Task *__restrict__ tasks, int ntasks, const InstDesc *__restrict__ insts,
     const uint32_t *__restrict__ start, const uint32_t *__restrict__ skeys,
     const float4 *__restrict__ rec, const float2 *__restrict__ le,
@@ -583,7 +588,7 @@ __global__ void __launch_bounds__(256, 3) k_sm_final(
     const int64_t r = d.poff + j;
     const uint32_t m = skeys[r] & ((1u << (2 * d.L)) - 1u);
     const float4 rr = rec[r];
-    const uint32_t mask = sb.lmask[d.loff + m];
+    const uint32_t mask = sb.lmask[d.loff + m], rank = sb.lrank[d.loff + m];  // (if by expansions)
     const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
     float2 w = make_float2(0.f, 0.f);
     if (d.L >= 2) {
@@ -591,15 +596,9 @@ __global__ void __launch_bounds__(256, 3) k_sm_final(
         const int p = d.p;
         const float2 *c =
             le + d.eoff + (lvl_off(d.L) + box_index(d.L, uint32_t(ix), uint32_t(iy))) * p;
-        float2 z = __ldg(c + p - 1);
-        for (int k = p - 2; k >= 0; --k) {
-            const float2 ck = __ldg(c + k);
-            z = make_float2(fmaf(z.x, rr.x, fmaf(-z.y, rr.y, ck.x)),
-                            fmaf(z.x, rr.y, fmaf(z.y, rr.x, ck.y)));
-        }
+        const float2 z = far_series(c, p, rr.x, rr.y);
         w = make_float2(d.cfar * z.y, d.cfar * z.x);
     }
-    const uint32_t rank = mask >> LM_EXP ? sb.lrank[d.loff + m] : 0u;
     if ((mask >> LM_EXP) && PF_IN(rank, sb.rows)) {
         const float *l = sb.loc + size_t(rank) * sb.row;
         const float s = 2.f * rr.x, q = 2.f * rr.y;
