@@ -35,9 +35,9 @@
 // in double; mixed path: float4 (xi, eta, zeta, q), the position relative to
 // the leaf centre in leaf widths), ME and LE of every level (8^l boxes in
 // Morton order, level l at box offset (8^l - 1) / 7), the operator tables, and
-// on the mixed path the parts of the pairwise near field, 26 + 1 float4 planes
-// of one entry per charge (432 B a charge; without room for them, or above
-// 2^26 charges, every leaf pair is summed one-sided).
+// the parts of the pairwise near field: planes of one entry per charge (mixed
+// 416, FP64 864 bytes a charge; without room for them, or above 28 GB, every
+// leaf pair is summed one-sided).
 // Every sum runs in a fixed order: results are bitwise reproducible.
 #include <algorithm>
 #include <cmath>
@@ -1788,7 +1788,10 @@ __device__ __forceinline__ void store3(void *o, int64_t i, double v) {
 // ---------------------------------------------------------------------------
 constexpr uint32_t P3_PAIR_MIN = 24;
 constexpr int P3_DIRS = 13;
-constexpr int P3_SLOTS = 2 * P3_DIRS;  // fwd[13], bwd[13]: planes of one float4 per charge
+// planes of one entry per charge, fwd and bwd: mixed (the leaf itself in its
+// first group) and FP64 (a group by itself in the heaviest leaves)
+constexpr int P3_SLOTS = P3_DIRS + P3_DIRS, P3_GROUPS64 = P3_DIRS + 1;
+constexpr int P3_SLOTS64 = P3_GROUPS64 + P3_DIRS;
 
 // forward direction k of 13: (dx, dy, dz) with (dz, dy, dx) above zero
 __host__ __device__ __forceinline__ void fwd3(int k, int *dx, int *dy, int *dz) {
@@ -1798,11 +1801,15 @@ __host__ __device__ __forceinline__ void fwd3(int k, int *dx, int *dy, int *dz) 
     *dz = o / 9 - 1;
 }
 // groups of a leaf of n charges, and group g's directions [first, last)
-__host__ __device__ __forceinline__ int groups3(uint32_t n) {
-    return n <= 96 ? 2 : n <= 384 ? 4 : P3_DIRS;
+template <int MAX = P3_DIRS> __host__ __device__ __forceinline__ int groups3(uint32_t n) {
+    return n <= 16 && MAX == P3_GROUPS64 ? 1 : n <= 96 ? 2 : n <= 384 ? 4 : MAX;
 }
 __host__ __device__ __forceinline__ int group_first3(int g, int groups) {
-    return g * P3_DIRS / groups;
+    return groups == P3_GROUPS64 ? (g < P3_DIRS ? g : P3_DIRS) : g * P3_DIRS / groups;
+}
+// the group that sums the leaf itself
+__host__ __device__ __forceinline__ int own_group3(int groups) {
+    return groups == P3_GROUPS64 ? P3_DIRS : 0;
 }
 // leaf flags of the final pass: bit d: bwd[d] holds a part; bit 13: own does;
 // bit 14: fwd of the leaf's groups do
@@ -1839,14 +1846,14 @@ __device__ __forceinline__ int class3(uint32_t n, uint64_t src) {
 }
 
 // Calls f(class, group) for the pair items of leaf b (n charges).
-template <typename F>
+template <int MAX, typename F>
 __device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, int L, uint32_t b,
                                             uint32_t n, uint32_t pmin, F &&f) {
     const int side = 1 << L;
     const int ix = int(compact3(b)), iy = int(compact3(b >> 1)), iz = int(compact3(b >> 2));
-    const int groups = groups3(n);
+    const int groups = groups3<MAX>(n);
     for (int g = 0; g < groups; ++g) {
-        uint64_t src = g ? 0 : n;
+        uint64_t src = g == own_group3(groups) ? n : 0;
         for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
             int dx, dy, dz;
             fwd3(k, &dx, &dy, &dz);
@@ -1861,7 +1868,7 @@ __device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, 
 // class, EMIT = true writes them, heaviest class first, the directed items and
 // the leaf flags.  A block counts in shared memory and takes its run of each
 // list by one atomic (the order of items changes no result).
-template <bool EMIT>
+template <bool EMIT, int MAX>
 __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__restrict__ start,
                                                      Near3 w) {
     __shared__ uint32_t hist[C3_CLASSES], base[C3_CLASSES], ndir, dbase;
@@ -1873,8 +1880,8 @@ __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__re
     const uint32_t s0 = b < nleaf ? start[b] : 0u, n = b < nleaf ? start[b + 1] - s0 : 0u;
     const bool big = n >= w.pmin;
     if (big)
-        leaf_items3(start, L, uint32_t(b), n, w.pmin,
-                    [&](int c, int) { atomicAdd(&hist[c], 1u); });
+        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin,
+                         [&](int c, int) { atomicAdd(&hist[c], 1u); });
     if (!EMIT) {
         __syncthreads();
         if (threadIdx.x < C3_CLASSES && hist[threadIdx.x]) {
@@ -1919,7 +1926,7 @@ __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__re
     for (uint32_t i = 0; i < mine; ++i)
         w.directed[dbase + at + i] = make_uint2(uint32_t(b), s0 + 32 * i);
     if (big)
-        leaf_items3(start, L, uint32_t(b), n, w.pmin, [&](int c, int g) {
+        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int g) {
             w.items[base[c] + atomicAdd(&hist[c], 1u)] = make_uint2(uint32_t(b), uint32_t(g));
         });
 }
@@ -2395,7 +2402,8 @@ __device__ __forceinline__ double rsqrt_f64(double x) {
 // out over an item's few targets as in the mixed kernel.  Bound by the FP64
 // pipe (two lanes a cycle and SM): 18 operations a pair.  Measured (one
 // GB300, 262,144 uniform charges, L = 4): 32.9 ms with a division and a square
-// root per pair and a warp per leaf -> 16.6 ms.
+// root per pair and a warp per leaf -> 16.6 ms.  Used without k3_pairs_f64's
+// memory.
 template <typename TOut>
 __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
                                                        const uint32_t *__restrict__ start,
@@ -2450,8 +2458,9 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
                     // self and coincident pairs (r2 = 0, tested on the bits)
                     const bool pair = (__double2hiint(r2) | __double2loint(r2)) != 0;
                     const double ri = pair ? rsqrt_f64(r2) : 0.0;
-                    const double qr = s.w * ri, qr3 = qr * (ri * ri);
-                    f = fma(s.w, ri, f);
+                    const double q = pair ? s.w : 0.0;  // (an infinite charge adds 0 to itself)
+                    const double qr = q * ri, qr3 = qr * (ri * ri);
+                    f = fma(q, ri, f);
                     gx = fma(qr3, ddx, gx);
                     gy = fma(qr3, ddy, gy);
                     gz = fma(qr3, ddz, gz);
@@ -2476,6 +2485,188 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
             store3<TOut>(ez, o, gz - fz / (w * w));
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// FP64 near field, pairwise: a warp per pair item (leaf A, group of forward
+// directions, as k3_near_items lists them with pmin = 1).  The charges of the
+// group's neighbours, and of A itself in one group, form one list; each lane
+// takes one of 32 and keeps its reaction in registers while A's targets pass
+// by: lane l meets target (l + step) mod 32 of a run of 32, so that the sums of
+// the targets, in shared memory, have one writer a step.  A last run of c < 32
+// targets is shared by groups of c lanes, each with its own copy of the sums,
+// and no lane idles for want of targets.  Targets go 128 at a time (the
+// reactions of later passes are added to those of the first).
+// Bound by the FP64 pipe (two lanes a cycle and SM): 24 operations a pair for
+// both charges, where the one-sided sums take 18 for each; loads, shuffles and
+// selects cost nothing beside it.
+// The near field whole, one GB300, one-sided / now: 262,144 uniform charges, 64
+// a leaf, 16.4 / 9.7 ms (the pipe busy throughout); 8 a leaf, 6.2 / 2.3 ms;
+// 200,000 clustered charges, up to 760 a leaf, 61.2 / 41.1 ms (47 with the leaf
+// itself in its first group, 58 with 24 warps an SM instead of 8 besides).
+constexpr int PW64 = 2;               // warps a block
+constexpr int PT64 = 128;             // targets of a pass
+constexpr int PA64 = PT64 + 32;       // sums of a pass, copies of the last run's among them
+// Shared memory asked for per block, so that no more than four are resident:
+// two warps a scheduler keep the pipe busy, and with more the heaviest items
+// all start at once and the schedulers that got them end last.
+constexpr size_t kPairs64Smem = 56 * 1024;
+
+// f, gx, gy, gz of target and source: one pair, both ways (d = target -
+// source); self, coincident and padding pairs add nothing.
+__device__ __forceinline__ void pair64(const Dbl4 &t, const Dbl4 &s, bool live, Dbl4 &ta, Dbl4 &sa) {
+    const double dx = t.x - s.x, dy = t.y - s.y, dz = t.z - s.z;
+    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+    const bool pair = live && (__double2hiint(r2) | __double2loint(r2)) != 0;
+    const double ri = pair ? rsqrt_f64(r2) : 0.0;
+    const double qs = pair ? s.w : 0.0, qt = pair ? t.w : 0.0;
+    const double r3 = ri * ri * ri, a = qs * r3, c = qt * r3;
+    ta.x = fma(qs, ri, ta.x);
+    ta.y = fma(a, dx, ta.y);
+    ta.z = fma(a, dy, ta.z);
+    ta.w = fma(a, dz, ta.w);
+    sa.x = fma(qt, ri, sa.x);
+    sa.y = fma(-c, dx, sa.y);
+    sa.z = fma(-c, dy, sa.z);
+    sa.w = fma(-c, dz, sa.w);
+}
+
+__global__ void __launch_bounds__(PW64 * 32) k3_pairs_f64(int L, const uint32_t *__restrict__ start,
+                                                    const Dbl4 *__restrict__ xs, const Near3 w,
+                                                    Dbl4 *__restrict__ slots) {
+    __shared__ Dbl4 stgt[PW64][PT64], sacc[PW64][PA64];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t it = blockIdx.x * PW64 + wid;
+    if (it >= w.ctrl[C3_PAIRS]) return;
+    const uint2 item = w.items[it];
+    const uint32_t leaf = item.x;
+    if (!PF_IN(leaf, int64_t(1) << (3 * L))) return;
+    const int g = int(item.y), side = 1 << L;
+    const int ix = int(compact3(leaf)), iy = int(compact3(leaf >> 1)), iz = int(compact3(leaf >> 2));
+    const uint32_t a0 = start[leaf], a1 = start[leaf + 1];
+    const int groups = groups3<P3_GROUPS64>(a1 - a0);
+    const int k0 = group_first3(g, groups), nk = group_first3(g + 1, groups) - k0;
+    Dbl4 *tgt = stgt[wid], *acc = sacc[wid];
+    // lane 0: the leaf itself (its group only); lane 1 + i: forward direction k0 + i
+    uint32_t beg = 0, cnt = 0;
+    if (lane == 0 && g == own_group3(groups)) {
+        beg = a0;
+        cnt = a1 - a0;
+    } else if (lane >= 1 && lane <= nk) {
+        int dx, dy, dz;
+        fwd3(k0 + lane - 1, &dx, &dy, &dz);
+        const int nx = ix + dx, ny = iy + dy, nz = iz + dz;
+        if (nx >= 0 && ny >= 0 && nz >= 0 && nx < side && ny < side && nz < side) {
+            const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
+            beg = start[nb];
+            cnt = start[nb + 1] - beg;
+        }
+    }
+    uint32_t end = cnt;  // of the lane's range in the list
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, end, o);
+        if (lane >= o) end += v;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, end, 31);
+    for (uint32_t t0 = a0; t0 < a1; t0 += PT64) {
+        const uint32_t nt = min(a1 - t0, uint32_t(PT64)), whole = nt & ~31u, c = nt & 31u;
+        for (uint32_t i = lane; i < nt; i += 32) tgt[i] = xs[t0 + i];
+        for (uint32_t i = lane; i < PA64; i += 32) acc[i] = Dbl4{0.0, 0.0, 0.0, 0.0};
+        __syncwarp();
+        for (uint32_t m0 = 0; m0 < total; m0 += 32) {
+            const uint32_t m = m0 + uint32_t(lane);
+            const bool live = m < total;
+            int r = 0;  // the range that holds entry m
+            for (int i = 0; i <= nk; ++i) r += m >= __shfl_sync(0xffffffffu, end, i);
+            r = min(r, nk);
+            const uint32_t j = __shfl_sync(0xffffffffu, beg + cnt - end, r) + m;
+            const Dbl4 s = live ? xs[j] : tgt[0];
+            Dbl4 sa{0.0, 0.0, 0.0, 0.0};
+            for (uint32_t b = 0; b < whole; b += 32)
+                for (uint32_t st = 0; st < 32; ++st) {
+                    const uint32_t i = b + ((uint32_t(lane) + st) & 31u);
+                    Dbl4 ta = acc[i];
+                    pair64(tgt[i], s, live, ta, sa);
+                    acc[i] = ta;
+                    __syncwarp();
+                }
+            if (c) {
+                const uint32_t copy = uint32_t(lane) / c * c;
+                uint32_t i = uint32_t(lane) - copy;
+                for (uint32_t st = 0; st < c; ++st) {
+                    Dbl4 ta = acc[whole + copy + i];
+                    pair64(tgt[whole + i], s, live, ta, sa);
+                    acc[whole + copy + i] = ta;
+                    __syncwarp();
+                    i = i + 1 == c ? 0 : i + 1;
+                }
+            }
+            if (live && r > 0 && PF_IN(j, w.n)) {
+                Dbl4 *o = slots + int64_t(P3_GROUPS64 + k0 + r - 1) * w.n + j;
+                if (t0 != a0) {
+                    const Dbl4 p = *o;
+                    sa = Dbl4{p.x + sa.x, p.y + sa.y, p.z + sa.z, p.w + sa.w};
+                }
+                *o = sa;
+            }
+        }
+        for (uint32_t i = lane; i < nt; i += 32) {
+            Dbl4 v = acc[i];
+            if (i >= whole)
+                for (uint32_t o = c; o < 32; o += c) {
+                    const Dbl4 u = acc[i + o];
+                    v = Dbl4{v.x + u.x, v.y + u.y, v.z + u.z, v.w + u.w};
+                }
+            slots[int64_t(g) * w.n + t0 + i] = v;
+        }
+        __syncwarp();
+    }
+}
+
+// The parts of each charge and L2P, in the caller's order.
+template <typename TOut>
+__global__ void __launch_bounds__(128) k3_final_f64(int L, int p, Dom3 d,
+                                                    const uint32_t *__restrict__ skeys,
+                                                    const uint32_t *__restrict__ start,
+                                                    const Dbl4 *__restrict__ xs,
+                                                    const double2 *__restrict__ le,
+                                                    const uint32_t *__restrict__ perm,
+                                                    const Near3 nr, const Dbl4 *__restrict__ slots,
+                                                    void *phi, void *ex, void *ey, void *ez) {
+    const int64_t i = int64_t(blockIdx.x) * 128 + threadIdx.x;
+    if (i >= nr.n) return;
+    const uint32_t b = skeys[i];
+    if (!PF_IN(b, int64_t(1) << (3 * L))) return;
+    const uint32_t flags = nr.flags[b];
+    Dbl4 s{0.0, 0.0, 0.0, 0.0};
+    auto add = [&](const Dbl4 v) {
+        s.x += v.x;
+        s.y += v.y;
+        s.z += v.z;
+        s.w += v.w;
+    };
+    const int groups = groups3<P3_GROUPS64>(start[b + 1] - start[b]);
+    for (int g = 0; g < groups; ++g) add(slots[int64_t(g) * nr.n + i]);
+#pragma unroll
+    for (int k = 0; k < P3_DIRS; ++k)
+        if ((flags >> k) & 1u) add(slots[int64_t(P3_GROUPS64 + k) * nr.n + i]);
+    const double w = d.width / double(1 << L);
+    double ff = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
+    if (L >= 2) {
+        const double cx = d.x0 + (int(compact3(b)) + 0.5) * w,
+                     cy = d.y0 + (int(compact3(b >> 1)) + 0.5) * w,
+                     cz = d.z0 + (int(compact3(b >> 2)) + 0.5) * w;
+        const Dbl4 t = xs[i];
+        l2p3<double, double2>(le + (lvl_off3(L) + int64_t(b)) * nc3(p), p, (t.x - cx) / w,
+                              (t.y - cy) / w, (t.z - cz) / w, ff, fx, fy, fz);
+    }
+    const int64_t o = perm[i];
+    if (!PF_IN(o, nr.n)) return;
+    store3<TOut>(phi, o, s.x + ff / w);
+    store3<TOut>(ex, o, s.y - fx / (w * w));
+    store3<TOut>(ey, o, s.z - fy / (w * w));
+    store3<TOut>(ez, o, s.w - fz / (w * w));
 }
 
 // ---------------------------------------------------------------------------
@@ -2706,9 +2897,10 @@ struct petfmm3d_ctx {
 
 namespace {
 
-// Most charges summed pairwise (416 bytes of parts each); more are summed
-// one-sided, as they are where that memory cannot be had.
-constexpr int64_t kPairs3MaxN = int64_t(1) << 26;
+// Most bytes for the parts of pairwise sums (67M charges of the mixed path, 32M
+// of the FP64 path); above it, or where that memory cannot be had, leaf
+// pairs are summed one-sided.
+constexpr size_t kPairs3MaxBytes = (size_t(1) << 26) * P3_SLOTS * sizeof(float4);
 
 #define P3_TRY(x) do { int rc_ = (x); if (rc_) return rc_; } while (0)
 #define P3_CUDA(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { cudaGetLastError(); \
@@ -3012,6 +3204,32 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
     return PETFMM_OK;
 }
 
+// The lists, flags and counters of the near field and, where they are allowed
+// and there is room, the slots of the pairwise sums (parts bytes a charge); else
+// nr->pmin stays all ones and every leaf pair is summed one-sided.
+int near_pairs3(petfmm3d_ctx *c, int64_t n, int64_t nleaf, uint32_t pmin, size_t parts, Near3 *nr,
+                int64_t *icap) {
+    cudaStream_t st = c->stream;
+    nr->n = n;
+    nr->pmin = ~0u;
+    if (n >= 2 * int64_t(pmin) && n * parts <= kPairs3MaxBytes && !c->no_pairs) {
+        // up to 2 groups of a leaf of at least pmin, 4 above 96 charges, 14 above 384
+        *icap = 2 * std::min<int64_t>(nleaf, n / pmin) + 2 * (n / 97) + 10 * (n / 385) + 1;
+        int rc = ensure3(c->slots, n * parts, st);
+        if (rc == PETFMM_OK) rc = ensure3(c->pitems, size_t(*icap) * sizeof(uint2), st);
+        if (rc == PETFMM_OK) nr->pmin = pmin;
+        else if (rc == PETFMM_ENOMEM) c->no_pairs = true;  // one-sided sums need no slots
+        else return rc;
+    }
+    P3_TRY(ensure3(c->nflags, size_t(nleaf) * 4, st));
+    P3_TRY(ensure3(c->nctrl, C3_WORDS * 4, st));
+    nr->flags = static_cast<uint32_t *>(c->nflags.p);
+    nr->ctrl = static_cast<uint32_t *>(c->nctrl.p);
+    nr->items = static_cast<uint2 *>(c->pitems.p);
+    P3_CUDA(cudaMemsetAsync(nr->ctrl, 0, C3_WORDS * 4, st));
+    return PETFMM_OK;
+}
+
 int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const void *z,
               const void *q, void *phi, void *ex, void *ey, void *ez) {
     cudaStream_t st = c->stream;
@@ -3097,44 +3315,27 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
     mark3(c, PETFMM3D_STAGE_NEAR);
     const double w = c->dom.width / double(int64_t(1) << L);
     const unsigned gb = unsigned((nleaf + 255) / 256);
-    // work items of up to 32 targets: at most min(8^L, n) + n / 32
+    // one-sided work items of up to 32 targets: at most min(8^L, n) + n / 32
     const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
     const unsigned gi = grid_w(cap);
     if (mixed) {
-        // pair items: 2 groups of a leaf of at least P3_PAIR_MIN, 4 above 96
-        // charges, 13 above 384
         Near3 nr{};
-        nr.n = n;
-        nr.pmin = ~0u;
         int64_t icap = 0;
-        if (n >= 2 * int64_t(P3_PAIR_MIN) && n <= kPairs3MaxN && !c->no_pairs) {
-            icap = 2 * std::min<int64_t>(nleaf, n / P3_PAIR_MIN) + 2 * (n / 97) + 9 * (n / 385) + 1;
-            int rc = ensure3(c->slots, size_t(P3_SLOTS) * n * sizeof(float4), st);
-            if (rc == PETFMM_OK) rc = ensure3(c->pitems, size_t(icap) * sizeof(uint2), st);
-            if (rc == PETFMM_OK) nr.pmin = P3_PAIR_MIN;
-            else if (rc == PETFMM_ENOMEM) c->no_pairs = true;  // one-sided sums need no slots
-            else return rc;
-        }
+        P3_TRY(near_pairs3(c, n, nleaf, P3_PAIR_MIN, P3_SLOTS * sizeof(float4), &nr, &icap));
         P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
         P3_TRY(ensure3(c->nown, size_t(n) * sizeof(float4), st));
-        P3_TRY(ensure3(c->nflags, size_t(nleaf) * 4, st));
-        P3_TRY(ensure3(c->nctrl, C3_WORDS * 4, st));
         nr.own = static_cast<float4 *>(c->nown.p);
         nr.slots = static_cast<float4 *>(c->slots.p);
-        nr.flags = static_cast<uint32_t *>(c->nflags.p);
-        nr.ctrl = static_cast<uint32_t *>(c->nctrl.p);
         nr.directed = static_cast<uint2 *>(c->nitems.p);
-        nr.items = static_cast<uint2 *>(c->pitems.p);
         const float4 *rec = static_cast<const float4 *>(c->rec.p);
         const float2 *le = static_cast<const float2 *>(c->le.p);
         const bool pairs = nr.pmin != ~0u;
-        P3_CUDA(cudaMemsetAsync(nr.ctrl, 0, C3_WORDS * 4, st));
         if (pairs) {
-            k3_near_items<false><<<gb, 256, 0, st>>>(L, start, nr);
+            k3_near_items<false, P3_DIRS><<<gb, 256, 0, st>>>(L, start, nr);
             P3_CUDA(cudaGetLastError());
             c->launches++;
         }
-        k3_near_items<true><<<gb, 256, 0, st>>>(L, start, nr);
+        k3_near_items<true, P3_DIRS><<<gb, 256, 0, st>>>(L, start, nr);
         P3_CUDA(cudaGetLastError());
         if (pairs) {
             k3_pairs<<<unsigned((icap + 3) / 4), 128, 0, st>>>(L, start, rec, nr);
@@ -3151,28 +3352,53 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
             k3_near_final<double><<<gp, 256, 0, st>>>(L, p, w, skeys, start, rec, le, perm, nr, phi,
                                                       ex, ey, ez);
     } else {
-        P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
-        P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
-        P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
-        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-        uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
-        uint32_t *nit = off + nleaf;  // the item count, after the offsets
-        uint2 *items = static_cast<uint2 *>(c->nitems.p);
-        k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
-        P3_CUDA(cudaGetLastError());
-        P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
-                               &c->launches));
-        k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
-        P3_CUDA(cudaGetLastError());
-        c->launches += 2;
         const Dbl4 *xs = static_cast<const Dbl4 *>(c->xs.p);
         const double2 *le = static_cast<const double2 *>(c->le.p);
-        if (f32)
-            k3_near_f64<float><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
-                                                       phi, ex, ey, ez);
-        else
-            k3_near_f64<double><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
-                                                        phi, ex, ey, ez);
+        Near3 nr{};
+        int64_t icap = 0;
+        P3_TRY(near_pairs3(c, n, nleaf, 1, P3_SLOTS64 * sizeof(Dbl4), &nr, &icap));
+        if (nr.pmin == 1) {
+            Dbl4 *slots = static_cast<Dbl4 *>(c->slots.p);
+            constexpr int pad = int(kPairs64Smem - PW64 * (PT64 + PA64) * sizeof(Dbl4));
+            P3_CUDA(cudaFuncSetAttribute(k3_pairs_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         pad));
+            k3_near_items<false, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
+            P3_CUDA(cudaGetLastError());
+            k3_near_items<true, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
+            P3_CUDA(cudaGetLastError());
+            k3_pairs_f64<<<unsigned((icap + PW64 - 1) / PW64), PW64 * 32, pad, st>>>(L, start, xs, nr,
+                                                                                   slots);
+            P3_CUDA(cudaGetLastError());
+            c->launches += 3;
+            const unsigned gf = unsigned((n + 127) / 128);
+            if (f32)
+                k3_final_f64<float><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr,
+                                                        slots, phi, ex, ey, ez);
+            else
+                k3_final_f64<double><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr,
+                                                         slots, phi, ex, ey, ez);
+        } else {
+            P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
+            P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
+            P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
+            P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
+            uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
+            uint32_t *nit = off + nleaf;  // the item count, after the offsets
+            uint2 *items = static_cast<uint2 *>(c->nitems.p);
+            k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
+            P3_CUDA(cudaGetLastError());
+            P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
+                                   &c->launches));
+            k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
+            P3_CUDA(cudaGetLastError());
+            c->launches += 2;
+            if (f32)
+                k3_near_f64<float><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
+                                                           phi, ex, ey, ez);
+            else
+                k3_near_f64<double><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
+                                                            phi, ex, ey, ez);
+        }
     }
     P3_CUDA(cudaGetLastError());
     c->launches++;

@@ -54,3 +54,31 @@ def test_coincident_and_face_to_face():
     rc, ref = T._run(w, "fp64")
     rest = np.setdiff1d(np.arange(w.n), [10, 11])
     assert T._rel(mixed[0][rest], ref[0][rest]) <= 1e-5
+
+
+# One level: all eight leaves touch, so the FP64 result is the whole sum, up to
+# the rounding of some thousand terms of mixed sign (n eps of the absolute sum,
+# 1e-12 here; a dropped or doubled pair shows at 1e-5 or more).
+@pytest.mark.parametrize("dtype", ["f32", "f64"])
+@pytest.mark.parametrize("seed", [1, 2, 3, 4])
+def test_fp64_leaf_counts(seed, dtype):
+    rng = np.random.default_rng(seed)
+    counts = rng.choice(COUNTS + [2, 15, 16, 17, 127, 160, 256, 257], size=(2, 2, 2))
+    w = by_counts(counts, seed, dtype)
+    if w.n > 8:
+        w.x[1], w.y[1], w.z[1] = w.x[0], w.y[0], w.z[0]  # a coincident pair
+    rc, got = T._run(w, "fp64")
+    assert rc == 0
+    rc, again = T._run(w, "fp64")
+    assert all(np.array_equal(a, b) for a, b in zip(got, again))
+    x, y, z, q = (a.astype(np.float64) for a in (w.x, w.y, w.z, w.q))
+    tol = 1e-12 if dtype == "f64" else 1e-7  # FP32 outputs round at 6e-8
+    for i0 in range(0, w.n, 512):
+        i = slice(i0, i0 + 512)
+        d = [a[i, None] - a[None, :] for a in (x, y, z)]
+        r2 = sum(a * a for a in d)
+        same = r2 == 0
+        r2[same] = 1.0
+        p = np.where(same, 0.0, q[None, :] / np.sqrt(r2))
+        for a, t in zip(got, [p] + [p / r2 * a for a in d]):
+            assert np.all(np.abs(a[i] - t.sum(1)) <= tol * np.abs(t).sum(1) + 1e-30)
