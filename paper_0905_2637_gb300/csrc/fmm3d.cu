@@ -44,6 +44,7 @@
 #include <complex>
 #include <cstring>
 #include <new>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/petfmm.h"
@@ -57,7 +58,7 @@ namespace {
 constexpr int P3_MAX = PETFMM3D_MAX_P;           // terms
 constexpr int L3_MAX = PETFMM3D_MAX_L;           // levels (3L <= 30 key bits)
 constexpr int NC3_MAX = P3_MAX * (P3_MAX + 1) / 2;  // stored coefficients
-constexpr int OUT3 = (NC3_MAX + 31) / 32;          // per lane, one warp per box
+constexpr int TC3_MAXP = 8;                        // terms of the tensor-core M2L
 constexpr int NSLOT3 = 343;                        // offsets in [-3, 3]^3
 constexpr int W3 = 8;                              // warps per block
 
@@ -105,23 +106,6 @@ __host__ __device__ __forceinline__ uint32_t morton3(uint32_t ix, uint32_t iy, u
 __device__ __forceinline__ uint32_t box_count3(const uint32_t *start, int L, int l, uint32_t b) {
     const int sh = 3 * (L - l);
     return start[(uint64_t(b) + 1) << sh] - start[uint64_t(b) << sh];
-}
-
-// coefficient (n, m) of a stored series; m < 0 by X_n^-m = (-1)^m conj(X_n^m)
-template <typename V>
-__device__ __forceinline__ V coef3(const V *a, int n, int m) {
-    if (m >= 0) return a[n * (n + 1) / 2 + m];
-    const V v = a[n * (n + 1) / 2 - m];
-    return (m & 1) ? mk<V>(-v.x, v.y) : mk<V>(v.x, -v.y);
-}
-
-template <typename V> __device__ __forceinline__ void cmac(V &acc, V a, V b) {  // acc += a b
-    acc.x += a.x * b.x - a.y * b.y;
-    acc.y += a.x * b.y + a.y * b.x;
-}
-template <typename V> __device__ __forceinline__ void cmac_conj(V &acc, V a, V b) {  // acc += conj(a) b
-    acc.x += a.x * b.x + a.y * b.y;
-    acc.y += a.x * b.y - a.y * b.x;
 }
 
 // ---------------------------------------------------------------------------
@@ -361,17 +345,20 @@ __global__ void __launch_bounds__(W3 * 32) k3_p2m(int L, int p, Dom3 d, const ui
     }
 }
 
-// P2M of the mixed path for p <= 8: a warp per leaf with a lane per charge
+// P2M for p <= 8: a warp per leaf with a lane per charge
 // (charges j, j + 32, ... of the leaf), each lane computing all p (p + 1) / 2
 // terms q R_n^m column by column with compile-time constants and summing
 // them over its charges; then a reduce-scatter across the warp (three
 // halving exchanges, offsets 16, 8, 4, then a butterfly over offsets 2 and
 // 1) leaves each group of four lanes the full sums of a ninth of the 2 NC
 // values, which one lane of the group writes.
-template <int P>
-__global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, const uint32_t *__restrict__ start,
-                                                        const float4 *__restrict__ rec,
-                                                        float2 *__restrict__ me) {
+// FP64: bound by its pipe; 262,144 charges, 64 a leaf, p = 8: 622 us by columns
+// (k3_p2m, few lanes of a group busy in the short columns) -> 235 us.
+template <int P, typename T, typename Rec>
+__global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, Dom3 d,
+                                                        const uint32_t *__restrict__ start,
+                                                        const Rec *__restrict__ rec,
+                                                        typename C3<T>::V *__restrict__ me) {
     constexpr int NC = P * (P + 1) / 2, NV = 2 * NC;  // values: Re of all, then Im of all
     constexpr int NV8 = (NV + 7) / 8, NVP = 8 * NV8;  // padded to eight equal parts
     const int lane = threadIdx.x & 31;
@@ -379,29 +366,33 @@ __global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, const uint32_t *_
     if (b >= (int64_t(1) << (3 * L))) return;
     const uint32_t s0 = start[b], s1 = start[b + 1];
     if (s0 == s1) return;
-    float v[NVP];
+    const double w = d.width / double(1u << L), inv_w = 1.0 / w;
+    const double cx = d.x0 + (double(compact3(uint32_t(b))) + 0.5) * w;
+    const double cy = d.y0 + (double(compact3(uint32_t(b) >> 1)) + 0.5) * w;
+    const double cz = d.z0 + (double(compact3(uint32_t(b) >> 2)) + 0.5) * w;
+    T v[NVP];
 #pragma unroll
-    for (int k = 0; k < NVP; ++k) v[k] = 0.f;
+    for (int k = 0; k < NVP; ++k) v[k] = T(0);
     for (uint32_t j = s0 + uint32_t(lane); j < s1; j += 32u) {
-        const float4 a = rec[j];
-        const float r2 = a.x * a.x + a.y * a.y + a.z * a.z;
-        float pr = a.w, pi = 0.f;  // q R_m^m
+        const Part3<T> a = leaf_part(rec, j, cx, cy, cz, inv_w);
+        const T r2 = a.x * a.x + a.y * a.y + a.z * a.z;
+        T pr = a.q, pi = T(0);  // q R_m^m
 #pragma unroll
         for (int m = 0; m < P; ++m) {
             if (m > 0) {
-                const float sc = 1.f / float(2 * m);
-                const float tr = (pr * a.x - pi * a.y) * sc, ti = (pr * a.y + pi * a.x) * sc;
+                const T sc = T(1) / T(2 * m);
+                const T tr = (pr * a.x - pi * a.y) * sc, ti = (pr * a.y + pi * a.x) * sc;
                 pr = tr;
                 pi = ti;
             }
-            float r1r = pr, r1i = pi, r0r = 0.f, r0i = 0.f;
+            T r1r = pr, r1i = pi, r0r = T(0), r0i = T(0);
             v[m * (m + 1) / 2 + m] += r1r;
             v[NC + m * (m + 1) / 2 + m] += r1i;
 #pragma unroll
             for (int n = m + 1; n < P; ++n) {
-                const float c1 = float(2 * n - 1) * a.z;
-                const float inv = 1.f / float(n * n - m * m);
-                const float rr = (c1 * r1r - r2 * r0r) * inv, ri = (c1 * r1i - r2 * r0i) * inv;
+                const T c1 = T(2 * n - 1) * a.z;
+                const T inv = T(1) / T(n * n - m * m);
+                const T rr = (c1 * r1r - r2 * r0r) * inv, ri = (c1 * r1i - r2 * r0i) * inv;
                 r0r = r1r;
                 r0i = r1i;
                 r1r = rr;
@@ -417,22 +408,22 @@ __global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, const uint32_t *_
 #pragma unroll
     for (int k = 0; k < NVP / 2; ++k) {
         const bool up = lane & 16;
-        const float send = up ? v[k] : v[k + NVP / 2];
-        const float keep = up ? v[k + NVP / 2] : v[k];
+        const T send = up ? v[k] : v[k + NVP / 2];
+        const T keep = up ? v[k + NVP / 2] : v[k];
         v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
     }
 #pragma unroll
     for (int k = 0; k < NVP / 4; ++k) {
         const bool up = lane & 8;
-        const float send = up ? v[k] : v[k + NVP / 4];
-        const float keep = up ? v[k + NVP / 4] : v[k];
+        const T send = up ? v[k] : v[k + NVP / 4];
+        const T keep = up ? v[k + NVP / 4] : v[k];
         v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
     }
 #pragma unroll
     for (int k = 0; k < NV8; ++k) {
         const bool up = lane & 4;
-        const float send = up ? v[k] : v[k + NV8];
-        const float keep = up ? v[k + NV8] : v[k];
+        const T send = up ? v[k] : v[k + NV8];
+        const T keep = up ? v[k + NV8] : v[k];
         v[k] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
     }
 #pragma unroll
@@ -443,7 +434,7 @@ __global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, const uint32_t *_
     // this group's values: index 4 NVP/8 bit4 + 2 NVP/8 bit3 + NVP/8 bit2 + k
     if ((lane & 3) == 0) {
         const int base = NV8 * (4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1));
-        float *dst = reinterpret_cast<float *>(me + (lvl_off3(L) + b) * NC);
+        T *dst = reinterpret_cast<T *>(me + (lvl_off3(L) + b) * NC);
 #pragma unroll
         for (int k = 0; k < NV8; ++k) {
             const int vi = base + k;
@@ -455,78 +446,18 @@ __global__ void __launch_bounds__(W3 * 32) k3_p2m_lanes(int L, const uint32_t *_
     }
 }
 
-template <int P>
-cudaError_t p2m_lanes_p(int L, const uint32_t *start, const float4 *rec, float2 *me, cudaStream_t st) {
-    k3_p2m_lanes<P><<<unsigned(((int64_t(1) << (3 * L)) + W3 - 1) / W3), W3 * 32, 0, st>>>(L, start,
-                                                                                          rec, me);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_p2m_lanes(int p, int L, const uint32_t *start, const float4 *rec, float2 *me,
-                             cudaStream_t st) {
+template <typename T, typename Rec>
+cudaError_t launch_p2m_lanes(int p, int L, const Dom3 &d, const uint32_t *start, const Rec *rec,
+                             typename C3<T>::V *me, cudaStream_t st) {
+    const unsigned grid = unsigned(((int64_t(1) << (3 * L)) + W3 - 1) / W3);
     switch (p) {
-#define PL_CASE(P) case P: return p2m_lanes_p<P>(L, start, rec, me, st);
+#define PL_CASE(P) \
+    case P: k3_p2m_lanes<P, T><<<grid, W3 * 32, 0, st>>>(L, d, start, rec, me); break;
         PL_CASE(1) PL_CASE(2) PL_CASE(3) PL_CASE(4) PL_CASE(5) PL_CASE(6) PL_CASE(7) PL_CASE(8)
 #undef PL_CASE
         default: return cudaErrorInvalidValue;
     }
-}
-
-// ---------------------------------------------------------------------------
-// M2M (parent level l from level l + 1): M~'_n^m = sum_children sum_{k,l}
-// conj(R_k^l(e_c)) 2^-(n-k) M~_{n-k}^{m-l}.  A warp per parent box, lanes over
-// output coefficients, children in octant order.
-// ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(W3 * 32) k3_m2m(int l, int L, int p, const uint32_t *__restrict__ start,
-                                                  const typename C3<T>::V *__restrict__ rtab,
-                                                  typename C3<T>::V *__restrict__ me) {
-    using V = typename C3<T>::V;
-    const int lane = threadIdx.x & 31;
-    const int64_t b = int64_t(blockIdx.x) * W3 + (threadIdx.x >> 5);
-    if (b >= (int64_t(1) << (3 * l))) return;
-    if (box_count3(start, L, l, uint32_t(b)) == 0) return;
-    const int nc = nc3(p);
-    V acc[OUT3];
-    int on[OUT3], om[OUT3];
-#pragma unroll
-    for (int u = 0; u < OUT3; ++u) {
-        acc[u] = mk<V>(T(0), T(0));
-        const int j = lane + 32 * u;
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= j) ++n;
-        on[u] = n;
-        om[u] = j - n * (n + 1) / 2;
-    }
-    for (int c = 0; c < 8; ++c) {
-        const uint32_t cb = uint32_t(b) * 8u + uint32_t(c);
-        if (box_count3(start, L, l + 1, cb) == 0) continue;
-        const V *mc = me + (lvl_off3(l + 1) + cb) * nc;
-        const V *rt = rtab + c * nc;
-#pragma unroll
-        for (int u = 0; u < OUT3; ++u) {
-            if (lane + 32 * u >= nc) continue;
-            const int n = on[u], m = om[u];
-            V s = mk<V>(T(0), T(0));
-            for (int k = 0; k <= n; ++k) {
-                V sk = mk<V>(T(0), T(0));
-                for (int ll = -k; ll <= k; ++ll) {
-                    const int mm = m - ll;
-                    if (mm < -(n - k) || mm > n - k) continue;
-                    cmac_conj(sk, coef3(rt, k, ll), coef3(mc, n - k, mm));
-                }
-                const T sc = T(ldexp(1.0, -(n - k)));
-                s.x += sk.x * sc;
-                s.y += sk.y * sc;
-            }
-            acc[u].x += s.x;
-            acc[u].y += s.y;
-        }
-    }
-    V *dst = me + (lvl_off3(l) + b) * nc;
-#pragma unroll
-    for (int u = 0; u < OUT3; ++u)
-        if (lane + 32 * u < nc) dst[lane + 32 * u] = acc[u];
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -1549,170 +1480,124 @@ __global__ void __launch_bounds__(TC3_THREADS, 1) k3_m2l_tc(int L, const uint32_
 }
 
 // ---------------------------------------------------------------------------
-// L2L (child level l >= 3): L~'_j^s += 2^-(j+1) sum_{k,l} L~_{j+k}^{s+l}(parent)
-// conj(R_k^l(e_c)).  A warp per child box.
+// M2M and L2L by reflections.  In the real basis of the M2L matrices the
+// operator of child octant c is S_c A S_c with the one of octant 0 and S_c the
+// signs of the coefficients under the reflections c (bits of c against a
+// coefficient's parities q).  So all eight children of a box share one real
+// p^2 x p^2 product:
+//   M2M  M'_r = sum_k A[k][r] H[q(r) ^ q(k)][k],
+//        H[g][k] = sum_c (-1)^popc(g & c) M_c[k]  (three butterfly stages)
+//   L2L  L_c[r] = sum_f (-1)^popc((f ^ q(r)) & c) Z_f[r],
+//        Z_f[r] = sum over the k of parity class f of B[k][r] L[k]
+// (the rows of B and L sorted by class).  A thread per (box, coefficient),
+// about 256 a block; operators come through L1.  Bound by launches and load
+// latency: one GB300, M2M / L2L together, all levels:
+//   262,144 charges, L = 4, p = 8, FP64    1.22 / 0.08 ms
+//   2 M uniform charges, L = 5, p = 8, FP32    0.135 / 0.088 ms
+// (a warp per box over the complex sums, in FP32 eight real matrices).
 // ---------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(W3 * 32) k3_l2l(int l, int L, int p, const uint32_t *__restrict__ start,
-                                                  const typename C3<T>::V *__restrict__ rtab,
-                                                  typename C3<T>::V *__restrict__ le) {
-    using V = typename C3<T>::V;
-    const int lane = threadIdx.x & 31;
-    const int64_t cb = int64_t(blockIdx.x) * W3 + (threadIdx.x >> 5);
-    if (cb >= (int64_t(1) << (3 * l))) return;
-    if (box_count3(start, L, l, uint32_t(cb)) == 0) return;
-    const int nc = nc3(p);
-    const V *lp = le + (lvl_off3(l - 1) + (cb >> 3)) * nc;
-    const V *rt = rtab + int(cb & 7) * nc;
-    V *dst = le + (lvl_off3(l) + cb) * nc;
-    for (int j0 = lane; j0 < nc; j0 += 32) {
-        int j = 0;
-        while ((j + 1) * (j + 2) / 2 <= j0) ++j;
-        const int s = j0 - j * (j + 1) / 2;
-        V acc = mk<V>(T(0), T(0));
-        for (int k = 0; j + k < p; ++k)
-            for (int ll = -k; ll <= k; ++ll) {
-                const int ss = s + ll;
-                if (ss < -(j + k) || ss > j + k) continue;
-                cmac_conj(acc, coef3(rt, k, ll), coef3(lp, j + k, ss));
-            }
-        const T sc = T(ldexp(1.0, -(j + 1)));
-        V o = dst[j0];
-        o.x += acc.x * sc;
-        o.y += acc.y * sc;
-        dst[j0] = o;
-    }
-}
+struct Shift3 {
+    int p, nr, boxes;           // terms, p^2, boxes per block
+    int cls[9];                 // rows of class f: cls[f] .. cls[f + 1]
+};
 
-// ---------------------------------------------------------------------------
-// M2M and L2L of the mixed path for p <= 8 as real matrix-vector products:
-// each of the eight child octants has a fixed real P^2 x P^2 operator in the
-// real basis of the M2L matrices (the sums of k3_m2m / k3_l2l applied to the
-// basis vectors on the host in FP64), staged in shared memory for a block.
-// ---------------------------------------------------------------------------
-constexpr int TT_MAXP = 8;  // operators of up to 64 x 64 in shared memory
-
-// A warp per parent box of level l: ME = sum over occupied children c of
-// A_c x_c, x_c the child's ME in the real basis; lanes over output rows.
-template <int P>
-__global__ void __launch_bounds__(W3 * 32) k3_m2m_real(int l, int L, const uint32_t *__restrict__ start,
-                                                       const float *__restrict__ op,
-                                                       const short2 *__restrict__ rmap,
-                                                       float2 *__restrict__ me) {
-    constexpr int NC = P * (P + 1) / 2, NR = P * P, RL = (NR + 31) / 32;
-    __shared__ float sA[NR * NR];  // sA[k_in * NR + r_out]
-    __shared__ float sx[W3][NR];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t b = int64_t(blockIdx.x) * W3 + wid;
-    const bool act = b < (int64_t(1) << (3 * l)) && box_count3(start, L, l, uint32_t(b)) != 0;
-    short2 rm[RL];
-    float acc[RL];
+// Boxes of level l (M2M: from level l + 1; L2L: to level l + 1).
+template <typename T, bool L2L>
+__global__ void __launch_bounds__(256) k3_shift(int l, int L, const Shift3 s,
+                                                const uint32_t *__restrict__ start,
+                                                const T *__restrict__ op,
+                                                const short2 *__restrict__ rmap,
+                                                const uint8_t *__restrict__ par,
+                                                const uint16_t *__restrict__ order,
+                                                typename C3<T>::V *__restrict__ ex) {
+    __shared__ T sh[L2L ? 256 : 256 * 8];
+    __shared__ uint8_t spar[256];
+    const int nr = s.nr, nc = nc3(s.p);
+    const int w = int(threadIdx.x) / nr, r = int(threadIdx.x) - w * nr;
+    const int64_t b = int64_t(blockIdx.x) * s.boxes + w;
+    const bool act = w < s.boxes && b < (int64_t(1) << (3 * l)) &&
+                     box_count3(start, L, l, uint32_t(b)) != 0;
+    const short2 rm = w < s.boxes ? rmap[r] : make_short2(0, 0);
+    const int q = w < s.boxes ? par[r] : 0;
+    // real element rm of a series: component 2 coefficient + (Im: 1)
+    const int at = 2 * rm.x + (rm.y == 1 ? 1 : 0);
+    if (w == 0) spar[r] = uint8_t(q);
+    T v[8];
 #pragma unroll
-    for (int i = 0; i < RL; ++i) {
-        const int r = lane + 32 * i;
-        rm[i] = r < NR ? rmap[r] : make_short2(0, 0);
-        acc[i] = 0.f;
-    }
-    for (int c = 0; c < 8; ++c) {
-        __syncthreads();  // the previous operator is no longer read
-        for (int t = threadIdx.x; t < NR * NR; t += W3 * 32) sA[t] = op[size_t(c) * NR * NR + t];
-        const uint32_t cb = uint32_t(b) * 8u + uint32_t(c);
-        const bool use = act && box_count3(start, L, l + 1, cb) != 0;
-        if (use) {
-            const float2 *mc = me + (lvl_off3(l + 1) + cb) * NC;
+    for (int c = 0; c < 8; ++c) v[c] = T(0);
+    if (!L2L) {
+        if (act) {
 #pragma unroll
-            for (int i = 0; i < RL; ++i) {
-                const int r = lane + 32 * i;
-                if (r < NR) {
-                    const float2 v = mc[rm[i].x];
-                    sx[wid][r] = rm[i].y == 1 ? v.y : v.x;
-                }
+            for (int c = 0; c < 8; ++c) {
+                const uint32_t cb = uint32_t(b) * 8u + uint32_t(c);
+                if (box_count3(start, L, l + 1, cb) != 0)
+                    v[c] = reinterpret_cast<const T *>(ex + (lvl_off3(l + 1) + cb) * nc)[at];
             }
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (!(c & o)) {
+                        const T a = v[c], d = v[c | o];
+                        v[c] = a + d;
+                        v[c | o] = a - d;
+                    }
+        }
+        if (w < s.boxes)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sh[threadIdx.x * 8 + c] = v[c];
+        __syncthreads();
+        if (!act) return;
+        const T *h = sh + w * nr * 8;
+        T acc = T(0);
+#pragma unroll 8
+        for (int k = 0; k < nr; ++k) acc = fma(op[k * nr + r], h[k * 8 + (q ^ spar[k])], acc);
+        T *dst = reinterpret_cast<T *>(ex + (lvl_off3(l) + b) * nc);
+        dst[at] = acc;
+        if (rm.y == 2) dst[at + 1] = T(0);  // Im of m = 0
+    } else {
+        if (act) {  // row r of the sorted order
+            const short2 o = rmap[order[r]];
+            sh[threadIdx.x] = reinterpret_cast<const T *>(
+                ex + (lvl_off3(l) + b) * nc)[2 * o.x + (o.y == 1 ? 1 : 0)];
         }
         __syncthreads();
-        if (use)
-            for (int k = 0; k < NR; ++k) {
-                const float xk = sx[wid][k];
+        if (!act) return;
+        const T *y = sh + w * nr;
 #pragma unroll
-                for (int i = 0; i < RL; ++i)
-                    if (lane + 32 * i < NR) acc[i] = fmaf(sA[k * NR + lane + 32 * i], xk, acc[i]);
-            }
-    }
-    if (!act) return;
-    float *dst = reinterpret_cast<float *>(me + (lvl_off3(l) + b) * NC);
-#pragma unroll
-    for (int i = 0; i < RL; ++i)
-        if (lane + 32 * i < NR) {
-            dst[2 * rm[i].x + (rm[i].y == 1 ? 1 : 0)] = acc[i];
-            if (rm[i].y == 2) dst[2 * rm[i].x + 1] = 0.f;  // Im of m = 0
+        for (int f = 0; f < 8; ++f) {
+            T acc = T(0);
+#pragma unroll 8
+            for (int k = s.cls[f]; k < s.cls[f + 1]; ++k) acc = fma(op[k * nr + r], y[k], acc);
+            v[f] = acc;
         }
-}
-
-// L2L: a block per (child octant o, W3 parents of level l - 1), a warp per
-// parent; its child of octant o adds B_o y to the local expansion that M2L
-// wrote, y the parent's LE in the real basis.
-template <int P>
-__global__ void __launch_bounds__(W3 * 32) k3_l2l_real(int l, int L, const uint32_t *__restrict__ start,
-                                                       const float *__restrict__ op,
-                                                       const short2 *__restrict__ rmap,
-                                                       float2 *__restrict__ le) {
-    constexpr int NC = P * (P + 1) / 2, NR = P * P, RL = (NR + 31) / 32;
-    __shared__ float sA[NR * NR];
-    __shared__ float sx[W3][NR];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int o = int(blockIdx.x & 7u);
-    const int64_t pb = int64_t(blockIdx.x >> 3) * W3 + wid;
-    const int64_t cb = pb * 8 + o;
-    const bool act = pb < (int64_t(1) << (3 * (l - 1))) && box_count3(start, L, l, uint32_t(cb)) != 0;
-    for (int t = threadIdx.x; t < NR * NR; t += W3 * 32) sA[t] = op[size_t(o) * NR * NR + t];
-    short2 rm[RL];
 #pragma unroll
-    for (int i = 0; i < RL; ++i) {
-        const int r = lane + 32 * i;
-        rm[i] = r < NR ? rmap[r] : make_short2(0, 0);
-        if (act && r < NR) {
-            const float2 v = le[(lvl_off3(l - 1) + pb) * NC + rm[i].x];
-            sx[wid][r] = rm[i].y == 1 ? v.y : v.x;
+        for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                if (!(c & o)) {
+                    const T a = v[c], d = v[c | o];
+                    v[c] = a + d;
+                    v[c | o] = a - d;
+                }
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            const uint32_t cb = uint32_t(b) * 8u + uint32_t(c);
+            if (box_count3(start, L, l + 1, cb) == 0) continue;
+            T *dst = reinterpret_cast<T *>(ex + (lvl_off3(l + 1) + cb) * nc) + at;
+            *dst += __popc(q & c) & 1 ? -v[c] : v[c];
         }
     }
-    __syncthreads();
-    if (!act) return;
-    float acc[RL];
-#pragma unroll
-    for (int i = 0; i < RL; ++i) acc[i] = 0.f;
-    for (int k = 0; k < NR; ++k) {
-        const float xk = sx[wid][k];
-#pragma unroll
-        for (int i = 0; i < RL; ++i)
-            if (lane + 32 * i < NR) acc[i] = fmaf(sA[k * NR + lane + 32 * i], xk, acc[i]);
-    }
-    float *dst = reinterpret_cast<float *>(le + (lvl_off3(l) + cb) * NC);
-#pragma unroll
-    for (int i = 0; i < RL; ++i)
-        if (lane + 32 * i < NR) dst[2 * rm[i].x + (rm[i].y == 1 ? 1 : 0)] += acc[i];
 }
 
-template <int P>
-cudaError_t m2m_l2l_real_p(bool m2m, int l, int L, const uint32_t *start, const float *op,
-                           const short2 *rmap, float2 *ex, cudaStream_t st) {
-    if (m2m)
-        k3_m2m_real<P><<<unsigned(((int64_t(1) << (3 * l)) + W3 - 1) / W3), W3 * 32, 0, st>>>(
-            l, L, start, op, rmap, ex);
-    else
-        k3_l2l_real<P><<<unsigned(8 * (((int64_t(1) << (3 * (l - 1))) + W3 - 1) / W3)), W3 * 32, 0,
-                         st>>>(l, L, start, op, rmap, ex);
+template <typename T, bool L2L>
+cudaError_t launch_shift3(int l, int L, const Shift3 &s, const uint32_t *start, const T *op,
+                          const short2 *rmap, const uint8_t *par, const uint16_t *order,
+                          typename C3<T>::V *ex, cudaStream_t st) {
+    const int64_t blocks = ((int64_t(1) << (3 * l)) + s.boxes - 1) / s.boxes;
+    k3_shift<T, L2L><<<unsigned(blocks), unsigned(s.boxes * s.nr + 31) / 32 * 32, 0, st>>>(
+        l, L, s, start, op, rmap, par, order, ex);
     return cudaGetLastError();
-}
-
-// m2m: level l's parents from level l + 1; else level l's children from l - 1
-cudaError_t launch_m2m_l2l_real(bool m2m, int p, int l, int L, const uint32_t *start,
-                                const float *op, const short2 *rmap, float2 *ex, cudaStream_t st) {
-    switch (p) {
-#define TT_CASE(P) case P: return m2m_l2l_real_p<P>(m2m, l, L, start, op, rmap, ex, st);
-        TT_CASE(1) TT_CASE(2) TT_CASE(3) TT_CASE(4) TT_CASE(5) TT_CASE(6) TT_CASE(7) TT_CASE(8)
-#undef TT_CASE
-        default: return cudaErrorInvalidValue;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2772,37 +2657,31 @@ cd host_coef(const cd *a, int n, int m) {
     return (m & 1) ? -v : v;
 }
 
-// The M2M sum of k3_m2m for one child (rt: R_k^l of the child's offset):
-// out_n^m = sum_k 2^-(n-k) sum_l conj(R_k^l) M_{n-k}^{m-l}.
-void host_m2m_one(int p, const cd *rt, const cd *mc, cd *out) {
-    for (int n = 0; n < p; ++n)
+// The M2M sum for one child (rt: R_k^l of the child's offset) of a series mc
+// whose only degree is n0: out_n^m = sum_l conj(R_k^l) M_{n0}^{m-l} 2^-n0,
+// k = n - n0.
+void host_m2m_one(int p, int n0, const cd *rt, const cd *mc, cd *out) {
+    std::fill(out, out + p * (p + 1) / 2, cd(0.0, 0.0));
+    for (int n = n0; n < p; ++n)
         for (int m = 0; m <= n; ++m) {
+            const int k = n - n0;
             cd s(0.0, 0.0);
-            for (int k = 0; k <= n; ++k) {
-                cd sk(0.0, 0.0);
-                for (int ll = -k; ll <= k; ++ll) {
-                    const int mm = m - ll;
-                    if (mm < -(n - k) || mm > n - k) continue;
-                    sk += std::conj(host_coef(rt, k, ll)) * host_coef(mc, n - k, mm);
-                }
-                s += sk * std::ldexp(1.0, -(n - k));
-            }
-            out[n * (n + 1) / 2 + m] = s;
+            for (int ll = std::max(-k, m - n0); ll <= std::min(k, m + n0); ++ll)
+                s += std::conj(host_coef(rt, k, ll)) * host_coef(mc, n0, m - ll);
+            out[n * (n + 1) / 2 + m] = s * std::ldexp(1.0, -n0);
         }
 }
 
-// The L2L sum of k3_l2l for one child: out_j^s = 2^-(j+1) sum_{k, l}
-// conj(R_k^l) L_{j+k}^{s+l}.
-void host_l2l_one(int p, const cd *rt, const cd *lp, cd *out) {
-    for (int j = 0; j < p; ++j)
+// The L2L sum for one child of a series lp whose only degree is n0:
+// out_j^s = 2^-(j+1) sum_l conj(R_k^l) L_{n0}^{s+l}, k = n0 - j.
+void host_l2l_one(int p, int n0, const cd *rt, const cd *lp, cd *out) {
+    std::fill(out, out + p * (p + 1) / 2, cd(0.0, 0.0));
+    for (int j = 0; j <= n0; ++j)
         for (int s = 0; s <= j; ++s) {
+            const int k = n0 - j;
             cd acc(0.0, 0.0);
-            for (int k = 0; j + k < p; ++k)
-                for (int ll = -k; ll <= k; ++ll) {
-                    const int ss = s + ll;
-                    if (ss < -(j + k) || ss > j + k) continue;
-                    acc += std::conj(host_coef(rt, k, ll)) * host_coef(lp, j + k, ss);
-                }
+            for (int ll = std::max(-k, -n0 - s); ll <= std::min(k, n0 - s); ++ll)
+                acc += std::conj(host_coef(rt, k, ll)) * host_coef(lp, n0, s + ll);
             out[j * (j + 1) / 2 + s] = acc * std::ldexp(1.0, -(j + 1));
         }
 }
@@ -2814,14 +2693,17 @@ template <typename F> void host_real_matrix(int p, F apply, double *a) {
     const int nc = p * (p + 1) / 2, nr = p * p;
     // real index -> (coefficient, imaginary part?)
     std::vector<int> jof(static_cast<size_t>(nr)), imof(static_cast<size_t>(nr), 0);
+    std::vector<int> nof(static_cast<size_t>(nr));  // its degree
     std::vector<int> imidx(size_t(nc), -1);
     for (int n = 0, r = nc; n < p; ++n)
         for (int m = 0; m <= n; ++m) {
             const int j = n * (n + 1) / 2 + m;
             jof[size_t(j)] = j;
+            nof[size_t(j)] = n;
             if (m > 0) {
                 imidx[size_t(j)] = r;
                 jof[size_t(r)] = j;
+                nof[size_t(r)] = n;
                 imof[size_t(r++)] = 1;
             }
         }
@@ -2829,7 +2711,7 @@ template <typename F> void host_real_matrix(int p, F apply, double *a) {
     for (int k = 0; k < nr; ++k) {
         std::fill(in.begin(), in.end(), cd(0.0, 0.0));
         in[size_t(jof[size_t(k)])] = imof[size_t(k)] ? cd(0.0, 1.0) : cd(1.0, 0.0);
-        apply(in.data(), out.data());
+        apply(nof[size_t(k)], in.data(), out.data());
         for (int j = 0; j < nc; ++j) {
             a[size_t(k) * nr + j] = out[size_t(j)].real();
             if (imidx[size_t(j)] >= 0) a[size_t(k) * nr + imidx[size_t(j)]] = out[size_t(j)].imag();
@@ -2844,9 +2726,9 @@ void host_shift_real(int p, int kind, int octant, double *a) {
     host_rec_r((octant & 1) ? 0.25 : -0.25, (octant & 2) ? 0.25 : -0.25,
                (octant & 4) ? 0.25 : -0.25, p, ro.data());
     if (kind == 0)
-        host_real_matrix(p, [&](const cd *in, cd *out) { host_m2m_one(p, ro.data(), in, out); }, a);
+        host_real_matrix(p, [&](int n, const cd *in, cd *out) { host_m2m_one(p, n, ro.data(), in, out); }, a);
     else
-        host_real_matrix(p, [&](const cd *in, cd *out) { host_l2l_one(p, ro.data(), in, out); }, a);
+        host_real_matrix(p, [&](int n, const cd *in, cd *out) { host_l2l_one(p, n, ro.data(), in, out); }, a);
 }
 
 struct DevBuf3 {
@@ -2884,8 +2766,9 @@ struct petfmm3d_ctx {
     DevBuf3 pitems, slots, nown, nflags, nctrl;
     bool no_pairs = false;  // no room for the parts of pairwise sums
     // operator tables of the context's precision only
-    DevBuf3 rtab32, rtab64, atab32, atab64, rmap, parity;
-    DevBuf3 m2m32, l2l32;  // p <= 8: the real M2M / L2L operators of the 8 octants
+    DevBuf3 atab32, atab64, rmap, parity;
+    DevBuf3 shift, order;  // the M2M and L2L operators of octant 0, rows by parity class
+    Shift3 sh{};
     DevBuf3 tcimg;  // p <= 8: TF32 hi / lo images of the M2L operators (tensor-core M2L)
     bool m2l_tc = true;  // PETFMM3D_OPT_M2L_TC
     bool timing = false, ev_recorded = false;
@@ -2908,10 +2791,6 @@ constexpr size_t kPairs3MaxBytes = (size_t(1) << 26) * P3_SLOTS * sizeof(float4)
 
 int upload_tables(petfmm3d_ctx *c) {
     const int p = c->p, nc = nc3(p), nci = nci3(p);
-    std::vector<cd> rt(size_t(8) * nc);
-    for (int o = 0; o < 8; ++o)
-        host_rec_r((o & 1) ? 0.25 : -0.25, (o & 2) ? 0.25 : -0.25, (o & 4) ? 0.25 : -0.25, p,
-                   rt.data() + size_t(o) * nc);
     // the real basis of the M2L matrices: real index r < nc is Re of
     // coefficient r, r >= nc Im of the coefficients with m > 0 in order;
     // parity: bit d set if the solid harmonic changes sign with axis d
@@ -2930,7 +2809,33 @@ int upload_tables(petfmm3d_ctx *c) {
         }
     P3_TRY(ensure3(c->rmap, rm.size() * sizeof(short2), c->stream));
     P3_CUDA(cudaMemcpy(c->rmap.p, rm.data(), rm.size() * sizeof(short2), cudaMemcpyHostToDevice));
+    P3_TRY(ensure3(c->parity, par.size(), c->stream));
+    P3_CUDA(cudaMemcpy(c->parity.p, par.data(), par.size(), cudaMemcpyHostToDevice));
     std::vector<double> a64(size_t(nr) * nr);
+    // M2M [k_in][r_out], then L2L with the rows k_in by parity class
+    c->sh = Shift3{p, nr, std::max(1, 256 / nr), {}};
+    std::vector<uint16_t> order;
+    for (int f = 0; f < 8; ++f) {
+        c->sh.cls[f] = int(order.size());
+        for (int r = 0; r < nr; ++r)
+            if (par[size_t(r)] == f) order.push_back(uint16_t(r));
+    }
+    c->sh.cls[8] = nr;
+    std::vector<double> ops(size_t(2) * nr * nr);
+    host_shift_real(p, 0, 0, ops.data());
+    host_shift_real(p, 1, 0, a64.data());
+    for (int k = 0; k < nr; ++k)
+        std::copy_n(a64.data() + size_t(order[size_t(k)]) * nr, nr,
+                    ops.data() + size_t(nr + k) * nr);
+    const std::vector<float> ops32(ops.begin(), ops.end());
+    const bool f64 = c->precision == PETFMM_FP64;
+    const size_t es = f64 ? sizeof(double) : sizeof(float);
+    P3_TRY(ensure3(c->shift, ops.size() * es, c->stream));
+    P3_TRY(ensure3(c->order, order.size() * sizeof(uint16_t), c->stream));
+    P3_CUDA(cudaMemcpy(c->shift.p, f64 ? static_cast<const void *>(ops.data()) : ops32.data(),
+                       ops.size() * es, cudaMemcpyHostToDevice));
+    P3_CUDA(cudaMemcpy(c->order.p, order.data(), order.size() * sizeof(uint16_t),
+                       cudaMemcpyHostToDevice));
     std::vector<cd> iv(static_cast<size_t>(nci));
     if (c->precision == PETFMM_FP64) {
         // [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
@@ -2941,14 +2846,8 @@ int upload_tables(petfmm3d_ctx *c) {
             host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
             host_m2l_real(p, iv.data(), at.data() + size_t(o) * nr * nr);
         }
-        std::vector<double2> r64(rt.size());
-        for (size_t i = 0; i < rt.size(); ++i) r64[i] = make_double2(rt[i].real(), rt[i].imag());
         P3_TRY(ensure3(c->atab64, at.size() * sizeof(double), c->stream));
-        P3_TRY(ensure3(c->parity, par.size(), c->stream));
-        P3_TRY(ensure3(c->rtab64, r64.size() * sizeof(double2), c->stream));
         P3_CUDA(cudaMemcpy(c->atab64.p, at.data(), at.size() * sizeof(double), cudaMemcpyHostToDevice));
-        P3_CUDA(cudaMemcpy(c->parity.p, par.data(), par.size(), cudaMemcpyHostToDevice));
-        P3_CUDA(cudaMemcpy(c->rtab64.p, r64.data(), r64.size() * sizeof(double2), cudaMemcpyHostToDevice));
         return PETFMM_OK;
     }
     // The mixed path's M2L matrices, FP32: ap[k_in * nrp + r_out]; for p <= 8
@@ -2956,7 +2855,7 @@ int upload_tables(petfmm3d_ctx *c) {
     // [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero padding), K in the
     // input basis of the tensor-core M2L (coefficient by coefficient: Re, then
     // Im if m > 0), N in the M2L matrices' basis.
-    const bool tc = p <= TT_MAXP;
+    const bool tc = p <= TC3_MAXP;
     std::vector<float> at(size_t(NSLOT3) * nrp * nrp, 0.f);
     std::vector<float> img(tc ? size_t(NSLOT3) * 2 * nrp * nrp : 0, 0.f);
     std::vector<int> tc3_kin(static_cast<size_t>(nr));
@@ -2993,24 +2892,6 @@ int upload_tables(petfmm3d_ctx *c) {
     }
     P3_TRY(ensure3(c->atab32, at.size() * sizeof(float), c->stream));
     P3_CUDA(cudaMemcpy(c->atab32.p, at.data(), at.size() * sizeof(float), cudaMemcpyHostToDevice));
-    std::vector<float2> r32(rt.size());
-    for (size_t i = 0; i < rt.size(); ++i) r32[i] = make_float2(float(rt[i].real()), float(rt[i].imag()));
-    P3_TRY(ensure3(c->rtab32, r32.size() * sizeof(float2), c->stream));
-    P3_CUDA(cudaMemcpy(c->rtab32.p, r32.data(), r32.size() * sizeof(float2), cudaMemcpyHostToDevice));
-    if (p <= TT_MAXP) {
-        // op[(octant * p^2 + k_in) * p^2 + r_out]
-        std::vector<float> mm(size_t(8) * nr * nr), ll(size_t(8) * nr * nr);
-        for (int o = 0; o < 8; ++o) {
-            host_shift_real(p, 0, o, a64.data());
-            for (size_t i = 0; i < size_t(nr) * nr; ++i) mm[size_t(o) * nr * nr + i] = float(a64[i]);
-            host_shift_real(p, 1, o, a64.data());
-            for (size_t i = 0; i < size_t(nr) * nr; ++i) ll[size_t(o) * nr * nr + i] = float(a64[i]);
-        }
-        P3_TRY(ensure3(c->m2m32, mm.size() * sizeof(float), c->stream));
-        P3_TRY(ensure3(c->l2l32, ll.size() * sizeof(float), c->stream));
-        P3_CUDA(cudaMemcpy(c->m2m32.p, mm.data(), mm.size() * sizeof(float), cudaMemcpyHostToDevice));
-        P3_CUDA(cudaMemcpy(c->l2l32.p, ll.data(), ll.size() * sizeof(float), cudaMemcpyHostToDevice));
-    }
     return PETFMM_OK;
 }
 
@@ -3124,35 +3005,23 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
     const int L = c->L, p = c->p;
     cudaStream_t st = c->stream;
     V *me = static_cast<V *>(c->me.p), *le = static_cast<V *>(c->le.p);
-    const bool f32 = sizeof(T) == 4;
-    const V *rtab = static_cast<const V *>(f32 ? c->rtab32.p : c->rtab64.p);
     const Dom3 d = make_dom3(c->dom, L);
     mark3(c, PETFMM3D_STAGE_P2M);
-    if constexpr (sizeof(T) == 4) {
-        if (p <= 8)
-            P3_CUDA(launch_p2m_lanes(p, L, start, static_cast<const float4 *>(c->rec.p), me, st));
-        else
-            k3_p2m<T, float4><<<grid_w(int64_t(1) << (3 * L)), W3 * 32, 0, st>>>(
-                L, p, d, start, static_cast<const float4 *>(c->rec.p), me);
-    } else
-        k3_p2m<T, Dbl4><<<grid_w(int64_t(1) << (3 * L)), W3 * 32, 0, st>>>(
-            L, p, d, start, static_cast<const Dbl4 *>(c->xs.p), me);
+    using Rec = std::conditional_t<sizeof(T) == 4, float4, Dbl4>;
+    const Rec *rec = static_cast<const Rec *>(sizeof(T) == 4 ? c->rec.p : c->xs.p);
+    if (p <= 8)
+        P3_CUDA(launch_p2m_lanes<T>(p, L, d, start, rec, me, st));
+    else
+        k3_p2m<T, Rec><<<grid_w(int64_t(1) << (3 * L)), W3 * 32, 0, st>>>(L, p, d, start, rec, me);
     P3_CUDA(cudaGetLastError());
     c->launches++;
     mark3(c, PETFMM3D_STAGE_M2M);
-    // mixed path with p <= 8: M2M and L2L as real matrix-vector products
-    const bool real_tt = sizeof(T) == 4 && p <= TT_MAXP;
+    const T *op = static_cast<const T *>(c->shift.p);
+    const short2 *rmap = static_cast<const short2 *>(c->rmap.p);
+    const uint8_t *par = static_cast<const uint8_t *>(c->parity.p);
+    const uint16_t *order = static_cast<const uint16_t *>(c->order.p);
     for (int l = L - 1; l >= 2; --l) {
-        if constexpr (sizeof(T) == 4) {
-            if (real_tt) {
-                P3_CUDA(launch_m2m_l2l_real(true, p, l, L, start, static_cast<const float *>(c->m2m32.p),
-                                            static_cast<const short2 *>(c->rmap.p), me, st));
-                c->launches++;
-                continue;
-            }
-        }
-        k3_m2m<T><<<grid_w(int64_t(1) << (3 * l)), W3 * 32, 0, st>>>(l, L, p, start, rtab, me);
-        P3_CUDA(cudaGetLastError());
+        P3_CUDA((launch_shift3<T, false>(l, L, c->sh, start, op, rmap, par, order, me, st)));
         c->launches++;
     }
     mark3(c, PETFMM3D_STAGE_M2L);
@@ -3160,7 +3029,7 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
     // p <= 8 (launch_m2l_gemm launches at l = L)
     const bool one = sizeof(T) == 8 || mg_nrp(p) <= 64;
     // mixed path, p <= 8, PETFMM3D_OPT_M2L_TC: all levels on the tensor cores
-    const bool tc = sizeof(T) == 4 && c->m2l_tc && p <= TT_MAXP;
+    const bool tc = sizeof(T) == 4 && c->m2l_tc && p <= TC3_MAXP;
     if constexpr (sizeof(T) == 4) {
         if (tc) {
             P3_CUDA(launch_m2l_tc3(p, L, start, static_cast<const float *>(c->tcimg.p), me, le,
@@ -3188,17 +3057,9 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
         c->launches++;
     }
     mark3(c, PETFMM3D_STAGE_L2L);
-    for (int l = 3; l <= L; ++l) {
-        if constexpr (sizeof(T) == 4) {
-            if (real_tt) {
-                P3_CUDA(launch_m2m_l2l_real(false, p, l, L, start, static_cast<const float *>(c->l2l32.p),
-                                            static_cast<const short2 *>(c->rmap.p), le, st));
-                c->launches++;
-                continue;
-            }
-        }
-        k3_l2l<T><<<grid_w(int64_t(1) << (3 * l)), W3 * 32, 0, st>>>(l, L, p, start, rtab, le);
-        P3_CUDA(cudaGetLastError());
+    for (int l = 2; l < L; ++l) {
+        P3_CUDA((launch_shift3<T, true>(l, L, c->sh, start, op + size_t(c->sh.nr) * c->sh.nr, rmap,
+                                        par, order, le, st)));
         c->launches++;
     }
     return PETFMM_OK;
@@ -3540,8 +3401,8 @@ int petfmm3d_destroy(petfmm3d_ctx *c) {
                        &c->nown, &c->nflags, &c->nctrl,
                        &c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->sortw, &c->start,
                        &c->recu,  &c->rec,   &c->xs,    &c->me,    &c->le,    &c->status,
-                       &c->rtab32, &c->rtab64, &c->atab32, &c->atab64, &c->parity, &c->rmap,
-                       &c->m2m32, &c->l2l32, &c->tcimg};
+                       &c->atab32, &c->atab64, &c->parity, &c->rmap,
+                       &c->shift, &c->order, &c->tcimg};
     for (DevBuf3 *b : bufs)
         if (b->p) cudaFree(b->p);
     for (int i = 0; i <= PETFMM3D_STAGE_COUNT; ++i)
