@@ -319,7 +319,10 @@ void free_op_tables(OpTables *t) {
 // cluster spread over all SMs.  Per leaf, lanes take 32 particles at a time,
 // write the gamma * zeta^k powers to shared memory, and lane k sums column k
 // in a fixed order: each leaf's expansion does not depend on which warp or
-// in which order the leaves were processed.
+// in which order the leaves were processed.  Two leaves of at most 16 blobs
+// share a warp: the FP64 pipe, two lanes a cycle and SM, bounds the FP64 path,
+// and half of the lanes held no blob (1M blobs, 16 a leaf, p = 17: 583 -> 294
+// us).
 // ----------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_occ_list(const Task *__restrict__ tasks, int ntasks,
                                                   const InstDesc *__restrict__ insts,
@@ -370,66 +373,97 @@ __global__ void __launch_bounds__(P2M_WARPS * 32) k_p2m(
     const int lane = threadIdx.x & 31;
     const uint32_t nocc = ctrl[CTRL_NOCC];
     const uint32_t nwarps = gridDim.x * P2M_WARPS;
-    for (uint32_t i = blockIdx.x * P2M_WARPS + (threadIdx.x >> 5); i < nocc; i += nwarps) {
-        const uint2 e = occ[i];
+    // leaf range of occupied-leaf entry i (empty past the end, and in the
+    // checked build when it lies outside its instance)
+    auto range = [&](uint32_t i, uint2 &e, uint32_t &s0, uint32_t &s1) {
+        e = occ[min(i, nocc - 1)];
         const InstDesc &d = insts[e.x];
-        const int p = d.p, L = d.L;
-        const uint32_t m = e.y;
-        uint32_t s0 = start[d.soff + m], s1 = start[d.soff + m + 1];
-        if (!(PF_IN(m, int64_t(1) << (2 * L)) && PF_IN(int64_t(s0) - d.poff, d.n + 1) &&
+        s0 = start[d.soff + e.y];
+        s1 = i < nocc ? start[d.soff + e.y + 1] : s0;
+        if (!(PF_IN(e.y, int64_t(1) << (2 * d.L)) && PF_IN(int64_t(s0) - d.poff, d.n + 1) &&
               PF_IN(int64_t(s1) - d.poff, d.n + 1)) || s1 < s0)
-            s1 = s0;  // checked build: a leaf range outside the instance is skipped
-        const uint32_t ix = compact_bits(m), iy = compact_bits(m >> 1);
-        const double cx = d.x0 + (double(ix) + 0.5) * d.wleaf;
-        const double cy = d.y0 + (double(iy) + 0.5) * d.wleaf;
-        C2 acc0 = mk2<R>(R(0), R(0)), acc1 = mk2<R>(R(0), R(0));
-        for (uint32_t c0 = s0; c0 < s1; c0 += 32) {
-            const uint32_t j = c0 + lane;
-            C2 z, w;
-            if (j < s1) {
-                if (rec) {
-                    const float4 r = rec[j];
-                    z = mk2<R>(R(r.x), R(r.y));
-                    w = mk2<R>(R(r.z), R(0));
-                } else {
-                    z = mk2<R>(R((xs[j] - cx) * d.scale), R((ys[j] - cy) * d.scale));
-                    w = mk2<R>(R(gs[j]), R(0));
-                }
+            s1 = s0;
+    };
+    // gamma zeta^k of sorted blob j (nothing from end on) in this lane's row;
+    // Laplace: q, then -q zeta^k / k.  (Explicit multiply-adds: the same bits
+    // wherever this is inlined.)
+    auto powers = [&](const InstDesc &d, uint32_t leaf, uint32_t j, uint32_t end) {
+        C2 z = mk2<R>(R(0), R(0)), w = z;
+        if (j < end) {
+            if (rec) {
+                const float4 r = rec[j];
+                z = mk2<R>(R(r.x), R(r.y));
+                w = mk2<R>(R(r.z), R(0));
             } else {
-                z = mk2<R>(R(0), R(0));
-                w = mk2<R>(R(0), R(0));
+                const double cx = fma(double(compact_bits(leaf)) + 0.5, d.wleaf, d.x0);
+                const double cy = fma(double(compact_bits(leaf >> 1)) + 0.5, d.wleaf, d.y0);
+                z = mk2<R>(R((xs[j] - cx) * d.scale), R((ys[j] - cy) * d.scale));
+                w = mk2<R>(R(gs[j]), R(0));
             }
-            // vortex: gamma zeta^k; Laplace: q, then -q zeta^k / k
-            const bool lap = d.kernel == KERNEL_LAPLACE;
-            for (int k = 0; k < p; ++k) {
-                C2 wk = w;
-                if (lap && k) {
-                    const R s = R(-1) / R(k);
-                    wk = mk2<R>(w.x * s, w.y * s);
-                }
-                buf[lane * pmax + k] = wk;
-                w = cmul(w, z);
-            }
-            __syncwarp();
-            if (lane < p) {
-                for (int q = 0; q < 32; ++q) {
-                    const C2 b = buf[q * pmax + lane];
-                    acc0.x += b.x;
-                    acc0.y += b.y;
-                }
-            }
-            if (lane + 32 < p) {
-                for (int q = 0; q < 32; ++q) {
-                    const C2 b = buf[q * pmax + lane + 32];
-                    acc1.x += b.x;
-                    acc1.y += b.y;
-                }
-            }
-            __syncwarp();
         }
-        C2 *dst = me + d.eoff + (lvl_off(L) + box_index(L, ix, iy)) * p;
-        if (lane < p) dst[lane] = acc0;
-        if (lane + 32 < p) dst[lane + 32] = acc1;
+        const bool lap = d.kernel == KERNEL_LAPLACE;
+        for (int k = 0; k < d.p; ++k) {
+            C2 wk = w;
+            if (lap && k) {
+                const R s = R(-1) / R(k);
+                wk = mk2<R>(w.x * s, w.y * s);
+            }
+            buf[lane * pmax + k] = wk;
+            w = mk2<R>(fma(w.x, z.x, -(w.y * z.y)), fma(w.x, z.y, w.y * z.x));
+        }
+    };
+    auto add_rows = [&](C2 &acc, int k, int row, uint32_t rows) {
+#pragma unroll 4
+        for (uint32_t q = 0; q < rows; ++q) {
+            const C2 b = buf[(row + q) * pmax + k];
+            acc.x += b.x;
+            acc.y += b.y;
+        }
+    };
+    auto series = [&](const InstDesc &d, uint32_t leaf) {
+        return me + d.eoff +
+               (lvl_off(d.L) + box_index(d.L, compact_bits(leaf), compact_bits(leaf >> 1))) * d.p;
+    };
+    // two entries at a time once there are more than warps
+    const uint32_t per = nocc > nwarps ? 2 : 1;
+    for (uint32_t i = per * (blockIdx.x * P2M_WARPS + (threadIdx.x >> 5)); i < nocc;
+         i += per * nwarps) {
+        uint2 e[2];
+        uint32_t s0[2], s1[2];
+        range(i, e[0], s0[0], s1[0]);
+        range(per == 2 ? i + 1 : nocc, e[1], s0[1], s1[1]);
+        if (per == 2 && s1[0] - s0[0] <= 16 && s1[1] - s0[1] <= 16) {
+            // a half-warp each
+            const int h = lane >> 4;
+            powers(insts[h ? e[1].x : e[0].x], h ? e[1].y : e[0].y,
+                   (h ? s0[1] : s0[0]) + uint32_t(lane & 15), h ? s1[1] : s1[0]);
+            __syncwarp();
+            const int p0 = insts[e[0].x].p, cols = p0 + insts[e[1].x].p;
+            for (int c = lane; c < cols; c += 32) {
+                const int u = c >= p0, k = u ? c - p0 : c;
+                const uint32_t rows = u ? s1[1] - s0[1] : s1[0] - s0[0];
+                C2 acc = mk2<R>(R(0), R(0));
+                add_rows(acc, k, 16 * u, rows);
+                if (!u || i + 1 < nocc) series(insts[u ? e[1].x : e[0].x], u ? e[1].y : e[0].y)[k] = acc;
+            }
+            __syncwarp();
+            continue;
+        }
+        for (uint32_t u = 0; u < per && i + u < nocc; ++u) {
+            const InstDesc &d = insts[e[u].x];
+            C2 acc0 = mk2<R>(R(0), R(0)), acc1 = acc0;
+            for (uint32_t c0 = s0[u]; c0 < s1[u]; c0 += 32) {
+                const uint32_t rows = min(32u, s1[u] - c0);
+                powers(d, e[u].y, c0 + uint32_t(lane), s1[u]);
+                __syncwarp();
+                if (lane < d.p) add_rows(acc0, lane, 0, rows);
+                if (lane + 32 < d.p) add_rows(acc1, lane + 32, 0, rows);
+                __syncwarp();
+            }
+            C2 *dst = series(d, e[u].y);
+            if (lane < d.p) dst[lane] = acc0;
+            if (lane + 32 < d.p) dst[lane + 32] = acc1;
+        }
     }
 }
 
