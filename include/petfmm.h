@@ -479,7 +479,7 @@ enum {
     PETFMM_OPT_P2P_MODE = 3,   /* order in which persistent P2P warps (FP64 path, and mixed
                                   path with PETFMM_OPT_P2P_PAIRS 0 or 1) take the work
                                   items from their queue: 0 (default) heaviest first by
-                                  the targets x sources cost of Eq. 14, 1 leaf (Morton)
+                                  the targets x sources cost of Eq. 14, 1 about leaf (Morton)
                                   order; the results are identical */
     PETFMM_OPT_POISON = 4,     /* 1: fill the expansion buffers with NaN bytes before each
                                   evaluation (testing: a read of a never-written

@@ -3,9 +3,9 @@
 // One evaluation (Sec. 2.2, Fig. 2) is this sequence of launches on the
 // context's stream, every one of them covering all instances of the batch:
 //   binning -> radix sort (ceil(bits / 8) passes) -> leaf starts -> gather
-//   -> P2M -> M2M (one launch per level, bottom-up) -> M2L (all levels in one
-//   launch) -> L2L (one launch per level, top-down) -> P2P work list
-//   -> P2P + L2P.
+//   -> P2M -> M2M (a launch per level, bottom-up, the top levels in one)
+//   -> M2L (all levels in one launch per kernel) -> L2L (as M2M, top-down)
+//   -> near field (its lists, sums or moments) -> final pass.
 // The host only plans (task tables, offsets) and launches; nothing is read
 // back until petfmm_sync().
 #include <algorithm>
@@ -142,8 +142,8 @@ struct petfmm_ctx {
     int64_t spin_limit = 0;
     uint64_t launches = 0, evaluations = 0;
 
-    DevBuf keysA, keysB, valsA, valsB, hist, scratch, start, xs, ys, gs, rec, me, le, cnt, off,
-        items, ctrl, plan_dev, busy, ucount, recu, occ, items_u, ikA, ikB, ivA, ivB, ihist, own,
+    DevBuf keysA, keysB, valsA, valsB, hist, start, xs, ys, gs, rec, me, le,
+        items, ctrl, plan_dev, busy, ucount, recu, occ, own,
         part, pitems, pxtra, pxs, ustage, smleaf, smlist, smmom, smloc, gtab;
     DevBuf hx, hy, hg, hu, hv;  // device staging for petfmm_evaluate_host
     std::map<int, OpTables> tables;
@@ -746,11 +746,10 @@ uint64_t graph_key(const petfmm_ctx *c, const Plan &pl, int grid) {
     k.put(c->precision); k.put(c->dtype); k.put(c->timing); k.put(c->p2p_mode); k.put(c->poison);
     k.put(c->tc_dense_pct); k.put(c->spin_limit); k.put(c->p2p_pairs); k.put(c->kernel);
     k.put(c->tc_blocks); k.put(c->tc_pipe); k.put(c->overlap);
-    for (const DevBuf *b : {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist, &c->scratch,
-                            &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le, &c->cnt,
-                            &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount,
-                            &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB,
-                            &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs,
+    for (const DevBuf *b : {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist,
+                            &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le,
+                            &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount,
+                            &c->recu, &c->occ, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs,
                             &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc})
         k.put(b->p);
     return k.h;
@@ -813,11 +812,6 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         PF_TRY(ensure(c->me, size_t(pl.ncoef) * sizeof(double2), st));
         PF_TRY(ensure(c->le, size_t(pl.ncoef) * sizeof(double2), st));
     }
-    if (pl.items_any) {
-        PF_TRY(ensure(c->cnt, size_t(pl.nleaves) * 4, st));
-        PF_TRY(ensure(c->off, size_t(pl.nleaves) * 4, st));
-        PF_TRY(ensure(c->scratch, size_t(scan_scratch_words(pl.nleaves)) * 4, st));
-    }
     PF_TRY(ensure(c->occ, size_t(pl.nleaves) * sizeof(uint2), st));
     if (pl.items_any) PF_TRY(ensure(c->items, size_t(pl.items_cap) * sizeof(uint4), st));
     PF_TRY(ensure(c->ucount,
@@ -855,23 +849,6 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         pb.xs = static_cast<float2 *>(c->pxs.p);
         pb.xcap = N;  // scratch of split pairs; more wanted: no pair is split
     }
-    P2POrder order{};
-    if (c->p2p_mode == 0 && pl.items_any) {
-        const size_t cap = size_t(pl.items_cap);
-        PF_TRY(ensure(c->items_u, cap * sizeof(uint4), st));
-        PF_TRY(ensure(c->ikA, cap * 4, st));
-        PF_TRY(ensure(c->ikB, cap * 4, st));
-        PF_TRY(ensure(c->ivA, cap * 4, st));
-        PF_TRY(ensure(c->ivB, cap * 4, st));
-        PF_TRY(ensure(c->ihist, size_t(radix_scratch_words(pl.items_cap)) * 4, st));
-        order.cap = pl.items_cap;
-        order.items_unsorted = static_cast<uint4 *>(c->items_u.p);
-        order.kA = static_cast<uint32_t *>(c->ikA.p);
-        order.kB = static_cast<uint32_t *>(c->ikB.p);
-        order.vA = static_cast<uint32_t *>(c->ivA.p);
-        order.vB = static_cast<uint32_t *>(c->ivB.p);
-        order.hist = static_cast<uint32_t *>(c->ihist.p);
-    }
     const bool lap = c->kernel == KERNEL_LAPLACE;
     const int grid = pl.items_any ? p2p_grid(mixed, pl.deg, pl.general, lap ? 1 : 0) : 0;
     if (pl.items_any && grid <= 0) return PETFMM_EINVAL;
@@ -898,7 +875,6 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     uint32_t *kA = static_cast<uint32_t *>(c->keysA.p), *kB = static_cast<uint32_t *>(c->keysB.p);
     uint32_t *vA = static_cast<uint32_t *>(c->valsA.p), *vB = static_cast<uint32_t *>(c->valsB.p);
     uint32_t *start = static_cast<uint32_t *>(c->start.p);
-    uint32_t *scratch = static_cast<uint32_t *>(c->scratch.p);
     const int f32 = c->dtype == PETFMM_F32;
     uint64_t *lc = &c->launches;
 
@@ -1073,11 +1049,8 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     const int tpi = mixed ? P2P_TPI_MIXED : P2P_TPI_F64;
     if (pl.items_any)
         PF_CUDA(launch_p2p_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count,
-                                    pl.leaves_wl.nblocks, dinst, start, pl.nleaves, tpi,
-                                    static_cast<uint32_t *>(c->cnt.p),
-                                    static_cast<uint32_t *>(c->off.p), scratch,
-                                    static_cast<uint4 *>(c->items.p), ctrl,
-                                    c->p2p_mode == 0 ? &order : nullptr, st, lc));
+                                    pl.leaves_wl.nblocks, dinst, start, tpi, c->p2p_mode == 0,
+                                    static_cast<uint4 *>(c->items.p), pl.items_cap, ctrl, st, lc));
     if (pairs)
         PF_CUDA(launch_pair_worklist(dtask + pl.leaves_wl.first, pl.leaves_wl.count,
                                      pl.leaves_wl.nblocks, dinst, start, c->p2p_mode == 0,
@@ -1272,9 +1245,9 @@ int petfmm_create(const petfmm_domain *dom, int levels, int order, double sigma,
 int petfmm_destroy(petfmm_ctx *c) {
     if (!c) return PETFMM_EINVAL;
     cudaStreamSynchronize(c->stream);
-    DevBuf *bufs[] = {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist, &c->scratch,
-                      &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le, &c->cnt,
-                      &c->off, &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->items_u, &c->ikA, &c->ikB, &c->ivA, &c->ivB, &c->ihist, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->gtab, &c->hx, &c->hy,
+    DevBuf *bufs[] = {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist,
+                      &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le,
+                      &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->gtab, &c->hx, &c->hy,
                       &c->hg, &c->hu, &c->hv};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);

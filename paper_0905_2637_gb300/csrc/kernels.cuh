@@ -35,14 +35,12 @@ cudaError_t exclusive_scan(const uint32_t *in, uint32_t *out, int64_t n, uint32_
 // digits, at most 4 passes, n < 2^32); the initial values are the element
 // indices.  Result ends up in (k0, v0) or (k1, v1): *result_in_first tells
 // which.  scratch: radix_scratch_words(n) words (per-tile digit counts and
-// their scan).  n_live (device, optional): sort only the
-// first min(n, *n_live) elements (the grid stays sized for n; tiles past the
-// live ones return at once).
+// their scan).
 int64_t radix_blocks(int64_t n);
 int64_t radix_scratch_words(int64_t n);
 cudaError_t radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, int64_t n,
                        int nbits, uint32_t *scratch, bool *result_in_first, cudaStream_t st,
-                       uint64_t *launches, const uint32_t *n_live = nullptr);
+                       uint64_t *launches);
 
 // start[soff + b] = first sorted rank of leaf b (b = 0..4^L).
 cudaError_t launch_leaf_start(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
@@ -192,20 +190,11 @@ constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block in the p
 // occupied leaf, tpi targets per item.  ctrl[CTRL_NITEMS] receives the count.
 enum { CTRL_STATUS = 0, CTRL_NITEMS = 1, CTRL_QUEUE = 2, CTRL_PAIRS_LO = 4, CTRL_NOCC = 6,
        CTRL_NPAIRS = 7, CTRL_QUEUE2 = 8, CTRL_NXTRA = 9, CTRL_SYM_LO = 10, CTRL_NSMOOTH = 12,
-       CTRL_CLASSES = 16, CTRL_WORDS = 288 };  // from CTRL_CLASSES: the pair items' classes
-// Buffers for dispatching the items heaviest first (order != nullptr): the
-// items are emitted to items_unsorted, sorted by work class (one stable radix
-// pass over cap entries) and permuted into the item array.
-struct P2POrder {
-    int64_t cap;
-    uint4 *items_unsorted;
-    uint32_t *kA, *kB, *vA, *vB, *hist;  // hist: radix_scratch_words(cap) words
-};
+       CTRL_CLASSES = 16, CTRL_WORDS = 288 };  // from CTRL_CLASSES: the items' work classes
 cudaError_t launch_p2p_worklist(const Task *tasks, int ntasks, int64_t nblocks,
-                                const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                int tpi, uint32_t *cnt, uint32_t *off,
-                                uint32_t *scan_scratch, uint4 *items, uint32_t *ctrl,
-                                const P2POrder *order, cudaStream_t st, uint64_t *launches);
+                                const InstDesc *insts, const uint32_t *start, int tpi, int ordered,
+                                uint4 *items, int64_t cap, uint32_t *ctrl, cudaStream_t st,
+                                uint64_t *launches);
 cudaError_t launch_p2p_f64(int grid, const uint4 *items, uint32_t *ctrl, const InstDesc *insts,
                            const uint32_t *start, const double *xs, const double *ys,
                            const double *gs, const uint32_t *perm, const double2 *le,

@@ -2,8 +2,12 @@
 // leaf and its 8 neighbours with the regularised kernel of Eq. 8, fused with
 // L2P of the leaf's local expansion, written back in the caller's order.
 //
-// Work list.  Every occupied leaf is cut into items of at most TPI targets
-// (one warp per item); an item's cost is (targets) x (sources in the 9
+// Mixed path: a thread per target (k_near_direct) unless the core is wide
+// against the leaf (smooth.cu) or PETFMM_OPT_P2P_PAIRS asks for items (0) or
+// for leaf pairs (1).
+//
+// Work list (FP64, and option 0).  Every occupied leaf is cut into items
+// of at most TPI targets (one warp per item); an item's cost is (targets) x (sources in the 9
 // leaves), the n_nd N_i^2 term of the work estimate of Eq. 14.  Warps of a
 // persistent grid take items from a queue, so equal-cost items of one leaf
 // spread across SMs and the heavy leaves of clustered inputs do not pin one
@@ -25,7 +29,7 @@
 // variant switches to (1 - exp(-q)) / q from the special-function unit above
 // the split.  The self pair has d = 0 and adds exactly zero.
 //
-// FP64 path: the same loop in FP64 (see k_p2p_f64).
+// FP64 path: the same loop in FP64, g from a table (see k_p2p_f64).
 #include <cmath>
 #include <vector>
 
@@ -104,140 +108,133 @@ enum : uint32_t {
     LF_SELF = 4096u     // the leaf's own pairs (slot 8)
 };
 
-__global__ void __launch_bounds__(256) k_p2p_count(const Task *__restrict__ tasks, int ntasks,
-                                                   const InstDesc *__restrict__ insts,
-                                                   const uint32_t *__restrict__ start, int tpi,
-                                                   uint32_t *__restrict__ cnt, uint32_t *ctrl) {
+// The work list takes two launches, both walking every leaf's items in the same
+// way: the first counts the items of each work class, the second puts the
+// items down class after class, heaviest first, their places within a class by
+// atomics (the order of items changes no result).  ordered = 0
+// (PETFMM_OPT_P2P_MODE = 1): one class, about leaf order.  Launches bound it:
+// 10,000 blobs 35 us with a scan and a radix pass, 16 us now.
+constexpr int WORK_CLASSES = 128;
+
+// log2(cost) in quarter steps, heaviest = smallest class
+__device__ __forceinline__ uint32_t work_class(uint32_t cost) {
+    if (cost < 1) cost = 1;
+    const int e = 31 - __clz(int(cost));
+    const uint32_t frac = e >= 2 ? (cost >> (e - 2)) & 3u : (cost << (2 - e)) & 3u;
+    return 127u - (uint32_t(e) * 4u + frac);
+}
+
+// Calls emit(class, item) for every item of leaf m; the leaf's ordered pairs.
+// The class is that of the n_nd N_i^2 term of Eq. 14 (targets x sources):
+// every lane of the warp runs the source loop of its group, target slot filled
+// or not, so the cost is the sources per lane group, ceil(src / S) with S
+// groups.
+template <typename F>
+__device__ __forceinline__ unsigned long long leaf_items(const InstDesc &d, const uint32_t *st,
+                                                         uint32_t m, uint32_t inst, uint32_t tpi,
+                                                         int ordered, F &&emit) {
+    const uint32_t s0 = st[m], n = st[m + 1] - s0;
+    if (!n) return 0;
+    const int nside = 1 << d.L;
+    const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
+    uint32_t src = 0;  // the blobs of the leaf and its neighbours
+    for (int dy = -1; dy <= 1; ++dy)
+        for (int dx = -1; dx <= 1; ++dx) src += leaf_count(st, nside, ix + dx, iy + dy);
+    for (uint32_t f = 0; f < n; f += tpi) {
+        const uint32_t nt = min(n - f, tpi);
+        const int ns = 5 - p2p_group_log2(nt, int(tpi) / 32);  // log2 S
+        emit(ordered ? work_class((src + (1u << ns) - 1) >> ns) : 0u,
+             make_uint4(inst, m, s0 + f, nt));
+    }
+    return (unsigned long long)n * (src - 1);
+}
+
+__global__ void __launch_bounds__(256) k_item_count(const Task *__restrict__ tasks, int ntasks,
+                                                    const InstDesc *__restrict__ insts,
+                                                    const uint32_t *__restrict__ start,
+                                                    uint32_t tpi, int ordered, uint32_t *ctrl) {
+    __shared__ uint32_t hist[WORK_CLASSES];
+    __shared__ unsigned long long sums;
+    for (int i = threadIdx.x; i < WORK_CLASSES; i += 256) hist[i] = 0;
+    if (threadIdx.x == 0) sums = 0;
+    __syncthreads();
     const int ti = find_task(tasks, ntasks, blockIdx.x);
     const Task t = tasks[ti];
     const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
     unsigned long long pairs = 0;
     if (m < t.count) {
         const InstDesc &d = insts[t.inst];
-        const uint32_t *st = start + d.soff;
-        const uint32_t n = st[m + 1] - st[m];
-        const int nside = 1 << d.L;
-        const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
-        cnt[d.loff + m] = (n + tpi - 1) / tpi;
-        if (n) {
-            uint32_t src = 0;
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    const int sx = ix + dx, sy = iy + dy;
-                    if (sx < 0 || sy < 0 || sx >= nside || sy >= nside) continue;
-                    const uint32_t nm = morton_key(uint32_t(sx), uint32_t(sy));
-                    src += st[nm + 1] - st[nm];
-                }
-            pairs = (unsigned long long)n * (src - 1);
-        }
+        pairs = leaf_items(d, start + d.soff, uint32_t(m), uint32_t(t.inst), tpi, ordered,
+                           [&](uint32_t c, const uint4 &) { atomicAdd(&hist[c], 1u); });
     }
-    // block reduction of the ordered pair count (for the statistics)
+    // the ordered pair count, for the statistics
 #pragma unroll
     for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
-    __shared__ unsigned long long ws[8];
-    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = pairs;
+    if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&sums, pairs);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long s = 0;
-        for (int w = 0; w < 8; ++w) s += ws[w];
-        if (s) atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), s);
+    if (threadIdx.x < WORK_CLASSES && hist[threadIdx.x]) {
+        atomicAdd(ctrl + CTRL_CLASSES + threadIdx.x, hist[threadIdx.x]);
+        atomicAdd(ctrl + CTRL_NITEMS, hist[threadIdx.x]);
     }
+    if (threadIdx.x == 0 && sums)
+        atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), sums);
 }
 
-__global__ void __launch_bounds__(256) k_p2p_emit(const Task *__restrict__ tasks, int ntasks,
-                                                  const InstDesc *__restrict__ insts,
-                                                  const uint32_t *__restrict__ start, int tpi,
-                                                  const uint32_t *__restrict__ cnt,
-                                                  const uint32_t *__restrict__ off,
-                                                  uint4 *__restrict__ items,
-                                                  uint32_t *__restrict__ wclass) {
+__global__ void __launch_bounds__(256) k_item_emit(const Task *__restrict__ tasks, int ntasks,
+                                                   const InstDesc *__restrict__ insts,
+                                                   const uint32_t *__restrict__ start,
+                                                   uint32_t tpi, int ordered, uint32_t *ctrl,
+                                                   uint4 *__restrict__ items, int64_t cap) {
+    __shared__ uint32_t hist[WORK_CLASSES], first[WORK_CLASSES];
     const int ti = find_task(tasks, ntasks, blockIdx.x);
     const Task t = tasks[ti];
     const int64_t m = (int64_t(blockIdx.x) - t.block0) * blockDim.x + threadIdx.x;
-    if (m >= t.count) return;
     const InstDesc &d = insts[t.inst];
-    const uint32_t c = cnt[d.loff + m];
-    if (!c) return;
     const uint32_t *st = start + d.soff;
-    const uint32_t s0 = st[m], s1 = st[m + 1];
-    const uint32_t o = off[d.loff + m];
-    // sources of the item: the blobs of the leaf and its neighbours
-    uint32_t src = 0;
-    if (wclass) {
-        const int nside = 1 << d.L;
-        const int ix = int(compact_bits(uint32_t(m))), iy = int(compact_bits(uint32_t(m) >> 1));
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int sx = ix + dx, sy = iy + dy;
-                if (sx < 0 || sy < 0 || sx >= nside || sy >= nside) continue;
-                const uint32_t nm = morton_key(uint32_t(sx), uint32_t(sy));
-                src += st[nm + 1] - st[nm];
-            }
+    if (threadIdx.x < WORK_CLASSES) {
+        hist[threadIdx.x] = 0;
+        first[threadIdx.x] = ctrl[CTRL_CLASSES + threadIdx.x];
     }
-    for (uint32_t i = 0; i < c; ++i) {
-        const uint32_t f = s0 + i * uint32_t(tpi);
-        const uint32_t nt = (s1 - f) < uint32_t(tpi) ? (s1 - f) : uint32_t(tpi);
-        items[o + i] = make_uint4(uint32_t(t.inst), uint32_t(m), f, nt);
-        // work class of the item (Eq. 14, n_nd N_i^2 term: targets x sources).
-        // Every lane of the warp runs the source loop of its group, target
-        // slot filled or not, so the cost is the sources per lane group,
-        // ceil(src / S) with S groups.  Class = log2(cost) in quarter steps,
-        // stored as 127 - class so that an ascending sort is heaviest first.
-        if (wclass) {
-            const int ns = 5 - p2p_group_log2(nt, tpi / 32);  // log2 S
-            const uint32_t cost = (src + (1u << ns) - 1) >> ns;
-            const int e = 31 - __clz(int(cost));  // cost >= 1: the leaf's own blobs
-            const uint32_t frac = e >= 2 ? (cost >> (e - 2)) & 3u : (cost << (2 - e)) & 3u;
-            wclass[o + i] = 127u - (uint32_t(e) * 4u + frac);
-        }
+    __syncthreads();
+    if (m < t.count)
+        leaf_items(d, st, uint32_t(m), uint32_t(t.inst), tpi, ordered,
+                   [&](uint32_t c, const uint4 &) { atomicAdd(&hist[c], 1u); });
+    __syncthreads();
+    // this block's run within each class
+    uint32_t base = 0, n = 0;
+    if (threadIdx.x < WORK_CLASSES && (n = hist[threadIdx.x])) {
+        for (int i = 0; i < int(threadIdx.x); ++i) base += first[i];
+        base += atomicAdd(ctrl + CTRL_CLASSES + WORK_CLASSES + threadIdx.x, n);
     }
-}
-
-// Invalid tail of the item array (beyond the device-side count) sorts last.
-__global__ void __launch_bounds__(256) k_item_permute(const uint4 *__restrict__ in,
-                                                      const uint32_t *__restrict__ perm,
-                                                      uint4 *__restrict__ out, int64_t cap,
-                                                      const uint32_t *count) {
-    const int64_t r = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (r < cap && r < int64_t(*count) && PF_IN(perm[r], cap)) out[r] = in[perm[r]];
-}
-
-// heaviest items first: one stable 8-bit radix pass over the work classes in
-// order->kA, then the items permuted from order->items_unsorted to items
-static cudaError_t order_items(const P2POrder *order, uint4 *items, const uint32_t *count,
-                               uint32_t *scan_scratch, cudaStream_t st, uint64_t *launches) {
-    const int64_t cap = order->cap;
-    const unsigned g = unsigned((cap + 255) / 256);
-    bool in_first = true;
-    cudaError_t e = radix_sort(order->kA, order->vA, order->kB, order->vB, cap, 8, order->hist,
-                               &in_first, st, launches, count);
-    if (e != cudaSuccess) return e;
-    k_item_permute<<<g, 256, 0, st>>>(order->items_unsorted, in_first ? order->vA : order->vB,
-                                      items, cap, count);
-    PF_LAUNCHED(1);
-    return cudaGetLastError();
+    __syncthreads();
+    if (threadIdx.x < WORK_CLASSES) {
+        first[threadIdx.x] = base;
+        hist[threadIdx.x] = 0;
+    }
+    __syncthreads();
+    if (m < t.count)
+        leaf_items(d, st, uint32_t(m), uint32_t(t.inst), tpi, ordered,
+                   [&](uint32_t c, const uint4 &item) {
+                       const uint32_t o = first[c] + atomicAdd(&hist[c], 1u);
+                       if (PF_IN(o, cap)) items[o] = item;
+                   });
 }
 
 cudaError_t launch_p2p_worklist(const Task *tasks, int ntasks, int64_t nblocks,
-                                const InstDesc *insts, const uint32_t *start, int64_t nleaves,
-                                int tpi, uint32_t *cnt, uint32_t *off,
-                                uint32_t *scan_scratch, uint4 *items, uint32_t *ctrl,
-                                const P2POrder *order, cudaStream_t st, uint64_t *launches) {
+                                const InstDesc *insts, const uint32_t *start, int tpi, int ordered,
+                                uint4 *items, int64_t cap, uint32_t *ctrl, cudaStream_t st,
+                                uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
-    k_p2p_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, tpi, cnt, ctrl);
+    k_item_count<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, uint32_t(tpi),
+                                                    ordered, ctrl);
     PF_LAUNCHED(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    e = exclusive_scan(cnt, off, nleaves, scan_scratch, ctrl + CTRL_NITEMS, st, launches);
-    if (e != cudaSuccess) return e;
-    uint4 *emit_to = order ? order->items_unsorted : items;
-    k_p2p_emit<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, tpi, cnt, off, emit_to,
-                                                  order ? order->kA : nullptr);
+    k_item_emit<<<unsigned(nblocks), 256, 0, st>>>(tasks, ntasks, insts, start, uint32_t(tpi),
+                                                   ordered, ctrl, items, cap);
     PF_LAUNCHED(1);
-    if ((e = cudaGetLastError()) != cudaSuccess || !order) return e;
-    return order_items(order, items, ctrl + CTRL_NITEMS, scan_scratch, st, launches);
+    return cudaGetLastError();
 }
-
 
 // ----------------------------------------------------------------------------
 // Mixed-precision P2P + L2P
@@ -654,15 +651,7 @@ __device__ __forceinline__ uint32_t pair_cost(uint32_t nt, uint32_t ns) {
     return c * ((ns & ~31u) + (tail == 0 ? 0u : tail <= 16 ? 16u : 32u));
 }
 
-// work class of an item of `cost` (64-target chunk, 32-source chunk) tiles:
-// heaviest first = smallest class, quarter steps of log2
-__device__ __forceinline__ uint32_t pair_wclass(uint32_t cost) {
-    if (cost < 1) cost = 1;
-    const int e = 31 - __clz(int(cost));
-    const uint32_t frac = e >= 2 ? (cost >> (e - 2)) & 3u : (cost << (2 - e)) & 3u;
-    return 127u - (uint32_t(e) * 4u + frac);
-}
-constexpr int PAIR_CLASSES = 128;
+constexpr int PAIR_CLASSES = WORK_CLASSES;
 
 // The work list takes two launches, both walking every leaf's items in the
 // same way: the first counts the items of each work class (and the scratch
@@ -689,13 +678,13 @@ __device__ __forceinline__ void leaf_pair_items(const InstDesc &d, const uint32_
             // a warp spends 32 steps per (64-target chunk, 32-source chunk)
             const uint32_t nt = min(pc, na - i * pc);
             const uint32_t cls =
-                ordered ? pair_wclass(((nt + 63) / 64) * ((nb + 31) / 32)) : 0u;
+                ordered ? work_class(((nt + 63) / 64) * ((nb + 31) / 32)) : 0u;
             emit(cls, make_uint4(inst, m, uint32_t(k) | (swap << 3) | (i << 4), 0u),
                  i ? 0u : (np - 1) * nb, (unsigned long long)(i ? 0u : na) * nb);
         }
     }
     // the leaf's own pairs (direction 4): half the tiles of the leaf with itself
-    const uint32_t cls = ordered ? pair_wclass(((na + 63) / 64) * ((na + 31) / 32) / 2) : 0u;
+    const uint32_t cls = ordered ? work_class(((na + 63) / 64) * ((na + 31) / 32) / 2) : 0u;
     emit(cls, make_uint4(inst, m, 4u, 0u), 0u, (unsigned long long)na * (na - 1) / 2);
 }
 
@@ -1208,7 +1197,7 @@ __device__ __forceinline__ void pair_item(const uint4 item, const InstDesc *__re
 
 // The pair items of the pairwise mode, heaviest first, in one persistent
 // launch (64 registers for the four targets per lane: 4 CTAs per SM); the
-// directed items of the leaves' own and not-pairwise neighbours follow in
+// leaves' not-pairwise neighbours follow in
 // k_p2p_mixed<.., PAIRS = true> at its higher occupancy.  Measured on GB300,
 // one queue over both kinds of item (the directed ones filling the pairs'
 // tail) was slower: the directed items ran at this kernel's occupancy.

@@ -277,14 +277,6 @@ int64_t radix_scratch_words(int64_t n) {
     return c + scan_scratch_words(c);
 }
 
-// n_live (device, may be null): only the first *n_live of the n elements
-// take part; tiles past them count nothing and move nothing.
-__device__ __forceinline__ int64_t live_count(int64_t n, const uint32_t *n_live) {
-    if (!n_live) return n;
-    const int64_t m = int64_t(*n_live);
-    return m < n ? m : n;
-}
-
 // Exclusive sums of (a, b) over the block's NT threads.
 template <int NT>
 __device__ __forceinline__ void block_exclusive_sum2(uint32_t a, uint32_t b, uint32_t *ea,
@@ -325,7 +317,7 @@ __device__ __forceinline__ void block_exclusive_sum2(uint32_t a, uint32_t b, uin
 // count[d * nblocks + tile]: elements of the tile whose digit
 // (key >> shift) & mask is d (tiles past the live elements count zero).
 __global__ void __launch_bounds__(RC_THREADS) k_radix_counts(const uint32_t *__restrict__ keys,
-                                                             int64_t n, const uint32_t *n_live,
+                                                             int64_t n,
                                                              int shift, uint32_t mask,
                                                              uint32_t *__restrict__ count,
                                                              int64_t nblocks) {
@@ -333,7 +325,6 @@ __global__ void __launch_bounds__(RC_THREADS) k_radix_counts(const uint32_t *__r
     const int tid = threadIdx.x;
     h[tid] = 0;
     __syncthreads();
-    n = live_count(n, n_live);
     const int64_t t0 = int64_t(blockIdx.x) * RS_TILE;
     uint32_t k[RS_TILE / RC_THREADS];
 #pragma unroll
@@ -353,7 +344,7 @@ __global__ void __launch_bounds__(RC_THREADS) k_radix_counts(const uint32_t *__r
 template <bool FIRST>
 __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(
     const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin, uint32_t *__restrict__ kout,
-    uint32_t *__restrict__ vout, int64_t n, const uint32_t *n_live, int shift, uint32_t mask,
+    uint32_t *__restrict__ vout, int64_t n, int shift, uint32_t mask,
     const uint32_t *__restrict__ offs, int64_t nblocks) {
     __shared__ uint16_t wcnt[RS_WARPS][256];  // per-warp digit counts, then warp offsets
     __shared__ uint32_t lstart[256];          // start of each digit's run in the sorted tile
@@ -362,7 +353,6 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(
     __shared__ uint2 wsum[RS_WARPS];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t lt_mask = (1u << lane) - 1u;
-    n = live_count(n, n_live);
     const int64_t t0 = int64_t(blockIdx.x) * RS_TILE;
     if (t0 >= n) return;
     const int64_t tile_n = n - t0 < RS_TILE ? n - t0 : RS_TILE;
@@ -431,7 +421,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3) k_radix_scatter(
 
 cudaError_t radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, int64_t n,
                        int nbits, uint32_t *scratch, bool *result_in_first, cudaStream_t st,
-                       uint64_t *launches, const uint32_t *n_live) {
+                       uint64_t *launches) {
     *result_in_first = true;
     if (n <= 0) return cudaSuccess;
     const int passes = (nbits + 7) / 8;
@@ -445,16 +435,16 @@ cudaError_t radix_sort(uint32_t *k0, uint32_t *v0, uint32_t *k1, uint32_t *v1, i
         const int shift = 8 * pass;
         const int bits = nbits - shift < 8 ? nbits - shift : 8;
         const uint32_t mask = (1u << bits) - 1u;
-        k_radix_counts<<<unsigned(nb), RC_THREADS, 0, st>>>(kin, n, n_live, shift, mask, count, nb);
+        k_radix_counts<<<unsigned(nb), RC_THREADS, 0, st>>>(kin, n, shift, mask, count, nb);
         PF_LAUNCHED(1);
         cudaError_t e = exclusive_scan(count, count, 256 * nb, scan, nullptr, st, launches);
         if (e != cudaSuccess) return e;
         if (pass == 0)
             k_radix_scatter<true><<<unsigned(nb), RS_THREADS, 0, st>>>(
-                kin, vin, kout, vout, n, n_live, shift, mask, count, nb);
+                kin, vin, kout, vout, n, shift, mask, count, nb);
         else
             k_radix_scatter<false><<<unsigned(nb), RS_THREADS, 0, st>>>(
-                kin, vin, kout, vout, n, n_live, shift, mask, count, nb);
+                kin, vin, kout, vout, n, shift, mask, count, nb);
         PF_LAUNCHED(1);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
