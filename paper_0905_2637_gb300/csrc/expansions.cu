@@ -1,7 +1,7 @@
 // expansions.cu -- the upward and downward sweeps of Sec. 2.2 (Fig. 2):
-// P2M, M2M, M2L over the interaction list, L2L.  SIMT kernels, templated on
-// the real type (double for the FP64 path, float for the mixed path's
-// non-tensor stages).
+// P2M, the per-box M2L of the mixed path's sparse units, and the operator
+// tables of all translations (M2M and L2L: shifts.cu; the other M2L kernels:
+// m2l_tc.cu, m2l_orbits.cu).
 //
 // Series (Cauchy kernel; the paper leaves the mathematics to Greengard-
 // Rokhlin, Sec. 2.2).  With z = x + i y, the far field is

@@ -19,9 +19,9 @@
 // cheaper summed directly, by the final pass with one thread per target.
 //
 // Measured on one GB300, the whole evaluation against the pairwise near field
-// (p2p.cu): 16.8M clustered blobs, kappa = 0.12: 18.3 -> 2.7 ms; 4.2M with the
-// copies from and to the host: 5.2 -> 1.3 ms; 765k blobs, one per leaf (direct
-// pairs only, without their work lists): 2.89 -> 2.38 ms then, 1.57 ms now.
+// (p2p.cu): 16.8M clustered blobs, kappa = 0.12: 18.3 -> 2.4 ms; 4.2M with the
+// copies from and to the host: 5.2 -> 1.15 ms; 765k blobs, one per leaf (direct
+// pairs only, without their work lists, with the other steps): 2.89 -> 1.57 ms.
 //
 // kappa <= 1.95 (degree 14) is where the line lies: the degree needed grows
 // with the core's steepness (a translation costs the square of (n + 1)(n + 2)
