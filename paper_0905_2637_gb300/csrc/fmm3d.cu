@@ -461,7 +461,8 @@ cudaError_t launch_p2m_lanes(int p, int L, const Dom3 &d, const uint32_t *start,
 }
 
 // ---------------------------------------------------------------------------
-// M2L of the FP64 path (all levels in one launch).  The coefficients of a
+// M2L by reflection orbits (all levels in one launch): the FP64 path, and the
+// mixed path's small trees.  The coefficients of a
 // real potential with degrees < p are p^2 real numbers (host_m2l_real); in
 // that basis a reflection of an axis is a diagonal of signs, so the operator
 // of delta = (+-a, +-b, +-c) is S T S with the one of (a, b, c) and S the
@@ -471,69 +472,87 @@ cudaError_t launch_p2m_lanes(int p, int L, const Dom3 &d, const uint32_t *start,
 //   H[q][k] = sum_s (-1)^popc(q & s) a_s[k]
 // (q: a coefficient's parity along x, y, z; s: the reflected axes), 56 real
 // p^2 x p^2 products for the up to 189 boxes of the interaction list and
-// three butterfly stages for H.  Bound by the FP64 pipe (two lanes a cycle
+// three butterfly stages for H.  FP64 is bound by its pipe (two lanes a cycle
 // and SM on this part), so the work is laid out to leave no lane idle: a
-// block takes M2L64_ITEMS (target box, coefficient) pairs flat over its
-// threads, four each; operators come through L1, H from shared memory.
-// Measured (one GB300, 262,144 uniform charges, L = 4, p = 8): M2L 76.6 ms with
-// a warp per target box and the complex sums of every source -> 2.45 ms.
+// group of threads takes (target box, coefficient) pairs flat, NI each, and
+// GROUPS groups of a block every GROUPS-th orbit, their sums added at the end
+// in group order; operators come through L1, H from shared memory.
+// Measured (one GB300, 262,144 uniform charges, L = 4, p = 8, FP64): 76.6 ms
+// with a warp per target box and the complex sums of every source -> 2.3 ms;
+// the FP32 sides are at use_orbits3 and launch_m2l_orbits.
 // ---------------------------------------------------------------------------
-constexpr int M2L64_THREADS = 256, M2L64_NI = 4, M2L64_ITEMS = M2L64_THREADS * M2L64_NI;
+constexpr int ORB_THREADS = 256;
 
-// the largest dynamic shared memory of any order (p = 1: 1,024 targets)
-constexpr size_t M2L64_SMEM_MAX = size_t(8) * (M2L64_ITEMS + 2) * 8 + size_t(8) * M2L64_ITEMS * 4;
+// the offsets (|dx| + 4 |dy| + 16 |dz|) of the interaction list
+struct Orbits3 {
+    uint8_t o[56];
+};
+constexpr Orbits3 orbits3() {
+    Orbits3 r{};
+    for (int o = 1, n = 0; o < 64; ++o)
+        if ((o & 3) >= 2 || ((o >> 2) & 3) >= 2 || (o >> 4) >= 2) r.o[n++] = uint8_t(o);
+    return r;
+}
+__constant__ Orbits3 c_orbits = orbits3();
 
-__host__ __device__ __forceinline__ int m2l64_rows(int p) { return M2L64_ITEMS / (p * p); }
+// targets of a block, from the (target, coefficient) pairs of a group
+__host__ __device__ constexpr int orb_items(int ni, int groups) { return ORB_THREADS / groups * ni; }
+__host__ __device__ constexpr int orb_rows(int items, int p) { return items / (p * p); }
 // blocks of level l: ceil(8^(l-1) / rows) x 8 child classes
-__host__ __device__ __forceinline__ int64_t m2l64_blocks(int l, int rows) {
+__host__ __device__ __forceinline__ int64_t orb_blocks(int l, int rows) {
     return ((int64_t(1) << (3 * (l - 1))) + rows - 1) / rows * 8;
 }
-// doubles between the H of two parity classes (two of padding keep the eight
+// values between the H of two parity classes (two of padding keep the eight
 // classes on different banks)
-__host__ __device__ __forceinline__ int m2l64_stride(int p) { return m2l64_rows(p) * p * p + 2; }
+__host__ __device__ constexpr int orb_stride(int rows, int p) { return rows * p * p + 2; }
 
-__global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
-    int L, int p, const uint32_t *__restrict__ start, const double *__restrict__ atab,
+template <typename T, int NI, int GROUPS>
+__global__ void __launch_bounds__(ORB_THREADS) k3_m2l_orbits(
+    int L, int p, const uint32_t *__restrict__ start, const T *__restrict__ atab,
     const short2 *__restrict__ rmap, const uint8_t *__restrict__ parity,
-    const double2 *__restrict__ me, double2 *__restrict__ le) {
-    extern __shared__ __align__(16) double m64_h[];
-    int *srow = reinterpret_cast<int *>(m64_h + 8 * m2l64_stride(p));  // source box of
-                                                                       // (target, member), -1: none
+    const typename C3<T>::V *__restrict__ me, typename C3<T>::V *__restrict__ le) {
+    constexpr int GT = ORB_THREADS / GROUPS;  // threads of a group
+    extern __shared__ __align__(16) unsigned char orb_smem[];
     __shared__ uint8_t sq[P3_MAX * P3_MAX];    // parity class of each real index
     __shared__ uint16_t soff[P3_MAX * P3_MAX]; // its place in a box's stored doubles
-    const int tid = threadIdx.x, nr = p * p, nc = nc3(p);
-    const int rows = m2l64_rows(p), qs = m2l64_stride(p);
+    const int g = int(threadIdx.x) / GT, tid = int(threadIdx.x) % GT;
+    const int nr = p * p, nc = nc3(p);
+    const int rows = orb_rows(orb_items(NI, GROUPS), p), qs = orb_stride(rows, p);
+    T *const hall = reinterpret_cast<T *>(orb_smem), *const hs = hall + g * 8 * qs;
+    // source box of (target, member), -1: none
+    int *const srow = reinterpret_cast<int *>(hall + GROUPS * 8 * qs) + g * 8 * rows;
     int l = 2;
     int64_t bid = blockIdx.x;
-    while (l < L && bid >= m2l64_blocks(l, rows)) bid -= m2l64_blocks(l++, rows);
+    while (l < L && bid >= orb_blocks(l, rows)) bid -= orb_blocks(l++, rows);
     const int c = int(bid & 7);
     const int64_t np = int64_t(1) << (3 * (l - 1)), p0 = (bid >> 3) * rows;
     const int side = 1 << l;
     bool mine = false;
-    for (int t = tid; t < rows; t += M2L64_THREADS)
+    for (int t = tid; t < rows; t += GT)
         if (p0 + t < np) mine |= box_count3(start, L, l, uint32_t((p0 + t) * 8 + c)) != 0;
     if (!__syncthreads_or(mine)) return;  // no target holds particles
-    for (int r = tid; r < nr; r += M2L64_THREADS) {
+    for (int r = threadIdx.x; r < nr; r += ORB_THREADS) {
         sq[r] = parity[r];
         const short2 mp = rmap[r];
         soff[r] = uint16_t(2 * mp.x + (mp.y == 1));
     }
     // this thread's (target, coefficient) pairs
-    int it_r[M2L64_NI], it_t[M2L64_NI], it_q[M2L64_NI];
-    double acc[M2L64_NI];
+    int it_r[NI], it_t[NI], it_q[NI];
+    T acc[NI];
 #pragma unroll
-    for (int i = 0; i < M2L64_NI; ++i) {
-        const int e = tid + i * M2L64_THREADS;
+    for (int i = 0; i < NI; ++i) {
+        const int e = tid + i * GT;
         const bool in = e < rows * nr;
         it_t[i] = in ? e / nr : 0;
         it_r[i] = in ? e % nr : 0;
         it_q[i] = parity[it_r[i]];
-        acc[i] = 0.0;
+        acc[i] = T(0);
     }
-    const double *lev = reinterpret_cast<const double *>(me + lvl_off3(l) * nc);
-    for (int o = 1; o < 64; ++o) {
+    const T *lev = reinterpret_cast<const T *>(me + lvl_off3(l) * nc);
+    static_assert(56 % GROUPS == 0, "orbits per group");
+    for (int step = g; step < 56; step += GROUPS) {
+        const int o = c_orbits.o[step];
         const int a[3] = {o & 3, (o >> 2) & 3, o >> 4};
-        if (a[0] < 2 && a[1] < 2 && a[2] < 2) continue;  // near field
         // axis d: both signs of the offset, or one (0; 3 reaches out of the
         // parent's neighbours on one side); delta = target - source
         bool both[3], neg[3];
@@ -544,7 +563,7 @@ __global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
         }
         __syncthreads();  // the previous orbit's products are done
         bool have = false;
-        for (int e = tid; e < 8 * rows; e += M2L64_THREADS) {
+        for (int e = tid; e < 8 * rows; e += GT) {
             const int s = e & 7, t = e >> 3;
             int src = -1;
             bool member = p0 + t < np;
@@ -565,13 +584,13 @@ __global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
             have |= src >= 0;
         }
         if (!__syncthreads_or(have)) continue;
-        for (int e = tid; e < rows * nr; e += M2L64_THREADS) {
+        for (int e = tid; e < rows * nr; e += GT) {
             const int t = e / nr, k = e - t * nr;
-            double v[8];
+            T v[8];
 #pragma unroll
             for (int s = 0; s < 8; ++s) {
                 const int sb = srow[8 * t + s];
-                v[s] = sb >= 0 ? lev[int64_t(sb) * (2 * nc) + soff[k]] : 0.0;
+                v[s] = sb >= 0 ? lev[int64_t(sb) * (2 * nc) + soff[k]] : T(0);
             }
             // butterflies along the axes with both signs (entries reflected
             // along another axis are not there yet), then copies
@@ -585,7 +604,7 @@ __global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
 #pragma unroll
                         for (int f = 0; f < 3; ++f) there = there && (both[f] || !((s >> f) & 1));
                         if (!there) continue;
-                        const double x = v[s], y = v[s | (1 << d)];
+                        const T x = v[s], y = v[s | (1 << d)];
                         v[s] = x + y;
                         v[s | (1 << d)] = x - y;
                     }
@@ -596,28 +615,84 @@ __global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
                     for (int s = 0; s < 8; ++s)
                         if (!((s >> d) & 1)) v[s | (1 << d)] = neg[d] ? -v[s] : v[s];
 #pragma unroll
-            for (int s = 0; s < 8; ++s) m64_h[s * qs + e] = v[s];
+            for (int s = 0; s < 8; ++s) hs[s * qs + e] = v[s];
         }
         __syncthreads();
-        const double *at = atab + size_t(o) * nr * nr;
-#pragma unroll 2
+        const T *at = atab + size_t(o) * nr * nr;
+#pragma unroll 4
         for (int k = 0; k < nr; ++k) {
             const int qk = sq[k];
 #pragma unroll
-            for (int i = 0; i < M2L64_NI; ++i)
+            for (int i = 0; i < NI; ++i)
                 acc[i] = fma(__ldg(at + size_t(k) * nr + it_r[i]),
-                             m64_h[(it_q[i] ^ qk) * qs + it_t[i] * nr + k], acc[i]);
+                             hs[(it_q[i] ^ qk) * qs + it_t[i] * nr + k], acc[i]);
         }
     }
-    double *lef = reinterpret_cast<double *>(le + lvl_off3(l) * nc);
+    if (GROUPS > 1) {
+        __syncthreads();
+        if (g)
 #pragma unroll
-    for (int i = 0; i < M2L64_NI; ++i) {
-        if (tid + i * M2L64_THREADS >= rows * nr || p0 + it_t[i] >= np) continue;
-        const short2 mp = rmap[it_r[i]];
-        double *dst = lef + ((p0 + it_t[i]) * 8 + c) * (2 * nc) + 2 * mp.x;
-        dst[mp.y == 1] = acc[i];
-        if (mp.y == 2) dst[1] = 0.0;  // Im of m = 0
+            for (int i = 0; i < NI; ++i) hall[((g - 1) * NI + i) * GT + tid] = acc[i];
+        __syncthreads();
+        if (g) return;
+        for (int k = 0; k + 1 < GROUPS; ++k)
+#pragma unroll
+            for (int i = 0; i < NI; ++i) acc[i] += hall[(k * NI + i) * GT + tid];
     }
+    T *lef = reinterpret_cast<T *>(le + lvl_off3(l) * nc);
+#pragma unroll
+    for (int i = 0; i < NI; ++i) {
+        if (tid + i * GT >= rows * nr || p0 + it_t[i] >= np) continue;
+        const short2 mp = rmap[it_r[i]];
+        T *dst = lef + ((p0 + it_t[i]) * 8 + c) * (2 * nc) + 2 * mp.x;
+        dst[mp.y == 1] = acc[i];
+        if (mp.y == 2) dst[1] = T(0);  // Im of m = 0
+    }
+}
+
+template <typename T, int NI, int GROUPS>
+cudaError_t launch_orbits3(int L, int p, const uint32_t *start, const T *atab, const short2 *rmap,
+                           const uint8_t *parity, const typename C3<T>::V *me,
+                           typename C3<T>::V *le, cudaStream_t st) {
+    const int rows = orb_rows(orb_items(NI, GROUPS), p);
+    const size_t smem = GROUPS * (size_t(8) * orb_stride(rows, p) * sizeof(T) +
+                                  size_t(8) * rows * sizeof(int));
+    cudaError_t e = cudaFuncSetAttribute(k3_m2l_orbits<T, NI, GROUPS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    if (e != cudaSuccess) return e;
+    int64_t grid = 0;
+    for (int k = 2; k <= L; ++k) grid += orb_blocks(k, rows);
+    k3_m2l_orbits<T, NI, GROUPS><<<unsigned(grid), ORB_THREADS, smem, st>>>(L, p, start, atab, rmap,
+                                                                            parity, me, le);
+    return cudaGetLastError();
+}
+
+// NI and GROUPS by size: four groups of orbits shorten the serial chain, small
+// runs of targets make more blocks; runs of 1,024 pairs (one group) reuse the
+// operators best.  M2L of one GB300, us, <4,1> / <2,4> / <1,4>:
+//   FP64  L = 2, p = 6   954 / 131 / 84      FP32  443 / 55 / 45
+//         L = 3, p = 8   1421 / 320 / 324          713 / 90 / 94
+//         L = 4, p = 8   2459 / 2305 / 2241        899 / 549 / 545
+// and above the 128 pairs that <2,4> holds, <4,1> / <4,4>: FP64 L = 4, p = 11
+// 8258 / 7618, FP32 L = 4, p = 12 2845 / 4434.
+template <typename T>
+cudaError_t launch_m2l_orbits(int L, int p, const uint32_t *start, const T *atab,
+                              const short2 *rmap, const uint8_t *parity,
+                              const typename C3<T>::V *me, typename C3<T>::V *le,
+                              cudaStream_t st) {
+    const int64_t sms = device_sm_count();
+    auto blocks = [&](int ni, int groups) {
+        int64_t n = 0;
+        for (int k = 2; k <= L; ++k) n += orb_blocks(k, orb_rows(orb_items(ni, groups), p));
+        return n;
+    };
+    if (p <= 8 && blocks(2, 4) < sms)
+        return launch_orbits3<T, 1, 4>(L, p, start, atab, rmap, parity, me, le, st);
+    if (p <= 11 && (sizeof(T) == 8 || p <= 8))
+        return launch_orbits3<T, 2, 4>(L, p, start, atab, rmap, parity, me, le, st);
+    if (sizeof(T) == 8 || blocks(4, 1) < 2 * sms)
+        return launch_orbits3<T, 4, 4>(L, p, start, atab, rmap, parity, me, le, st);
+    return launch_orbits3<T, 4, 1>(L, p, start, atab, rmap, parity, me, le, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -627,163 +702,15 @@ __global__ void __launch_bounds__(M2L64_THREADS) k3_m2l_f64(
 // translation is a fixed real p^2 x p^2 matrix A_delta (built on the host in
 // FP64 from the M2L sum, rounded to FP32; stored transposed, k-major, padded
 // to NRP = p^2 rounded up to 32); rmap[r] = (coefficient, part) of real index
-// r, part 0 = Re, 1 = Im, 2 = Re of an m = 0 coefficient (its Im is zero).  A block takes 64 consecutive parent cells
-// (Morton order) of level l - 1 and one target child class c: 64 target rows.
-// For each (source class cs, parent offset d) of the interaction list of
-// class c (delta = c - cs - 2d, |delta|_inf >= 2), the 64 source rows (parent
-// P + d, class cs; zero when outside the domain or empty) are staged k-major
-// in shared memory and multiplied by A_delta in K chunks of 32: every thread
-// owns 4 rows x NRP / 8 columns, reading its 4 rows with one 16-byte load and
-// its columns with 16-byte loads (conflict-free: a warp spans 4 row groups x
-// 8 column groups).  Sums in a fixed order; the result is written, the L2L
-// that follows adds the parent's part.
+// r, part 0 = Re, 1 = Im, 2 = Re of an m = 0 coefficient (its Im is zero).
+// (p <= 8: above, and on small trees, M2L goes by orbits.)
 // ---------------------------------------------------------------------------
-constexpr int MG_ROWS = 64, MG_THREADS = 128, MG_XS = MG_ROWS + 4;
+constexpr int MG_THREADS = 128;
 #ifndef MG_PIPE_ROWS
 #define MG_PIPE_ROWS 128  // target rows per block of the pipelined M2L (64 or 128)
 #endif
 
 __host__ __device__ constexpr int mg_nrp(int p) { return (p * p + 31) / 32 * 32; }
-// K chunk of A staged at once: all of it up to 64 rows, else 64 or 32 rows,
-// whichever divides NRP (so no chunk reads past its operator)
-__host__ __device__ constexpr int mg_kt(int p) {
-    return mg_nrp(p) <= 64 ? mg_nrp(p) : (mg_nrp(p) % 64 == 0 ? 64 : 32);
-}
-
-template <int P>
-__global__ void __launch_bounds__(MG_THREADS) k3_m2l_gemm(int l, int L, const uint32_t *__restrict__ start,
-                                                        const float *__restrict__ atab,
-                                                        const short2 *__restrict__ rmap,
-                                                        const float2 *__restrict__ me,
-                                                        float2 *__restrict__ le) {
-    constexpr int NC = P * (P + 1) / 2, NR = P * P, NRP = mg_nrp(P), CG = NRP / 8;
-    constexpr int KT = mg_kt(P);
-    static_assert(NRP % KT == 0 && KT % 4 == 0 && CG % 4 == 0, "chunking");
-    constexpr int NLOAD = (MG_ROWS * NC + MG_THREADS - 1) / MG_THREADS;
-    extern __shared__ __align__(16) float mg_smem[];
-    float *xs = mg_smem;                 // [NRP][MG_XS]: X^T, k-major
-    float *as = xs + NRP * MG_XS;        // [KT][NRP]: a K chunk of A^T
-    __shared__ int srow[MG_ROWS];
-    __shared__ short imr[NC];            // real index of Im of coefficient j (m > 0), else -1
-    const int tid = threadIdx.x, rg = tid >> 3, g = tid & 7;
-    const int c = int(blockIdx.x & 7);
-    const int64_t np = int64_t(1) << (3 * (l - 1));  // parent cells of level l - 1
-    const int64_t p0 = int64_t(blockIdx.x >> 3) * MG_ROWS;
-    const int pside = 1 << (l - 1);
-    for (int i = tid; i < (NRP - NR) * MG_XS; i += MG_THREADS) xs[NR * MG_XS + i] = 0.f;
-    for (int j = tid; j < NC; j += MG_THREADS) {
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= j) ++n;
-        // the m > 0 coefficients before j, in order: j - n - 1
-        imr[j] = short(j == n * (n + 1) / 2 ? -1 : NC + j - n - 1);
-    }
-    float acc[4][CG];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < CG; ++j) acc[i][j] = 0.f;
-    const float2 *lev = me + lvl_off3(l) * NC;
-    for (int cs = 0; cs < 8; ++cs)
-        for (int dz = -1; dz <= 1; ++dz)
-            for (int dy = -1; dy <= 1; ++dy)
-                for (int dx = -1; dx <= 1; ++dx) {
-                    // delta = target - source, in box widths
-                    const int ex = (c & 1) - (cs & 1) - 2 * dx;
-                    const int ey = ((c >> 1) & 1) - ((cs >> 1) & 1) - 2 * dy;
-                    const int ez = (c >> 2) - (cs >> 2) - 2 * dz;
-                    if (ex >= -1 && ex <= 1 && ey >= -1 && ey <= 1 && ez >= -1 && ez <= 1)
-                        continue;  // near field
-                    // source rows (the barrier also ends the previous offset's reads)
-                    bool have = false;
-                    if (tid < MG_ROWS) {
-                        int sb = -1;
-                        const int64_t pc = p0 + tid;
-                        if (pc < np) {
-                            const int qx = int(compact3(uint32_t(pc))) + dx,
-                                      qy = int(compact3(uint32_t(pc) >> 1)) + dy,
-                                      qz = int(compact3(uint32_t(pc) >> 2)) + dz;
-                            if (qx >= 0 && qy >= 0 && qz >= 0 && qx < pside && qy < pside &&
-                                qz < pside) {
-                                const uint32_t b = morton3(uint32_t(qx), uint32_t(qy), uint32_t(qz)) *
-                                                       8u + uint32_t(cs);
-                                if (box_count3(start, L, l, b)) sb = int(b);
-                            }
-                        }
-                        srow[tid] = sb;
-                        have = sb >= 0;
-                    }
-                    if (!__syncthreads_or(have)) continue;
-                    {
-                        // every load of the rows in flight at once, then the
-                        // k-major scatter (Re to row j, Im to row imr[j])
-                        float2 v[NLOAD];
-#pragma unroll
-                        for (int u = 0; u < NLOAD; ++u) {
-                            const int i = tid + u * MG_THREADS;
-                            v[u] = make_float2(0.f, 0.f);
-                            if (i < MG_ROWS * NC) {
-                                const int sb = srow[i / NC];
-                                if (sb >= 0) v[u] = lev[int64_t(sb) * NC + i % NC];
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < NLOAD; ++u) {
-                            const int i = tid + u * MG_THREADS;
-                            if (i < MG_ROWS * NC) {
-                                const int row = i / NC, j = i % NC;
-                                xs[j * MG_XS + row] = v[u].x;
-                                if (imr[j] >= 0) xs[imr[j] * MG_XS + row] = v[u].y;
-                            }
-                        }
-                    }
-                    const float *at = atab + size_t((ex + 3) + 7 * (ey + 3) + 49 * (ez + 3)) * NRP * NRP;
-                    for (int k0 = 0; k0 < NRP; k0 += KT) {
-                        __syncthreads();
-#pragma unroll
-                        for (int u = 0; u < (KT * NRP / 4 + MG_THREADS - 1) / MG_THREADS; ++u) {
-                            const int i = tid + u * MG_THREADS;
-                            if (i < KT * NRP / 4)
-                                reinterpret_cast<float4 *>(as)[i] =
-                                    __ldg(reinterpret_cast<const float4 *>(at + size_t(k0) * NRP) + i);
-                        }
-                        __syncthreads();
-#pragma unroll 4
-                        for (int kk = 0; kk < KT; ++kk) {
-                            const float4 x4 = *reinterpret_cast<const float4 *>(
-                                xs + (k0 + kk) * MG_XS + 4 * rg);
-                            const float *ar = as + kk * NRP + g * CG;
-#pragma unroll
-                            for (int j4 = 0; j4 < CG; j4 += 4) {
-                                const float4 a4 = *reinterpret_cast<const float4 *>(ar + j4);
-                                const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-                                for (int t = 0; t < 4; ++t) {
-                                    acc[0][j4 + t] = fmaf(x4.x, av[t], acc[0][j4 + t]);
-                                    acc[1][j4 + t] = fmaf(x4.y, av[t], acc[1][j4 + t]);
-                                    acc[2][j4 + t] = fmaf(x4.z, av[t], acc[2][j4 + t]);
-                                    acc[3][j4 + t] = fmaf(x4.w, av[t], acc[3][j4 + t]);
-                                }
-                            }
-                        }
-                    }
-                }
-    float *lef = reinterpret_cast<float *>(le + lvl_off3(l) * NC);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t pc = p0 + 4 * rg + i;
-        if (pc >= np) continue;
-        const int64_t box = pc * 8 + c;
-#pragma unroll
-        for (int j = 0; j < CG; ++j) {
-            const int r = g * CG + j;
-            if (r >= NR) continue;
-            const short2 mp = rmap[r];
-            lef[(box * NC + mp.x) * 2 + (mp.y == 1)] = acc[i][j];
-            if (mp.y == 2) lef[(box * NC + mp.x) * 2 + 1] = 0.f;  // Im of m = 0
-        }
-    }
-}
-
 // The same GEMMs with the operands of the next offset in flight: for p <= 8
 // (a whole operator is one K chunk) the operator and the source rows of
 // offset i + 1 are copied with cp.async (16-byte chunks; 8 when a box's
@@ -2766,11 +2693,11 @@ struct petfmm3d_ctx {
     DevBuf3 pitems, slots, nown, nflags, nctrl;
     bool no_pairs = false;  // no room for the parts of pairwise sums
     // operator tables of the context's precision only
-    DevBuf3 atab32, atab64, rmap, parity;
+    DevBuf3 orbits, atab32, rmap, parity;  // M2L operators: by orbit, by offset
     DevBuf3 shift, order;  // the M2M and L2L operators of octant 0, rows by parity class
     Shift3 sh{};
     DevBuf3 tcimg;  // p <= 8: TF32 hi / lo images of the M2L operators (tensor-core M2L)
-    bool m2l_tc = true;  // PETFMM3D_OPT_M2L_TC
+    int m2l_tc = 2;  // PETFMM3D_OPT_M2L_TC
     bool timing = false, ev_recorded = false;
     cudaEvent_t ev[PETFMM3D_STAGE_COUNT + 1] = {};
     uint64_t launches = 0, evaluations = 0;
@@ -2788,6 +2715,16 @@ constexpr size_t kPairs3MaxBytes = (size_t(1) << 26) * P3_SLOTS * sizeof(float4)
 #define P3_TRY(x) do { int rc_ = (x); if (rc_) return rc_; } while (0)
 #define P3_CUDA(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { cudaGetLastError(); \
     return e_ == cudaErrorMemoryAllocation ? PETFMM_ENOMEM : PETFMM_ECUDA; } } while (0)
+
+// M2L by reflection orbits: FP64, p > 8, and by default the mixed path's trees
+// of up to four levels, where the tensor-core kernel waits on its serial chain
+// of offsets (us, tensor cores / orbits: L = 3, p = 8 653 / 90; L = 4, p = 8
+// 733 / 549, p = 5 496 / 170; L = 5, p = 8 799 / 4132, p = 5 518 / 983).  p > 8,
+// against a SIMT GEMM over every offset: L = 4, p = 12 7.87 / 2.84 ms, L = 5,
+// p = 16 181 / 51 ms.
+bool use_orbits3(const petfmm3d_ctx *c) {
+    return c->precision == PETFMM_FP64 || c->p > TC3_MAXP || (c->m2l_tc == 2 && c->L <= 4);
+}
 
 int upload_tables(petfmm3d_ctx *c) {
     const int p = c->p, nc = nc3(p), nci = nci3(p);
@@ -2837,27 +2774,28 @@ int upload_tables(petfmm3d_ctx *c) {
     P3_CUDA(cudaMemcpy(c->order.p, order.data(), order.size() * sizeof(uint16_t),
                        cudaMemcpyHostToDevice));
     std::vector<cd> iv(static_cast<size_t>(nci));
-    if (c->precision == PETFMM_FP64) {
-        // [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
-        std::vector<double> at(size_t(64) * nr * nr, 0.0);
-        for (int o = 0; o < 64; ++o) {
-            const int dx = o & 3, dy = (o >> 2) & 3, dz = o >> 4;
-            if (dx < 2 && dy < 2 && dz < 2) continue;
-            host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
-            host_m2l_real(p, iv.data(), at.data() + size_t(o) * nr * nr);
-        }
-        P3_TRY(ensure3(c->atab64, at.size() * sizeof(double), c->stream));
-        P3_CUDA(cudaMemcpy(c->atab64.p, at.data(), at.size() * sizeof(double), cudaMemcpyHostToDevice));
-        return PETFMM_OK;
+    // the orbits' operators [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
+    std::vector<double> orb(size_t(64) * nr * nr, 0.0);
+    for (int o = 0; o < 64; ++o) {
+        const int dx = o & 3, dy = (o >> 2) & 3, dz = o >> 4;
+        if (dx < 2 && dy < 2 && dz < 2) continue;
+        host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
+        host_m2l_real(p, iv.data(), orb.data() + size_t(o) * nr * nr);
     }
+    if (use_orbits3(c)) {
+        const std::vector<float> orb32(orb.begin(), orb.end());
+        P3_TRY(ensure3(c->orbits, orb.size() * es, c->stream));
+        P3_CUDA(cudaMemcpy(c->orbits.p, f64 ? static_cast<const void *>(orb.data()) : orb32.data(),
+                           orb.size() * es, cudaMemcpyHostToDevice));
+    }
+    if (f64 || p > TC3_MAXP) return PETFMM_OK;
     // The mixed path's M2L matrices, FP32: ap[k_in * nrp + r_out]; for p <= 8
     // also their TF32 hi / lo images for the tensor cores:
     // [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero padding), K in the
     // input basis of the tensor-core M2L (coefficient by coefficient: Re, then
     // Im if m > 0), N in the M2L matrices' basis.
-    const bool tc = p <= TC3_MAXP;
     std::vector<float> at(size_t(NSLOT3) * nrp * nrp, 0.f);
-    std::vector<float> img(tc ? size_t(NSLOT3) * 2 * nrp * nrp : 0, 0.f);
+    std::vector<float> img(size_t(NSLOT3) * 2 * nrp * nrp, 0.f);
     std::vector<int> tc3_kin(static_cast<size_t>(nr));
     for (int n = 0, k = 0, t = 0; n < p; ++n)
         for (int m = 0; m <= n; ++m) {
@@ -2868,12 +2806,19 @@ int upload_tables(petfmm3d_ctx *c) {
     for (int slot = 0; slot < NSLOT3; ++slot) {
         const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
         if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
-        host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
-        host_m2l_real(p, iv.data(), a64.data());
+        // its orbit's operator between the signs of the reflected axes
+        const int o = std::abs(dx) + 4 * std::abs(dy) + 16 * std::abs(dz);
+        const double *ao = orb.data() + size_t(o) * nr * nr;
+        const int refl = (dx < 0) | (dy < 0) << 1 | (dz < 0) << 2;
+        for (int k = 0; k < nr; ++k)
+            for (int r = 0; r < nr; ++r) {
+                const double v = ao[size_t(k) * nr + r];
+                const bool odd = __builtin_popcount((par[size_t(k)] ^ par[size_t(r)]) & refl) & 1;
+                a64[size_t(k) * nr + r] = odd ? -v : v;
+            }
         float *ap = at.data() + size_t(slot) * nrp * nrp;
         for (int k = 0; k < nr; ++k)
             for (int r = 0; r < nr; ++r) ap[size_t(k) * nrp + r] = float(a64[size_t(k) * nr + r]);
-        if (!tc) continue;
         float *hi = img.data() + size_t(slot) * 2 * nrp * nrp, *lo = hi + size_t(nrp) * nrp;
         for (int k = 0; k < nr; ++k) {
             const int kin = tc3_kin[size_t(k)];
@@ -2886,10 +2831,8 @@ int upload_tables(petfmm3d_ctx *c) {
             }
         }
     }
-    if (tc) {
-        P3_TRY(ensure3(c->tcimg, img.size() * sizeof(float), c->stream));
-        P3_CUDA(cudaMemcpy(c->tcimg.p, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
-    }
+    P3_TRY(ensure3(c->tcimg, img.size() * sizeof(float), c->stream));
+    P3_CUDA(cudaMemcpy(c->tcimg.p, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
     P3_TRY(ensure3(c->atab32, at.size() * sizeof(float), c->stream));
     P3_CUDA(cudaMemcpy(c->atab32.p, at.data(), at.size() * sizeof(float), cudaMemcpyHostToDevice));
     return PETFMM_OK;
@@ -2920,36 +2863,20 @@ void mark3(petfmm3d_ctx *c, int s) {
 unsigned grid_w(int64_t warps) { return unsigned((warps + W3 - 1) / W3); }
 
 template <int P>
-cudaError_t m2l_gemm_p(int l, int L, const uint32_t *start, const float *atab, const short2 *rmap,
-                       const float2 *me, float2 *le, cudaStream_t st) {
-    if constexpr (mg_nrp(P) <= 64) {
-        constexpr int R = MG_PIPE_ROWS;
-        constexpr size_t smem = mgp_smem_bytes<P, R>();
-        static bool pattr = false;
-        if (!pattr) {
-            cudaError_t e = cudaFuncSetAttribute(k3_m2l_pipe<P, R>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 int(smem));
-            if (e != cudaSuccess) return e;
-            pattr = true;
-        }
-        if (l != L) return cudaSuccess;  // one launch covers levels 2..L
-        int64_t grid = 0;
-        for (int k = 2; k <= L; ++k) grid += mg_blocks(k, R);
-        k3_m2l_pipe<P, R><<<unsigned(grid), MG_THREADS, smem, st>>>(L, start, atab, me, le);
-        return cudaGetLastError();
-    }
-    const size_t smem = size_t(mg_nrp(P) * MG_XS + mg_kt(P) * mg_nrp(P)) * sizeof(float);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k3_m2l_gemm<P>,
+cudaError_t m2l_gemm_p(int L, const uint32_t *start, const float *atab, const float2 *me,
+                       float2 *le, cudaStream_t st) {
+    constexpr int R = MG_PIPE_ROWS;
+    constexpr size_t smem = mgp_smem_bytes<P, R>();
+    static bool pattr = false;
+    if (!pattr) {
+        cudaError_t e = cudaFuncSetAttribute(k3_m2l_pipe<P, R>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
         if (e != cudaSuccess) return e;
-        attr = true;
+        pattr = true;
     }
-    const int64_t np = int64_t(1) << (3 * (l - 1));
-    const unsigned grid = unsigned((np + MG_ROWS - 1) / MG_ROWS * 8);
-    k3_m2l_gemm<P><<<grid, MG_THREADS, smem, st>>>(l, L, start, atab, rmap, me, le);
+    int64_t grid = 0;
+    for (int k = 2; k <= L; ++k) grid += mg_blocks(k, R);
+    k3_m2l_pipe<P, R><<<unsigned(grid), MG_THREADS, smem, st>>>(L, start, atab, me, le);
     return cudaGetLastError();
 }
 
@@ -2987,13 +2914,12 @@ cudaError_t launch_m2l_tc3(int p, int L, const uint32_t *start, const float *bim
     }
 }
 
-cudaError_t launch_m2l_gemm(int p, int l, int L, const uint32_t *start, const float *atab,
-                            const short2 *rmap, const float2 *me, float2 *le, cudaStream_t st) {
+// all levels 2..L in one launch, p <= 8
+cudaError_t launch_m2l_gemm(int p, int L, const uint32_t *start, const float *atab,
+                            const float2 *me, float2 *le, cudaStream_t st) {
     switch (p) {
-#define MG_CASE(P) case P: return m2l_gemm_p<P>(l, L, start, atab, rmap, me, le, st);
+#define MG_CASE(P) case P: return m2l_gemm_p<P>(L, start, atab, me, le, st);
         MG_CASE(1) MG_CASE(2) MG_CASE(3) MG_CASE(4) MG_CASE(5) MG_CASE(6) MG_CASE(7) MG_CASE(8)
-        MG_CASE(9) MG_CASE(10) MG_CASE(11) MG_CASE(12) MG_CASE(13) MG_CASE(14) MG_CASE(15)
-        MG_CASE(16)
 #undef MG_CASE
         default: return cudaErrorInvalidValue;
     }
@@ -3025,37 +2951,17 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
         c->launches++;
     }
     mark3(c, PETFMM3D_STAGE_M2L);
-    // one launch for all levels: the FP64 path, and the mixed path with
-    // p <= 8 (launch_m2l_gemm launches at l = L)
-    const bool one = sizeof(T) == 8 || mg_nrp(p) <= 64;
-    // mixed path, p <= 8, PETFMM3D_OPT_M2L_TC: all levels on the tensor cores
-    const bool tc = sizeof(T) == 4 && c->m2l_tc && p <= TC3_MAXP;
-    if constexpr (sizeof(T) == 4) {
-        if (tc) {
+    if (use_orbits3(c)) {
+        P3_CUDA(launch_m2l_orbits<T>(L, p, start, static_cast<const T *>(c->orbits.p), rmap, par, me,
+                                     le, st));
+    } else if constexpr (sizeof(T) == 4) {
+        if (c->m2l_tc)
             P3_CUDA(launch_m2l_tc3(p, L, start, static_cast<const float *>(c->tcimg.p), me, le,
                                    static_cast<int *>(c->status.p), st));
-            c->launches++;
-        }
+        else
+            P3_CUDA(launch_m2l_gemm(p, L, start, static_cast<const float *>(c->atab32.p), me, le, st));
     }
-    for (int l = tc ? L + 1 : one ? L : 2; l <= L; ++l) {
-        if constexpr (sizeof(T) == 4) {
-            P3_CUDA(launch_m2l_gemm(p, l, L, start, static_cast<const float *>(c->atab32.p),
-                                    static_cast<const short2 *>(c->rmap.p), me, le, st));
-        } else {
-            const size_t smem = size_t(8) * m2l64_stride(p) * sizeof(double) +
-                                size_t(8) * m2l64_rows(p) * sizeof(int);
-            P3_CUDA(cudaFuncSetAttribute(k3_m2l_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(M2L64_SMEM_MAX)));
-            int64_t grid = 0;
-            for (int k = 2; k <= L; ++k) grid += m2l64_blocks(k, m2l64_rows(p));
-            k3_m2l_f64<<<unsigned(grid), M2L64_THREADS, smem, st>>>(
-                L, p, start, static_cast<const double *>(c->atab64.p),
-                static_cast<const short2 *>(c->rmap.p), static_cast<const uint8_t *>(c->parity.p),
-                me, le);
-        }
-        P3_CUDA(cudaGetLastError());
-        c->launches++;
-    }
+    c->launches++;
     mark3(c, PETFMM3D_STAGE_L2L);
     for (int l = 2; l < L; ++l) {
         P3_CUDA((launch_shift3<T, true>(l, L, c->sh, start, op + size_t(c->sh.nr) * c->sh.nr, rmap,
@@ -3332,7 +3238,7 @@ int petfmm3d_set_option(petfmm3d_ctx *c, int option, int64_t value) {
         case PETFMM3D_OPT_TIMING: c->timing = value != 0; return PETFMM_OK;
         case PETFMM3D_OPT_M2L_TC:
             if (value != 0 && value != 1) return PETFMM_EINVAL;
-            c->m2l_tc = value != 0;
+            c->m2l_tc = value == 2 ? 2 : value != 0;
             return PETFMM_OK;
         default: return PETFMM_EINVAL;
     }
@@ -3401,7 +3307,7 @@ int petfmm3d_destroy(petfmm3d_ctx *c) {
                        &c->nown, &c->nflags, &c->nctrl,
                        &c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->sortw, &c->start,
                        &c->recu,  &c->rec,   &c->xs,    &c->me,    &c->le,    &c->status,
-                       &c->atab32, &c->atab64, &c->parity, &c->rmap,
+                       &c->orbits, &c->atab32, &c->parity, &c->rmap,
                        &c->shift, &c->order, &c->tcimg};
     for (DevBuf3 *b : bufs)
         if (b->p) cudaFree(b->p);

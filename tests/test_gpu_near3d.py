@@ -82,3 +82,23 @@ def test_fp64_leaf_counts(seed, dtype):
         p = np.where(same, 0.0, q[None, :] / np.sqrt(r2))
         for a, t in zip(got, [p] + [p / r2 * a for a in d]):
             assert np.all(np.abs(a[i] - t.sum(1)) <= tol * np.abs(t).sum(1) + 1e-30)
+
+
+# M2L by reflection orbits, at the orders where the split over a block changes
+# (one or several targets a group, 64, 128, 256 and 1,024 pairs), against the
+# tensor-core kernel and the FP64 path: the mixed path's bar.
+@pytest.mark.parametrize("L,p", [(2, 1), (2, 4), (2, 8), (3, 3), (3, 7), (3, 8), (4, 5), (2, 9),
+                                 (3, 11), (3, 12), (4, 12), (3, 16)])
+def test_orbit_m2l(L, p):
+    from paper_0905_2637_gb300 import fmm3d
+    w = W.tiny3d(6000 * 4 ** (L - 2), 50 + p, L=L, p=p, dtype="f32", clustered_frac=0.3)
+    rc, got = T._run(w, "mixed")
+    assert rc == 0
+    rc, ref = T._run(w, "fp64")
+    assert rc == 0
+    assert T._rel(got[0], ref[0]) <= 1e-5 and T._field_rel(got, ref) <= 1e-5
+    ctx = T._ctx(w, "mixed")
+    ctx.set_option(fmm3d.PETFMM3D_OPT_M2L_TC, 1)
+    rc, tc = T._run(w, "mixed", ctx)
+    ctx.close()
+    assert rc == 0 and T._field_rel(got, tc) <= 1e-5
