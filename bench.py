@@ -144,6 +144,16 @@ def _p2p_traffic(kernel):
     return float(m.group(1))
 
 
+def _smooth_terms(w):
+    """Terms of the smooth near field's expansions (0: summed pair by pair):
+    kappa = w^2 / (2 sigma^2) of a leaf sets the degree."""
+    kappa = (w.domain[2] / 2 ** w.L / w.sigma) ** 2 / 2
+    for bound, degree in ((0.17, 8), (0.50, 10), (1.04, 12), (1.95, 14)):
+        if kappa <= bound:
+            return (degree + 1) * (degree + 2) // 2
+    return 0
+
+
 def _hbm_traffic():
     """DRAM bytes per evaluation of each bandwidth-bound step from the
     committed ncu summary: lines ``traffic[<step>]: <bytes> sources <file>:<sha16>
@@ -518,10 +528,11 @@ def threed_leg(torch, stream, steps=5, tf32_flops=None):
                                      "microbenchmark (petfmm_measure_peaks); frac_of_fp32_fma "
                                      "against 152 SMs x 128 lanes x 2 x 2070 MHz, the SIMT "
                                      "kernel's bound"},
-            "near_roofline": {"bound": "fp32", "achieved": 13 * near_pairs / near_s,
+            "near_roofline": {"bound": "fp32", "achieved": 9 * near_pairs / near_s,
                               "peak": fp32_ops, "unit": "ops/s",
-                              "frac": 13 * near_pairs / near_s / fp32_ops,
-                              "note": "13 FP32 operations per ordered pair against 152 x 128 x "
+                              "frac": 9 * near_pairs / near_s / fp32_ops,
+                              "note": "18 FP32 operations per unordered pair (k3_pairs: both "
+                                      "charges served), 9 per ordered pair, against 152 x 128 x "
                                       "2070 MHz; the stage includes L2P and the output"},
             "data": "synthetic: x, y, z ~ U(0,1), q ~ U(-1,1)/N, seed 1, fp32 storage"}
 
@@ -763,8 +774,22 @@ def main():
                 f"both blobs served) x {sym} pairs / mean pair-kernel launch "
                 f"{1e3 * pairs_t:.3f} ms (CUDA events on the launching stream); {peak_note}. "
                 f"The directed kernel + final pass take {1e3 * p2p_t:.3f} ms more")
+    elif _smooth_terms(w):
+        # the smooth near field by expansions: moments and gradients of a
+        # polynomial per blob, no pair sums but those of sparse leaf pairs
+        kernel = "k_sm_moments + k_sm_translate + k_sm_final"
+        terms = _smooth_terms(w)
+        final_t = statistics.mean(r["final"] for r in stage_runs) / 1e3
+        per_blob = 4 * terms + 4 * w.p
+        achieved = per_blob * w.n / (pairs_t + final_t) / 1e12
+        note = (f"{per_blob} FP32 ops per blob ({terms} moments, {3 * terms} of the gradient, "
+                f"{4 * w.p} of the far-field series) x {w.n} blobs / mean of the moments + "
+                f"translation and final stages {1e3 * (pairs_t + final_t):.3f} ms (CUDA events on "
+                f"the launching stream); {peak_note}. Bound by load latency and the scattered "
+                f"output, not by the FP32 pipe; pair by pair this near field has {pairs} ordered "
+                f"pairs")
     else:
-        kernel = "k_p2p_mixed"
+        kernel = "k_near_direct"
         achieved = pairs * P2P_OPS_PER_PAIR / p2p_t / 1e12
         note = (f"{P2P_OPS_PER_PAIR} FP32 ops per ordered pair x {pairs} pairs / mean P2P "
                 f"stage {1e3 * p2p_t:.3f} ms (CUDA events on the launching stream); {peak_note}")
@@ -778,7 +803,7 @@ def main():
     # measured dense TF32 rate: 8 p^2 real flops per (target, source) pair
     m2l_t = statistics.mean(m2l_ms) / 1e3
     m2l_ach = 8.0 * w.p * w.p * stats["m2l_pairs"] / m2l_t / 1e12
-    m2l = {"bound": "tensor", "stage": "M2L (k_m2l_tcb + k_m2l_tile + k_m2l)", "achieved": m2l_ach,
+    m2l = {"bound": "tensor", "stage": "M2L (k_m2l_tcb + k_m2l_orbits + k_m2l)", "achieved": m2l_ach,
            "peak_measured": pipes["tf32_flops"] / 1e12, "unit": "TFLOP/s",
            "frac_of_measured": m2l_ach / (pipes["tf32_flops"] / 1e12),
            "note": (f"8 p^2 flops x {stats['m2l_pairs']} translations / mean M2L stage "
