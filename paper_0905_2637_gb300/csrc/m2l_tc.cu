@@ -451,6 +451,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tcb(
         asm volatile("fence.mbarrier_init.release.cluster;");
         sany = 0;
     }
+    __syncthreads();  // sany is zero before any thread sets a bit of it
     uint32_t ncols = 32;
     while (ncols < uint32_t(NC)) ncols <<= 1;
     if (warp == 0) {
