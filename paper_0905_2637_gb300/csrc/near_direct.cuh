@@ -2,6 +2,8 @@
 // per target: the sums of k_near_direct (p2p.cu) and of the smooth near
 // field's small leaf pairs (smooth.cu).
 #pragma once
+#include <cfloat>
+
 #include "common.cuh"
 
 namespace petfmm {
@@ -19,6 +21,11 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 __device__ __forceinline__ float lg2_ftz(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float lg2_full(float x) {  // subnormal x too
+    float y;
+    asm("lg2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 
@@ -169,7 +176,9 @@ __device__ __forceinline__ float2 near_vortex_of(const NearLeaves &q, const floa
 
 // Laplace kernel: sum of q_j log r over the leaves (global units, logw the
 // log of the leaf width), coincident pairs excluded: log r = ln 2 / 2 log2
-// rho^2 + logw, the constant taken out of the sum.
+// rho^2 + logw, the constant taken out of the sum.  Pairs so close that rho^2
+// is subnormal (the flushing logarithm would take them for coincident, log 0)
+// stand apart with those, behind one test for the four.
 __device__ __forceinline__ float near_laplace(const NearLeaves &q, const float4 *__restrict__ rec,
                                               float x, float y, float logw, uint32_t &total) {
     const float none = -2.88539008f * logw;  // log2 rho^2 that makes log r zero
@@ -177,12 +186,21 @@ __device__ __forceinline__ float near_laplace(const NearLeaves &q, const float4 
     total = near_sources(
         q, rec, x, y,
         [&](const float4(&r)[4], float xt, float yt) {
+            float r2[4], l[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float dx = xt - r[i].x, dy = yt - r[i].y;
-                const float r2 = fmaf(dx, dx, dy * dy);
-                const float l = r2 > 0.f ? lg2_ftz(r2) : none;
-                ps = fmaf(r[i].z, l, ps);
+                r2[i] = fmaf(dx, dx, dy * dy);
+                l[i] = lg2_ftz(r2[i]);
+            }
+            if (fminf(fminf(r2[0], r2[1]), fminf(r2[2], r2[3])) < FLT_MIN) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (r2[i] < FLT_MIN) l[i] = r2[i] > 0.f ? lg2_full(r2[i]) : none;
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                ps = fmaf(r[i].z, l[i], ps);
                 pq += r[i].z;
             }
         },

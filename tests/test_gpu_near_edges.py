@@ -1,0 +1,25 @@
+"""The 2D near field at the edges of its arithmetic: pairs at subnormal
+squared distances, coincident and lone blobs, infinite strengths, cores of
+every width; against the FP64 oracle FMM or the exact value."""
+import numpy as np
+import pytest
+
+import gpu_util as G
+from paper_0905_2637_gb300 import workloads as W
+from test_gpu_laplace import rel, run_laplace
+
+pytestmark = pytest.mark.gpu
+
+
+# A leaf centre of this domain lies at the coordinate origin, where FP32
+# offsets far below the leaf's resolution elsewhere are kept.  1e-20 and 3e-20
+# leaf widths: rho^2 is subnormal, of 17 bits or more, so its logarithm (about
+# -92) is good to 1e-7.  Bar: the mixed path's 1e-5.
+def test_laplace_pairs_at_subnormal_squared_distance(orc):
+    rng = np.random.default_rng(1)
+    x = np.concatenate([[0.0, 1e-20, 0.0, 0.3], rng.uniform(-1.5, 2.5, 60)])
+    y = np.concatenate([[0.0, 0.0, 3e-20, 0.2], rng.uniform(-1.5, 2.5, 60)])
+    w = W.Workload("close", x, y, rng.uniform(0.5, 1.0, x.size), 1.0, (-1.5, -1.5, 4.0), 2, 17, "f64")
+    u, _ = run_laplace(w, precision="mixed")
+    assert np.all(np.isfinite(u))
+    assert rel(u, orc.laplace_fmm(w.x, w.y, w.gamma, w.domain, w.L, w.p)) <= 1e-5
