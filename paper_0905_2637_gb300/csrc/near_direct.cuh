@@ -178,30 +178,34 @@ __device__ __forceinline__ float2 near_vortex_of(const NearLeaves &q, const floa
 // log of the leaf width), coincident pairs excluded: log r = ln 2 / 2 log2
 // rho^2 + logw, the constant taken out of the sum.  Pairs so close that rho^2
 // is subnormal (the flushing logarithm would take them for coincident, log 0)
-// stand apart with those, behind one test for the four.
+// stand apart with those, behind one test for the four; coincident ones have no
+// strength there (a logarithm that cancels the constant leaves its rounding).
 __device__ __forceinline__ float near_laplace(const NearLeaves &q, const float4 *__restrict__ rec,
                                               float x, float y, float logw, uint32_t &total) {
-    const float none = -2.88539008f * logw;  // log2 rho^2 that makes log r zero
     float s = 0.f, qs = 0.f, ps = 0.f, pq = 0.f;
     total = near_sources(
         q, rec, x, y,
         [&](const float4(&r)[4], float xt, float yt) {
-            float r2[4], l[4];
+            float r2[4], l[4], z[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const float dx = xt - r[i].x, dy = yt - r[i].y;
                 r2[i] = fmaf(dx, dx, dy * dy);
                 l[i] = lg2_ftz(r2[i]);
+                z[i] = r[i].z;
             }
             if (fminf(fminf(r2[0], r2[1]), fminf(r2[2], r2[3])) < FLT_MIN) {
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
-                    if (r2[i] < FLT_MIN) l[i] = r2[i] > 0.f ? lg2_full(r2[i]) : none;
+                    if (r2[i] < FLT_MIN) {
+                        l[i] = r2[i] > 0.f ? lg2_full(r2[i]) : 0.f;
+                        if (!(r2[i] > 0.f)) z[i] = 0.f;
+                    }
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                ps = fmaf(r[i].z, l[i], ps);
-                pq += r[i].z;
+                ps = fmaf(z[i], l[i], ps);
+                pq += z[i];
             }
         },
         [&] {

@@ -23,3 +23,14 @@ def test_laplace_pairs_at_subnormal_squared_distance(orc):
     u, _ = run_laplace(w, precision="mixed")
     assert np.all(np.isfinite(u))
     assert rel(u, orc.laplace_fmm(w.x, w.y, w.gamma, w.domain, w.L, w.p)) <= 1e-5
+
+
+# A charge has no potential of its own, nor has one at the same place: exactly
+# zero, whatever the leaf width (its logarithm is a constant of the sum).
+@pytest.mark.parametrize("width", [4.0, 1.0, 1e-6, 1e9])
+def test_laplace_lone_and_coincident_charges_have_no_potential(width):
+    x = np.full(5, 0.3 * width)
+    for n in (1, 5):
+        w = W.Workload("alone", x[:n], x[:n], np.arange(1.0, n + 1), 1.0, (0.0, 0.0, width), 1, 8, "f64")
+        u, v = run_laplace(w, precision="mixed")
+        assert np.all(u == 0.0) and np.all(v == 0.0)
