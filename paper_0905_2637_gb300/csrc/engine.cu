@@ -161,7 +161,7 @@ struct petfmm_ctx {
     Plan plan;
     bool sorted_in_first = true;
     int p2p_grid = 0, pairs_grid = 0;  // CTAs of the persistent near-field launches
-    int direct_sms = 0;                // SMs of the one-thread-per-target kernel, if it ran
+    int direct_sms = 0;                // busy entries of the one-thread-per-target kernel, if it ran
     // CUDA-graph replay of the launch sequence (PETFMM_OPT_GRAPH)
     bool use_graph = false;
     bool capturing = false;
@@ -1070,7 +1070,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
         if (pl.direct)
             PF_CUDA(launch_near_direct(dtask + pl.particles.first, pl.particles.count,
                                        pl.particles.nblocks, dinst, start, skeys, srec, pb.own,
-                                       ctrl, dbusy, st, lc));
+                                       ctrl, dbusy, c->direct_sms, st, lc));
         else if (pl.items_any)
             PF_CUDA(launch_p2p_mixed(grid, pl.deg, pl.general,
                                      static_cast<const uint4 *>(c->items.p), ctrl, dinst, start,

@@ -213,9 +213,10 @@ cudaError_t launch_p2p_mixed(int grid, int deg, int general, const uint4 *items,
 // leaves not summed pairwise with its own (tasks over blobs).
 cudaError_t launch_near_direct(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
                                const uint32_t *start, const uint32_t *skeys, const float4 *rec,
-                               float2 *own, uint32_t *ctrl, unsigned long long *busy,
+                               float2 *own, uint32_t *ctrl, unsigned long long *busy, int nbusy,
                                cudaStream_t st, uint64_t *launches);
-// (busy: per SM the first start, preset to all ones, and the last end.)
+// (busy: of the SMs with identifiers below nbusy the first start, preset to
+// all ones, and the last end.)
 // Fewest blobs in both leaves of a pair for the pair kernel.
 constexpr uint32_t P2P_PAIR_MIN = 32;
 // Pairwise near field between neighbouring leaves (mixed path).  Buffers:

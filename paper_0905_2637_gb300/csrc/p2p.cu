@@ -1370,15 +1370,17 @@ __global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
     const Task *__restrict__ tasks, int ntasks, const InstDesc *__restrict__ insts,
     const uint32_t *__restrict__ start, const uint32_t *__restrict__ skeys,
     const float4 *__restrict__ rec, float2 *__restrict__ own, uint32_t *ctrl,
-    unsigned long long *busy) {
+    unsigned long long *busy, uint32_t nbusy) {
     __shared__ unsigned long long spairs;
-    // busy: first start and last end of this kernel's blocks on each SM
+    // busy: first start and last end of this kernel's blocks on each SM, by
+    // %smid; the identifiers need not be contiguous, and those from nbusy on
+    // have no entry
     uint32_t sm = 0;
     if (threadIdx.x == 0) {
         spairs = 0;
         if (busy) {
             asm volatile("mov.u32 %0, %%smid;" : "=r"(sm));
-            atomicMin(busy + 2 * sm, (unsigned long long)global_ns());
+            if (sm < nbusy) atomicMin(busy + 2 * sm, (unsigned long long)global_ns());
         }
     }
     __syncthreads();
@@ -1417,17 +1419,17 @@ __global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
     if (threadIdx.x == 0) {
         if (spairs)
             atomicAdd(reinterpret_cast<unsigned long long *>(ctrl + CTRL_PAIRS_LO), spairs);
-        if (busy) atomicMax(busy + 2 * sm + 1, (unsigned long long)global_ns());
+        if (busy && sm < nbusy) atomicMax(busy + 2 * sm + 1, (unsigned long long)global_ns());
     }
 }
 
 cudaError_t launch_near_direct(const Task *tasks, int ntasks, int64_t nblocks, const InstDesc *insts,
                                const uint32_t *start, const uint32_t *skeys, const float4 *rec,
-                               float2 *own, uint32_t *ctrl, unsigned long long *busy,
+                               float2 *own, uint32_t *ctrl, unsigned long long *busy, int nbusy,
                                cudaStream_t st, uint64_t *launches) {
     if (nblocks <= 0) return cudaSuccess;
     k_near_direct<<<unsigned(nblocks * (256 / NEAR_THREADS)), NEAR_THREADS, 0, st>>>(
-        tasks, ntasks, insts, start, skeys, rec, own, ctrl, busy);
+        tasks, ntasks, insts, start, skeys, rec, own, ctrl, busy, uint32_t(nbusy));
     PF_LAUNCHED(1);
     return cudaGetLastError();
 }

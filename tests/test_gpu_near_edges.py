@@ -34,3 +34,15 @@ def test_laplace_lone_and_coincident_charges_have_no_potential(width):
         w = W.Workload("alone", x[:n], x[:n], np.arange(1.0, n + 1), 1.0, (0.0, 0.0, width), 1, 8, "f64")
         u, v = run_laplace(w, precision="mixed")
         assert np.all(u == 0.0) and np.all(v == 0.0)
+
+
+# The busy times of the direct kernel (timing on) are kept by SM: a value for
+# the SMs that have an entry, no effect on the result.
+def test_busy_times_of_the_direct_kernel():
+    w = W.tiny(40_000, 3, L=6, p=8, sigma=0.002)
+    keep = []
+    timed = G.run(w, "mixed", timing=True, ctx_out=keep)
+    st = keep[0].stats()
+    keep[0].close()
+    assert 0.0 < st["p2p_load_balance"] <= 1.0
+    assert all(np.array_equal(a, b) for a, b in zip(timed, G.run(w, "mixed")))
