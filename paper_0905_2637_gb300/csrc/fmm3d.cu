@@ -3237,8 +3237,8 @@ int petfmm3d_set_option(petfmm3d_ctx *c, int option, int64_t value) {
     switch (option) {
         case PETFMM3D_OPT_TIMING: c->timing = value != 0; return PETFMM_OK;
         case PETFMM3D_OPT_M2L_TC:
-            if (value != 0 && value != 1) return PETFMM_EINVAL;
-            c->m2l_tc = value == 2 ? 2 : value != 0;
+            if (value < 0 || value > 2) return PETFMM_EINVAL;
+            c->m2l_tc = int(value);
             return PETFMM_OK;
         default: return PETFMM_EINVAL;
     }
