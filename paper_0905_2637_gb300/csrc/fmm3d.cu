@@ -57,7 +57,6 @@ namespace {
 
 constexpr int P3_MAX = PETFMM3D_MAX_P;           // terms
 constexpr int L3_MAX = PETFMM3D_MAX_L;           // levels (3L <= 30 key bits)
-constexpr int NC3_MAX = P3_MAX * (P3_MAX + 1) / 2;  // stored coefficients
 constexpr int TC3_MAXP = 8;                        // terms of the tensor-core M2L
 constexpr int NSLOT3 = 343;                        // offsets in [-3, 3]^3
 constexpr int W3 = 8;                              // warps per block
@@ -1594,11 +1593,26 @@ __device__ __forceinline__ void store3(void *o, int64_t i, double v) {
 // and the parts are added in a fixed order.
 //
 // A pair item is (leaf A, group of the 13 forward directions); a heavier leaf
-// has more groups, so that no item outlasts the launch.  Parts: fwd[g] of A's
-// charges (from group g's neighbours; group 0 also the leaf itself), bwd[d] of
-// a leaf's charges from the leaf behind it in direction d, own (one-sided).
+// has more groups.  Parts: fwd[g] of A's charges (from group g's neighbours;
+// group 0 also the leaf itself), bwd[d] of a leaf's charges from the leaf behind
+// it in direction d, own (one-sided).
+//
+// One warp evaluates a leaf pair, all of it (its reactions have one writer), so
+// a pair is left to the one-sided sums, which any number of warps share, where
+// it is more than a small part of the whole: na nb above P3_SHARE / 4096 of the
+// pairs of all leaf pairs that could be pairwise, and above P3_LEAST (a group
+// of three such pairs is no more than the six of 96 charges that two groups a
+// leaf give).
+// Measured (one GB300, whole evaluations, p = 6, us; all pairs pairwise / at this
+// limit): mixed, 5,000 clustered charges 714 / 390, 150,000 16,800 / 2,440,
+// 100,000 charges in eight leaves 342,000 / 6,900; FP64, 60,000 clustered 338,000
+// / 68,300.  Shares of 1/2048, 1/4096, 1/8192 (mixed): 600,000 clustered 27.5 /
+// 22.9 / 21.9 ms, but 1,000,000 uniform charges, 1,950 a leaf, 18.0 / 18.0 /
+// 21.8; of 1/256, 1/410, 1/512 (FP64): 150,000 clustered 135 / 110 / 104 ms,
+// 100,000 uniform, 1,560 a leaf, 99 / 99 / 126.
 // ---------------------------------------------------------------------------
 constexpr uint32_t P3_PAIR_MIN = 24;
+constexpr uint32_t P3_SHARE = 1, P3_SHARE64 = 10, P3_LEAST = 16384;
 constexpr int P3_DIRS = 13;
 // planes of one entry per charge, fwd and bwd: mixed (the leaf itself in its
 // first group) and FP64 (a group by itself in the heaviest leaves)
@@ -1627,9 +1641,12 @@ __host__ __device__ __forceinline__ int own_group3(int groups) {
 // bit 14: fwd of the leaf's groups do
 constexpr uint32_t LF3_OWN = 1u << 13, LF3_FWD = 1u << 14;
 // counters: directed items, pair items, then per work class the pair items
-// counted and placed
+// counted and placed, then (64 bits) the pairs of all leaf pairs of at least
+// pmin charges each
 constexpr int C3_DIRECTED = 0, C3_PAIRS = 1, C3_COUNT = 2, C3_CLASSES = 64,
-              C3_PLACED = C3_COUNT + C3_CLASSES, C3_WORDS = C3_PLACED + C3_CLASSES;
+              C3_PLACED = C3_COUNT + C3_CLASSES, C3_TOTAL = C3_PLACED + C3_CLASSES,
+              C3_WORDS = C3_TOTAL + 2;
+static_assert(C3_TOTAL % 2 == 0, "64-bit counter");
 
 struct Near3 {
     float4 *own, *slots;  // slots[P3_SLOTS][n], or no pairs
@@ -1639,7 +1656,22 @@ struct Near3 {
     uint2 *items;         // (leaf, group)
     int64_t n;
     uint32_t pmin;        // P3_PAIR_MIN, or all ones: no pairs
+    uint32_t share;       // most3's limit, in 1/4096 of the total
 };
+
+// Most charges of a leaf that is summed pairwise with one of n charges (n >= 1;
+// na nb <= limit is the same for both leaves), 0: none is.
+__device__ __forceinline__ uint32_t most3(const Near3 &w, uint32_t n) {
+    if (n < w.pmin) return 0;
+    const uint64_t total = *reinterpret_cast<const unsigned long long *>(w.ctrl + C3_TOTAL);
+    const uint64_t limit = (total >> 12) * w.share;
+    return max(uint32_t(min(limit, uint64_t(0xffffffffu))), P3_LEAST) / n;
+}
+// Whether a leaf with most = most3 of its charges and a neighbour of n (or
+// itself) are summed pairwise.
+__device__ __forceinline__ bool pairwise3(const Near3 &w, uint32_t most, uint32_t n) {
+    return n >= w.pmin && n <= most;
+}
 
 __device__ __forceinline__ uint32_t leaf_count3(const uint32_t *start, int side, int x, int y,
                                                 int z) {
@@ -1657,7 +1689,8 @@ __device__ __forceinline__ int class3(uint32_t n, uint64_t src) {
     return c >= C3_CLASSES ? 0 : C3_CLASSES - 1 - c;
 }
 
-// Calls f(class, group) for the pair items of leaf b (n charges).
+// Calls f(class, group, pairs) for the pair items of leaf b (n charges), as if
+// every leaf pair of at least pmin charges each were summed pairwise.
 template <int MAX, typename F>
 __device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, int L, uint32_t b,
                                             uint32_t n, uint32_t pmin, F &&f) {
@@ -1672,7 +1705,7 @@ __device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, 
             const uint32_t c = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
             if (c >= pmin) src += c;
         }
-        f(class3(n, src), g);
+        f(class3(n, src), g, uint64_t(n) * src);
     }
 }
 
@@ -1684,18 +1717,30 @@ template <bool EMIT, int MAX>
 __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__restrict__ start,
                                                      Near3 w) {
     __shared__ uint32_t hist[C3_CLASSES], base[C3_CLASSES], ndir, dbase;
+    __shared__ unsigned long long sum;
     const int64_t nleaf = int64_t(1) << (3 * L);
     const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (threadIdx.x < C3_CLASSES) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) ndir = 0;
+    if (threadIdx.x == 0) {
+        ndir = 0;
+        sum = 0;
+    }
     __syncthreads();
     const uint32_t s0 = b < nleaf ? start[b] : 0u, n = b < nleaf ? start[b + 1] - s0 : 0u;
     const bool big = n >= w.pmin;
+    unsigned long long pairs = 0;
     if (big)
-        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin,
-                         [&](int c, int) { atomicAdd(&hist[c], 1u); });
+        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int, uint64_t q) {
+            atomicAdd(&hist[c], 1u);
+            pairs += q;
+        });
     if (!EMIT) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
+        if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&sum, pairs);
         __syncthreads();
+        if (threadIdx.x == 0 && sum)
+            atomicAdd(reinterpret_cast<unsigned long long *>(w.ctrl + C3_TOTAL), sum);
         if (threadIdx.x < C3_CLASSES && hist[threadIdx.x]) {
             atomicAdd(w.ctrl + C3_COUNT + threadIdx.x, hist[threadIdx.x]);
             atomicAdd(w.ctrl + C3_PAIRS, hist[threadIdx.x]);
@@ -1708,14 +1753,16 @@ __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__re
         const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
                   iz = int(compact3(uint32_t(b) >> 2));
         uint32_t flags = big ? LF3_FWD : 0u;
-        bool directed = !big;
+        const uint32_t most = most3(w, n);
+        bool directed = !pairwise3(w, most, n);
         for (int k = 0; big && k < P3_DIRS; ++k) {
             int dx, dy, dz;
             fwd3(k, &dx, &dy, &dz);
             const uint32_t f = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
             const uint32_t r = leaf_count3(start, side, ix - dx, iy - dy, iz - dz);
-            if (r >= w.pmin) flags |= 1u << k;
-            directed |= (f && f < w.pmin) || (r && r < w.pmin);
+            const bool rp = pairwise3(w, most, r);
+            if (rp) flags |= 1u << k;
+            directed |= (f && !pairwise3(w, most, f)) || (r && !rp);
         }
         if (directed) {
             flags |= LF3_OWN;
@@ -1738,7 +1785,7 @@ __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__re
     for (uint32_t i = 0; i < mine; ++i)
         w.directed[dbase + at + i] = make_uint2(uint32_t(b), s0 + 32 * i);
     if (big)
-        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int g) {
+        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int g, uint64_t) {
             w.items[base[c] + atomicAdd(&hist[c], 1u)] = make_uint2(uint32_t(b), uint32_t(g));
         });
 }
@@ -1841,7 +1888,8 @@ constexpr int P3_REST = 16;
 // targets a lane and whole-warp rings the eight shuffles of a step were a
 // quarter of its instructions.)  first: the reactions are stored, else added
 // to those of A's earlier runs (the same warp's).
-__device__ __forceinline__ void pairs_run3(const Near3 &w, int L, const uint32_t *__restrict__ start,
+__device__ __forceinline__ void pairs_run3(const Near3 &w, uint32_t most, int L,
+                                           const uint32_t *__restrict__ start,
                                            const float4 *__restrict__ rec, uint32_t leaf, int g,
                                            uint32_t t0, uint32_t t1, bool first, int lane) {
     const int side = 1 << L;
@@ -1863,7 +1911,7 @@ __device__ __forceinline__ void pairs_run3(const Near3 &w, int L, const uint32_t
         t.z[i] = make_float2(r[2 * i].z, r[2 * i + 1].z);
         t.q[i] = make_float2(r[2 * i].w, r[2 * i + 1].w);
     }
-    if (g == 0)
+    if (g == 0 && pairwise3(w, most, a1 - a0))
 #pragma unroll 2
         for (uint32_t j = a0 + half; j < a1; j += 2) own3(t, rec[j]);
     const int groups = groups3(a1 - a0);
@@ -1874,7 +1922,7 @@ __device__ __forceinline__ void pairs_run3(const Near3 &w, int L, const uint32_t
         if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side) continue;
         const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
         const uint32_t b0 = start[nb], b1 = start[nb + 1];
-        if (b1 - b0 < w.pmin) continue;
+        if (!pairwise3(w, most, b1 - b0)) continue;
         float4 *out = w.slots + int64_t(P3_DIRS + k) * w.n;
         const float ox = float(dx), oy = float(dy), oz = float(dz);
         uint32_t c = b0;
@@ -1951,7 +1999,8 @@ __device__ __forceinline__ void pairs_run3(const Near3 &w, int L, const uint32_t
 // The targets left over after whole runs (up to 16), four at a time: the
 // lanes hold the neighbours' charges, so that no lane idles for want of
 // targets; the reactions are added to those of the leaf's first run.
-__device__ __forceinline__ void pairs_rest3(const Near3 &w, int L, const uint32_t *__restrict__ start,
+__device__ __forceinline__ void pairs_rest3(const Near3 &w, uint32_t most, int L,
+                                            const uint32_t *__restrict__ start,
                                             const float4 *__restrict__ rec, uint32_t leaf, int g,
                                             uint32_t t0, uint32_t t1, int lane) {
     const int side = 1 << L;
@@ -1972,7 +2021,7 @@ __device__ __forceinline__ void pairs_rest3(const Near3 &w, int L, const uint32_
             t.z[i] = make_float2(r[2 * i].z, r[2 * i + 1].z);
             t.q[i] = make_float2(r[2 * i].w, r[2 * i + 1].w);
         }
-        if (g == 0)
+        if (g == 0 && pairwise3(w, most, a1 - a0))
             for (uint32_t j = a0 + uint32_t(lane); j < a1; j += 32) own3(t, rec[j]);
         for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
             int dx, dy, dz;
@@ -1981,7 +2030,7 @@ __device__ __forceinline__ void pairs_rest3(const Near3 &w, int L, const uint32_
             if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side) continue;
             const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
             const uint32_t b0 = start[nb], b1 = start[nb + 1];
-            if (b1 - b0 < w.pmin) continue;
+            if (!pairwise3(w, most, b1 - b0)) continue;
             float4 *out = w.slots + int64_t(P3_DIRS + k) * w.n;
             for (uint32_t j = b0 + uint32_t(lane); j < b1; j += 32) {
                 const float4 u = rec[j], p = out[j];
@@ -2027,14 +2076,15 @@ __global__ void __launch_bounds__(128, 6) k3_pairs(int L, const uint32_t *__rest
     if (!PF_IN(leaf, int64_t(1) << (3 * L))) return;
     const int g = int(item.y);
     const uint32_t a0 = start[leaf], a1 = start[leaf + 1];
+    const uint32_t most = most3(w, a1 - a0);
     bool first = true;
     for (uint32_t t = a0; t < a1;) {
         const uint32_t left = a1 - t;
         if (left <= 16 && !first) {
-            pairs_rest3(w, L, start, rec, leaf, g, t, a1, lane);
+            pairs_rest3(w, most, L, start, rec, leaf, g, t, a1, lane);
             break;
         }
-        pairs_run3(w, L, start, rec, leaf, g, t, min(a1, t + 64), first, lane);
+        pairs_run3(w, most, L, start, rec, leaf, g, t, min(a1, t + 64), first, lane);
         t += 64;
         first = false;
     }
@@ -2063,6 +2113,7 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_directed(int L,
     if (!PF_IN(b, int64_t(1) << (3 * L))) return;
     const uint32_t s0 = item.y;
     const uint32_t nme = start[b + 1] - start[b];
+    const uint32_t most = most3(w, nme);
     const uint32_t s1 = min(start[b + 1], s0 + 32u);
     const int k = int(s1 - s0);  // 1..32 (an item holds at least one target)
     int lg = 0;
@@ -2083,7 +2134,7 @@ __global__ void __launch_bounds__(W3 * 32, 4) k3_near_directed(int L,
                     continue;
                 const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
                 const uint32_t a = start[nb], e = start[nb + 1];
-                if (nme >= w.pmin && e - a >= w.pmin) continue;  // pairwise
+                if (pairwise3(w, most, e - a)) continue;
                 const float ox = tg.x - float(dx), oy = tg.y - float(dy), oz = tg.z - float(dz);
                 // |d| = 0 only within the target's own leaf (self, and
                 // coincident particles, which bin to the same leaf); the
@@ -2173,29 +2224,6 @@ __global__ void __launch_bounds__(256) k3_near_final(int L, int p, double w,
     store3<TOut>(ez, o, double((s.w - fz) * inv_w2));
 }
 
-// ---------------------------------------------------------------------------
-// The FP64 near field's work items: leaf b with n_b particles gives ceil(n_b /
-// 32) items (b, first sorted rank of the chunk), in leaf order (a hot leaf's
-// chunks go to consecutive warps, so they spread over the SMs).
-__global__ void __launch_bounds__(256) k3_near_count(const uint32_t *__restrict__ start,
-                                                     int64_t nleaf, uint32_t *__restrict__ cnt) {
-    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    cnt[b] = (start[b + 1] - start[b] + 31u) / 32u;
-}
-__global__ void __launch_bounds__(256) k3_near_emit(const uint32_t *__restrict__ start,
-                                                    int64_t nleaf, const uint32_t *__restrict__ off,
-                                                    const uint32_t *__restrict__ nitems,
-                                                    int64_t cap, uint2 *__restrict__ items) {
-    const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    const uint32_t s0 = start[b], k = (start[b + 1] - s0 + 31u) / 32u;
-    for (uint32_t c = 0; c < k; ++c) {
-        const int64_t o = int64_t(off[b]) + c;
-        if (o < cap && o < int64_t(*nitems)) items[o] = make_uint2(uint32_t(b), s0 + 32u * c);
-    }
-}
-
 // 1/sqrt(x): the hardware's approximation y and one step of Householder's
 // third-order iteration, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y^2
 // (|e| < 2^-18 leaves |e|^3 below 2^-54): five FP64 operations, where a
@@ -2210,30 +2238,26 @@ __device__ __forceinline__ double rsqrt_f64(double x) {
     return fma(y * e, fma(0.375, e, 0.5), y);
 }
 
-// The FP64 path: global coordinates; a warp per work item, its lanes shared
-// out over an item's few targets as in the mixed kernel.  Bound by the FP64
-// pipe (two lanes a cycle and SM): 18 operations a pair.  Measured (one
-// GB300, 262,144 uniform charges, L = 4): 32.9 ms with a division and a square
-// root per pair and a warp per leaf -> 16.6 ms.  Used without k3_pairs_f64's
-// memory.
-template <typename TOut>
-__global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
-                                                       const uint32_t *__restrict__ start,
-                                                       const Dbl4 *__restrict__ xs,
-                                                       const double2 *__restrict__ le,
-                                                       const uint32_t *__restrict__ perm,
-                                                       const uint2 *__restrict__ items,
-                                                       const uint32_t *__restrict__ nitems,
-                                                       int64_t n, void *phi, void *ex, void *ey,
-                                                       void *ez) {
-    __shared__ double2 sle[W3][NC3_MAX];
+// The FP64 path's leaf pairs not evaluated pairwise: global coordinates; work
+// items, and lanes shared out over an item's few targets, as in the mixed
+// kernel.  Bound by the FP64 pipe (two lanes a cycle and SM): 18 operations a
+// pair.  Measured with every leaf pair (one GB300, 262,144 uniform charges, L =
+// 4): 32.9 ms with a division and a square root per pair and a warp per leaf ->
+// 16.6 ms.
+__global__ void __launch_bounds__(W3 * 32) k3_near_directed64(int L,
+                                                              const uint32_t *__restrict__ start,
+                                                              const Dbl4 *__restrict__ xs,
+                                                              const Near3 w,
+                                                              Dbl4 *__restrict__ own) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t it = int64_t(blockIdx.x) * W3 + wid;
-    if (it >= int64_t(*nitems)) return;
+    if (it >= int64_t(w.ctrl[C3_DIRECTED])) return;
     // one item: the targets s0 .. s1 - 1 of leaf b, rep lanes each
-    const uint2 item = items[it];
+    const uint2 item = w.directed[it];
     const int64_t b = item.x;
     if (!PF_IN(b, int64_t(1) << (3 * L))) return;
+    const uint32_t nme = start[b + 1] - start[b];
+    const uint32_t most = most3(w, nme);
     const uint32_t s0 = item.y, s1 = min(start[b + 1], s0 + 32u);
     const int k = int(s1 - s0);
     int lg = 0;
@@ -2241,18 +2265,10 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
     const uint32_t rep = 1u << lg, c = uint32_t(lane) & (rep - 1u);
     const uint32_t i = s0 + uint32_t(lane >> lg);
     const bool live = i < s1;
-    const int nc = nc3(p);
-    const bool far = L >= 2;
-    if (far)
-        for (int t = lane; t < nc; t += 32) sle[wid][t] = le[(lvl_off3(L) + b) * nc + t];
-    __syncwarp();
     const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
               iz = int(compact3(uint32_t(b) >> 2));
     const int side = 1 << L;
-    const double w = d.width / double(side);
-    const double cx = d.x0 + (ix + 0.5) * w, cy = d.y0 + (iy + 0.5) * w,
-                 cz = d.z0 + (iz + 0.5) * w;
-    const Dbl4 tg = live ? xs[i] : Dbl4{cx, cy, cz, 0.0};
+    const Dbl4 tg = xs[live ? i : s0];
     double f = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
     for (int dz = -1; dz <= 1; ++dz)
         for (int dy = -1; dy <= 1; ++dy)
@@ -2261,9 +2277,10 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
                 if (nx < 0 || ny < 0 || nz < 0 || nx >= side || ny >= side || nz >= side)
                     continue;
                 const uint32_t nb = morton3(uint32_t(nx), uint32_t(ny), uint32_t(nz));
-                const uint32_t e = start[nb + 1];
+                const uint32_t a = start[nb], e = start[nb + 1];
+                if (pairwise3(w, most, e - a)) continue;
 #pragma unroll 2
-                for (uint32_t j = start[nb] + c; j < e; j += rep) {
+                for (uint32_t j = a + c; j < e; j += rep) {
                     const Dbl4 s = xs[j];
                     const double ddx = tg.x - s.x, ddy = tg.y - s.y, ddz = tg.z - s.z;
                     const double r2 = fma(ddx, ddx, fma(ddy, ddy, ddz * ddz));
@@ -2284,25 +2301,14 @@ __global__ void __launch_bounds__(W3 * 32) k3_near_f64(int L, int p, Dom3 d,
         gy += __shfl_xor_sync(0xffffffffu, gy, int(o));
         gz += __shfl_xor_sync(0xffffffffu, gz, int(o));
     }
-    if (c == 0 && live) {
-        double ff = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
-        if (far)
-            l2p3<double, double2>(sle[wid], p, (tg.x - cx) / w, (tg.y - cy) / w, (tg.z - cz) / w,
-                                  ff, fx, fy, fz);
-        const int64_t o = perm[i];
-        if (PF_IN(o, n)) {
-            store3<TOut>(phi, o, f + ff / w);
-            store3<TOut>(ex, o, gx - fx / (w * w));
-            store3<TOut>(ey, o, gy - fy / (w * w));
-            store3<TOut>(ez, o, gz - fz / (w * w));
-        }
-    }
+    if (c == 0 && live) own[i] = Dbl4{f, gx, gy, gz};
 }
 
 // ---------------------------------------------------------------------------
 // FP64 near field, pairwise: a warp per pair item (leaf A, group of forward
-// directions, as k3_near_items lists them with pmin = 1).  The charges of the
-// group's neighbours, and of A itself in one group, form one list; each lane
+// directions, as k3_near_items lists them with pmin = 1; the leaf pairs above
+// limit left out).  The charges of the group's neighbours, and of A itself in
+// one group, form one list; each lane
 // takes one of 32 and keeps its reaction in registers while A's targets pass
 // by: lane l meets target (l + step) mod 32 of a run of 32, so that the sums of
 // the targets, in shared memory, have one writer a step.  A last run of c < 32
@@ -2359,6 +2365,7 @@ __global__ void __launch_bounds__(PW64 * 32) k3_pairs_f64(int L, const uint32_t 
     const int groups = groups3<P3_GROUPS64>(a1 - a0);
     const int k0 = group_first3(g, groups), nk = group_first3(g + 1, groups) - k0;
     Dbl4 *tgt = stgt[wid], *acc = sacc[wid];
+    const uint32_t most = most3(w, a1 - a0);
     // lane 0: the leaf itself (its group only); lane 1 + i: forward direction k0 + i
     uint32_t beg = 0, cnt = 0;
     if (lane == 0 && g == own_group3(groups)) {
@@ -2374,6 +2381,7 @@ __global__ void __launch_bounds__(PW64 * 32) k3_pairs_f64(int L, const uint32_t 
             cnt = start[nb + 1] - beg;
         }
     }
+    if (!pairwise3(w, most, cnt)) cnt = 0;
     uint32_t end = cnt;  // of the lane's range in the list
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -2445,7 +2453,8 @@ __global__ void __launch_bounds__(128) k3_final_f64(int L, int p, Dom3 d,
                                                     const double2 *__restrict__ le,
                                                     const uint32_t *__restrict__ perm,
                                                     const Near3 nr, const Dbl4 *__restrict__ slots,
-                                                    void *phi, void *ex, void *ey, void *ez) {
+                                                    const Dbl4 *__restrict__ own, void *phi,
+                                                    void *ex, void *ey, void *ez) {
     const int64_t i = int64_t(blockIdx.x) * 128 + threadIdx.x;
     if (i >= nr.n) return;
     const uint32_t b = skeys[i];
@@ -2458,8 +2467,11 @@ __global__ void __launch_bounds__(128) k3_final_f64(int L, int p, Dom3 d,
         s.z += v.z;
         s.w += v.w;
     };
-    const int groups = groups3<P3_GROUPS64>(start[b + 1] - start[b]);
-    for (int g = 0; g < groups; ++g) add(slots[int64_t(g) * nr.n + i]);
+    if (flags & LF3_OWN) add(own[i]);
+    if (flags & LF3_FWD) {
+        const int groups = groups3<P3_GROUPS64>(start[b + 1] - start[b]);
+        for (int g = 0; g < groups; ++g) add(slots[int64_t(g) * nr.n + i]);
+    }
 #pragma unroll
     for (int k = 0; k < P3_DIRS; ++k)
         if ((flags >> k) & 1u) add(slots[int64_t(P3_GROUPS64 + k) * nr.n + i]);
@@ -2688,9 +2700,8 @@ struct petfmm3d_ctx {
     int L = 0, p = 0, precision = 0, dtype = 0;
     cudaStream_t stream = nullptr;
     DevBuf3 keysA, keysB, valsA, valsB, sortw, start, recu, rec, xs, me, le, status;
-    DevBuf3 ncnt, noff, nscan, nitems;  // the near field's work items
-    // mixed near field: pair items, parts of the charges' sums, flags, counters
-    DevBuf3 pitems, slots, nown, nflags, nctrl;
+    // near field: one-sided and pair items, parts of the charges' sums, flags, counters
+    DevBuf3 nitems, pitems, slots, nown, nflags, nctrl;
     bool no_pairs = false;  // no room for the parts of pairwise sums
     // operator tables of the context's precision only
     DevBuf3 orbits, atab32, rmap, parity;  // M2L operators: by orbit, by offset
@@ -3092,6 +3103,7 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
         P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
         P3_TRY(ensure3(c->nown, size_t(n) * sizeof(float4), st));
         nr.own = static_cast<float4 *>(c->nown.p);
+        nr.share = P3_SHARE;
         nr.slots = static_cast<float4 *>(c->slots.p);
         nr.directed = static_cast<uint2 *>(c->nitems.p);
         const float4 *rec = static_cast<const float4 *>(c->rec.p);
@@ -3124,48 +3136,38 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
         Near3 nr{};
         int64_t icap = 0;
         P3_TRY(near_pairs3(c, n, nleaf, 1, P3_SLOTS64 * sizeof(Dbl4), &nr, &icap));
-        if (nr.pmin == 1) {
-            Dbl4 *slots = static_cast<Dbl4 *>(c->slots.p);
+        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
+        P3_TRY(ensure3(c->nown, size_t(n) * sizeof(Dbl4), st));
+        nr.directed = static_cast<uint2 *>(c->nitems.p);
+        nr.share = P3_SHARE64;
+        Dbl4 *slots = static_cast<Dbl4 *>(c->slots.p), *own = static_cast<Dbl4 *>(c->nown.p);
+        const bool pairs = nr.pmin != ~0u;
+        if (pairs) {
+            k3_near_items<false, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
+            P3_CUDA(cudaGetLastError());
+            c->launches++;
+        }
+        k3_near_items<true, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
+        P3_CUDA(cudaGetLastError());
+        if (pairs) {
             constexpr int pad = int(kPairs64Smem - PW64 * (PT64 + PA64) * sizeof(Dbl4));
             P3_CUDA(cudaFuncSetAttribute(k3_pairs_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          pad));
-            k3_near_items<false, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
-            P3_CUDA(cudaGetLastError());
-            k3_near_items<true, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
-            P3_CUDA(cudaGetLastError());
             k3_pairs_f64<<<unsigned((icap + PW64 - 1) / PW64), PW64 * 32, pad, st>>>(L, start, xs, nr,
                                                                                    slots);
             P3_CUDA(cudaGetLastError());
-            c->launches += 3;
-            const unsigned gf = unsigned((n + 127) / 128);
-            if (f32)
-                k3_final_f64<float><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr,
-                                                        slots, phi, ex, ey, ez);
-            else
-                k3_final_f64<double><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr,
-                                                         slots, phi, ex, ey, ez);
-        } else {
-            P3_TRY(ensure3(c->ncnt, size_t(nleaf) * 4, st));
-            P3_TRY(ensure3(c->noff, size_t(nleaf) * 4 + 16, st));
-            P3_TRY(ensure3(c->nscan, size_t(scan_scratch_words(nleaf)) * 4, st));
-            P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-            uint32_t *cnt = static_cast<uint32_t *>(c->ncnt.p), *off = static_cast<uint32_t *>(c->noff.p);
-            uint32_t *nit = off + nleaf;  // the item count, after the offsets
-            uint2 *items = static_cast<uint2 *>(c->nitems.p);
-            k3_near_count<<<gb, 256, 0, st>>>(start, nleaf, cnt);
-            P3_CUDA(cudaGetLastError());
-            P3_CUDA(exclusive_scan(cnt, off, nleaf, static_cast<uint32_t *>(c->nscan.p), nit, st,
-                                   &c->launches));
-            k3_near_emit<<<gb, 256, 0, st>>>(start, nleaf, off, nit, cap, items);
-            P3_CUDA(cudaGetLastError());
-            c->launches += 2;
-            if (f32)
-                k3_near_f64<float><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
-                                                           phi, ex, ey, ez);
-            else
-                k3_near_f64<double><<<gi, W3 * 32, 0, st>>>(L, p, d, start, xs, le, perm, items, nit, n,
-                                                            phi, ex, ey, ez);
+            c->launches++;
         }
+        k3_near_directed64<<<gi, W3 * 32, 0, st>>>(L, start, xs, nr, own);
+        P3_CUDA(cudaGetLastError());
+        c->launches += 2;
+        const unsigned gf = unsigned((n + 127) / 128);
+        if (f32)
+            k3_final_f64<float><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr, slots,
+                                                    own, phi, ex, ey, ez);
+        else
+            k3_final_f64<double><<<gf, 128, 0, st>>>(L, p, d, skeys, start, xs, le, perm, nr, slots,
+                                                     own, phi, ex, ey, ez);
     }
     P3_CUDA(cudaGetLastError());
     c->launches++;
@@ -3303,7 +3305,7 @@ int petfmm3d_debug_shift_operator(int order, int kind, int octant, double *out, 
 int petfmm3d_destroy(petfmm3d_ctx *c) {
     if (!c) return PETFMM_EINVAL;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    DevBuf3 *bufs[] = {&c->ncnt, &c->noff, &c->nscan, &c->nitems, &c->pitems, &c->slots,
+    DevBuf3 *bufs[] = {&c->nitems, &c->pitems, &c->slots,
                        &c->nown, &c->nflags, &c->nctrl,
                        &c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->sortw, &c->start,
                        &c->recu,  &c->rec,   &c->xs,    &c->me,    &c->le,    &c->status,
