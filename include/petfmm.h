@@ -706,12 +706,22 @@ int petfmm3d_evaluate(petfmm3d_ctx *ctx, int64_t n, const void *x, const void *y
 int petfmm3d_sync(petfmm3d_ctx *ctx);
 enum {
     PETFMM3D_OPT_TIMING = 1, /* 1: record CUDA events per stage */
-    PETFMM3D_OPT_M2L_TC = 2  /* mixed path, p <= 8: 1 run M2L on the tensor cores
+    PETFMM3D_OPT_M2L_TC = 2, /* mixed path, p <= 8: 1 run M2L on the tensor cores
                                 (tcgen05, TF32 hi/lo split, FP32 accumulation);
                                 0 the SIMT GEMM kernel; 2 (default) the tensor
                                 cores from 5 levels on, below that FP32 sums by
                                 reflection orbits (which p > 8 always takes).
                                 Results differ by FP32-level rounding. */
+    PETFMM3D_OPT_PAIR_BYTES = 3 /* most bytes of device memory for near-field sums
+                                that evaluate a pair of charges once for both (416
+                                bytes a charge, FP64 path 864; default 26 x 2^30).
+                                An evaluation that needs more, or more than can be
+                                allocated beside the buffers that it cannot do
+                                without, sums every pair from both sides instead,
+                                more slowly; the results differ by rounding (of
+                                the path's precision).  After a failed allocation
+                                the context stays with that until this option is
+                                set.  0: always from both sides. */
 };
 int petfmm3d_set_option(petfmm3d_ctx *ctx, int option, int64_t value);
 enum {

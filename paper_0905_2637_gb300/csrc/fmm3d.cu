@@ -35,10 +35,12 @@
 // in double; mixed path: float4 (xi, eta, zeta, q), the position relative to
 // the leaf centre in leaf widths), ME and LE of every level (8^l boxes in
 // Morton order, level l at box offset (8^l - 1) / 7), the operator tables, and
-// the parts of the pairwise near field: planes of one entry per charge (mixed
-// 416, FP64 864 bytes a charge; without room for them, or above 28 GB, every
-// leaf pair is summed one-sided).
-// Every sum runs in a fixed order: results are bitwise reproducible.
+// the parts of the near field: one entry per charge of the one-sided sums (16
+// bytes, FP64 32) and planes of one entry per charge of the pairwise ones (mixed
+// 416, FP64 864 bytes a charge; without room for them, or above
+// PETFMM3D_OPT_PAIR_BYTES, every leaf pair is summed one-sided).
+// Every sum runs in a fixed order: results are bitwise reproducible, as long as
+// the planes are had or not had alike.
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -2670,6 +2672,11 @@ void host_shift_real(int p, int kind, int octant, double *a) {
         host_real_matrix(p, [&](int n, const cd *in, cd *out) { host_l2l_one(p, n, ro.data(), in, out); }, a);
 }
 
+// Default of PETFMM3D_OPT_PAIR_BYTES, the most bytes for the planes of the
+// pairwise sums (67M charges of the mixed path, 32M of the FP64 path); above it,
+// or where that memory cannot be had, leaf pairs are summed one-sided.
+constexpr size_t kPairs3MaxBytes = (size_t(1) << 26) * P3_SLOTS * sizeof(float4);
+
 struct DevBuf3 {
     void *p = nullptr;
     size_t cap = 0;
@@ -2693,6 +2700,14 @@ int ensure3(DevBuf3 &b, size_t bytes, cudaStream_t st) {
     return PETFMM_OK;
 }
 
+int free3(DevBuf3 &b, cudaStream_t st) {
+    if (!b.p) return PETFMM_OK;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return PETFMM_ECUDA;
+    cudaFree(b.p);
+    b = DevBuf3();
+    return PETFMM_OK;
+}
+
 }  // namespace
 
 struct petfmm3d_ctx {
@@ -2702,7 +2717,8 @@ struct petfmm3d_ctx {
     DevBuf3 keysA, keysB, valsA, valsB, sortw, start, recu, rec, xs, me, le, status;
     // near field: one-sided and pair items, parts of the charges' sums, flags, counters
     DevBuf3 nitems, pitems, slots, nown, nflags, nctrl;
-    bool no_pairs = false;  // no room for the parts of pairwise sums
+    bool no_pairs = false;  // no room for the planes of pairwise sums
+    size_t pair_bytes = kPairs3MaxBytes;  // PETFMM3D_OPT_PAIR_BYTES
     // operator tables of the context's precision only
     DevBuf3 orbits, atab32, rmap, parity;  // M2L operators: by orbit, by offset
     DevBuf3 shift, order;  // the M2M and L2L operators of octant 0, rows by parity class
@@ -2717,11 +2733,6 @@ struct petfmm3d_ctx {
 };
 
 namespace {
-
-// Most bytes for the parts of pairwise sums (67M charges of the mixed path, 32M
-// of the FP64 path); above it, or where that memory cannot be had, leaf
-// pairs are summed one-sided.
-constexpr size_t kPairs3MaxBytes = (size_t(1) << 26) * P3_SLOTS * sizeof(float4);
 
 #define P3_TRY(x) do { int rc_ = (x); if (rc_) return rc_; } while (0)
 #define P3_CUDA(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) { cudaGetLastError(); \
@@ -2982,27 +2993,86 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
     return PETFMM_OK;
 }
 
-// The lists, flags and counters of the near field and, where they are allowed
-// and there is room, the slots of the pairwise sums (parts bytes a charge); else
-// nr->pmin stays all ones and every leaf pair is summed one-sided.
-int near_pairs3(petfmm3d_ctx *c, int64_t n, int64_t nleaf, uint32_t pmin, size_t parts, Near3 *nr,
-                int64_t *icap) {
+// One-sided work items of up to 32 targets: at most min(8^L, n) + n / 32.
+int64_t directed_cap3(int64_t n, int64_t nleaf) { return std::min(nleaf, n) + n / 32 + 1; }
+
+// The buffers that an evaluation of n charges cannot do without: those of the
+// tree and the expansions, those of the near field.
+int tree_buffers3(petfmm3d_ctx *c, int64_t n) {
     cudaStream_t st = c->stream;
-    nr->n = n;
-    nr->pmin = ~0u;
-    if (n >= 2 * int64_t(pmin) && n * parts <= kPairs3MaxBytes && !c->no_pairs) {
-        // up to 2 groups of a leaf of at least pmin, 4 above 96 charges, 14 above 384
-        *icap = 2 * std::min<int64_t>(nleaf, n / pmin) + 2 * (n / 97) + 10 * (n / 385) + 1;
-        int rc = ensure3(c->slots, n * parts, st);
-        if (rc == PETFMM_OK) rc = ensure3(c->pitems, size_t(*icap) * sizeof(uint2), st);
-        if (rc == PETFMM_OK) nr->pmin = pmin;
-        else if (rc == PETFMM_ENOMEM) c->no_pairs = true;  // one-sided sums need no slots
-        else return rc;
+    const bool mixed = c->precision == PETFMM_MIXED;
+    const int64_t nleaf = int64_t(1) << (3 * c->L), nbox = lvl_off3(c->L + 1);
+    const size_t series = size_t(nbox) * nc3(c->p) * (mixed ? sizeof(float2) : sizeof(double2));
+    P3_TRY(ensure3(c->keysA, size_t(n) * 4, st));
+    P3_TRY(ensure3(c->keysB, size_t(n) * 4, st));
+    P3_TRY(ensure3(c->valsA, size_t(n) * 4, st));
+    P3_TRY(ensure3(c->valsB, size_t(n) * 4, st));
+    P3_TRY(ensure3(c->sortw, size_t(radix_scratch_words(n)) * 4, st));
+    P3_TRY(ensure3(c->start, size_t(nleaf + 1) * 4, st));
+    P3_TRY(ensure3(c->me, series, st));
+    P3_TRY(ensure3(c->le, series, st));
+    if (mixed) {
+        P3_TRY(ensure3(c->recu, size_t(n) * sizeof(float4), st));
+        P3_TRY(ensure3(c->rec, size_t(n) * sizeof(float4), st));
+    } else {
+        P3_TRY(ensure3(c->xs, size_t(n) * sizeof(Dbl4), st));
     }
+    return PETFMM_OK;
+}
+int near_buffers3(petfmm3d_ctx *c, int64_t n) {
+    cudaStream_t st = c->stream;
+    const int64_t nleaf = int64_t(1) << (3 * c->L);
+    P3_TRY(ensure3(c->nown, size_t(n) * (c->precision == PETFMM_MIXED ? sizeof(float4) : sizeof(Dbl4)),
+                   st));
+    P3_TRY(ensure3(c->nitems, size_t(directed_cap3(n, nleaf)) * sizeof(uint2), st));
     P3_TRY(ensure3(c->nflags, size_t(nleaf) * 4, st));
     P3_TRY(ensure3(c->nctrl, C3_WORDS * 4, st));
+    return PETFMM_OK;
+}
+
+// Either of them; the planes of the pairwise sums give way where a needed buffer
+// cannot be had beside them.
+int needed3(petfmm3d_ctx *c, int64_t n, int (*buffers)(petfmm3d_ctx *, int64_t)) {
+    const int rc = buffers(c, n);
+    if (rc != PETFMM_ENOMEM || !c->slots.p) return rc;
+    P3_TRY(free3(c->slots, c->stream));
+    c->no_pairs = true;
+    return buffers(c, n);
+}
+
+// The near field's buffers: where they are allowed and there is room, the planes
+// and items of the pairwise sums too (*icap of them), else nr->pmin stays all
+// ones and every leaf pair is summed one-sided.
+int near3(petfmm3d_ctx *c, int64_t n, Near3 *nr, int64_t *icap) {
+    cudaStream_t st = c->stream;
+    const bool mixed = c->precision == PETFMM_MIXED;
+    const int64_t nleaf = int64_t(1) << (3 * c->L);
+    const uint32_t pmin = mixed ? P3_PAIR_MIN : 1;
+    const size_t parts = mixed ? P3_SLOTS * sizeof(float4) : P3_SLOTS64 * sizeof(Dbl4);
+    nr->n = n;
+    nr->pmin = ~0u;
+    nr->share = mixed ? P3_SHARE : P3_SHARE64;
+    P3_TRY(needed3(c, n, near_buffers3));
+    if (n >= 2 * int64_t(pmin) && n * parts <= c->pair_bytes && !c->no_pairs) {
+        // up to 2 groups of a leaf of at least pmin, 4 above 96 charges, 14 above 384
+        *icap = 2 * std::min<int64_t>(nleaf, n / pmin) + 2 * (n / 97) + 10 * (n / 385) + 1;
+        int rc = ensure3(c->pitems, size_t(*icap) * sizeof(uint2), st);
+        if (rc == PETFMM_OK) rc = ensure3(c->slots, n * parts, st);
+        if (rc == PETFMM_OK) {
+            nr->pmin = pmin;
+        } else if (rc == PETFMM_ENOMEM) {
+            P3_TRY(free3(c->slots, st));
+            P3_TRY(free3(c->pitems, st));
+            c->no_pairs = true;
+        } else {
+            return rc;
+        }
+    }
+    nr->own = static_cast<float4 *>(c->nown.p);
+    nr->slots = static_cast<float4 *>(c->slots.p);
     nr->flags = static_cast<uint32_t *>(c->nflags.p);
     nr->ctrl = static_cast<uint32_t *>(c->nctrl.p);
+    nr->directed = static_cast<uint2 *>(c->nitems.p);
     nr->items = static_cast<uint2 *>(c->pitems.p);
     P3_CUDA(cudaMemsetAsync(nr->ctrl, 0, C3_WORDS * 4, st));
     return PETFMM_OK;
@@ -3019,22 +3089,7 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
     c->ev_recorded = false;
     if (n == 0) return PETFMM_OK;
     const int64_t nleaf = int64_t(1) << (3 * L);
-    const int64_t nbox = lvl_off3(L + 1);
-    const size_t es = mixed ? sizeof(float2) : sizeof(double2);
-    P3_TRY(ensure3(c->keysA, size_t(n) * 4, st));
-    P3_TRY(ensure3(c->keysB, size_t(n) * 4, st));
-    P3_TRY(ensure3(c->valsA, size_t(n) * 4, st));
-    P3_TRY(ensure3(c->valsB, size_t(n) * 4, st));
-    P3_TRY(ensure3(c->sortw, size_t(radix_scratch_words(n)) * 4, st));
-    P3_TRY(ensure3(c->start, size_t(nleaf + 1) * 4, st));
-    P3_TRY(ensure3(c->me, size_t(nbox) * nc3(p) * es, st));
-    P3_TRY(ensure3(c->le, size_t(nbox) * nc3(p) * es, st));
-    if (mixed) {
-        P3_TRY(ensure3(c->recu, size_t(n) * sizeof(float4), st));
-        P3_TRY(ensure3(c->rec, size_t(n) * sizeof(float4), st));
-    } else {
-        P3_TRY(ensure3(c->xs, size_t(n) * sizeof(Dbl4), st));
-    }
+    P3_TRY(needed3(c, n, tree_buffers3));
     uint32_t *kA = static_cast<uint32_t *>(c->keysA.p), *kB = static_cast<uint32_t *>(c->keysB.p);
     uint32_t *vA = static_cast<uint32_t *>(c->valsA.p), *vB = static_cast<uint32_t *>(c->valsB.p);
     uint32_t *start = static_cast<uint32_t *>(c->start.p);
@@ -3093,22 +3148,14 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
     mark3(c, PETFMM3D_STAGE_NEAR);
     const double w = c->dom.width / double(int64_t(1) << L);
     const unsigned gb = unsigned((nleaf + 255) / 256);
-    // one-sided work items of up to 32 targets: at most min(8^L, n) + n / 32
-    const int64_t cap = std::min<int64_t>(nleaf, n) + n / 32 + 1;
-    const unsigned gi = grid_w(cap);
+    const unsigned gi = grid_w(directed_cap3(n, nleaf));
+    Near3 nr{};
+    int64_t icap = 0;
+    P3_TRY(near3(c, n, &nr, &icap));
+    const bool pairs = nr.pmin != ~0u;
     if (mixed) {
-        Near3 nr{};
-        int64_t icap = 0;
-        P3_TRY(near_pairs3(c, n, nleaf, P3_PAIR_MIN, P3_SLOTS * sizeof(float4), &nr, &icap));
-        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-        P3_TRY(ensure3(c->nown, size_t(n) * sizeof(float4), st));
-        nr.own = static_cast<float4 *>(c->nown.p);
-        nr.share = P3_SHARE;
-        nr.slots = static_cast<float4 *>(c->slots.p);
-        nr.directed = static_cast<uint2 *>(c->nitems.p);
         const float4 *rec = static_cast<const float4 *>(c->rec.p);
         const float2 *le = static_cast<const float2 *>(c->le.p);
-        const bool pairs = nr.pmin != ~0u;
         if (pairs) {
             k3_near_items<false, P3_DIRS><<<gb, 256, 0, st>>>(L, start, nr);
             P3_CUDA(cudaGetLastError());
@@ -3133,15 +3180,7 @@ int evaluate3(petfmm3d_ctx *c, int64_t n, const void *x, const void *y, const vo
     } else {
         const Dbl4 *xs = static_cast<const Dbl4 *>(c->xs.p);
         const double2 *le = static_cast<const double2 *>(c->le.p);
-        Near3 nr{};
-        int64_t icap = 0;
-        P3_TRY(near_pairs3(c, n, nleaf, 1, P3_SLOTS64 * sizeof(Dbl4), &nr, &icap));
-        P3_TRY(ensure3(c->nitems, size_t(cap) * sizeof(uint2), st));
-        P3_TRY(ensure3(c->nown, size_t(n) * sizeof(Dbl4), st));
-        nr.directed = static_cast<uint2 *>(c->nitems.p);
-        nr.share = P3_SHARE64;
         Dbl4 *slots = static_cast<Dbl4 *>(c->slots.p), *own = static_cast<Dbl4 *>(c->nown.p);
-        const bool pairs = nr.pmin != ~0u;
         if (pairs) {
             k3_near_items<false, P3_GROUPS64><<<gb, 256, 0, st>>>(L, start, nr);
             P3_CUDA(cudaGetLastError());
@@ -3242,6 +3281,12 @@ int petfmm3d_set_option(petfmm3d_ctx *c, int option, int64_t value) {
             if (value < 0 || value > 2) return PETFMM_EINVAL;
             c->m2l_tc = int(value);
             return PETFMM_OK;
+        case PETFMM3D_OPT_PAIR_BYTES:
+            if (value < 0) return PETFMM_EINVAL;
+            c->pair_bytes = size_t(value);
+            c->no_pairs = false;
+            // (planes above the new limit are given back)
+            return c->slots.cap > c->pair_bytes ? free3(c->slots, c->stream) : PETFMM_OK;
         default: return PETFMM_EINVAL;
     }
 }
