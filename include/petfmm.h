@@ -686,8 +686,8 @@ typedef struct {
  * translations, near field and L2P in FP32 on leaf-relative coordinates;
  * binning in FP64); dtype PETFMM_F64 or PETFMM_F32 storage of x, y, z, q and
  * of the outputs; cuda_stream: the cudaStream_t every launch goes to (NULL:
- * the legacy default stream).  Uploads the operator tables (synchronous).
- * Returns PETFMM_OK, PETFMM_EINVAL, PETFMM_ENOMEM or PETFMM_ECUDA. */
+ * the legacy default stream).  Uploads the operator tables (on
+ * that stream).  Returns PETFMM_OK, PETFMM_EINVAL, PETFMM_ENOMEM or PETFMM_ECUDA. */
 int petfmm3d_create(const petfmm_domain3d *dom, int levels, int order, int precision, int dtype,
                     void *cuda_stream, petfmm3d_ctx **out);
 /* One evaluation of n particles, asynchronous on the context's stream.

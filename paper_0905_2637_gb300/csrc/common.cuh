@@ -238,7 +238,7 @@ template <typename T2> __host__ __device__ __forceinline__ T2 cfma(T2 a, T2 b, T
 // Position of the M2L offset (dx, dy) among the 40 vectors of
 // [-3, 3]^2 \ [-1, 1]^2, taken row by row (increasing dy, then dx): the index
 // of its operator T_delta.
-__host__ __device__ __forceinline__ int m2l_op_index(int dx, int dy) {
+__host__ __device__ constexpr int m2l_op_index(int dx, int dy) {
     const int base = dy <= -1 ? 7 * (dy + 3) : (dy <= 2 ? 14 + 4 * (dy + 1) : 33);
     const int pos = (dy >= -1 && dy <= 1) ? (dx < 0 ? dx + 3 : dx) : dx + 3;
     return base + pos;

@@ -341,7 +341,7 @@ OpTables *get_tables(petfmm_ctx *c, int p, int kernel, int *err) {
     auto it = c->tables.find(key);
     if (it != c->tables.end()) return &it->second;
     OpTables t;
-    cudaError_t e = build_op_tables(p, kernel, &t);
+    cudaError_t e = build_op_tables(p, kernel, &t, c->stream);
     if (e != cudaSuccess) {
         free_op_tables(&t);
         *err = cuda_status(e);
@@ -377,8 +377,10 @@ int attach_sm_tables(petfmm_ctx *c, Plan &pl) {
             host_sm_operators(key.second, key.first, host);
             void *p = nullptr;
             cudaError_t e = cudaMalloc(&p, host.size() * sizeof(float));
+            // (on the context's stream: its launches wait for the copy)
             if (e == cudaSuccess)
-                e = cudaMemcpy(p, host.data(), host.size() * sizeof(float), cudaMemcpyHostToDevice);
+                e = cudaMemcpyAsync(p, host.data(), host.size() * sizeof(float),
+                                    cudaMemcpyHostToDevice, c->stream);
             if (e != cudaSuccess) {
                 cudaGetLastError();
                 if (p) cudaFree(p);
@@ -1226,7 +1228,8 @@ int petfmm_create(const petfmm_domain *dom, int levels, int order, double sigma,
         const size_t bytes = G64_WORDS * sizeof(double);
         rc = ensure(c->gtab, bytes, c->stream);
         if (rc == PETFMM_OK)
-            rc = cuda_status(cudaMemcpy(c->gtab.p, host_g64_table(), bytes, cudaMemcpyHostToDevice));
+            rc = cuda_status(cudaMemcpyAsync(c->gtab.p, host_g64_table(), bytes,
+                                             cudaMemcpyHostToDevice, c->stream));
         if (rc != PETFMM_OK) {
             cudaGetLastError();
             petfmm_destroy(c);

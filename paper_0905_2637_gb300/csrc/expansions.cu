@@ -36,43 +36,34 @@ namespace petfmm {
 // if cx = 1 (same for y), minus the 3x3 block around the target -- 27
 // offsets.  Each offset maps to one of the 40 vectors of [-3, 3]^2 \ [-1, 1]^2.
 // ----------------------------------------------------------------------------
-__constant__ IlEntry c_il[4][27];
-
-static int offset_op_index(int dx, int dy) { return m2l_op_index(dx, dy); }
-
-static void il_offsets(int c, IlEntry *out) {
-    const int cx = c & 1, cy = c >> 1;
-    const int x_lo = cx ? -3 : -2, y_lo = cy ? -3 : -2;
-    int n = 0;
-    for (int dy = y_lo; dy <= y_lo + 5; ++dy)
-        for (int dx = x_lo; dx <= x_lo + 5; ++dx) {
-            if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
-            out[n].dx = int8_t(dx);
-            out[n].dy = int8_t(dy);
-            out[n].op = int8_t(offset_op_index(dx, dy));
-            out[n].pad = 0;
-            ++n;
-        }
+struct IlTable {
+    IlEntry e[4][27];
+};
+constexpr IlTable il_table() {
+    IlTable t{};
+    for (int c = 0; c < 4; ++c) {
+        const int x_lo = (c & 1) ? -3 : -2, y_lo = (c >> 1) ? -3 : -2;
+        int n = 0;
+        for (int dy = y_lo; dy <= y_lo + 5; ++dy)
+            for (int dx = x_lo; dx <= x_lo + 5; ++dx) {
+                if (dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1) continue;
+                t.e[c][n].dx = int8_t(dx);
+                t.e[c][n].dy = int8_t(dy);
+                t.e[c][n].op = int8_t(m2l_op_index(dx, dy));
+                ++n;
+            }
+    }
+    return t;
 }
-
-static bool g_il_uploaded = false;
-
-static cudaError_t upload_il() {
-    if (g_il_uploaded) return cudaSuccess;
-    IlEntry h[4][27];
-    for (int c = 0; c < 4; ++c) il_offsets(c, h[c]);
-    cudaError_t e = cudaMemcpyToSymbol(c_il, h, sizeof(h));
-    if (e == cudaSuccess) g_il_uploaded = true;
-    return e;
-}
+static constexpr IlTable kIl = il_table();
+__constant__ IlTable c_il = il_table();
 
 int host_interaction_list(int level, int ix, int iy, int32_t *out) {
     if (level < 0 || level > MAX_L) return -1;
     const int nside = 1 << level;
     if (ix < 0 || iy < 0 || ix >= nside || iy >= nside) return -1;
     if (level < 2) return 0;
-    IlEntry e[27];
-    il_offsets((ix & 1) | ((iy & 1) << 1), e);
+    const IlEntry *e = kIl.e[(ix & 1) | ((iy & 1) << 1)];
     int n = 0;
     for (int i = 0; i < 27; ++i) {
         const int sx = ix + e[i].dx, sy = iy + e[i].dy;
@@ -271,9 +262,7 @@ void host_op_table(int p, int kernel, int which, std::vector<double> &out) {
     else (lap ? host_lap_m2l_table : host_m2l_table)(p, out.data());
 }
 
-cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
-    cudaError_t e = upload_il();
-    if (e != cudaSuccess) return e;
+cudaError_t build_op_tables(int p, int kernel, OpTables *t, cudaStream_t st) {
     t->p = p;
     std::vector<double> m2l(size_t(2) * 40 * p * p), shift, orbit;
     (kernel == KERNEL_LAPLACE ? host_lap_m2l_table : host_m2l_table)(p, m2l.data());
@@ -302,9 +291,11 @@ cudaError_t build_op_tables(int p, int kernel, OpTables *t) {
         host_m2l_tcb_images(p, kernel, img);
         put((void **)&t->m2l_tcb, img.data(), img.size() * 4);
     }
-    if ((e = cudaMalloc(&t->blob, blob.size())) != cudaSuccess) return e;
+    const cudaError_t e = cudaMalloc(&t->blob, blob.size());
+    if (e != cudaSuccess) return e;
     for (const auto &x : at) *x.first = static_cast<unsigned char *>(t->blob) + x.second;
-    return cudaMemcpy(t->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice);
+    // (the call returns once the pageable source is staged)
+    return cudaMemcpyAsync(t->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, st);
 }
 
 void free_op_tables(OpTables *t) {
@@ -743,7 +734,7 @@ __global__ void __launch_bounds__(M2L_WARPS * 32) k_m2l(const Task *__restrict__
         const C2 *lev = me + d.eoff + lvl_off(l) * p;
         C2 acc0 = mk2<R>(R(0), R(0)), acc1 = mk2<R>(R(0), R(0));
         for (int e = 0; e < 27; ++e) {
-            const IlEntry en = c_il[c][e];
+            const IlEntry en = c_il.e[c][e];
             const int sx = ix + en.dx, sy = iy + en.dy;
             if (sx < 0 || sy < 0 || sx >= nside || sy >= nside) continue;
             if (!box_count(st, d.L, l, morton_key(uint32_t(sx), uint32_t(sy)))) continue;
@@ -803,7 +794,7 @@ __global__ void __launch_bounds__(256) k_m2l_logterm(const Task *__restrict__ ta
     const C2 *lev = me + d.eoff + lvl_off(l) * p;
     R sr = R(0), si = R(0);
     for (int e = 0; e < 27; ++e) {
-        const IlEntry en = c_il[c][e];
+        const IlEntry en = c_il.e[c][e];
         const int sx = ix + en.dx, sy = iy + en.dy;
         if (sx < 0 || sy < 0 || sx >= nside || sy >= nside) continue;
         if (!box_count(st, d.L, l, morton_key(uint32_t(sx), uint32_t(sy)))) continue;

@@ -2700,6 +2700,16 @@ int ensure3(DevBuf3 &b, size_t bytes, cudaStream_t st) {
     return PETFMM_OK;
 }
 
+// A table, copied on the context's stream: the launches that follow there find it
+// complete (the call returns once the pageable source is staged).
+int upload3(DevBuf3 &b, const void *src, size_t bytes, cudaStream_t st) {
+    const int rc = ensure3(b, bytes, st);
+    if (rc) return rc;
+    if (cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess) return PETFMM_OK;
+    cudaGetLastError();
+    return PETFMM_ECUDA;
+}
+
 int free3(DevBuf3 &b, cudaStream_t st) {
     if (!b.p) return PETFMM_OK;
     if (cudaStreamSynchronize(st) != cudaSuccess) return PETFMM_ECUDA;
@@ -2766,10 +2776,8 @@ int upload_tables(petfmm3d_ctx *c) {
                 rm[size_t(r++)] = make_short2(short(j), 1);
             }
         }
-    P3_TRY(ensure3(c->rmap, rm.size() * sizeof(short2), c->stream));
-    P3_CUDA(cudaMemcpy(c->rmap.p, rm.data(), rm.size() * sizeof(short2), cudaMemcpyHostToDevice));
-    P3_TRY(ensure3(c->parity, par.size(), c->stream));
-    P3_CUDA(cudaMemcpy(c->parity.p, par.data(), par.size(), cudaMemcpyHostToDevice));
+    P3_TRY(upload3(c->rmap, rm.data(), rm.size() * sizeof(short2), c->stream));
+    P3_TRY(upload3(c->parity, par.data(), par.size(), c->stream));
     std::vector<double> a64(size_t(nr) * nr);
     // M2M [k_in][r_out], then L2L with the rows k_in by parity class
     c->sh = Shift3{p, nr, std::max(1, 256 / nr), {}};
@@ -2789,12 +2797,9 @@ int upload_tables(petfmm3d_ctx *c) {
     const std::vector<float> ops32(ops.begin(), ops.end());
     const bool f64 = c->precision == PETFMM_FP64;
     const size_t es = f64 ? sizeof(double) : sizeof(float);
-    P3_TRY(ensure3(c->shift, ops.size() * es, c->stream));
-    P3_TRY(ensure3(c->order, order.size() * sizeof(uint16_t), c->stream));
-    P3_CUDA(cudaMemcpy(c->shift.p, f64 ? static_cast<const void *>(ops.data()) : ops32.data(),
-                       ops.size() * es, cudaMemcpyHostToDevice));
-    P3_CUDA(cudaMemcpy(c->order.p, order.data(), order.size() * sizeof(uint16_t),
-                       cudaMemcpyHostToDevice));
+    P3_TRY(upload3(c->shift, f64 ? static_cast<const void *>(ops.data()) : ops32.data(),
+                   ops.size() * es, c->stream));
+    P3_TRY(upload3(c->order, order.data(), order.size() * sizeof(uint16_t), c->stream));
     std::vector<cd> iv(static_cast<size_t>(nci));
     // the orbits' operators [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
     std::vector<double> orb(size_t(64) * nr * nr, 0.0);
@@ -2806,9 +2811,8 @@ int upload_tables(petfmm3d_ctx *c) {
     }
     if (use_orbits3(c)) {
         const std::vector<float> orb32(orb.begin(), orb.end());
-        P3_TRY(ensure3(c->orbits, orb.size() * es, c->stream));
-        P3_CUDA(cudaMemcpy(c->orbits.p, f64 ? static_cast<const void *>(orb.data()) : orb32.data(),
-                           orb.size() * es, cudaMemcpyHostToDevice));
+        P3_TRY(upload3(c->orbits, f64 ? static_cast<const void *>(orb.data()) : orb32.data(),
+                       orb.size() * es, c->stream));
     }
     if (f64 || p > TC3_MAXP) return PETFMM_OK;
     // The mixed path's M2L matrices, FP32: ap[k_in * nrp + r_out]; for p <= 8
@@ -2853,10 +2857,8 @@ int upload_tables(petfmm3d_ctx *c) {
             }
         }
     }
-    P3_TRY(ensure3(c->tcimg, img.size() * sizeof(float), c->stream));
-    P3_CUDA(cudaMemcpy(c->tcimg.p, img.data(), img.size() * sizeof(float), cudaMemcpyHostToDevice));
-    P3_TRY(ensure3(c->atab32, at.size() * sizeof(float), c->stream));
-    P3_CUDA(cudaMemcpy(c->atab32.p, at.data(), at.size() * sizeof(float), cudaMemcpyHostToDevice));
+    P3_TRY(upload3(c->tcimg, img.data(), img.size() * sizeof(float), c->stream));
+    P3_TRY(upload3(c->atab32, at.data(), at.size() * sizeof(float), c->stream));
     return PETFMM_OK;
 }
 

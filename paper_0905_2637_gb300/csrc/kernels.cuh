@@ -69,7 +69,8 @@ struct OpTables {
     float *m2l_tc = nullptr;  // hi/lo B images for the tensor-core M2L (p <= 24)
     float *m2l_tcb = nullptr; // ... the four target classes side by side (block units)
 };
-cudaError_t build_op_tables(int p, int kernel, OpTables *out);
+// Copied on st: the launches that follow there find them complete.
+cudaError_t build_op_tables(int p, int kernel, OpTables *out, cudaStream_t st);
 // The FP64 table behind them: which = 0 M2M [c][l][k], 1 L2L [c][n][m],
 // 2 M2L [op][k][m], complex as (re, im) pairs.
 void host_op_table(int p, int kernel, int which, std::vector<double> &out);
