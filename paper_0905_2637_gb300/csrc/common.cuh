@@ -79,6 +79,7 @@ struct InstDesc {
     int general;            // 1: some near pairs exceed the polynomial range
     float poly[POLY_MAX + 1];
     uint32_t pair_min;      // pairwise near field: leaf pairs of at least this many blobs each
+    int direct;             // 1: near field by one thread per target (k_near_direct), else items
     int smdeg;              // > 0: near field by expansions of this degree (smooth.cu) ...
     const void *t_sm;       // ... and their operators
     // FP64 constants

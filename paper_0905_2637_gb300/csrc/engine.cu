@@ -95,8 +95,8 @@ struct Plan {
     uint32_t sm_degrees = 0;
     int sm_row = 0;
     int64_t sm_rows = 0;
-    // the others: pairs_any sums pairs of leaves pairwise (pair kernel),
-    // direct sums by one thread per target, else by work items
+    // the others: pairs_any sums pairs of leaves pairwise (pair kernel), direct
+    // by one thread per target (some instance), items_any by work items (some)
     bool pairs_any = false, direct = false, items_any = false;
 };
 
@@ -447,7 +447,7 @@ int64_t dump_tile_units(int l) {
 int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
 
 // Laplace kernel, mixed path: blobs per leaf (empty ones included) up to which
-// one thread per target sums its near field; denser trees take work items of
+// one thread per target sums a tree's near field; denser trees take work items of
 // 64 targets, two per lane, which share each source load.
 constexpr int64_t kLaplaceDirectMax = 64;
 
@@ -501,18 +501,16 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
             pl.sm_row = std::max(pl.sm_row, int(sm_row_floats(d.smdeg)));
             pl.sm_rows += sm_max_rows(d.smdeg, pb.n, nleaf);
         }
+        // (each instance by its own numbers: its bits are those it gets alone)
+        if (precision == PETFMM_MIXED && near != 0 && !d.smdeg)
+            d.direct = kernel == KERNEL_VORTEX || pb.n <= kLaplaceDirectMax * nleaf;
+        if (pb.n > 0 && !d.smdeg) (d.direct ? pl.direct : pl.items_any) = true;
         pl.inst.push_back(d);
         poff += pb.n;
         loff += nleaf;
         eoff += lvl_off(pb.L + 1) * pb.p;
     }
-    bool others = false;  // instances without expansions of the near field
-    for (const InstDesc &d : pl.inst) others |= d.smdeg == 0;
-    if (precision == PETFMM_MIXED && near != 0 && others) {
-        pl.direct = kernel == KERNEL_VORTEX || poff <= kLaplaceDirectMax * loff;
-        pl.pairs_any = kernel == KERNEL_VORTEX && near == 1;
-    }
-    pl.items_any = others && !pl.direct;
+    pl.pairs_any = pl.direct && kernel == KERNEL_VORTEX && near == 1;
     pl.N = poff;
     pl.nleaves = loff;
     pl.nstart = loff + ni;
@@ -1073,7 +1071,7 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
             PF_CUDA(launch_near_direct(dtask + pl.particles.first, pl.particles.count,
                                        pl.particles.nblocks, dinst, start, skeys, srec, pb.own,
                                        ctrl, dbusy, c->direct_sms, st, lc));
-        else if (pl.items_any)
+        if (pl.items_any)
             PF_CUDA(launch_p2p_mixed(grid, pl.deg, pl.general,
                                      static_cast<const uint4 *>(c->items.p), ctrl, dinst, start,
                                      srec, pb.own, lap ? 1 : 0, busy, st, lc));

@@ -134,7 +134,7 @@ __device__ __forceinline__ unsigned long long leaf_items(const InstDesc &d, cons
                                                          uint32_t m, uint32_t inst, uint32_t tpi,
                                                          int ordered, F &&emit) {
     const uint32_t s0 = st[m], n = st[m + 1] - s0;
-    if (!n) return 0;
+    if (!n || d.direct) return 0;
     const int nside = 1 << d.L;
     const int ix = int(compact_bits(m)), iy = int(compact_bits(m >> 1));
     uint32_t src = 0;  // the blobs of the leaf and its neighbours
@@ -1391,7 +1391,7 @@ __global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
                       threadIdx.x;
     const InstDesc &d = insts[t.inst];
     unsigned long long pairs = 0;
-    if (j < t.count && !d.smdeg) {
+    if (j < t.count && d.direct) {
         const int64_t r = d.poff + j;
         const uint32_t *st = start + d.soff;
         const uint32_t m = skeys[r] & ((1u << (2 * d.L)) - 1u);

@@ -46,3 +46,25 @@ def test_busy_times_of_the_direct_kernel():
     keep[0].close()
     assert 0.0 < st["p2p_load_balance"] <= 1.0
     assert all(np.array_equal(a, b) for a, b in zip(timed, G.run(w, "mixed")))
+
+
+# The Laplace near field goes by work items in dense trees and by one thread per
+# target in the others: a tree's form, and so its bits, are its own whatever
+# the rest of its batch.
+def test_laplace_batch_of_dense_and_sparse_trees_equals_alone():
+    _lib, torch = G.lib(), G.torch_cuda()
+    ws = [W.tiny(n, 20 + i, L=L, p=8, dtype="f32")
+          for i, (n, L) in enumerate([(2000, 2), (4000, 6), (0, 3), (3000, 2), (900, 5), (1, 1)])]
+    ctx = _lib.Context((0, 0, 1), 2, 8, 0.01, precision="mixed", dtype="f32", kernel="laplace")
+    insts, outs = [], []
+    for w in ws:
+        x, y, g = G.to_dev((w.x, w.y, w.gamma))
+        outs.append((torch.empty_like(x), torch.empty_like(x)))
+        insts.append(dict(domain=w.domain, levels=w.L, order=w.p, sigma=w.sigma, x=x, y=y, gamma=g,
+                          u=outs[-1][0], v=outs[-1][1]))
+    ctx.evaluate_batch(insts)
+    assert ctx.sync() == 0
+    ctx.close()
+    for w, (u, v) in zip(ws, outs):
+        if w.n:
+            assert np.array_equal(u.cpu().numpy().astype(np.float64), run_laplace(w, precision="mixed")[0])
