@@ -286,7 +286,11 @@ void fill_p2p_constants(InstDesc &d, double tol) {
     d.kappa = float(kappa);
     d.cnear = float(w / (4.0 * M_PI * d.sigma * d.sigma));
     d.cfar = float(1.0 / (2.0 * M_PI * w));
-    d.inv2s2 = 1.0 / (2.0 * d.sigma * d.sigma);
+    // Held where q = r^2 / 2 sigma^2 and its products stay finite: a narrower core
+    // gives every pair farther apart than 1e-133 leaf widths the same factor,
+    // the point vortex's.
+    d.inv2s2 = std::min({1.0 / (2.0 * d.sigma * d.sigma), std::ldexp(1.0, 900) / (w * w),
+                         std::ldexp(1.0, 1000)});
     d.cnear64 = 1.0 / (2.0 * M_PI);
     d.cfar64 = 1.0 / (2.0 * M_PI * w);
     // (1 - e^-q) / q loses about 2^-22.5 / q to the subtraction: the direct sums

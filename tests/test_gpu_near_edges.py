@@ -68,3 +68,18 @@ def test_laplace_batch_of_dense_and_sparse_trees_equals_alone():
     for w, (u, v) in zip(ws, outs):
         if w.n:
             assert np.array_equal(u.cpu().numpy().astype(np.float64), run_laplace(w, precision="mixed")[0])
+
+
+# Cores down to 1e-300: point vortices to every bit of the FP64 path, whatever
+# 1 / 2 sigma^2 overflows to.  The oracle's FMM in the unit square, at a core far
+# below every distance (the tree scales with a power of two exactly).
+@pytest.mark.parametrize("sigma,width", [(1e-100, 1.0), (1e-150, 1.0), (1e-160, 1.0), (1e-300, 1.0),
+                                         (1e-160, 2.0 ** 133), (1e-200, 2.0 ** -133),
+                                         (1e-260, 2.0 ** -133)])
+def test_fp64_point_vortices(orc, sigma, width):
+    w = W.tiny(1500, 8, L=3, p=12, clustered_frac=0.2)
+    w.x[:3], w.y[:3] = w.x[3], w.y[3]  # coincident: nothing from one another
+    ur, vr = orc.fmm(w.x, w.y, w.gamma, w.domain, w.L, w.p, 1e-9)
+    w = W.Workload("points", w.x * width, w.y * width, w.gamma, sigma, (0.0, 0.0, width), 3, 12, "f64")
+    u, v = G.run(w, "fp64")
+    assert G.rel_l2(u * width, v * width, ur, vr) <= 1e-12
