@@ -238,8 +238,9 @@ bool solve_dense(std::vector<double> &A, std::vector<double> &b, int n) {
     return true;
 }
 
-// Fits on q in [0, Q]; returns degree (0 on failure) and coefficients in rho^2.
-int fit_near_poly(double Q, double kappa, double tol, float *coef) {
+// Fits on q in [0, Q]; returns degree (0 on failure) and coefficients in rho^2
+// and in t = log2 e^-q (which stay of order one however narrow the core).
+int fit_near_poly(double Q, double kappa, double tol, float *coef, float *coeft) {
     for (int d = 4; d <= 12; ++d) {
         const int n = d + 1;
         std::vector<double> A(size_t(n) * n), b(n);
@@ -253,28 +254,32 @@ int fit_near_poly(double Q, double kappa, double tol, float *coef) {
             b[j] = g_exact(t * Q);
         }
         if (!solve_dense(A, b, n)) continue;
-        // coefficients in rho^2: a_k = b_k (kappa / Q)^k
-        double a[16];
-        const double r = kappa / Q;
-        double rp = 1.0;
-        for (int k = 0; k < n; ++k) {
-            a[k] = b[k] * rp;
-            rp *= r;
-        }
         double err = 0.0;
-        const double smax = Q / kappa;
         for (int i = 0; i <= 4000; ++i) {
-            const double s = smax * i / 4000.0;
-            double v = a[d];
-            for (int k = d - 1; k >= 0; --k) v = v * s + a[k];
-            err = std::max(err, std::fabs(v - g_exact(kappa * s)) / g_exact(kappa * s));
+            const double s = i / 4000.0;
+            double v = b[d];
+            for (int k = d - 1; k >= 0; --k) v = v * s + b[k];
+            err = std::max(err, std::fabs(v - g_exact(Q * s)) / g_exact(Q * s));
         }
         if (err < tol) {
-            for (int k = 0; k <= POLY_MAX; ++k) coef[k] = k <= d ? float(a[k]) : 0.0f;
+            double r = 1.0, t = 1.0;  // (kappa / Q)^k, (-ln 2 / Q)^k
+            for (int k = 0; k <= POLY_MAX; ++k) {
+                coef[k] = k <= d ? float(b[k] * r) : 0.0f;
+                coeft[k] = k <= d ? float(b[k] * t) : 0.0f;
+                r *= kappa / Q;
+                t *= -M_LN2 / Q;
+            }
             return d;
         }
     }
     return 0;
+}
+
+// w^2 / 2 sigma^2, held where the FP32 kernels' products stay finite: a narrower
+// core gives every pair farther apart than 1e-13 leaf widths the same factor,
+// the point vortex's.
+double near_kappa(double w, double sigma) {
+    return std::min(w * w / (2.0 * sigma * sigma), std::ldexp(1.0, 90));
 }
 
 // Largest q the polynomial alone may cover.
@@ -282,9 +287,9 @@ constexpr double kPolyQMax = 2.0;
 
 void fill_p2p_constants(InstDesc &d, double tol) {
     const double w = d.wleaf;
-    const double kappa = w * w / (2.0 * d.sigma * d.sigma);
+    const double kappa = near_kappa(w, d.sigma);
     d.kappa = float(kappa);
-    d.cnear = float(w / (4.0 * M_PI * d.sigma * d.sigma));
+    d.cnear = float(kappa / (2.0 * M_PI * w));  // w / (4 pi sigma^2)
     d.cfar = float(1.0 / (2.0 * M_PI * w));
     // Held where q = r^2 / 2 sigma^2 and its products stay finite: a narrower core
     // gives every pair farther apart than 1e-133 leaf widths the same factor,
@@ -302,7 +307,7 @@ void fill_p2p_constants(InstDesc &d, double tol) {
     struct Fit {
         int general, deg;
         float split;
-        float poly[POLY_MAX + 1];
+        float poly[POLY_MAX + 1], polyt[POLY_MAX + 1];
     };
     static std::mutex mu;
     static std::map<std::pair<double, double>, Fit> cache;
@@ -315,6 +320,7 @@ void fill_p2p_constants(InstDesc &d, double tol) {
             d.deg = it->second.deg;
             d.qsplit_rho2 = it->second.split;
             std::memcpy(d.poly, it->second.poly, sizeof(d.poly));
+            std::memcpy(d.polyt, it->second.polyt, sizeof(d.polyt));
             return;
         }
     }
@@ -323,11 +329,11 @@ void fill_p2p_constants(InstDesc &d, double tol) {
     const double qmax = kappa * rho2max;
     if (qmax <= kPolyQMax) {
         d.general = 0;
-        d.deg = fit_near_poly(qmax, kappa, tol, d.poly);
+        d.deg = fit_near_poly(qmax, kappa, tol, d.poly, d.polyt);
         d.qsplit_rho2 = float(rho2max);
     } else {
         d.general = 1;
-        d.deg = fit_near_poly(1.0, kappa, tol, d.poly);
+        d.deg = fit_near_poly(1.0, kappa, tol, d.poly, d.polyt);
         d.qsplit_rho2 = float(1.0 / kappa);
     }
     Fit f;
@@ -335,6 +341,7 @@ void fill_p2p_constants(InstDesc &d, double tol) {
     f.deg = d.deg;
     f.split = d.qsplit_rho2;
     std::memcpy(f.poly, d.poly, sizeof(f.poly));
+    std::memcpy(f.polyt, d.polyt, sizeof(f.polyt));
     std::lock_guard<std::mutex> lk(mu);
     if (cache.size() > 4096) cache.clear();
     cache[key] = f;
@@ -360,7 +367,7 @@ OpTables *get_tables(petfmm_ctx *c, int p, int kernel, int *err) {
 // stream is done with them) before the next evaluation's are made.
 constexpr size_t kMaxSmTables = 64;
 
-double sm_kappa(const InstDesc &d) { return d.wleaf * d.wleaf / (2.0 * d.sigma * d.sigma); }
+double sm_kappa(const InstDesc &d) { return near_kappa(d.wleaf, d.sigma); }
 
 int attach_sm_tables(petfmm_ctx *c, Plan &pl) {
     if (!pl.sm_degrees) return PETFMM_OK;
@@ -499,15 +506,20 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
         const int64_t nleaf = int64_t(1) << (2 * pb.L);
         if (near == 2 && precision == PETFMM_MIXED && kernel == KERNEL_VORTEX)
             d.smdeg = sm_degree(sm_kappa(d), near_tol);
-        d.pair_min = kernel == KERNEL_VORTEX && near == 1 ? P2P_PAIR_MIN : ~0u;
+        // the polynomial in rho^2 of the items and pairs leaves FP32's range in very
+        // narrow cores (kappa above some 1e8): summed by one thread per target
+        bool ranged = true;
+        for (float a : d.poly) ranged = ranged && std::isfinite(a);
+        d.pair_min = kernel == KERNEL_VORTEX && near == 1 && ranged ? P2P_PAIR_MIN : ~0u;
         if (d.smdeg) {
             pl.sm_degrees |= 1u << d.smdeg;
             pl.sm_row = std::max(pl.sm_row, int(sm_row_floats(d.smdeg)));
             pl.sm_rows += sm_max_rows(d.smdeg, pb.n, nleaf);
         }
         // (each instance by its own numbers: its bits are those it gets alone)
-        if (precision == PETFMM_MIXED && near != 0 && !d.smdeg)
-            d.direct = kernel == KERNEL_VORTEX || pb.n <= kLaplaceDirectMax * nleaf;
+        if (precision == PETFMM_MIXED && !d.smdeg)
+            d.direct = kernel == KERNEL_VORTEX ? near != 0 || !ranged
+                                               : near != 0 && pb.n <= kLaplaceDirectMax * nleaf;
         if (pb.n > 0 && !d.smdeg) (d.direct ? pl.direct : pl.items_any) = true;
         pl.inst.push_back(d);
         poff += pb.n;

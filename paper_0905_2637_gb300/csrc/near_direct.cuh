@@ -29,12 +29,12 @@ __device__ __forceinline__ float lg2_full(float x) {  // subnormal x too
     return y;
 }
 
-// kappa g(kappa rho^2) by the polynomial fitted on the host
+// kappa g(q) by the polynomial fitted on the host, in t = log2 e^-q
 template <int DEG>
-__device__ __forceinline__ float near_poly(const float (&a)[DEG + 1], float r2, float kappa) {
+__device__ __forceinline__ float near_poly(const float (&a)[DEG + 1], float t, float kappa) {
     float g = a[DEG];
 #pragma unroll
-    for (int k = DEG - 1; k >= 0; --k) g = fmaf(g, r2, a[k]);
+    for (int k = DEG - 1; k >= 0; --k) g = fmaf(g, t, a[k]);
     return kappa * g;
 }
 
@@ -47,23 +47,24 @@ template <int DEG, bool GENERAL>
 __device__ __forceinline__ void near_four(const float4 (&r)[4], float xt, float yt,
                                           const float (&a)[DEG + 1], float kappa, float split,
                                           float ek, float &u, float &v) {
-    float dx[4], dy[4], r2[4], f[4];
+    float dx[4], dy[4], r2[4], t[4], f[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         dx[i] = xt - r[i].x;
         dy[i] = yt - r[i].y;
         r2[i] = fmaf(dx[i], dx[i], dy[i] * dy[i]);
+        t[i] = ek * r2[i];
         if (GENERAL) {
             f[i] = r[i].z * rcp_ftz(r2[i]);
-            f[i] = fmaf(-ex2_ftz(ek * r2[i]), f[i], f[i]);
+            f[i] = fmaf(-ex2_ftz(t[i]), f[i], f[i]);
         } else {
-            f[i] = r[i].z * near_poly<DEG>(a, r2[i], kappa);
+            f[i] = r[i].z * near_poly<DEG>(a, t[i], kappa);
         }
     }
     if (GENERAL && fminf(fminf(r2[0], r2[1]), fminf(r2[2], r2[3])) < split) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (r2[i] < split) f[i] = r[i].z * near_poly<DEG>(a, r2[i], kappa);
+            if (r2[i] < split) f[i] = r[i].z * near_poly<DEG>(a, t[i], kappa);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -147,7 +148,7 @@ __device__ __forceinline__ float2 near_vortex(const NearLeaves &q, const float4 
     const InstDesc &d = *q.d;
     float a[DEG + 1];
 #pragma unroll
-    for (int k = 0; k <= DEG; ++k) a[k] = d.poly[k];
+    for (int k = 0; k <= DEG; ++k) a[k] = d.polyt[k];
     const float kappa = d.kappa, split = d.direct_rho2;
     const float ek = -1.44269504f * kappa;  // e^-q = 2^(ek rho^2)
     float u = 0.f, v = 0.f, pu = 0.f, pv = 0.f;

@@ -83,3 +83,16 @@ def test_fp64_point_vortices(orc, sigma, width):
     w = W.Workload("points", w.x * width, w.y * width, w.gamma, sigma, (0.0, 0.0, width), 3, 12, "f64")
     u, v = G.run(w, "fp64")
     assert G.rel_l2(u * width, v * width, ur, vr) <= 1e-12
+
+
+# Cores far narrower than a leaf, down to points, in every form of the mixed
+# near field: the polynomial's coefficients in rho^2 grow as kappa^5 and leave
+# FP32's range, those in q do not.  Bar: the mixed path's 1e-5.
+@pytest.mark.parametrize("form", [0, 1, 2])
+@pytest.mark.parametrize("sigma", [1e-3, 3e-5, 1e-5, 1e-6, 1e-9, 1e-13, 1e-20, 1e-100, 1e-300])
+def test_mixed_narrow_cores(orc, sigma, form):
+    w = W.tiny(3000, 8, L=3, p=12, clustered_frac=0.2, sigma=sigma)
+    w.x[:3], w.y[:3] = w.x[3], w.y[3]  # coincident: nothing from one another
+    u, v = G.run(w, "mixed", options={G.lib().PETFMM_OPT_P2P_PAIRS: form})
+    ur, vr = orc.fmm(w.x, w.y, w.gamma, w.domain, w.L, w.p, max(sigma, 1e-9))
+    assert np.all(np.isfinite(u)) and G.rel_l2(u, v, ur, vr) <= 1e-5
