@@ -78,7 +78,7 @@ struct InstDesc {
     int deg;                // polynomial degree (in rho^2) of g(q) = (1 - e^-q) / q
     int general;            // 1: some near pairs exceed the polynomial range
     float poly[POLY_MAX + 1];   // in rho^2
-    float polyt[POLY_MAX + 1];  // the same polynomial in log2 e^-q
+    float polyt[POLY_MAX + 1];  // one thread per target: kappa g in log2 e^-q
     uint32_t pair_min;      // pairwise near field: leaf pairs of at least this many blobs each
     int direct;             // 1: near field by one thread per target (k_near_direct), else items
     int smdeg;              // > 0: near field by expansions of this degree (smooth.cu) ...

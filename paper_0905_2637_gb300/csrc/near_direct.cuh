@@ -31,22 +31,21 @@ __device__ __forceinline__ float lg2_full(float x) {  // subnormal x too
 
 // kappa g(q) by the polynomial fitted on the host, in t = log2 e^-q
 template <int DEG>
-__device__ __forceinline__ float near_poly(const float (&a)[DEG + 1], float t, float kappa) {
+__device__ __forceinline__ float near_poly(const float (&a)[DEG + 1], float t) {
     float g = a[DEG];
 #pragma unroll
     for (int k = DEG - 1; k >= 0; --k) g = fmaf(g, t, a[k]);
-    return kappa * g;
+    return g;
 }
 
 // Four sources' factors gamma kappa g: GENERAL, most pairs of a narrow core lie
 // beyond the polynomial and take (1 - e^-q) / rho^2, two special-function
-// operations; the polynomial only where q is so small that the subtraction
-// would lose the fit's tolerance (InstDesc::direct_rho2), behind one test for
-// the four.
+// operations; below q = kDirectQ the subtraction loses more than the polynomial
+// does, which takes over behind one test for the four.
 template <int DEG, bool GENERAL>
 __device__ __forceinline__ void near_four(const float4 (&r)[4], float xt, float yt,
-                                          const float (&a)[DEG + 1], float kappa, float split,
-                                          float ek, float &u, float &v) {
+                                          const float (&a)[DEG + 1], float split, float ek,
+                                          float &u, float &v) {
     float dx[4], dy[4], r2[4], t[4], f[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -58,13 +57,13 @@ __device__ __forceinline__ void near_four(const float4 (&r)[4], float xt, float 
             f[i] = r[i].z * rcp_ftz(r2[i]);
             f[i] = fmaf(-ex2_ftz(t[i]), f[i], f[i]);
         } else {
-            f[i] = r[i].z * near_poly<DEG>(a, t[i], kappa);
+            f[i] = r[i].z * near_poly<DEG>(a, t[i]);
         }
     }
     if (GENERAL && fminf(fminf(r2[0], r2[1]), fminf(r2[2], r2[3])) < split) {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-            if (r2[i] < split) f[i] = r[i].z * near_poly<DEG>(a, t[i], kappa);
+            if (r2[i] < split) f[i] = r[i].z * near_poly<DEG>(a, t[i]);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -149,13 +148,13 @@ __device__ __forceinline__ float2 near_vortex(const NearLeaves &q, const float4 
     float a[DEG + 1];
 #pragma unroll
     for (int k = 0; k <= DEG; ++k) a[k] = d.polyt[k];
-    const float kappa = d.kappa, split = d.direct_rho2;
-    const float ek = -1.44269504f * kappa;  // e^-q = 2^(ek rho^2)
+    const float split = d.direct_rho2;
+    const float ek = -1.44269504f * d.kappa;  // e^-q = 2^(ek rho^2)
     float u = 0.f, v = 0.f, pu = 0.f, pv = 0.f;
     total = near_sources(
         q, rec, x, y,
         [&](const float4(&r)[4], float xt, float yt) {
-            near_four<DEG, GENERAL>(r, xt, yt, a, kappa, split, ek, pu, pv);
+            near_four<DEG, GENERAL>(r, xt, yt, a, split, ek, pu, pv);
         },
         [&] {
             u += pu;
@@ -168,8 +167,9 @@ __device__ __forceinline__ float2 near_vortex(const NearLeaves &q, const float4 
 // ... by the instance's degree and range
 __device__ __forceinline__ float2 near_vortex_of(const NearLeaves &q, const float4 *__restrict__ rec,
                                                  float x, float y, uint32_t &total) {
+    // (5: the degree of the default tolerance)
     if (q.d->general)
-        return q.d->deg <= 6 ? near_vortex<6, true>(q, rec, x, y, total)
+        return q.d->deg <= 5 ? near_vortex<5, true>(q, rec, x, y, total)
                              : near_vortex<12, true>(q, rec, x, y, total);
     return q.d->deg <= 6 ? near_vortex<6, false>(q, rec, x, y, total)
                          : near_vortex<12, false>(q, rec, x, y, total);

@@ -96,3 +96,33 @@ def test_mixed_narrow_cores(orc, sigma, form):
     u, v = G.run(w, "mixed", options={G.lib().PETFMM_OPT_P2P_PAIRS: form})
     ur, vr = orc.fmm(w.x, w.y, w.gamma, w.domain, w.L, w.p, max(sigma, 1e-9))
     assert np.all(np.isfinite(u)) and G.rel_l2(u, v, ur, vr) <= 1e-5
+
+
+# The pair factor alone, trees of two blobs, q = r^2 / 2 sigma^2 over the line
+# between its two forms.  FP32's bound per bin of q: the polynomial's 11e-8 rms or
+# the exponential form's 7e-8, and some six roundings of 3.4e-8 rms: 14e-8.
+@pytest.mark.parametrize("kappa", [3.5, 27.0])
+def test_pair_factor_keeps_fp32_accuracy(kappa):
+    _lib, torch = G.lib(), G.torch_cuda()
+    rng = np.random.default_rng(2)
+    edges = np.array([0.02, 0.05, 0.07, 0.1, 0.15, 0.2, 0.3, 0.4, 0.5, 0.6, 0.7, 0.8, 1.0, 1.5])
+    per = 160
+    q = np.concatenate([rng.uniform(a, b, per) for a, b in zip(edges, edges[1:])])
+    sigma = float(0.5 / np.sqrt(2 * kappa))  # leaves of 1/2
+    r, th = sigma * np.sqrt(2 * q), rng.uniform(0, 2 * np.pi, q.size)
+    ax, ay = rng.uniform(0.45, 0.55, (2, q.size))
+    x = np.stack([ax, ax + r * np.cos(th)], 1).astype(np.float32)
+    y = np.stack([ay, ay + r * np.sin(th)], 1).astype(np.float32)
+    dx, dy, g = *G.to_dev((x, y)), torch.ones(q.size, 2, device="cuda")
+    u, v = torch.empty_like(dx), torch.empty_like(dx)
+    ctx = _lib.Context((0, 0, 1), 1, 4, 0.01, precision="mixed", dtype="f32")
+    ctx.evaluate_batch([dict(domain=(0.0, 0.0, 1.0), levels=1, order=4, sigma=sigma, x=dx[i], y=dy[i],
+                             gamma=g[i], u=u[i], v=v[i]) for i in range(q.size)])
+    assert ctx.sync() == 0
+    ctx.close()
+    ex, ey = (a[:, 0].astype(np.float64) - a[:, 1] for a in (x, y))
+    r2 = ex ** 2 + ey ** 2
+    f = -np.expm1(-r2 / (2 * sigma ** 2)) / (2 * np.pi * r2)
+    err = np.hypot(u[:, 0].cpu().numpy() + f * ey, v[:, 0].cpu().numpy() - f * ex) / (f * np.sqrt(r2))
+    rms = np.sqrt((err.reshape(-1, per) ** 2).mean(1))
+    assert np.all(rms <= 2e-7), dict(zip(edges.round(2), rms))
