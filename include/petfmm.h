@@ -417,6 +417,10 @@ int petfmm_debug_near_fit(double sigma, double wleaf, double tol, double *out);
  * PETFMM_EINVAL (out too short: cap < 9 M S).  out may be NULL with cap 0 to
  * ask for the degree. */
 int petfmm_debug_smooth_operators(double kappa, float *out, int64_t cap);
+/* The same of instance inst of the last evaluation, as made on the device (host
+ * copy; waits for the stream).  Returns the degree, 0 if the evaluation had no
+ * need of them, PETFMM_EINVAL or PETFMM_ECUDA. */
+int petfmm_debug_smooth_table(petfmm_ctx *ctx, int inst, float *out, int64_t cap);
 
 /* The FP64 translation operators of Sec. 2.2 for order p (1..40) and kernel,
  * in the rescaled coefficients (box width r: ME a~_k = a_k / r^k; LE

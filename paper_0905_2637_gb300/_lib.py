@@ -149,6 +149,7 @@ def load():
             "petfmm_debug_op_table": (I, [I, I, I, P, ctypes.c_int64]),
             "petfmm_debug_near_fit": (I, [ctypes.c_double, ctypes.c_double, ctypes.c_double, P]),
             "petfmm_debug_smooth_operators": (I, [ctypes.c_double, P, ctypes.c_int64]),
+            "petfmm_debug_smooth_table": (I, [P, I, P, ctypes.c_int64]),
             "petfmm_debug_plan": (I, [I, I, ctypes.POINTER(Instance), P, I]),
             "petfmm_set_option": (I, [P, I, I64]),
             "petfmm_stage_times": (I, [P, P, I]),
@@ -409,6 +410,19 @@ class Context:
         st = Stats()
         _ck(load().petfmm_get_stats(self.handle, ctypes.byref(st)), "petfmm_get_stats")
         return {f: getattr(st, f) for f, _ in Stats._fields_}
+
+    def debug_smooth_table(self, inst=0):
+        """(degree, operators as petfmm_debug_smooth_operators gives them) of an
+        instance of the last evaluation, from the device; (0, None) without."""
+        lib = load()
+        n = _ck(lib.petfmm_debug_smooth_table(self.handle, inst, None, 0), "petfmm_debug_smooth_table")
+        if n == 0:
+            return 0, None
+        m = (n + 1) * (n + 2) // 2
+        out = np.zeros((9, m, (m + 3) // 4 * 4), np.float32)
+        _ck(lib.petfmm_debug_smooth_table(self.handle, inst, out.ctypes.data, out.size),
+            "petfmm_debug_smooth_table")
+        return n, out[:, :, :m]
 
     def debug_tree(self, n):
         keys = np.zeros(n, np.uint32)

@@ -141,14 +141,19 @@ struct petfmm_ctx {
     double near_tol = kNearTolDefault;
     int64_t spin_limit = 0;
     uint64_t launches = 0, evaluations = 0;
+    bool ctrl_zeroed = false;  // the status word starts at zero
 
     DevBuf keysA, keysB, valsA, valsB, hist, start, xs, ys, gs, rec, me, le,
         items, ctrl, plan_dev, busy, ucount, recu, occ, own,
         part, pitems, pxtra, pxs, ustage, smleaf, smlist, smmom, smloc, gtab;
     DevBuf hx, hy, hg, hu, hv;  // device staging for petfmm_evaluate_host
     std::map<int, OpTables> tables;
-    // operators of the near-field expansions by (degree, kappa), see get_sm_table
-    std::map<std::pair<int, double>, void *> sm_tables;
+    // operators of the near-field expansions (attach_sm_tables): the buffer, the
+    // place in it of those held, by (degree, kappa), the floats in use; the
+    // degrees' fixed tables; scratch
+    DevBuf smops, smfixed[15], smwork;
+    std::map<std::pair<int, double>, size_t> sm_held;
+    size_t sm_used = 0;
 
     // plan upload
     std::vector<unsigned char> last_upload;
@@ -202,6 +207,13 @@ int cuda_status(cudaError_t e) {
     if (e == cudaErrorMemoryAllocation) return PETFMM_ENOMEM;
     return PETFMM_ECUDA;
 }
+
+#define PF_TRY(expr)                         \
+    do {                                     \
+        int rc_ = (expr);                    \
+        if (rc_ != PETFMM_OK) return rc_;    \
+    } while (0)
+#define PF_CUDA(expr) PF_TRY(cuda_status(expr))
 
 // ---------------------------------------------------------------------------
 // Near-field polynomial: Chebyshev interpolation of g(q) = (1 - e^-q) / q on
@@ -353,46 +365,77 @@ OpTables *get_tables(petfmm_ctx *c, int p, int kernel, int *err) {
     return &(c->tables[key] = t);
 }
 
-// Operators of the near field by expansions for one (degree, kappa): a few
-// hundred KB each.  A server that refits domains meets new values of kappa
-// now and then: when kMaxSmTables are held, they are dropped (after the
-// stream is done with them) before the next evaluation's are made.
-constexpr size_t kMaxSmTables = 64;
-
 double sm_kappa(const InstDesc &d) { return near_kappa(d.wleaf, d.sigma); }
+
+// Operators of the near field by expansions for one (degree, kappa), 80 to 520 KB
+// each, made on the device when a plan first needs them and kept while they fit
+// the buffer (a simulation or a server that refits domains meets new values of
+// kappa all the time): where the next plan's do not fit beside them, they make
+// room.  All of it is ordered by the context's stream.
+constexpr size_t kSmOperatorBytes = size_t(4) << 20;  // smallest buffer
 
 int attach_sm_tables(petfmm_ctx *c, Plan &pl) {
     if (!pl.sm_degrees) return PETFMM_OK;
-    size_t missing = 0;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    PF_CUDA(cudaStreamIsCapturing(c->stream, &cap));
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    // (a captured graph makes its own operators, and nothing here relies on when)
+    if (captured) c->sm_held.clear();
+    typedef std::pair<int, double> Key;
+    std::map<Key, size_t> need;  // operators of the plan (leaves of few blobs need none)
     for (const InstDesc &d : pl.inst)
-        if (d.smdeg && !c->sm_tables.count({d.smdeg, sm_kappa(d)})) ++missing;
-    if (missing && c->sm_tables.size() + missing > kMaxSmTables && !c->sm_tables.empty()) {
-        if (cudaStreamSynchronize(c->stream) != cudaSuccess) return PETFMM_ECUDA;
-        for (auto &kv : c->sm_tables) cudaFree(kv.second);
-        c->sm_tables.clear();
+        if (d.smdeg && sm_max_rows(d.smdeg, d.n, int64_t(1) << (2 * d.L)) > 0)
+            need[Key(d.smdeg, sm_kappa(d))] = 0;
+    size_t all = 0, more = 0;  // floats
+    for (const auto &kv : need) {
+        const size_t f = sm_operator_floats(kv.first.first);
+        all += f;
+        if (!c->sm_held.count(kv.first)) more += f;
     }
-    std::vector<float> host;
+    if (more) {
+        if (c->sm_held.empty() || (c->sm_used + more) * sizeof(float) > c->smops.cap) {
+            c->sm_held.clear();
+            c->sm_used = 0;
+            PF_TRY(ensure(c->smops, std::max(all * sizeof(float), kSmOperatorBytes), c->stream));
+        }
+        std::vector<SmOperator> ops;
+        int nmax = 0;
+        for (const auto &kv : need) {
+            if (c->sm_held.count(kv.first)) continue;
+            const int n = kv.first.first;
+            DevBuf &fixed = c->smfixed[n];
+            if (!fixed.p) {
+                const std::vector<double> &t = host_sm_fixed(n);
+                PF_TRY(ensure(fixed, t.size() * sizeof(double), c->stream));
+                const cudaError_t e = cudaMemcpyAsync(fixed.p, t.data(), t.size() * sizeof(double),
+                                                      cudaMemcpyHostToDevice, c->stream);
+                if (e != cudaSuccess) {
+                    cudaFree(fixed.p);
+                    fixed = DevBuf();
+                    return cuda_status(e);
+                }
+            }
+            ops.push_back({n, kv.first.second, static_cast<const double *>(fixed.p),
+                           static_cast<float *>(c->smops.p) + c->sm_used});
+            c->sm_held[kv.first] = c->sm_used;
+            c->sm_used += sm_operator_floats(n);
+            nmax = std::max(nmax, n);
+        }
+        int rc = ensure(c->smwork, sm_work_bytes(nmax, ops.size()), c->stream);
+        if (rc == PETFMM_OK)
+            rc = cuda_status(launch_sm_operators(ops, nmax, static_cast<double *>(c->smwork.p),
+                                                 c->stream, &c->launches));
+        if (rc != PETFMM_OK) {
+            c->sm_held.clear();
+            return rc;
+        }
+    }
     for (InstDesc &d : pl.inst) {
         if (!d.smdeg) continue;
-        const std::pair<int, double> key(d.smdeg, sm_kappa(d));
-        auto it = c->sm_tables.find(key);
-        if (it == c->sm_tables.end()) {
-            host_sm_operators(key.second, key.first, host);
-            void *p = nullptr;
-            cudaError_t e = cudaMalloc(&p, host.size() * sizeof(float));
-            // (on the context's stream: its launches wait for the copy)
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(p, host.data(), host.size() * sizeof(float),
-                                    cudaMemcpyHostToDevice, c->stream);
-            if (e != cudaSuccess) {
-                cudaGetLastError();
-                if (p) cudaFree(p);
-                return cuda_status(e);
-            }
-            it = c->sm_tables.emplace(key, p).first;
-        }
-        d.t_sm = it->second;
+        const auto it = c->sm_held.find(Key(d.smdeg, sm_kappa(d)));
+        if (it != c->sm_held.end()) d.t_sm = static_cast<float *>(c->smops.p) + it->second;
     }
+    if (captured) c->sm_held.clear();
     return PETFMM_OK;
 }
 
@@ -717,13 +760,6 @@ int upload_plan(petfmm_ctx *c, const Plan &pl) {
     return PETFMM_OK;
 }
 
-#define PF_TRY(expr)                         \
-    do {                                     \
-        int rc_ = (expr);                    \
-        if (rc_ != PETFMM_OK) return rc_;    \
-    } while (0)
-#define PF_CUDA(expr) PF_TRY(cuda_status(expr))
-
 // FNV-1a over everything a kernel argument of the launch sequence depends on.
 struct KeyHash {
     uint64_t h = 1469598103934665603ull;
@@ -789,7 +825,8 @@ int run(petfmm_ctx *c, const std::vector<Problem> &probs) {
     const int64_t N = pl.N;
     // buffers
     PF_TRY(ensure(c->ctrl, CTRL_WORDS * sizeof(uint32_t), st));
-    if (c->evaluations == 0 && c->launches == 0) PF_CUDA(cudaMemsetAsync(c->ctrl.p, 0, CTRL_WORDS * 4, st));
+    if (!c->ctrl_zeroed) PF_CUDA(cudaMemsetAsync(c->ctrl.p, 0, CTRL_WORDS * 4, st));
+    c->ctrl_zeroed = true;
     PF_TRY(upload_plan(c, pl));
     if (N == 0) {
         c->evaluations++;
@@ -1256,12 +1293,13 @@ int petfmm_destroy(petfmm_ctx *c) {
     cudaStreamSynchronize(c->stream);
     DevBuf *bufs[] = {&c->keysA, &c->keysB, &c->valsA, &c->valsB, &c->hist,
                       &c->start, &c->xs, &c->ys, &c->gs, &c->rec, &c->me, &c->le,
-                      &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->gtab, &c->hx, &c->hy,
+                      &c->items, &c->ctrl, &c->plan_dev, &c->busy, &c->ucount, &c->recu, &c->occ, &c->own, &c->part, &c->pitems, &c->pxtra, &c->pxs, &c->ustage, &c->smleaf, &c->smlist, &c->smmom, &c->smloc, &c->smops, &c->smwork, &c->gtab, &c->hx, &c->hy,
                       &c->hg, &c->hu, &c->hv};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     for (auto &kv : c->tables) free_op_tables(&kv.second);
-    for (auto &kv : c->sm_tables) cudaFree(kv.second);
+    for (DevBuf &b : c->smfixed)
+        if (b.p) cudaFree(b.p);
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->pinned) cudaFreeHost(c->pinned);
@@ -1839,6 +1877,22 @@ int petfmm_debug_smooth_operators(double kappa, float *out, int64_t cap) {
     if (cap < int64_t(t.size())) return PETFMM_EINVAL;
     std::memcpy(out, t.data(), t.size() * sizeof(float));
     return n;
+}
+
+int petfmm_debug_smooth_table(petfmm_ctx *c, int inst, float *out, int64_t cap) {
+    if (!c || inst < 0 || cap < 0 || (cap > 0 && !out)) return PETFMM_EINVAL;
+    if (size_t(inst) >= c->plan.inst.size()) return PETFMM_EINVAL;
+    const InstDesc &d = c->plan.inst[size_t(inst)];
+    if (!d.smdeg || !d.t_sm) return 0;
+    if (!out) return d.smdeg;
+    const size_t n = sm_operator_floats(d.smdeg);
+    if (cap < int64_t(n)) return PETFMM_EINVAL;
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess ||
+        cudaMemcpy(out, d.t_sm, n * sizeof(float), cudaMemcpyDeviceToHost) != cudaSuccess) {
+        cudaGetLastError();
+        return PETFMM_ECUDA;
+    }
+    return d.smdeg;
 }
 
 int petfmm_debug_op_table(int order, int kernel, int which, double *out, int64_t cap) {

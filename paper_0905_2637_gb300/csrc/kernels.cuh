@@ -271,6 +271,20 @@ int sm_degree(double kappa, double near_tol);
 size_t sm_row_floats(int n);
 int64_t sm_max_rows(int n, int64_t blobs, int64_t leaves);
 void host_sm_operators(double kappa, int n, std::vector<float> &out);
+// The operators of one (degree, kappa) on the device: sm_operator_floats(n)
+// floats at out, from the degree's host_sm_fixed table (a device copy), launched
+// on st; work: sm_work_bytes of the largest degree and the number of operators.
+const std::vector<double> &host_sm_fixed(int n);
+size_t sm_operator_floats(int n);
+size_t sm_work_bytes(int n, size_t ops);
+struct SmOperator {
+    int n;
+    double kappa;
+    const double *fixed;
+    float *out;
+};
+cudaError_t launch_sm_operators(const std::vector<SmOperator> &ops, int nmax, double *work,
+                                cudaStream_t st, uint64_t *launches);
 // lmask, lrank: per leaf, its neighbours summed directly / by expansion, and
 // its row of mom (moments) and loc (local expansions); list: (instance, leaf)
 // of each row; rows of `row` floats.

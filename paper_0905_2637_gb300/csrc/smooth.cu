@@ -91,14 +91,36 @@ int64_t sm_max_rows(int n, int64_t blobs, int64_t leaves) {
 // 1e-12 for kappa < 2).
 constexpr int kSmCheb = 26;
 
-// V[a][b][k]: T_k(tau - s), tau, s in [-1/2, 1/2], projected onto
-// P_a(2 tau) P_b(2 s), a, b <= n; fixed per degree, built once.
-static const std::vector<double> &sm_shift_table(int n) {
+// What the operators of a degree have in common, FP64, built once per process
+// (one copy per context on the device): U[a][b][i], i < kSmCheb, with which
+// sum_ij U[a1][b1][i] f[i][j] U[a2][b2][j] is the coefficient of P_a1(2 tau_x)
+// P_b1(2 s_x) P_a2(2 tau_y) P_b2(2 s_y) in the function of tau - s that has the
+// values f at the Chebyshev nodes; the powers pw[a][e] of x in P_a(x); the nodes
+// cos(pi (i + 1/2) / kSmCheb); 1 / k for the series of Ein.
+constexpr int kSmSeries = 160;
+struct SmFixed {
+    const double *u, *pw, *node, *inv;
+    __host__ __device__ SmFixed(const double *t, int n) {
+        const int n1 = n + 1;
+        u = t;
+        pw = u + n1 * n1 * kSmCheb;
+        node = pw + n1 * n1;
+        inv = node + kSmCheb;
+    }
+};
+static size_t sm_fixed_words(int n) {
+    return size_t(n + 1) * (n + 1) * (kSmCheb + 1) + kSmCheb + kSmSeries;
+}
+
+const std::vector<double> &host_sm_fixed(int n) {
     static std::mutex mu;
     static std::map<int, std::vector<double>> tables;
     std::lock_guard<std::mutex> lk(mu);
-    std::vector<double> &V = tables[n];
-    if (!V.empty()) return V;
+    std::vector<double> &out = tables[n];
+    if (!out.empty()) return out;
+    // V[a][b][k]: T_k(tau - s), tau, s in [-1/2, 1/2], projected onto
+    // P_a(2 tau) P_b(2 s), a, b <= n
+    std::vector<double> V;
     const int n1 = n + 1, q = n + 12;  // Gauss nodes: exact for T_k P_a products
     // Gauss-Legendre nodes by Newton's method on P_q
     std::vector<double> xg(q), wg(q);
@@ -131,10 +153,16 @@ static const std::vector<double> &sm_shift_table(int n) {
         }
     }
     V.assign(size_t(n1) * n1 * kSmCheb, 0.0);
+    std::vector<double> t0(size_t(q) * q), t1(size_t(q) * q);  // T_{k-2}, T_{k-1}
     for (int k = 0; k < kSmCheb; ++k) {
         for (int i = 0; i < q; ++i)
-            for (int j = 0; j < q; ++j)
-                t[size_t(i) * q + j] = std::cos(k * std::acos(0.5 * (xg[i] - xg[j])));
+            for (int j = 0; j < q; ++j) {
+                const size_t e = size_t(i) * q + j;
+                const double x = 0.5 * (xg[i] - xg[j]);
+                t[e] = k == 0 ? 1.0 : k == 1 ? x : 2.0 * x * t1[e] - t0[e];
+                t0[e] = t1[e];
+                t1[e] = t[e];
+            }
         for (int a = 0; a < n1; ++a)
             for (int j = 0; j < q; ++j) {
                 double s = 0.0;
@@ -148,117 +176,229 @@ static const std::vector<double> &sm_shift_table(int n) {
                 V[size_t(a * n1 + b) * kSmCheb + k] = s;
             }
     }
-    return V;
-}
-
-// C^D of the 9 neighbour offsets, source = target + (ox, oy), block
-// (oy + 1) 3 + ox + 1, as [beta][alpha] with rows of sm_stride(n) floats;
-// beta: Legendre products of twice the source offset, alpha: powers of twice
-// the target offset.  Phi is interpolated in d by Chebyshev polynomials,
-// T_k(tau - s) projected onto Legendre products (fixed per degree), the
-// total degrees cut at n, and the target side turned into powers; FP64
-// throughout.
-void host_sm_operators(double kappa, int n, std::vector<float> &out) {
-    const int n1 = n + 1, M = sm_terms(n), S = sm_stride(n), mm = kSmCheb;
-    const std::vector<double> &V = sm_shift_table(n);  // [a][b][k]
-    // powers of x in P_a(x)
-    std::vector<double> pw(size_t(n1 + 1) * n1, 0.0);
+    out.assign(sm_fixed_words(n), 0.0);
+    double *U = out.data(), *pw = U + size_t(n1) * n1 * kSmCheb, *node = pw + n1 * n1,
+           *inv = node + kSmCheb;
+    for (int i = 0; i < kSmCheb; ++i) node[i] = std::cos(M_PI * (i + 0.5) / kSmCheb);
+    for (int k = 1; k < kSmSeries; ++k) inv[k] = 1.0 / k;
+    // Chebyshev coefficients from the values at the nodes
+    std::vector<double> cs(size_t(kSmCheb) * kSmCheb);
+    for (int k = 0; k < kSmCheb; ++k)
+        for (int i = 0; i < kSmCheb; ++i)
+            cs[size_t(k) * kSmCheb + i] =
+                std::cos(M_PI * k * (i + 0.5) / kSmCheb) * (k ? 2.0 : 1.0) / kSmCheb;
+    for (int e = 0; e < n1 * n1; ++e)
+        for (int i = 0; i < kSmCheb; ++i) {
+            double v = 0.0;
+            // (T_k has the parity of k)
+            for (int k = (e / n1 + e % n1) & 1; k < kSmCheb; k += 2)
+                v += V[size_t(e) * kSmCheb + k] * cs[size_t(k) * kSmCheb + i];
+            U[size_t(e) * kSmCheb + i] = v;
+        }
     pw[0] = 1.0;
-    if (n >= 1) pw[size_t(1) * n1 + 1] = 1.0;
+    if (n >= 1) pw[n1 + 1] = 1.0;
     for (int a = 2; a <= n; ++a)
         for (int k = 0; k <= a; ++k)
-            pw[size_t(a) * n1 + k] =
-                ((k ? (2 * a - 1) * pw[size_t(a - 1) * n1 + k - 1] : 0.0) -
-                 (a - 1) * pw[size_t(a - 2) * n1 + k]) / a;
-    auto phi = [&](double s) {  // Ein(kappa s) / (2 kappa), s = |d|^2
-        const double z = kappa * s;
-        double term = 1.0, sum = 0.0;  // sum_k (-z)^(k-1) / (k k!)
-        for (int k = 1; k < 160; ++k) {
-            sum += term / k;
-            term *= -z / (k + 1);
-            if (std::fabs(term) < 1e-18 && k > z) break;
-        }
-        return 0.5 * s * sum;
-    };
-    out.assign(size_t(9) * M * S, 0.0f);
-    const int kD[3][2] = {{0, 0}, {1, 0}, {1, 1}};
-    std::vector<double> f(size_t(mm) * mm), g(size_t(mm) * mm), c(size_t(mm) * mm);
-    std::vector<double> h(size_t(mm) * n1 * n1), C(size_t(M) * M), tr(size_t(n1) * n1);
-    std::vector<double> cs(size_t(mm) * mm);
-    for (int k = 0; k < mm; ++k)
-        for (int i = 0; i < mm; ++i)
-            cs[size_t(k) * mm + i] = std::cos(M_PI * k * (i + 0.5) / mm) * (k ? 2.0 : 1.0) / mm;
-    for (const auto &D : kD) {
-        for (int i = 0; i < mm; ++i)
-            for (int j = 0; j < mm; ++j) {
-                const double dx = D[0] + std::cos(M_PI * (i + 0.5) / mm);
-                const double dy = D[1] + std::cos(M_PI * (j + 0.5) / mm);
-                f[size_t(i) * mm + j] = phi(dx * dx + dy * dy);
-            }
-        for (int k = 0; k < mm; ++k)
-            for (int j = 0; j < mm; ++j) {
-                double s = 0.0;
-                for (int i = 0; i < mm; ++i) s += cs[size_t(k) * mm + i] * f[size_t(i) * mm + j];
-                g[size_t(k) * mm + j] = s;
-            }
-        for (int k = 0; k < mm; ++k)
-            for (int l = 0; l < mm; ++l) {
-                double s = 0.0;
-                for (int j = 0; j < mm; ++j) s += cs[size_t(l) * mm + j] * g[size_t(k) * mm + j];
-                c[size_t(k) * mm + l] = s;
-            }
-        // h[a2][b2][k] = sum_l c[k][l] V[a2][b2][l]; T_l has the parity of l
-        for (int e = 0; e < n1 * n1; ++e) {
-            const double *v = &V[size_t(e) * mm];
-            for (int k = 0; k < mm; ++k) {
-                double s = 0.0;
-                for (int l = (e / n1 + e % n1) & 1; l < mm; l += 2) s += c[size_t(k) * mm + l] * v[l];
-                h[size_t(e) * mm + k] = s;
-            }
-        }
-        for (int b2 = 0; b2 <= n; ++b2)          // source y, x
-            for (int b1 = 0; b1 + b2 <= n; ++b1) {
-                // Legendre coefficients of the target side, then powers
-                std::fill(tr.begin(), tr.end(), 0.0);
-                for (int a2 = 0; a2 <= n; ++a2)
-                    for (int a1 = 0; a1 + a2 <= n; ++a1) {
-                        double s = 0.0;
-                        const double *v = &V[size_t(a1 * n1 + b1) * mm];
-                        const double *w = &h[size_t(a2 * n1 + b2) * mm];
-                        for (int k = (a1 + b1) & 1; k < mm; k += 2) s += v[k] * w[k];
-                        for (int e = a1 & 1; e <= a1; e += 2)
-                            tr[size_t(a2) * n1 + e] += s * pw[size_t(a1) * n1 + e];
-                    }
-                for (int e2 = 0; e2 <= n; ++e2)
-                    for (int e1 = 0; e1 + e2 <= n; ++e1) {
-                        double s = 0.0;
-                        for (int a2 = e2; a2 + e1 <= n; a2 += 2)
-                            s += tr[size_t(a2) * n1 + e1] * pw[size_t(a2) * n1 + e2];
-                        C[size_t(sm_idx(n, b1, b2)) * M + sm_idx(n, e1, e2)] = s;
-                    }
-            }
-        // the offsets that mirror or swap to this one; D = -(source offset)
-        for (int oy = -1; oy <= 1; ++oy)
-            for (int ox = -1; ox <= 1; ++ox) {
-                const int hi = std::max(std::abs(ox), std::abs(oy));
-                const int lo = std::min(std::abs(ox), std::abs(oy));
-                if (hi != D[0] || lo != D[1]) continue;
-                const bool swap = std::abs(oy) > std::abs(ox);
-                const int sx = -ox < 0 ? -1 : 1, sy = -oy < 0 ? -1 : 1;
-                float *t = out.data() + size_t((oy + 1) * 3 + ox + 1) * M * S;
-                for (int b2 = 0; b2 <= n; ++b2)
-                    for (int b1 = 0; b1 + b2 <= n; ++b1)
-                        for (int e2 = 0; e2 <= n; ++e2)
-                            for (int e1 = 0; e1 + e2 <= n; ++e1) {
-                                const double v =
-                                    swap ? C[size_t(sm_idx(n, b2, b1)) * M + sm_idx(n, e2, e1)]
-                                         : C[size_t(sm_idx(n, b1, b2)) * M + sm_idx(n, e1, e2)];
-                                const int par = (sx < 0 ? b1 + e1 : 0) + (sy < 0 ? b2 + e2 : 0);
-                                t[size_t(sm_idx(n, b1, b2)) * S + sm_idx(n, e1, e2)] =
-                                    float(par & 1 ? -v : v);
-                            }
-            }
+            pw[a * n1 + k] = ((k ? (2 * a - 1) * pw[(a - 1) * n1 + k - 1] : 0.0) -
+                              (a - 1) * pw[(a - 2) * n1 + k]) / a;
+    return out;
+}
+
+// The operators C^D of the 9 neighbour offsets, source = target + (ox, oy), block
+// (oy + 1) 3 + ox + 1, as [beta][alpha] with rows of sm_stride(n) floats; beta:
+// Legendre products of twice the source offset, alpha: powers of twice the
+// target offset.  Phi is interpolated in d by Chebyshev polynomials, T_k(tau -
+// s) projected onto Legendre products (both in U), the total degrees cut at n,
+// and the target side turned into powers; FP64 throughout.  Three of the nine
+// are computed, D = (0, 0), (1, 0), (1, 1); the others mirror or swap them.  The
+// steps below make them on the device (k_sm_values, k_sm_half, k_sm_finish: an
+// evaluation meets a new kappa without the host's 0.6 to 1.6 ms) and on the host.
+
+// Phi = Ein(kappa s) / (2 kappa), s = |d|^2
+__host__ __device__ inline double sm_phi(const SmFixed &t, double kappa, double s) {
+    const double z = kappa * s;
+    double term = 1.0, sum = 0.0;  // sum_k (-z)^(k-1) / (k k!)
+    for (int k = 1; k < kSmSeries - 1; ++k) {
+        sum += term * t.inv[k];
+        term *= -z * t.inv[k + 1];
+        if (fabs(term) < 1e-18 && k > z) break;
     }
+    return 0.5 * s * sum;
+}
+// value e = (i, j) of offset D (0: (0, 0), 1: (1, 0), 2: (1, 1))
+__host__ __device__ inline double sm_value(const SmFixed &t, double kappa, int D, int e) {
+    const double dx = (D > 0) + t.node[e / kSmCheb], dy = (D > 1) + t.node[e % kSmCheb];
+    return sm_phi(t, kappa, dx * dx + dy * dy);
+}
+// w[a2][b2][i] = sum_j f[i][j] U[a2][b2][j], e = (a2, b2, i)
+__host__ __device__ inline double sm_half(const SmFixed &t, const double *f, int e) {
+    const double *u = t.u + e / kSmCheb * kSmCheb, *g = f + e % kSmCheb * kSmCheb;
+    double v = 0.0;
+    for (int j = 0; j < kSmCheb; ++j) v += g[j] * u[j];
+    return v;
+}
+// A term's degrees (a of x, b of y).
+__host__ __device__ inline void sm_degrees(int n, int t, int *a, int *b) {
+    int y = 0;
+    while (sm_idx(n, 0, y + 1) <= t && y < n) ++y;
+    *b = y;
+    *a = t - sm_idx(n, 0, y);
+}
+// Row (b1, b2) of C^D, term (a1, a2): Legendre coefficient ...
+__host__ __device__ inline double sm_legendre(const SmFixed &t, int n, const double *w, int b1,
+                                              int b2, int a1, int a2) {
+    const double *u = t.u + (a1 * (n + 1) + b1) * kSmCheb;
+    const double *v = w + (a2 * (n + 1) + b2) * kSmCheb;
+    double c = 0.0;
+    for (int i = 0; i < kSmCheb; ++i) c += u[i] * v[i];
+    return c;
+}
+// ... then powers of x (cl: the row's terms) ...
+__host__ __device__ inline double sm_power_x(const SmFixed &t, int n, const double *cl, int e1, int a2) {
+    double v = 0.0;
+    for (int a1 = e1; a1 + a2 <= n; a1 += 2) v += cl[sm_idx(n, a1, a2)] * t.pw[a1 * (n + 1) + e1];
+    return v;
+}
+// ... and of y.
+__host__ __device__ inline double sm_power_y(const SmFixed &t, int n, const double *cx, int e1, int e2) {
+    double v = 0.0;
+    for (int a2 = e2; e1 + a2 <= n; a2 += 2) v += cx[sm_idx(n, e1, a2)] * t.pw[a2 * (n + 1) + e2];
+    return v;
+}
+// Entry (b1, b2), (e1, e2) of C^D into the offsets that mirror or swap D; pad >=
+// 0: column pad of the row instead, which has no term, zero.
+__host__ __device__ inline void sm_store(int n, int D, int b1, int b2, int e1, int e2, int pad,
+                                         double v, float *out) {
+    const int M = sm_terms(n), S = sm_stride(n);
+    for (int o = 0; o < 9; ++o) {
+        const int ox = o % 3 - 1, oy = o / 3 - 1, ax = ox < 0 ? -ox : ox, ay = oy < 0 ? -oy : oy;
+        if (ax + ay != D) continue;
+        const bool swap = ay > ax;
+        const int p1 = swap ? b2 : b1, p2 = swap ? b1 : b2, q1 = swap ? e2 : e1, q2 = swap ? e1 : e2;
+        const int par = (ox > 0 ? p1 + q1 : 0) + (oy > 0 ? p2 + q2 : 0);
+        float *row = out + (size_t(o) * M + sm_idx(n, p1, p2)) * S;
+        if (pad >= 0) row[pad] = 0.0f;
+        else row[sm_idx(n, q1, q2)] = float(par & 1 ? -v : v);
+    }
+}
+
+void host_sm_operators(double kappa, int n, std::vector<float> &out) {
+    const int n1 = n + 1, M = sm_terms(n), S = sm_stride(n);
+    const SmFixed t(host_sm_fixed(n).data(), n);
+    out.assign(size_t(9) * M * S, 0.0f);
+    std::vector<double> f(size_t(kSmCheb) * kSmCheb), w(size_t(n1) * n1 * kSmCheb);
+    std::vector<double> cl(static_cast<size_t>(M)), cx(static_cast<size_t>(M));
+    for (int D = 0; D < 3; ++D) {
+        for (size_t e = 0; e < f.size(); ++e) f[e] = sm_value(t, kappa, D, int(e));
+        for (size_t e = 0; e < w.size(); ++e) w[e] = sm_half(t, f.data(), int(e));
+        for (int beta = 0; beta < M; ++beta) {
+            int b1, b2, x, y;
+            sm_degrees(n, beta, &b1, &b2);
+            for (int k = 0; k < M; ++k) {
+                sm_degrees(n, k, &x, &y);
+                cl[size_t(k)] = sm_legendre(t, n, w.data(), b1, b2, x, y);
+            }
+            for (int k = 0; k < M; ++k) {
+                sm_degrees(n, k, &x, &y);
+                cx[size_t(k)] = sm_power_x(t, n, cl.data(), x, y);
+            }
+            for (int k = 0; k < M; ++k) {
+                sm_degrees(n, k, &x, &y);
+                sm_store(n, D, b1, b2, x, y, -1, sm_power_y(t, n, cx.data(), x, y), out.data());
+            }
+        }
+    }
+}
+
+// ----------------------------------------------------------------------------
+// The same on the device: grid (entries, D, operator)
+// ----------------------------------------------------------------------------
+namespace {
+
+constexpr int SM_OPS = 64;  // operators per launch
+struct SmOps {
+    const double *fixed[SM_OPS];
+    float *out[SM_OPS];
+    double kappa[SM_OPS];
+    int n[SM_OPS];
+    double *work;   // per operator and D: values, then w
+    size_t stride;  // of one (operator, D)
+};
+
+__device__ __forceinline__ double *sm_work(const SmOps &o, int op, int D) {
+    return o.work + size_t(op * 3 + D) * o.stride;
+}
+
+__global__ void __launch_bounds__(128) k_sm_values(const __grid_constant__ SmOps o) {
+    const int op = int(blockIdx.z), D = int(blockIdx.y), e = int(blockIdx.x * 128 + threadIdx.x);
+    if (e >= kSmCheb * kSmCheb) return;
+    sm_work(o, op, D)[e] = sm_value(SmFixed(o.fixed[op], o.n[op]), o.kappa[op], D, e);
+}
+
+__global__ void __launch_bounds__(128) k_sm_half(const __grid_constant__ SmOps o) {
+    const int op = int(blockIdx.z), D = int(blockIdx.y), e = int(blockIdx.x * 128 + threadIdx.x);
+    const int n = o.n[op];
+    if (e >= (n + 1) * (n + 1) * kSmCheb) return;
+    double *f = sm_work(o, op, D);
+    f[kSmCheb * kSmCheb + e] = sm_half(SmFixed(o.fixed[op], n), f, e);
+}
+
+// A block per row of C^D, a thread per term.
+constexpr int SM_TERMS_MAX = sm_terms(14);
+static_assert(SM_TERMS_MAX <= 128 && sm_stride(14) <= 128, "a thread per term");
+__global__ void __launch_bounds__(128) k_sm_finish(const __grid_constant__ SmOps o) {
+    __shared__ double cl[SM_TERMS_MAX], cx[SM_TERMS_MAX];
+    const int op = int(blockIdx.z), D = int(blockIdx.y), beta = int(blockIdx.x);
+    const int n = o.n[op], M = sm_terms(n), k = int(threadIdx.x);
+    if (beta >= M) return;
+    const SmFixed t(o.fixed[op], n);
+    const double *w = sm_work(o, op, D) + kSmCheb * kSmCheb;
+    int b1, b2, x = 0, y = 0;
+    sm_degrees(n, beta, &b1, &b2);
+    if (k < M) {
+        sm_degrees(n, k, &x, &y);
+        cl[k] = sm_legendre(t, n, w, b1, b2, x, y);
+    }
+    __syncthreads();
+    if (k < M) cx[k] = sm_power_x(t, n, cl, x, y);
+    __syncthreads();
+    if (k < M) sm_store(n, D, b1, b2, x, y, -1, sm_power_y(t, n, cx, x, y), o.out[op]);
+    else if (k < sm_stride(n)) sm_store(n, D, b1, b2, 0, 0, k, 0.0, o.out[op]);
+}
+
+}  // namespace
+
+size_t sm_operator_floats(int n) { return size_t(9) * sm_terms(n) * sm_stride(n); }
+
+static size_t sm_work_stride(int n) {
+    return size_t(kSmCheb) * kSmCheb + size_t(n + 1) * (n + 1) * kSmCheb;
+}
+size_t sm_work_bytes(int n, size_t ops) {
+    return std::min(ops, size_t(SM_OPS)) * 3 * sm_work_stride(n) * sizeof(double);
+}
+
+cudaError_t launch_sm_operators(const std::vector<SmOperator> &ops, int nmax, double *work,
+                                cudaStream_t st, uint64_t *launches) {
+    for (size_t i0 = 0; i0 < ops.size(); i0 += SM_OPS) {
+        SmOps o{};
+        const size_t m = std::min(ops.size() - i0, size_t(SM_OPS));
+        for (size_t i = 0; i < m; ++i) {
+            o.fixed[i] = ops[i0 + i].fixed;
+            o.out[i] = ops[i0 + i].out;
+            o.kappa[i] = ops[i0 + i].kappa;
+            o.n[i] = ops[i0 + i].n;
+        }
+        o.work = work;
+        o.stride = sm_work_stride(nmax);
+        const unsigned z = unsigned(m);
+        k_sm_values<<<dim3((kSmCheb * kSmCheb + 127) / 128, 3, z), 128, 0, st>>>(o);
+        k_sm_half<<<dim3(unsigned((nmax + 1) * (nmax + 1) * kSmCheb + 127) / 128, 3, z), 128, 0, st>>>(o);
+        k_sm_finish<<<dim3(unsigned(sm_terms(nmax)), 3, z), 128, 0, st>>>(o);
+        PF_LAUNCHED(3);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 // ----------------------------------------------------------------------------
