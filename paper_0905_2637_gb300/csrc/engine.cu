@@ -356,7 +356,7 @@ OpTables *get_tables(petfmm_ctx *c, int p, int kernel, int *err) {
     auto it = c->tables.find(key);
     if (it != c->tables.end()) return &it->second;
     OpTables t;
-    cudaError_t e = build_op_tables(p, kernel, &t, c->stream);
+    cudaError_t e = build_op_tables(p, kernel, c->precision == PETFMM_FP64, &t, c->stream);
     if (e != cudaSuccess) {
         free_op_tables(&t);
         *err = cuda_status(e);
@@ -716,6 +716,8 @@ int attach_tables(petfmm_ctx *c, Plan &pl) {
             d.t_shift = t->shift32;
             d.t_m2l = t->orbit32;
             d.t_m2l_box = t->m2l32;
+            if (d.tc_levels) PF_CUDA(build_tc_image(c->kernel, false, t, c->stream));
+            if (d.tcb_levels) PF_CUDA(build_tc_image(c->kernel, true, t, c->stream));
             d.t_m2l_tc = t->m2l_tc;
             d.t_m2l_tcb = t->m2l_tcb;
         }
@@ -1280,7 +1282,11 @@ int petfmm_create(const petfmm_domain *dom, int levels, int order, double sigma,
         }
     }
     int err = PETFMM_OK;
-    if (!get_tables(c, order, KERNEL_VORTEX, &err)) {
+    OpTables *t = get_tables(c, order, KERNEL_VORTEX, &err);
+    // (an evaluation of this depth runs these levels on the tensor cores)
+    if (t && precision == PETFMM_MIXED && levels >= 8 && m2l_tcb_supported(order, levels))
+        err = cuda_status(build_tc_image(KERNEL_VORTEX, true, t, c->stream));
+    if (!t || err != PETFMM_OK) {
         petfmm_destroy(c);
         return err;
     }

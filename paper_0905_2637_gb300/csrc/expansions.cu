@@ -262,44 +262,64 @@ void host_op_table(int p, int kernel, int which, std::vector<double> &out) {
     else (lap ? host_lap_m2l_table : host_m2l_table)(p, out.data());
 }
 
-cudaError_t build_op_tables(int p, int kernel, OpTables *t, cudaStream_t st) {
+cudaError_t build_op_tables(int p, int kernel, bool fp64, OpTables *t, cudaStream_t st) {
     t->p = p;
-    std::vector<double> m2l(size_t(2) * 40 * p * p), shift, orbit;
-    (kernel == KERNEL_LAPLACE ? host_lap_m2l_table : host_m2l_table)(p, m2l.data());
+    std::vector<double> shift, orbit;
     host_shift_table(p, kernel, shift);
     host_m2l_orbit_table(p, kernel, orbit);
-    std::vector<float> m2l32(m2l.begin(), m2l.end()), shift32(shift.begin(), shift.end()),
-        orbit32(orbit.begin(), orbit.end());
     // one allocation and one copy for all of them
-    std::vector<unsigned char> blob;
-    std::vector<std::pair<void **, size_t>> at;
-    auto put = [&](void **dst, const void *src, size_t bytes) {
-        at.push_back({dst, blob.size()});
-        const unsigned char *b = static_cast<const unsigned char *>(src);
-        blob.insert(blob.end(), b, b + bytes);
-        blob.resize((blob.size() + 255) / 256 * 256);
+    std::vector<float> shift32, orbit32, m2l32;
+    struct Part {
+        void **dst;
+        const void *src;
+        size_t bytes;
     };
-    put((void **)&t->shift64, shift.data(), shift.size() * 8);
-    put((void **)&t->shift32, shift32.data(), shift32.size() * 4);
-    put((void **)&t->orbit64, orbit.data(), orbit.size() * 8);
-    put((void **)&t->orbit32, orbit32.data(), orbit32.size() * 4);
-    put((void **)&t->m2l32, m2l32.data(), m2l32.size() * 4);
-    if (((2 * p + 15) & ~15) <= 48) {
-        std::vector<float> img;
-        host_m2l_tc_images(p, kernel, img);
-        put((void **)&t->m2l_tc, img.data(), img.size() * 4);
-        host_m2l_tcb_images(p, kernel, img);
-        put((void **)&t->m2l_tcb, img.data(), img.size() * 4);
+    std::vector<Part> parts;
+    if (fp64) {
+        parts = {{(void **)&t->shift64, shift.data(), shift.size() * 8},
+                 {(void **)&t->orbit64, orbit.data(), orbit.size() * 8}};
+    } else {
+        std::vector<double> m2l(size_t(2) * 40 * p * p);
+        (kernel == KERNEL_LAPLACE ? host_lap_m2l_table : host_m2l_table)(p, m2l.data());
+        shift32.assign(shift.begin(), shift.end());
+        orbit32.assign(orbit.begin(), orbit.end());
+        m2l32.assign(m2l.begin(), m2l.end());
+        parts = {{(void **)&t->shift32, shift32.data(), shift32.size() * 4},
+                 {(void **)&t->orbit32, orbit32.data(), orbit32.size() * 4},
+                 {(void **)&t->m2l32, m2l32.data(), m2l32.size() * 4}};
     }
-    const cudaError_t e = cudaMalloc(&t->blob, blob.size());
+    size_t total = 0;
+    for (const Part &x : parts) total += (x.bytes + 255) / 256 * 256;
+    std::vector<unsigned char> blob(total);
+    const cudaError_t e = cudaMalloc(&t->blob, total);
     if (e != cudaSuccess) return e;
-    for (const auto &x : at) *x.first = static_cast<unsigned char *>(t->blob) + x.second;
+    size_t at = 0;
+    for (const Part &x : parts) {
+        std::memcpy(blob.data() + at, x.src, x.bytes);
+        *x.dst = static_cast<unsigned char *>(t->blob) + at;
+        at += (x.bytes + 255) / 256 * 256;
+    }
     // (the call returns once the pageable source is staged)
-    return cudaMemcpyAsync(t->blob, blob.data(), blob.size(), cudaMemcpyHostToDevice, st);
+    return cudaMemcpyAsync(t->blob, blob.data(), total, cudaMemcpyHostToDevice, st);
+}
+
+cudaError_t build_tc_image(int kernel, bool blocks, OpTables *t, cudaStream_t st) {
+    float *&dst = blocks ? t->m2l_tcb : t->m2l_tc;
+    if (dst) return cudaSuccess;
+    std::vector<float> img;
+    (blocks ? host_m2l_tcb_images : host_m2l_tc_images)(t->p, kernel, img);
+    void *p = nullptr;
+    cudaError_t e = cudaMalloc(&p, img.size() * 4);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p, img.data(), img.size() * 4, cudaMemcpyHostToDevice, st);
+    if (e != cudaSuccess) cudaFree(p);
+    else dst = static_cast<float *>(p);
+    return e;
 }
 
 void free_op_tables(OpTables *t) {
     cudaFree(t->blob);
+    cudaFree(t->m2l_tc);
+    cudaFree(t->m2l_tcb);
     *t = OpTables();
 }
 

@@ -2758,15 +2758,13 @@ bool use_orbits3(const petfmm3d_ctx *c) {
     return c->precision == PETFMM_FP64 || c->p > TC3_MAXP || (c->m2l_tc == 2 && c->L <= 4);
 }
 
-int upload_tables(petfmm3d_ctx *c) {
-    const int p = c->p, nc = nc3(p), nci = nci3(p);
-    // the real basis of the M2L matrices: real index r < nc is Re of
-    // coefficient r, r >= nc Im of the coefficients with m > 0 in order;
-    // parity: bit d set if the solid harmonic changes sign with axis d
-    const int nr = p * p, nrp = mg_nrp(p);
-    std::vector<short2> rm(static_cast<size_t>(nr));
-    std::vector<uint8_t> par(static_cast<size_t>(nr));
-    for (int n = 0, r = nc; n < p; ++n)
+// The real basis of the M2L matrices: real index r < nc is Re of coefficient r, r
+// >= nc Im of the coefficients with m > 0 in order; parity: bit d set if the
+// solid harmonic changes sign with axis d.
+void real_basis3(int p, std::vector<short2> &rm, std::vector<uint8_t> &par) {
+    rm.resize(size_t(p) * p);
+    par.resize(size_t(p) * p);
+    for (int n = 0, r = nc3(p); n < p; ++n)
         for (int m = 0; m <= n; ++m) {
             const int j = n * (n + 1) / 2 + m;
             rm[size_t(j)] = make_short2(short(j), short(m == 0 ? 2 : 0));
@@ -2776,6 +2774,83 @@ int upload_tables(petfmm3d_ctx *c) {
                 rm[size_t(r++)] = make_short2(short(j), 1);
             }
         }
+}
+
+// The M2L operators of the kernel that the options and the tree choose, made the
+// first time they are needed: by orbit, or for every offset the tensor cores'
+// images or the SIMT GEMM's matrices.
+int m2l_tables(petfmm3d_ctx *c) {
+    const int p = c->p, nc = nc3(p), nr = p * p, nrp = mg_nrp(p);
+    const bool f64 = c->precision == PETFMM_FP64, by_orbit = use_orbits3(c);
+    if (c->L < 2 || (by_orbit ? c->orbits : c->m2l_tc ? c->tcimg : c->atab32).p) return PETFMM_OK;
+    std::vector<cd> iv(static_cast<size_t>(nci3(p)));
+    // the orbits' operators [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
+    std::vector<double> orb(size_t(64) * nr * nr, 0.0);
+    for (int o = 0; o < 64; ++o) {
+        const int dx = o & 3, dy = (o >> 2) & 3, dz = o >> 4;
+        if (dx < 2 && dy < 2 && dz < 2) continue;
+        host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
+        host_m2l_real(p, iv.data(), orb.data() + size_t(o) * nr * nr);
+    }
+    if (by_orbit) {
+        if (f64) return upload3(c->orbits, orb.data(), orb.size() * sizeof(double), c->stream);
+        const std::vector<float> orb32(orb.begin(), orb.end());
+        return upload3(c->orbits, orb32.data(), orb32.size() * sizeof(float), c->stream);
+    }
+    // Each offset's operator is its orbit's between the signs of the reflected
+    // axes.  atab32: FP32, ap[k_in * nrp + r_out].  tcimg: TF32 hi / lo images for
+    // the tensor cores: [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero
+    // padding), K in the input basis of the tensor-core M2L (coefficient by
+    // coefficient: Re, then Im if m > 0), N in the M2L matrices' basis.
+    std::vector<short2> rm;
+    std::vector<uint8_t> par;
+    real_basis3(p, rm, par);
+    std::vector<int> tc3_kin(static_cast<size_t>(nr));
+    for (int n = 0, k = 0, t = 0; n < p; ++n)
+        for (int m = 0; m <= n; ++m) {
+            tc3_kin[size_t(k++)] = n * (n + 1) / 2 + m;
+            if (m > 0) tc3_kin[size_t(k++)] = nc + t++;
+        }
+    const size_t mat = size_t(nrp) * nrp;
+    std::vector<double> sign(static_cast<size_t>(nr));
+    std::vector<float> tab(size_t(NSLOT3) * mat * (c->m2l_tc ? 2 : 1), 0.f);
+    for (int slot = 0; slot < NSLOT3; ++slot) {
+        const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
+        if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
+        const int o = std::abs(dx) + 4 * std::abs(dy) + 16 * std::abs(dz);
+        const double *ao = orb.data() + size_t(o) * nr * nr;
+        const int refl = (dx < 0) | (dy < 0) << 1 | (dz < 0) << 2;
+        for (int r = 0; r < nr; ++r)
+            sign[size_t(r)] = __builtin_popcount(par[size_t(r)] & refl) & 1 ? -1.0 : 1.0;
+        auto entry = [&](int k, int r) {
+            return ao[size_t(k) * nr + r] * (sign[size_t(k)] * sign[size_t(r)]);
+        };
+        if (!c->m2l_tc) {
+            float *ap = tab.data() + size_t(slot) * mat;
+            for (int k = 0; k < nr; ++k)
+                for (int r = 0; r < nr; ++r) ap[size_t(k) * nrp + r] = float(entry(k, r));
+            continue;
+        }
+        float *hi = tab.data() + size_t(slot) * 2 * mat, *lo = hi + mat;
+        for (int k = 0; k < nr; ++k) {
+            const int kin = tc3_kin[size_t(k)];
+            for (int n = 0; n < nr; ++n) {
+                const double a = entry(kin, n);
+                const float h = host_tf32_rna(float(a));
+                const size_t at = (size_t(k / 4) * nrp + n) * 4 + size_t(k % 4);
+                hi[at] = h;
+                lo[at] = host_tf32_rna(float(a - double(h)));
+            }
+        }
+    }
+    return upload3(c->m2l_tc ? c->tcimg : c->atab32, tab.data(), tab.size() * sizeof(float), c->stream);
+}
+
+int upload_tables(petfmm3d_ctx *c) {
+    const int p = c->p, nr = p * p;
+    std::vector<short2> rm;
+    std::vector<uint8_t> par;
+    real_basis3(p, rm, par);
     P3_TRY(upload3(c->rmap, rm.data(), rm.size() * sizeof(short2), c->stream));
     P3_TRY(upload3(c->parity, par.data(), par.size(), c->stream));
     std::vector<double> a64(size_t(nr) * nr);
@@ -2800,66 +2875,7 @@ int upload_tables(petfmm3d_ctx *c) {
     P3_TRY(upload3(c->shift, f64 ? static_cast<const void *>(ops.data()) : ops32.data(),
                    ops.size() * es, c->stream));
     P3_TRY(upload3(c->order, order.data(), order.size() * sizeof(uint16_t), c->stream));
-    std::vector<cd> iv(static_cast<size_t>(nci));
-    // the orbits' operators [|dx| + 4 |dy| + 16 |dz|][k_in][r_out]
-    std::vector<double> orb(size_t(64) * nr * nr, 0.0);
-    for (int o = 0; o < 64; ++o) {
-        const int dx = o & 3, dy = (o >> 2) & 3, dz = o >> 4;
-        if (dx < 2 && dy < 2 && dz < 2) continue;
-        host_rec_i(dx, dy, dz, 2 * p - 1, iv.data());
-        host_m2l_real(p, iv.data(), orb.data() + size_t(o) * nr * nr);
-    }
-    if (use_orbits3(c)) {
-        const std::vector<float> orb32(orb.begin(), orb.end());
-        P3_TRY(upload3(c->orbits, f64 ? static_cast<const void *>(orb.data()) : orb32.data(),
-                       orb.size() * es, c->stream));
-    }
-    if (f64 || p > TC3_MAXP) return PETFMM_OK;
-    // The mixed path's M2L matrices, FP32: ap[k_in * nrp + r_out]; for p <= 8
-    // also their TF32 hi / lo images for the tensor cores:
-    // [slot][hi, lo][k / 4][n][k mod 4] = A[k][n] (zero padding), K in the
-    // input basis of the tensor-core M2L (coefficient by coefficient: Re, then
-    // Im if m > 0), N in the M2L matrices' basis.
-    std::vector<float> at(size_t(NSLOT3) * nrp * nrp, 0.f);
-    std::vector<float> img(size_t(NSLOT3) * 2 * nrp * nrp, 0.f);
-    std::vector<int> tc3_kin(static_cast<size_t>(nr));
-    for (int n = 0, k = 0, t = 0; n < p; ++n)
-        for (int m = 0; m <= n; ++m) {
-            const int j = n * (n + 1) / 2 + m;
-            tc3_kin[size_t(k++)] = j;
-            if (m > 0) tc3_kin[size_t(k++)] = nc + t++;
-        }
-    for (int slot = 0; slot < NSLOT3; ++slot) {
-        const int dx = slot % 7 - 3, dy = (slot / 7) % 7 - 3, dz = slot / 49 - 3;
-        if (std::max(std::abs(dx), std::max(std::abs(dy), std::abs(dz))) < 2) continue;
-        // its orbit's operator between the signs of the reflected axes
-        const int o = std::abs(dx) + 4 * std::abs(dy) + 16 * std::abs(dz);
-        const double *ao = orb.data() + size_t(o) * nr * nr;
-        const int refl = (dx < 0) | (dy < 0) << 1 | (dz < 0) << 2;
-        for (int k = 0; k < nr; ++k)
-            for (int r = 0; r < nr; ++r) {
-                const double v = ao[size_t(k) * nr + r];
-                const bool odd = __builtin_popcount((par[size_t(k)] ^ par[size_t(r)]) & refl) & 1;
-                a64[size_t(k) * nr + r] = odd ? -v : v;
-            }
-        float *ap = at.data() + size_t(slot) * nrp * nrp;
-        for (int k = 0; k < nr; ++k)
-            for (int r = 0; r < nr; ++r) ap[size_t(k) * nrp + r] = float(a64[size_t(k) * nr + r]);
-        float *hi = img.data() + size_t(slot) * 2 * nrp * nrp, *lo = hi + size_t(nrp) * nrp;
-        for (int k = 0; k < nr; ++k) {
-            const int kin = tc3_kin[size_t(k)];
-            for (int n = 0; n < nr; ++n) {
-                const double a = a64[size_t(kin) * nr + n];
-                const float h = host_tf32_rna(float(a));
-                const size_t o = (size_t(k / 4) * nrp + n) * 4 + size_t(k % 4);
-                hi[o] = h;
-                lo[o] = host_tf32_rna(float(a - double(h)));
-            }
-        }
-    }
-    P3_TRY(upload3(c->tcimg, img.data(), img.size() * sizeof(float), c->stream));
-    P3_TRY(upload3(c->atab32, at.data(), at.size() * sizeof(float), c->stream));
-    return PETFMM_OK;
+    return m2l_tables(c);
 }
 
 Dom3 make_dom3(const petfmm_domain3d &dom, int L) {
@@ -2974,6 +2990,7 @@ int expansions3(petfmm3d_ctx *c, const uint32_t *start) {
         P3_CUDA((launch_shift3<T, false>(l, L, c->sh, start, op, rmap, par, order, me, st)));
         c->launches++;
     }
+    P3_TRY(m2l_tables(c));  // (after an option changed the kernel)
     mark3(c, PETFMM3D_STAGE_M2L);
     if (use_orbits3(c)) {
         P3_CUDA(launch_m2l_orbits<T>(L, p, start, static_cast<const T *>(c->orbits.p), rmap, par, me,

@@ -57,7 +57,8 @@ cudaError_t launch_gather_mixed(const float4 *recu, const uint32_t *perm, float4
                                 cudaStream_t st, uint64_t *launches);
 
 // ---- expansions.cu ---------------------------------------------------------
-// Operator tables for p (FP64 build, also rounded to FP32), device-resident.
+// Operator tables for p (FP64 build; the mixed path's rounded to FP32),
+// device-resident.
 struct OpTables {
     int p = 0;
     void *blob = nullptr;       // the allocation behind the tables
@@ -69,8 +70,12 @@ struct OpTables {
     float *m2l_tc = nullptr;  // hi/lo B images for the tensor-core M2L (p <= 24)
     float *m2l_tcb = nullptr; // ... the four target classes side by side (block units)
 };
-// Copied on st: the launches that follow there find them complete.
-cudaError_t build_op_tables(int p, int kernel, OpTables *out, cudaStream_t st);
+// Those of one precision, copied on st: the launches that follow there find them
+// complete.  build_tc_image: one of the tensor cores' images (mixed path, p <=
+// 24), if it is not there yet; 0.35 ms of host time at p = 17, so only where a
+// plan has such units.
+cudaError_t build_op_tables(int p, int kernel, bool fp64, OpTables *out, cudaStream_t st);
+cudaError_t build_tc_image(int kernel, bool blocks, OpTables *t, cudaStream_t st);
 // The FP64 table behind them: which = 0 M2M [c][l][k], 1 L2L [c][n][m],
 // 2 M2L [op][k][m], complex as (re, im) pairs.
 void host_op_table(int p, int kernel, int which, std::vector<double> &out);
