@@ -500,7 +500,8 @@ enum {
                                   evaluates Eq. 8's factor (1 - e^-q)/q, in units of
                                   1e-9 (1 .. 1000000; default 2500 = 2.5e-6, a quarter
                                   of the 1e-5 budget against FP64; 100 = 1e-7 is the
-                                  FP32 rounding level).  Applies from the next
+                                  FP32 rounding level, and below 420 wide cores too
+                                  are summed pair by pair).  Applies from the next
                                   evaluation. */
     PETFMM_OPT_GRAPH = 10,     /* 1: run an evaluation's launch sequence as a CUDA graph,
                                   captured on the first evaluation of a launch shape
@@ -512,7 +513,7 @@ enum {
                                   blob core is wide against a leaf (w^2 / 2 sigma^2 <= 1.95)
                                   the near kernel is smooth, and leaf pairs of many blobs
                                   are summed by expansions of it (to FP32 rounding; not
-                                  below a PETFMM_OPT_NEAR_TOL of 100); elsewhere one
+                                  below a PETFMM_OPT_NEAR_TOL of 420); elsewhere one
                                   thread per target sums its 9 leaves.  1: each pair of
                                   blobs in the same or neighbouring leaves that both hold
                                   >= 32 blobs is evaluated once, its kernel value serving

@@ -65,10 +65,13 @@ constexpr uint32_t LM_EXP = 16;   // lmask: bits 0..8 direct neighbours, 16..24 
 // Host: degree and operators
 // ----------------------------------------------------------------------------
 // Largest error of the gradient over the near domain, against its largest
-// value there, of the projection below: at most 1.2e-7 up to each bound
-// (tests/test_smooth_operator.py), so the truncation stays at FP32 rounding.
+// value there, of the projection below: at most 1.2e-7 up to each bound, and
+// another 3e-7 by the FP32 rounding of the operators' entries
+// (tests/test_smooth_operator.py).  A caller who asks for less gets pair sums.
+constexpr double kSmTol = 4.2e-7;
+
 int sm_degree(double kappa, double near_tol) {
-    if (!(near_tol >= 1e-7)) return 0;
+    if (!(near_tol >= kSmTol)) return 0;
     static const struct { double kappa; int n; } kBound[] = {
         {0.17, 8}, {0.50, 10}, {1.04, 12}, {1.95, 14}};
     for (const auto &b : kBound)

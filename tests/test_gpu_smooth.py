@@ -76,3 +76,16 @@ def test_batch_of_degrees_equals_alone():
     for w, (u, v) in zip(ws, outs):
         ua, va = G.run(w, "mixed")
         assert np.array_equal(u.cpu().numpy(), ua) and np.array_equal(v.cpu().numpy(), va)
+
+
+# A near-field tolerance below what the expansions keep (4.2e-7 of the kernel's
+# largest value, tests/test_smooth_operator.py) is kept by pair sums.  No leaf
+# has the 32 blobs of the pair kernel, so those are option 1's, bit for bit.
+@pytest.mark.parametrize("tol,summed", [(100, True), (419, True), (420, False), (2500, False)])
+def test_small_tolerances_sum_pairs(tol, summed):
+    _lib = G.lib()
+    w = wide_core(0.119, np.random.default_rng(1).integers(16, 32, (8, 8)), 2)
+    got = [G.run(w, "mixed", options={_lib.PETFMM_OPT_NEAR_TOL: tol, _lib.PETFMM_OPT_P2P_PAIRS: form})
+           for form in (2, 1)]
+    assert np.array_equal(got[0][0], got[1][0]) == summed
+    assert np.array_equal(got[0][1], got[1][1]) == summed
