@@ -353,7 +353,10 @@ int petfmm_serve_stats(petfmm_server *s, petfmm_serve_counters *out);
  * resident at that moment.  Returns the number of rounds recorded, or
  * PETFMM_EINVAL.  Host only. */
 int petfmm_serve_trace(petfmm_server *s, double *t_ms, int32_t *queued, int32_t *active, int cap);
-/* Per-request device-memory estimate used for admission (Table 1 adapted). */
+/* Per-request device-memory estimate used for admission (Table 1 adapted).  A
+ * request whose levels make the core wide against a leaf is admitted beside
+ * others with the buffers of the near field's expansions added (at most about
+ * 240 bytes a blob); alone, this is what has to fit the budget. */
 size_t petfmm_serve_estimate_bytes(int64_t n, int levels, int order, int precision);
 
 /* ---------------------------------------------------------------------- */

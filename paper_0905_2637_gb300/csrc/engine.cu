@@ -112,8 +112,6 @@ struct Problem {
 }  // namespace
 
 namespace {
-// default relative tolerance of the near-field polynomial (PETFMM_OPT_NEAR_TOL)
-constexpr double kNearTolDefault = 2.5e-6;
 // default widest tensor-core M2L unit (PETFMM_OPT_TC_SEG)
 constexpr int kTcSegDefault = 128;
 }  // namespace

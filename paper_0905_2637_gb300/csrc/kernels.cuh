@@ -272,6 +272,8 @@ cudaError_t launch_unsort(const InstDesc *insts, const uint32_t *perm, const flo
 // (instances with InstDesc::smdeg > 0).  sm_degree: the degree for
 // kappa = w^2 / 2 sigma^2 and the context's near-field tolerance, 0 where
 // the pairs are summed.
+// (kNearTolDefault: that of a new context, PETFMM_OPT_NEAR_TOL.)
+constexpr double kNearTolDefault = 2.5e-6;
 int sm_degree(double kappa, double near_tol);
 size_t sm_row_floats(int n);
 int64_t sm_max_rows(int n, int64_t blobs, int64_t leaves);

@@ -28,6 +28,7 @@
 
 #include "../../include/petfmm.h"
 #include "common.cuh"
+#include "kernels.cuh"
 
 namespace {
 
@@ -172,6 +173,19 @@ size_t estimate(int64_t n, int L, int p, int precision) {
     const size_t coef = precision == PETFMM_FP64 ? 16 : 8;
     return size_t(n) * per_particle + size_t(2.0 * lam * p * coef) + size_t(leaves * 12.0) +
            size_t((n / 32 + leaves) * 16.0) + (1u << 20);
+}
+
+// What the near field's expansions add to that where the core is wide against a
+// leaf of the request's first domain.
+size_t near_bytes(const petfmm_request &q, const petfmm_domain &dom, int L) {
+    if (q.precision == PETFMM_FP64 || q.n <= 0) return 0;
+    const double w = std::ldexp(dom.width, -L);
+    const int degree = petfmm::sm_degree(w * w / (2.0 * q.sigma * q.sigma), petfmm::kNearTolDefault);
+    if (!degree) return 0;
+    const int64_t leaves = int64_t(1) << (2 * L);
+    return size_t(leaves) * 8 +
+           size_t(petfmm::sm_max_rows(degree, q.n, leaves)) *
+               (2 * petfmm::sm_row_floats(degree) * sizeof(float) + 8);
 }
 
 // Request state comes from the server's own stream-ordered memory pool:
@@ -577,6 +591,8 @@ int petfmm_serve_submit(petfmm_server *s, const petfmm_request *req, uint64_t *t
             delete r;
             return PETFMM_ENOMEM;
         }
+        // (they keep others out, not the request itself)
+        r->bytes = std::min(r->bytes + near_bytes(q, r->dom, L), s->budget);
         if (int(s->queue.size()) >= s->max_queue || s->stop) {
             delete r;
             return PETFMM_EBUSY;

@@ -123,3 +123,24 @@ def test_release_while_worker_runs():
     results += _wait(srv, pending)
     srv.close()
     assert len(results) == 300 and all(r["status"] == 0 for r in results)
+
+
+def test_admission_counts_the_near_field_expansions():
+    # wide cores at explicit levels: a row of 392 bytes for each of 16,384 leaves,
+    # 6.4 MB beside the estimate's 8.5, so that two such requests do not fit where
+    # two with narrow cores do, and each still fits alone
+    _lib = G.lib()
+    x, y, g, _ = _patch(200, 4)
+    base = _lib.petfmm_serve_estimate_bytes(x.size, 7, 8, _lib.PETFMM_MIXED)
+    active = []
+    for sigma in (0.1, 0.002):
+        srv = _lib.Server(int(2.2 * base), max_slots=8)
+        ts = [srv.submit(x, y, g, sigma, 8, 0.01, 3, precision="mixed", levels=7) for _ in range(4)]
+        assert all(r["status"] == 0 for r in _wait(srv, ts))
+        active.append(srv.stats()["max_active"])
+        srv.close()
+        srv = _lib.Server(base, max_slots=8)
+        r = _wait(srv, [srv.submit(x, y, g, sigma, 8, 0.01, 1, precision="mixed", levels=7)])[0]
+        srv.close()
+        assert r["status"] == 0
+    assert active == [1, 2]
