@@ -462,7 +462,7 @@ int petfmm_debug_op_table(int order, int kernel, int which, double *out, int64_t
  * bad arguments. */
 int petfmm_debug_m2l_images(int order, int kernel, int blocks, float *out, int64_t cap);
 
-/* Launch plan of a batch, built on the host without touching the device
+/* Work plan of a batch, built on the host without touching the device
  * (pointers in inst are not dereferenced).  Each task is written as five
  * int64 {range, instance, level, units, first block}; range 0 the scatter of
  * staged FP32 outputs to the caller's order (1024 blobs per block),
@@ -471,10 +471,19 @@ int petfmm_debug_m2l_images(int order, int kernel, int blocks, float *out, int64
  * blocks, 70 + c the mixed path's levels without tensor-core units for orders
  * up to 8, 12, 18 and 24 (units of 128 boxes of a class, or whole rows of 64),
  * 100 + r the r-th M2M level, 200 + r the r-th L2L level (units = (box,
- * coefficient) pairs), with default options.  Ranges 5 and 70 .. describe the
- * work; its launches group M2L's and M2M / L2L's boxes their own way.  Writes
+ * coefficient) pairs), with default options.  Ranges 5, 70 .. and 100 .. are
+ * the translations as work (petfmm_debug_launches has their launches).  Writes
  * at most cap tasks and returns the total count, or PETFMM_EINVAL. */
 int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, int64_t *out, int cap);
+/* The task lists that an evaluation with default options launches, in the same
+ * form: 0 .. 4 as above, 5 the per-box M2L of the tensor cores' sparse units
+ * (target boxes of a level, 32 per block), 6 and 7 as above, 8 M2L by orbits
+ * (units = blocks, a run of target boxes of one class each), 100 + r the r-th
+ * M2M launch and 200 + r the r-th L2L launch (level: the parents'; units =
+ * blocks, a run of parents each), 9 (mixed path) the one launch, a block per
+ * instance, of the M2M and L2L of the parents' levels 2 .. level. */
+int petfmm_debug_launches(int precision, int n_inst, const petfmm_instance *inst, int64_t *out,
+                          int cap);
 
 /* Options. */
 enum {

@@ -151,6 +151,7 @@ def load():
             "petfmm_debug_smooth_operators": (I, [ctypes.c_double, P, ctypes.c_int64]),
             "petfmm_debug_smooth_table": (I, [P, I, P, ctypes.c_int64]),
             "petfmm_debug_plan": (I, [I, I, ctypes.POINTER(Instance), P, I]),
+            "petfmm_debug_launches": (I, [I, I, ctypes.POINTER(Instance), P, I]),
             "petfmm_set_option": (I, [P, I, I64]),
             "petfmm_stage_times": (I, [P, P, I]),
             "petfmm_get_stats": (I, [P, ctypes.POINTER(Stats)]),
@@ -280,15 +281,24 @@ def petfmm_debug_interaction_list(level, ix, iy):
 
 
 def petfmm_debug_plan(precision, instances):
-    """Host-side launch plan: list of (range, inst, level, units, block0)."""
+    """Host-side work plan: list of (range, inst, level, units, block0)."""
+    return _dump("petfmm_debug_plan", precision, instances)
+
+
+def petfmm_debug_launches(precision, instances):
+    """The task lists an evaluation launches, in the same form."""
+    return _dump("petfmm_debug_launches", precision, instances)
+
+
+def _dump(name, precision, instances):
     arr = (Instance * max(1, len(instances)))()
     for i, it in enumerate(instances):
         arr[i] = Instance(Domain(*map(float, it["domain"])), int(it.get("levels", 0)),
                           int(it["order"]), float(it["sigma"]), int(it["n"]), 8, 8, 8, 8, 8)
-    n = _ck(load().petfmm_debug_plan(int(precision), len(instances), arr, None, 0), "petfmm_debug_plan")
+    fn = getattr(load(), name)
+    n = _ck(fn(int(precision), len(instances), arr, None, 0), name)
     out = np.zeros((max(n, 1), 5), np.int64)
-    _ck(load().petfmm_debug_plan(int(precision), len(instances), arr, out.ctypes.data, n),
-        "petfmm_debug_plan")
+    _ck(fn(int(precision), len(instances), arr, out.ctypes.data, n), name)
     return out[:n]
 
 

@@ -75,16 +75,11 @@ struct Plan {
     TaskRange orbits;
     int orbit_ni = 0;
     size_t orbit_smem = 0;
-    // the plan dump's units of 128 (or whole rows of 64) target boxes of those
-    // levels, by order class (p <= 8, 12, 18, 24)
-    static constexpr int kTileClasses = 4;
-    TaskRange m2l_tile[kTileClasses];
     // M2M and L2L, in launch order: a task's units are runs of parents (on the
     // mixed path the top levels run apart, shift_top)
     std::vector<TaskRange> up, down;
     size_t shift_smem = 0, shift_top_smem = 0;
     bool shift_top = false;
-    std::vector<TaskRange> m2m, l2l;  // the plan dump's (box, coefficient) pairs
     int64_t N = 0, nleaves = 0, nstart = 0, ncoef = 0, items_cap = 0;
     int nbits = 0, pmax = 1, Lmax = 0;
     int deg = 0, general = 0;          // mixed P2P variant (max over instances)
@@ -463,13 +458,10 @@ void flatten_tasks(Plan &pl) {
     put(pl.m2l);
     put(pl.m2l_tc);
     put(pl.m2l_tcb);
-    for (TaskRange &r : pl.m2l_tile) put(r);
     put(pl.m2l_log);
     put(pl.orbits);
     for (TaskRange &r : pl.up) put(r);
     for (TaskRange &r : pl.down) put(r);
-    for (TaskRange &r : pl.m2m) put(r);
-    for (TaskRange &r : pl.l2l) put(r);
 }
 
 // Fewest block units at levels 5 to 7 for which those levels run as blocks
@@ -482,14 +474,6 @@ constexpr int64_t kTcbShallowMinUnits = 512;
 // 0.036.  On the mixed path units of 128 were as fast or faster everywhere.
 constexpr int64_t kOrbitLargeUnits = 608;
 
-// The plan dump's units of a level without tensor-core units.
-int64_t dump_tile_units(int l) {
-    const int W = 1 << (l - 1), seg = std::min(W, 128);
-    const int rows = W < 128 ? std::max(1, std::min(64 / seg, W)) : 1;
-    return int64_t(4) * (W / rows) * (W / seg);
-}
-int tile_class(int p) { return p <= 8 ? 0 : p <= 12 ? 1 : p <= 18 ? 2 : 3; }
-
 // Laplace kernel, mixed path: blobs per leaf (empty ones included) up to which
 // one thread per target sums a tree's near field; denser trees take work items of
 // 64 targets, two per lane, which share each source load.
@@ -497,7 +481,7 @@ constexpr int64_t kLaplaceDirectMax = 64;
 
 // near: PETFMM_OPT_P2P_PAIRS
 int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_segmax, double near_tol,
-               int near, const std::vector<Problem> &probs, Plan &pl, bool dump = false) {
+               int near, const std::vector<Problem> &probs, Plan &pl) {
     pl = Plan();
     const int ni = int(probs.size());
     int inst_bits = 0;
@@ -625,14 +609,14 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
             }
         }
     }
-    // per box: the sparse units of the tensor cores' levels (the dump lists
-    // every level); by orbits: the levels without tensor-core units
+    // per box: the sparse units of the tensor cores' levels; by orbits: the levels
+    // without tensor-core units
     int64_t large = 0;
     for (int i = 0; i < ni; ++i) {
         const InstDesc &d = pl.inst[i];
         for (int l = 2; l <= d.L; ++l) {
             const bool tc = ((d.tc_levels | d.tcb_levels) >> l) & 1u;
-            if (tc || dump) add_task(pl.m2l, i, l, int64_t(1) << (2 * l), M2L_BOXES);
+            if (tc) add_task(pl.m2l, i, l, int64_t(1) << (2 * l), M2L_BOXES);
             if (!tc) large += m2l_orbit_units(d.p, l, M2L_ORBIT_NI_MAX);
         }
     }
@@ -646,15 +630,6 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
                                      m2l_orbit_smem(d.p, pl.orbit_ni, precision == PETFMM_FP64));
         }
     }
-    if (dump && precision == PETFMM_MIXED)
-        for (int cls = 0; cls < Plan::kTileClasses; ++cls)
-            for (int i = 0; i < ni; ++i) {
-                const InstDesc &d = pl.inst[i];
-                if (d.p > 24 || tile_class(d.p) != cls) continue;
-                for (int l = 2; l <= d.L; ++l)
-                    if (!(((d.tc_levels | d.tcb_levels) >> l) & 1u))
-                        add_task(pl.m2l_tile[cls], i, l, dump_tile_units(l), 1);
-            }
     // M2M rounds: round r computes level L_i - 1 - r of every instance, down to
     // the first level the top launch does not take; L2L rounds start there
     const int bottom = precision == PETFMM_FP64 ? 2 : kShiftTop + 1;
@@ -673,27 +648,6 @@ int build_plan(int precision, int kernel, bool use_tc, int tc_blocks, int tc_seg
         if (precision == PETFMM_MIXED && d.L >= 3) {
             pl.shift_top = true;
             pl.shift_top_smem = std::max(pl.shift_top_smem, shift_smem(d.p, false, true));
-        }
-    }
-    if (dump) {
-        // M2M rounds: round r computes level L_i - 1 - r (>= 2) of every instance.
-        for (int r = 0; r + 3 <= Lmax; ++r) {
-            TaskRange tr;
-            for (int i = 0; i < ni; ++i) {
-                const int l = pl.inst[i].L - 1 - r;
-                if (l >= 2) add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
-            }
-            if (tr.count) pl.m2m.push_back(tr);
-        }
-        // L2L rounds: round r translates level 2 + r into level 3 + r.
-        for (int r = 0; r + 3 <= Lmax; ++r) {
-            TaskRange tr;
-            for (int i = 0; i < ni; ++i) {
-                const int l = 3 + r;
-                if (l <= pl.inst[i].L)
-                    add_task(tr, i, l, (int64_t(1) << (2 * l)) * pl.inst[i].p, EXP_THREADS);
-            }
-            if (tr.count) pl.l2l.push_back(tr);
         }
     }
     pl.items_cap = items_cap;
@@ -1600,39 +1554,98 @@ int petfmm_tune_batch(petfmm_ctx *c, int n_inst, const petfmm_instance *inst, in
     return PETFMM_OK;
 }
 
-int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, int64_t *out, int cap) {
+// Rows {id, instance, level, units, first block} of a dump.
+struct DumpRows {
+    int64_t *out;
+    int cap, n;
+    void add(int64_t id, const Task &t) {
+        if (n < cap) {
+            int64_t *o = out + 5 * size_t(n);
+            o[0] = id; o[1] = t.inst; o[2] = t.level; o[3] = t.count; o[4] = t.block0;
+        }
+        ++n;
+    }
+    void add(int64_t id, const std::vector<Task> &tasks) {
+        for (const Task &t : tasks) add(id, t);
+    }
+    void add(int64_t id, const Plan &pl, const TaskRange &r) {
+        for (int i = 0; i < r.count; ++i) add(id, pl.tasks[size_t(r.first + i)]);
+    }
+};
+
+// The plan of a context with default options.
+static int dump_plan(int precision, int n_inst, const petfmm_instance *inst, const int64_t *out,
+                     int cap, Plan &pl) {
     if (n_inst < 0 || (n_inst > 0 && !inst) || cap < 0 || (cap > 0 && !out)) return PETFMM_EINVAL;
     if (precision != PETFMM_FP64 && precision != PETFMM_MIXED) return PETFMM_EINVAL;
     std::vector<Problem> probs;
-    int rc = problems_from(n_inst, inst, probs);
+    const int rc = problems_from(n_inst, inst, probs);
     if (rc) return rc;
+    return build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, 2, probs, pl);
+}
+
+int petfmm_debug_plan(int precision, int n_inst, const petfmm_instance *inst, int64_t *out, int cap) {
     Plan pl;
-    rc = build_plan(precision, KERNEL_VORTEX, true, 0, kTcSegDefault, kNearTolDefault, 2, probs, pl,
-                    true);
+    const int rc = dump_plan(precision, n_inst, inst, out, cap, pl);
     if (rc) return rc;
-    int n = 0;
-    auto emit = [&](int64_t id, const TaskRange &r) {
-        for (int i = 0; i < r.count; ++i) {
-            const Task &t = pl.tasks[size_t(r.first + i)];
-            if (n < cap) {
-                int64_t *o = out + 5 * size_t(n);
-                o[0] = id; o[1] = t.inst; o[2] = t.level; o[3] = t.count; o[4] = t.block0;
-            }
-            ++n;
-        }
+    DumpRows rows{out, cap, 0};
+    rows.add(0, pl, pl.outscatter);
+    rows.add(1, pl, pl.start);
+    rows.add(2, pl, pl.particles);
+    rows.add(3, pl, pl.leaves_p2m);
+    rows.add(4, pl, pl.leaves_wl);
+    // the translations as work, apart from the launches that do it: every list
+    // by itself, its rows numbered through
+    auto list = [&](int64_t id, int64_t per_block, auto &&units) {
+        TaskRange tr;
+        for (int i = 0; i < int(pl.inst.size()); ++i)
+            for (int l = 2; l <= pl.inst[size_t(i)].L; ++l)
+                add_task(tr, i, l, units(pl.inst[size_t(i)], l), per_block);
+        rows.add(id, tr.list);
     };
-    emit(0, pl.outscatter);
-    emit(1, pl.start);
-    emit(2, pl.particles);
-    emit(3, pl.leaves_p2m);
-    emit(4, pl.leaves_wl);
-    emit(5, pl.m2l);
-    emit(6, pl.m2l_tc);
-    emit(7, pl.m2l_tcb);
-    for (int cls = 0; cls < Plan::kTileClasses; ++cls) emit(70 + cls, pl.m2l_tile[cls]);
-    for (size_t r = 0; r < pl.m2m.size(); ++r) emit(100 + int64_t(r), pl.m2m[r]);
-    for (size_t r = 0; r < pl.l2l.size(); ++r) emit(200 + int64_t(r), pl.l2l[r]);
-    return n;
+    list(5, M2L_BOXES, [](const InstDesc &, int l) { return int64_t(1) << (2 * l); });
+    rows.add(6, pl, pl.m2l_tc);
+    rows.add(7, pl, pl.m2l_tcb);
+    for (int cls = 0; precision == PETFMM_MIXED && cls < 4; ++cls)
+        list(70 + cls, 1, [&](const InstDesc &d, int l) {
+            const int of = d.p <= 8 ? 0 : d.p <= 12 ? 1 : d.p <= 18 ? 2 : d.p <= 24 ? 3 : 4;
+            if (of != cls || ((d.tc_levels | d.tcb_levels) >> l) & 1u) return int64_t(0);
+            const int W = 1 << (l - 1), seg = std::min(W, 128);
+            const int r = W < 128 ? std::max(1, std::min(64 / seg, W)) : 1;
+            return int64_t(4) * (W / r) * (W / seg);
+        });
+    for (int r = 0; r + 3 <= pl.Lmax; ++r)
+        list(100 + r, EXP_THREADS, [&](const InstDesc &d, int l) {
+            return l == d.L - 1 - r ? (int64_t(1) << (2 * l)) * d.p : 0;
+        });
+    for (int r = 0; r + 3 <= pl.Lmax; ++r)
+        list(200 + r, EXP_THREADS, [&](const InstDesc &d, int l) {
+            return l == 3 + r ? (int64_t(1) << (2 * l)) * d.p : 0;
+        });
+    return rows.n;
+}
+
+int petfmm_debug_launches(int precision, int n_inst, const petfmm_instance *inst, int64_t *out,
+                          int cap) {
+    Plan pl;
+    const int rc = dump_plan(precision, n_inst, inst, out, cap, pl);
+    if (rc) return rc;
+    DumpRows rows{out, cap, 0};
+    const TaskRange *lists[] = {&pl.outscatter, &pl.start,  &pl.particles, &pl.leaves_p2m, &pl.leaves_wl,
+                                &pl.m2l,        &pl.m2l_tc, &pl.m2l_tcb,   &pl.orbits};
+    for (int id = 0; id < 9; ++id) rows.add(id, pl, *lists[id]);
+    if (pl.shift_top)
+        for (int i = 0; i < int(pl.inst.size()); ++i) {
+            Task t{};
+            t.inst = i;
+            t.level = std::min(pl.inst[size_t(i)].L - 1, kShiftTop);
+            t.count = 1;
+            t.block0 = i;
+            rows.add(9, t);
+        }
+    for (size_t r = 0; r < pl.up.size(); ++r) rows.add(100 + int64_t(r), pl, pl.up[r]);
+    for (size_t r = 0; r < pl.down.size(); ++r) rows.add(200 + int64_t(r), pl, pl.down[r]);
+    return rows.n;
 }
 
 int petfmm_choose_levels(int64_t n, int order, double sigma, const petfmm_domain *dom) {

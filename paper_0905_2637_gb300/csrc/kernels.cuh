@@ -189,7 +189,7 @@ constexpr int M2L_WARPS = 4;      // warps per block
 // scheduling.
 constexpr int BOX_RUN = 8;
 constexpr int M2L_BOXES = M2L_WARPS * BOX_RUN;   // target boxes per block
-constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block in the plan dump's M2M / L2L
+constexpr int EXP_THREADS = 256;  // (box, coefficient) pairs per block of petfmm_debug_plan's M2M / L2L
 
 // ---- p2p.cu ----------------------------------------------------------------
 // Work list: items (inst, leaf, first target rank, target count) for every
