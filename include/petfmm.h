@@ -405,6 +405,11 @@ int petfmm_debug_interaction_list(int level, int ix, int iy, int32_t *out);
  * PETFMM_OK or PETFMM_EINVAL. */
 int petfmm_debug_near_fit(double sigma, double wleaf, double tol, double *out);
 
+/* The FP64 path's pair factor g(q) = (1 - e^-q) / q, as its kernels compute it,
+ * of n values q >= 0 (device arrays, on the context's stream; a context with
+ * PETFMM_FP64, else PETFMM_EINVAL). */
+int petfmm_debug_pair_factor(petfmm_ctx *ctx, int64_t n, const double *q, double *g);
+
 /* The mixed path's near field where the blob core is wide against a leaf
  * (kappa = w^2 / 2 sigma^2 <= 1.95, leaf width w): Phi(d) = Ein(kappa |d|^2) /
  * (2 kappa), whose turned gradient is the pair velocity (-d_y, d_x) g(kappa
@@ -776,6 +781,9 @@ enum { PETFMM3D_SHIFT_M2M = 0, PETFMM3D_SHIFT_L2L = 1 };
  * rounds it to FP32); cap >= p^4 doubles; PETFMM_EINVAL for a bad kind,
  * octant, order or cap. */
 int petfmm3d_debug_shift_operator(int order, int kind, int octant, double *out, int64_t cap);
+/* 1 / sqrt(x) as the FP64 near field computes it, of n values x > 0 (device
+ * arrays, on the context's stream). */
+int petfmm3d_debug_rsqrt(petfmm3d_ctx *ctx, int64_t n, const double *x, double *y);
 int petfmm3d_destroy(petfmm3d_ctx *ctx);
 
 #ifdef __cplusplus

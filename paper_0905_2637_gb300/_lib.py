@@ -149,6 +149,7 @@ def load():
             "petfmm_debug_op_table": (I, [I, I, I, P, ctypes.c_int64]),
             "petfmm_debug_near_fit": (I, [ctypes.c_double, ctypes.c_double, ctypes.c_double, P]),
             "petfmm_debug_smooth_operators": (I, [ctypes.c_double, P, ctypes.c_int64]),
+            "petfmm_debug_pair_factor": (I, [P, I64, P, P]),
             "petfmm_debug_smooth_table": (I, [P, I, P, ctypes.c_int64]),
             "petfmm_debug_plan": (I, [I, I, ctypes.POINTER(Instance), P, I]),
             "petfmm_debug_launches": (I, [I, I, ctypes.POINTER(Instance), P, I]),
@@ -420,6 +421,13 @@ class Context:
         st = Stats()
         _ck(load().petfmm_get_stats(self.handle, ctypes.byref(st)), "petfmm_get_stats")
         return {f: getattr(st, f) for f, _ in Stats._fields_}
+
+    def debug_pair_factor(self, q):
+        """g(q) of a float64 device tensor as the FP64 near field takes it."""
+        g = _torch().empty_like(q)
+        _ck(load().petfmm_debug_pair_factor(self.handle, q.numel(), q.data_ptr(), g.data_ptr()),
+            "petfmm_debug_pair_factor")
+        return g
 
     def debug_smooth_table(self, inst=0):
         """(degree, operators as petfmm_debug_smooth_operators gives them) of an

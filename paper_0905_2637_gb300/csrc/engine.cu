@@ -1554,6 +1554,11 @@ int petfmm_tune_batch(petfmm_ctx *c, int n_inst, const petfmm_instance *inst, in
     return PETFMM_OK;
 }
 
+int petfmm_debug_pair_factor(petfmm_ctx *c, int64_t n, const double *q, double *g) {
+    if (!c || n < 0 || (n > 0 && (!q || !g)) || !c->gtab.p) return PETFMM_EINVAL;
+    return cuda_status(launch_g64(q, g, n, static_cast<const double *>(c->gtab.p), c->stream));
+}
+
 // Rows {id, instance, level, units, first block} of a dump.
 struct DumpRows {
     int64_t *out;

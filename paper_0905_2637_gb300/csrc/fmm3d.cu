@@ -2228,7 +2228,8 @@ __global__ void __launch_bounds__(256) k3_near_final(int L, int p, double w,
 
 // 1/sqrt(x): the hardware's approximation y and one step of Householder's
 // third-order iteration, y (1 + e / 2 + 3 e^2 / 8) with e = 1 - x y^2
-// (|e| < 2^-18 leaves |e|^3 below 2^-54): five FP64 operations, where a
+// (|e| < 2^-18 leaves |e|^3 below 2^-54; within 1.5 ulp,
+// tests/test_gpu_factors.py): five FP64 operations, where a
 // division by sqrt took about thirty.  Subnormal, infinite and NaN x (the
 // approximation flushes or saturates there) by division.
 __device__ __forceinline__ double rsqrt_f64(double x) {
@@ -2238,6 +2239,12 @@ __device__ __forceinline__ double rsqrt_f64(double x) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
     const double e = fma(-x * y, y, 1.0);
     return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+__global__ void __launch_bounds__(256) k3_rsqrt64(const double *__restrict__ x,
+                                                  double *__restrict__ y, int64_t n) {
+    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+    if (i < n) y[i] = rsqrt_f64(x[i]);
 }
 
 // The FP64 path's leaf pairs not evaluated pairwise: global coordinates; work
@@ -3364,6 +3371,12 @@ int petfmm3d_debug_shift_operator(int order, int kind, int octant, double *out, 
     if (cap < nr * nr) return PETFMM_EINVAL;
     host_shift_real(order, kind == PETFMM3D_SHIFT_M2M ? 0 : 1, octant, out);
     return PETFMM_OK;
+}
+
+int petfmm3d_debug_rsqrt(petfmm3d_ctx *c, int64_t n, const double *x, double *y) {
+    if (!c || n < 0 || (n > 0 && (!x || !y))) return PETFMM_EINVAL;
+    if (n > 0) k3_rsqrt64<<<unsigned((n + 255) / 256), 256, 0, c->stream>>>(x, y, n);
+    return cudaGetLastError() == cudaSuccess ? PETFMM_OK : PETFMM_ECUDA;
 }
 
 int petfmm3d_destroy(petfmm3d_ctx *c) {

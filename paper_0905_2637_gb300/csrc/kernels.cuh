@@ -209,6 +209,8 @@ cudaError_t launch_p2p_f64(int grid, const uint4 *items, uint32_t *ctrl, const I
 // The table behind its kernel factor (vortex), G64_WORDS doubles.
 constexpr int G64_CELLS = 640, G64_TERMS = 7, G64_WORDS = G64_CELLS * (G64_TERMS + 1);
 const double *host_g64_table();
+// g(q) by it, on the device.
+cudaError_t launch_g64(const double *q, double *g, int64_t n, const double *gtab, cudaStream_t st);
 // Mixed near field from work items, every leaf against all 9 leaves: own[r] =
 // the near sum of sorted blob r (launch_p2p_final then adds the far field).
 cudaError_t launch_p2p_mixed(int grid, int deg, int general, const uint4 *items, uint32_t *ctrl,

@@ -421,8 +421,8 @@ __global__ void __launch_bounds__(P2P_THREADS, 5) k_p2p_mixed(
 // Bound by the FP64 pipe (two lanes a cycle and SM on this part; every other
 // instruction is nearly free beside it), so a pair's factor g(q) = (1 - e^-q)
 // / q comes without division or exponential: below q = 40 a polynomial of
-// degree 6 in q on 640 cells of width 1/16, read from shared memory (about
-// 1 ulp, as -expm1(-q) / q is), above it 1 / q (e^-40 is below the rounding)
+// degree 6 in q on 640 cells of width 1/16, read from shared memory (within 2
+// ulp, tests/test_gpu_factors.py), above it 1 / q (e^-40 is below the rounding)
 // from the hardware's approximate reciprocal y and the series step
 // y (1 + e + e^2), e = 1 - q y.  15 operations a pair where expm1 and a
 // division took about 45.  Items hold 16 targets: two lanes a target, so that
@@ -489,6 +489,18 @@ const double *host_g64_table() {
         return out;
     }();
     return table.data();
+}
+
+__global__ void __launch_bounds__(256) k_g64(const double *__restrict__ q, double *__restrict__ g,
+                                             int64_t n, const double *__restrict__ tab) {
+    const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+    if (i < n) g[i] = g_f64(q[i], tab);
+}
+
+cudaError_t launch_g64(const double *q, double *g, int64_t n, const double *gtab, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_g64<<<unsigned((n + 255) / 256), 256, 0, st>>>(q, g, n, gtab);
+    return cudaGetLastError();
 }
 
 template <bool LAP>

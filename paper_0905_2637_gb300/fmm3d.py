@@ -42,6 +42,7 @@ def lib3():
                 ("petfmm3d_launches", ctypes.c_uint64, [P]),
                 ("petfmm3d_debug_m2l_operator", I, [I, I, I, I, P, I64]),
                 ("petfmm3d_debug_shift_operator", I, [I, I, I, P, I64]),
+                ("petfmm3d_debug_rsqrt", I, [P, I64, P, P]),
                 ("petfmm3d_destroy", I, [P])):
             fn = getattr(lib, name)
             fn.restype = res
@@ -143,6 +144,13 @@ class Context3D:
 
     def launches(self):
         return int(lib3().petfmm3d_launches(self.handle))
+
+    def debug_rsqrt(self, x):
+        """1 / sqrt(x) of a float64 device tensor as the FP64 near field takes it."""
+        y = _lib._torch().empty_like(x)
+        _lib._ck(lib3().petfmm3d_debug_rsqrt(self.handle, x.numel(), x.data_ptr(), y.data_ptr()),
+                 "petfmm3d_debug_rsqrt")
+        return y
 
     def debug_tree(self, n):
         """(sorted keys, perm, leaf starts) of the last evaluation."""
