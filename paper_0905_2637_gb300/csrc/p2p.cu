@@ -31,6 +31,7 @@
 //
 // FP64 path: the same loop in FP64, g from a table (see k_p2p_f64).
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "kernels.cuh"
@@ -539,29 +540,36 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_f64(
         double su = 0.0, sv = 0.0;
         const uint32_t *st = start + d.soff;
         const int nside = 1 << L;
-        for (int dy = -1; dy <= 1; ++dy) {
-            const int sy = iy + dy;
-            if (sy < 0 || sy >= nside) continue;
-            for (int dx = -1; dx <= 1; ++dx) {
-                const int sx = ix + dx;
-                if (sx < 0 || sx >= nside) continue;
-                const uint32_t nm = morton_key(uint32_t(sx), uint32_t(sy));
-                const uint32_t j0 = st[nm], j1 = st[nm + 1];
+        auto sum = [&](auto guard) {
+            su = sv = 0.0;
+            for (int dy = -1; dy <= 1; ++dy) {
+                const int sy = iy + dy;
+                if (sy < 0 || sy >= nside) continue;
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const int sx = ix + dx;
+                    if (sx < 0 || sx >= nside) continue;
+                    const uint32_t nm = morton_key(uint32_t(sx), uint32_t(sy));
+                    const uint32_t j0 = st[nm], j1 = st[nm + 1];
 #pragma unroll 2
-                for (uint32_t j = j0 + grp; j < j1; j += S) {
-                    const double ddx = x - __ldg(xs + j), ddy = y - __ldg(ys + j);
-                    const double r2 = fma(ddx, ddx, ddy * ddy);
-                    if (LAP) {
-                        if (r2 > 0.0) su += __ldg(gs + j) * (0.5 * log(r2));
-                    } else {
-                        // (the self pair has ddx = ddy = 0 and adds zero)
-                        const double f = __ldg(gs + j) * g_f64(r2 * inv2s2, tab);
-                        su = fma(-ddy, f, su);
-                        sv = fma(ddx, f, sv);
+                    for (uint32_t j = j0 + grp; j < j1; j += S) {
+                        const double ddx = x - __ldg(xs + j), ddy = y - __ldg(ys + j);
+                        const double r2 = fma(ddx, ddx, ddy * ddy);
+                        if (LAP) {
+                            if (r2 > 0.0) su += __ldg(gs + j) * (0.5 * log(r2));
+                        } else {
+                            // (the self pair and coincident blobs have ddx = ddy =
+                            // 0 and add zero, unless the strength is infinite)
+                            if (decltype(guard)::value && !(r2 > 0.0)) continue;
+                            const double f = __ldg(gs + j) * g_f64(r2 * inv2s2, tab);
+                            su = fma(-ddy, f, su);
+                            sv = fma(ddx, f, sv);
+                        }
                     }
                 }
             }
-        }
+        };
+        sum(std::false_type());
+        if (!LAP && (isnan(su) || isnan(sv))) sum(std::true_type());
         for (uint32_t o = W; o < 32u; o <<= 1) {
             su += __shfl_xor_sync(0xffffffffu, su, int(o));
             sv += __shfl_xor_sync(0xffffffffu, sv, int(o));

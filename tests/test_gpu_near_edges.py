@@ -126,3 +126,19 @@ def test_pair_factor_keeps_fp32_accuracy(kappa):
     err = np.hypot(u[:, 0].cpu().numpy() + f * ey, v[:, 0].cpu().numpy() - f * ex) / (f * np.sqrt(r2))
     rms = np.sqrt((err.reshape(-1, per) ** 2).mean(1))
     assert np.all(rms <= 2e-7), dict(zip(edges.round(2), rms))
+
+
+# A blob of infinite strength moves the others, not itself nor one at its place.
+def test_fp64_infinite_strength_adds_nothing_to_itself():
+    x = np.array([0.3, 0.3, 0.31, 0.8])
+    w = W.Workload("inf", x, x[::-1].copy(), np.array([np.inf, 2.0, 1.0, -1.0]), 0.05, (0, 0, 1.0), 1, 4,
+                   "f64")
+    w.y[:2] = 0.4
+    u, v = G.run(w, "fp64")
+    d = np.hypot(w.x[:, None] - w.x, w.y[:, None] - w.y)
+    f = np.where(d > 0, -np.expm1(-d ** 2 / (2 * w.sigma ** 2)) / (2 * np.pi * np.where(d > 0, d, 1) ** 2), 0)
+    for i in (0, 1):
+        k = [2, 3]  # the blobs elsewhere
+        want = (-(f[i, k] * w.gamma[k] * (w.y[i] - w.y[k])).sum(), (f[i, k] * w.gamma[k] * (w.x[i] - w.x[k])).sum())
+        assert np.allclose((u[i], v[i]), want, rtol=1e-12, atol=0)
+    assert np.all(np.isinf(u[2:])) and np.all(np.isinf(v[2:]))
