@@ -373,6 +373,10 @@ size_t petfmm_serve_estimate_bytes(int64_t n, int levels, int order, int precisi
  * PETFMM_EINVAL for a NULL pointer.  Section 6.2's verification support;
  * the paper has no counterpart of the checks themselves. */
 int petfmm_debug_checks(uint32_t *lines);
+/* The same of every file with checks: tree.cu, expansions.cu, p2p.cu, smooth.cu,
+ * shifts.cu, m2l_orbits.cu, fmm3d.cu, the first cap of them to lines (all are
+ * cleared).  Returns their number, 0 in the regular build, or PETFMM_EINVAL. */
+int petfmm_debug_checks_by_file(uint32_t *lines, int cap);
 
 /* Tree of the last petfmm_evaluate (after petfmm_sync): host arrays
  * keys[n] (Morton key of each particle, input order), perm[n] (input index

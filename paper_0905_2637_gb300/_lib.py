@@ -161,6 +161,7 @@ def load():
             "petfmm_measure_peaks": (I, [ctypes.POINTER(Peaks)]),
             "petfmm_tree_noalloc": (I, [ctypes.POINTER(Domain), I, I, I64, P, P, P, P, P, P]),
             "petfmm_debug_checks": (I, [P]),
+            "petfmm_debug_checks_by_file": (I, [P, I]),
             "petfmm_rule_levels": (I, [ctypes.POINTER(LevelRule), I, I64, I, D,
                                        ctypes.POINTER(Domain)]),
             "petfmm_set_level_rules": (I, [P, ctypes.POINTER(LevelRule), I]),

@@ -1801,10 +1801,24 @@ int petfmm_debug_checks(uint32_t *lines) {
     lines[0] = pf_checks_tree();
     lines[1] = pf_checks_expansions();
     lines[2] = pf_checks_p2p();
-    const unsigned sm_line = pf_checks_smooth();
-    if (!lines[2]) lines[2] = sm_line;
 #ifdef PETFMM_CHECKS
     return 3;
+#else
+    return 0;
+#endif
+}
+
+int petfmm_debug_checks_by_file(uint32_t *lines, int cap) {
+    if (!lines || cap < 0) return PETFMM_EINVAL;
+    unsigned (*const files[])() = {pf_checks_tree,   pf_checks_expansions, pf_checks_p2p, pf_checks_smooth,
+                                   pf_checks_shifts, pf_checks_orbits,     pf_checks_fmm3d};
+    const int n = int(sizeof(files) / sizeof(files[0]));
+    for (int i = 0; i < n; ++i) {
+        const uint32_t line = files[i]();
+        if (i < cap) lines[i] = line;
+    }
+#ifdef PETFMM_CHECKS
+    return n;
 #else
     return 0;
 #endif

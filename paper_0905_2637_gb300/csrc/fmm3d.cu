@@ -53,6 +53,9 @@
 #include "kernels.cuh"
 #include "tcgen05.cuh"
 
+namespace petfmm {
+PF_DEFINE_CHECK_READER(fmm3d)
+}
 using namespace petfmm;
 
 namespace {
@@ -591,7 +594,8 @@ __global__ void __launch_bounds__(ORB_THREADS) k3_m2l_orbits(
 #pragma unroll
             for (int s = 0; s < 8; ++s) {
                 const int sb = srow[8 * t + s];
-                v[s] = sb >= 0 ? lev[int64_t(sb) * (2 * nc) + soff[k]] : T(0);
+                v[s] = sb >= 0 && PF_IN(sb, int64_t(1) << (3 * l)) ? lev[int64_t(sb) * (2 * nc) + soff[k]]
+                                                                    : T(0);
             }
             // butterflies along the axes with both signs (entries reflected
             // along another axis are not there yet), then copies

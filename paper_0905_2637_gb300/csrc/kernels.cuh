@@ -15,6 +15,9 @@ unsigned pf_checks_tree();
 unsigned pf_checks_expansions();
 unsigned pf_checks_p2p();
 unsigned pf_checks_smooth();
+unsigned pf_checks_shifts();
+unsigned pf_checks_orbits();
+unsigned pf_checks_fmm3d();
 
 // ---- tree.cu ---------------------------------------------------------------
 // Sec. 2.1 binning + z-order key of every particle (composite key for batches);

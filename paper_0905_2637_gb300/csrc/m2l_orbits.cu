@@ -198,7 +198,8 @@ __global__ void __launch_bounds__(ORB_THREADS) k_m2l_orbits(
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int s = srow[(o * rows + b) * 4 + r];
-            a[r] = s >= 0 ? lev[int64_t(s) * p + k] : orb_c<C2>(R(0), R(0));
+            a[r] = s >= 0 && PF_IN(s, int64_t(1) << (2 * l)) ? lev[int64_t(s) * p + k]
+                                                              : orb_c<C2>(R(0), R(0));
         }
     };
     C2 ahead[4];
@@ -354,5 +355,7 @@ template cudaError_t launch_m2l_orbits<double>(const Task *, int, int64_t, int, 
 template cudaError_t launch_m2l_orbits<float>(const Task *, int, int64_t, int, size_t,
                                               const InstDesc *, const uint32_t *, const float2 *,
                                               float2 *, cudaStream_t, uint64_t *);
+
+PF_DEFINE_CHECK_READER(orbits)
 
 }  // namespace petfmm

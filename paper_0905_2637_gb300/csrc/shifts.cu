@@ -170,7 +170,7 @@ __device__ __forceinline__ void sh_m2m(const ShMem<R> &m, const InstDesc &d, int
         for (int r = 0; r < 4; ++r) {
             a[r].x = a[r].y = R(0);
             const int c = m.child[4 * b + r];
-            if (c >= 0) a[r] = kids[int64_t(c) * p + k];
+            if (c >= 0 && PF_IN(c, int64_t(4) << (2 * l))) a[r] = kids[int64_t(c) * p + k];
         }
         const C2 s02 = sh_add(a[0], a[2]), d02 = sh_sub(a[0], a[2]);
         const C2 s13 = sh_add(a[1], a[3]), d13 = sh_sub(a[1], a[3]);
@@ -240,7 +240,7 @@ __device__ __forceinline__ void sh_l2l(const ShMem<R> &m, const InstDesc &d, int
             for (int r = 0; r < 4; ++r) {
                 const int kid = m.child[4 * b + r];
                 own[which][r].x = own[which][r].y = R(0);
-                if (kid >= 0) own[which][r] = kids[int64_t(kid) * p + (which ? n2 : n1)];
+                if (kid >= 0 && PF_IN(kid, int64_t(4) << (2 * l))) own[which][r] = kids[int64_t(kid) * p + (which ? n2 : n1)];
             }
 #pragma unroll
         for (int which = 0; which < 2; ++which) {
@@ -282,7 +282,7 @@ __device__ __forceinline__ void sh_l2l(const ShMem<R> &m, const InstDesc &d, int
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 const int kid = m.child[4 * b + r];
-                if (kid >= 0)
+                if (kid >= 0 && PF_IN(kid, int64_t(4) << (2 * l)))
                     kids[int64_t(kid) * p + c] = sh_add(own[which][r], sh_mul(f[r], m.em[c]));
             }
         }
@@ -404,5 +404,7 @@ template cudaError_t launch_shift<float>(bool, const Task *, int, int64_t, size_
                                          const uint32_t *, float2 *, cudaStream_t, uint64_t *);
 template cudaError_t launch_shift<double>(bool, const Task *, int, int64_t, size_t, const InstDesc *,
                                           const uint32_t *, double2 *, cudaStream_t, uint64_t *);
+
+PF_DEFINE_CHECK_READER(shifts)
 
 }  // namespace petfmm
