@@ -787,22 +787,21 @@ template <int N>
 static cudaError_t sm_near(const uint32_t *ctrl, const InstDesc *insts, const uint32_t *start,
                            const float4 *rec, const SmBufs &sb, cudaStream_t st,
                            uint64_t *launches) {
-    static int per_sm_m = 0, per_sm_t = 0;
-    if (!per_sm_t) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_m, k_sm_moments<N>, 128, 0);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_t, k_sm_translate<N>,
-                                                      SmTile<N>::THREADS, 0);
-        if (per_sm_m < 1) per_sm_m = 1;
-        if (per_sm_t < 1) per_sm_t = 1;
-    }
+    // (found once, by whichever thread comes first; the others wait for it)
+    static const int2 per_sm = [] {
+        int2 n = make_int2(0, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.x, k_sm_moments<N>, 128, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n.y, k_sm_translate<N>, SmTile<N>::THREADS, 0);
+        return make_int2(std::max(n.x, 1), std::max(n.y, 1));
+    }();
     const int64_t sms = device_sm_count();
     if (sb.rows <= 0) return cudaSuccess;
-    const int64_t gm = std::min<int64_t>(sms * per_sm_m, (sb.rows + 3) / 4);
+    const int64_t gm = std::min<int64_t>(sms * per_sm.x, (sb.rows + 3) / 4);
     k_sm_moments<N><<<unsigned(gm), 128, 0, st>>>(ctrl, insts, start, rec, sb);
     PF_LAUNCHED(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int64_t gt = std::min<int64_t>(sms * per_sm_t, (sb.rows + SM_TGT - 1) / SM_TGT);
+    const int64_t gt = std::min<int64_t>(sms * per_sm.y, (sb.rows + SM_TGT - 1) / SM_TGT);
     k_sm_translate<N><<<unsigned(gt), SmTile<N>::THREADS, 0, st>>>(ctrl, insts, sb);
     PF_LAUNCHED(1);
     return cudaGetLastError();

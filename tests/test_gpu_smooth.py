@@ -89,3 +89,32 @@ def test_small_tolerances_sum_pairs(tol, summed):
            for form in (2, 1)]
     assert np.array_equal(got[0][0], got[1][0]) == summed
     assert np.array_equal(got[0][1], got[1][1]) == summed
+
+
+def test_first_evaluations_on_several_threads():
+    # contexts of their own on threads of their own, all at their first wide core
+    import threading
+    _lib, torch = G.lib(), G.torch_cuda()
+    ws = [wide_core(k, np.full((4, 4), 60), i) for i, k in enumerate([0.1, 0.3, 0.8, 1.7] * 2)]
+    dev = [G.to_dev((w.x, w.y, w.gamma)) for w in ws]
+    torch.cuda.synchronize()
+    out, go = [None] * len(ws), threading.Barrier(len(ws))
+
+    def work(i):
+        w, st = ws[i], torch.cuda.Stream()
+        go.wait()
+        with torch.cuda.stream(st):
+            ctx = _lib.Context(w.domain, w.L, w.p, w.sigma, precision="mixed", dtype="f32", stream=st)
+            u, v = ctx.evaluate(*dev[i])
+            assert ctx.sync() == 0
+            ctx.close()
+        out[i] = u.cpu().numpy(), v.cpu().numpy()
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(ws))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for w, got in zip(ws, out):
+        ref = G.run(w, "mixed")
+        assert got is not None and all(np.array_equal(a, b) for a, b in zip(got, ref))
