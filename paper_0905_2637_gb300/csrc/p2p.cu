@@ -67,11 +67,15 @@ __constant__ int8_t c_fwd[4][2] = {{1, 0}, {-1, 1}, {0, 1}, {1, 1}};
 // pmin (InstDesc::pair_min) blobs; the others are summed directly, one thread
 // per target (k_near_direct).  Both leaves of a pair decide from the same two
 // counts.  PETFMM_OPT_P2P_PAIRS = 1 sets pmin to a warp's worth, 32.  The
-// automatic choice never does: wide cores (kappa <= 1.95) go by expansions,
-// and beyond the polynomial's range the pair kernel ran at 0.2 to 1.06 of the
-// direct kernel's rate (349,185 clustered blobs, 530 per leaf, kappa = 7.6:
-// 3.2 ms, its few heavy items unbalanced, against 1.2; 4,000,000 blobs, 560 per
-// leaf, kappa = 3.9, its best case: 7.5 against 8.0).
+// automatic choice never does: wide cores (kappa <= 1.95) go by expansions, and
+// beyond them neither kernel is always the better one.  Whole evaluations,
+// direct / pairs, ms: where few heavy items decide, 349,185 clustered blobs, 530
+// per leaf, kappa = 6: 1.38 / 2.65; 131,072 even blobs, 512 per leaf, kappa = 3.9:
+// 0.51 / 0.81; 64 per leaf, kappa = 12: 0.60 / 0.63.  In dense trees with many
+// leaves pairs win: 1,048,576 even blobs, 256 per leaf, kappa = 3.9: 1.66 / 1.39;
+// 4,000,000 clustered ones, 560 per leaf: 8.96 / 7.28.  Which it is depends on how
+// the blobs lie, which the plan does not know; the option is there for dense
+// trees.
 __host__ __device__ __forceinline__ bool pairwise(uint32_t na, uint32_t nb, uint32_t pmin) {
     return na >= pmin && nb >= pmin;
 }
@@ -1375,15 +1379,15 @@ cudaError_t launch_pair_worklist(const Task *tasks, int ntasks, int64_t nblocks,
 // The near field outside the pair kernel, one thread per target blob: own[r]
 // = its sum over the leaves of its neighbourhood that are not summed pairwise
 // with its own (Laplace kernel, and vortex cores narrow against a leaf: all
-// nine).  Bound by issue (about 16 instructions a pair, two of them special
-// functions, 12 of the special-function pipe's cycles): every lane has a
-// target of its own, so leaves of any count fill the warps, where a warp per
+// nine).  Bound by issue (74 % of the slots; 26 instructions a pair and lane with
+// the idle lanes of uneven leaves, two of them special functions): every lane has
+// a target of its own, so leaves of any count fill the warps, where a warp per
 // leaf of 17 blobs kept 17 of 32 lanes busy; the lanes of a leaf read the
 // same source (one request), and no work list is needed.
 // Measured on one GB300 (this kernel alone, against work items and the pair
 // kernel with their lists): 512 uneven trees, 3.9e9 pairs: 9.0 -> 3.6 ms;
-// 1,048,576 blobs, 16 per leaf: 0.29 -> 0.12 ms; 349,185 clustered blobs, 530
-// per leaf, kappa = 7.6: 3.3 -> 1.2 ms.
+// 1,048,576 blobs, 16 per leaf: 0.29 -> 0.13 ms; 349,185 clustered blobs, 530
+// per leaf, kappa = 7.6: 3.3 -> 1.3 ms.
 constexpr int NEAR_THREADS = 128;  // half a particle task block: more blocks, better balance
 
 __global__ void __launch_bounds__(NEAR_THREADS, 8) k_near_direct(
