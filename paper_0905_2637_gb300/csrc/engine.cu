@@ -400,9 +400,11 @@ int attach_sm_tables(petfmm_ctx *c, Plan &pl) {
             if (!fixed.p) {
                 const std::vector<double> &t = host_sm_fixed(n);
                 PF_TRY(ensure(fixed, t.size() * sizeof(double), c->stream));
+                // (the table outlives the copy)
                 const cudaError_t e = cudaMemcpyAsync(fixed.p, t.data(), t.size() * sizeof(double),
                                                       cudaMemcpyHostToDevice, c->stream);
                 if (e != cudaSuccess) {
+                    cudaGetLastError();
                     cudaFree(fixed.p);
                     fixed = DevBuf();
                     return cuda_status(e);

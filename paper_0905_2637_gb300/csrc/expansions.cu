@@ -262,6 +262,14 @@ void host_op_table(int p, int kernel, int which, std::vector<double> &out) {
     else (lap ? host_lap_m2l_table : host_m2l_table)(p, out.data());
 }
 
+// A table on its stream, which the launches that use it follow.  The source goes
+// with the caller's frame, and a device that reads pageable memory itself need
+// not have it staged when the copy returns: wait for it.
+cudaError_t copy_table(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
+}
+
 cudaError_t build_op_tables(int p, int kernel, bool fp64, OpTables *t, cudaStream_t st) {
     t->p = p;
     std::vector<double> shift, orbit;
@@ -291,16 +299,18 @@ cudaError_t build_op_tables(int p, int kernel, bool fp64, OpTables *t, cudaStrea
     size_t total = 0;
     for (const Part &x : parts) total += (x.bytes + 255) / 256 * 256;
     std::vector<unsigned char> blob(total);
-    const cudaError_t e = cudaMalloc(&t->blob, total);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaMalloc(&t->blob, total);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return e;
+    }
     size_t at = 0;
     for (const Part &x : parts) {
         std::memcpy(blob.data() + at, x.src, x.bytes);
         *x.dst = static_cast<unsigned char *>(t->blob) + at;
         at += (x.bytes + 255) / 256 * 256;
     }
-    // (the call returns once the pageable source is staged)
-    return cudaMemcpyAsync(t->blob, blob.data(), total, cudaMemcpyHostToDevice, st);
+    return copy_table(t->blob, blob.data(), total, st);
 }
 
 cudaError_t build_tc_image(int kernel, bool blocks, OpTables *t, cudaStream_t st) {
@@ -310,9 +320,13 @@ cudaError_t build_tc_image(int kernel, bool blocks, OpTables *t, cudaStream_t st
     (blocks ? host_m2l_tcb_images : host_m2l_tc_images)(t->p, kernel, img);
     void *p = nullptr;
     cudaError_t e = cudaMalloc(&p, img.size() * 4);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p, img.data(), img.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) cudaFree(p);
-    else dst = static_cast<float *>(p);
+    if (e == cudaSuccess) e = copy_table(p, img.data(), img.size() * 4, st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(p);
+    } else {
+        dst = static_cast<float *>(p);
+    }
     return e;
 }
 

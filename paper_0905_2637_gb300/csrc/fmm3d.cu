@@ -2712,11 +2712,11 @@ int ensure3(DevBuf3 &b, size_t bytes, cudaStream_t st) {
 }
 
 // A table, copied on the context's stream: the launches that follow there find it
-// complete (the call returns once the pageable source is staged).
+// complete.
 int upload3(DevBuf3 &b, const void *src, size_t bytes, cudaStream_t st) {
     const int rc = ensure3(b, bytes, st);
     if (rc) return rc;
-    if (cudaMemcpyAsync(b.p, src, bytes, cudaMemcpyHostToDevice, st) == cudaSuccess) return PETFMM_OK;
+    if (copy_table(b.p, src, bytes, st) == cudaSuccess) return PETFMM_OK;
     cudaGetLastError();
     return PETFMM_ECUDA;
 }

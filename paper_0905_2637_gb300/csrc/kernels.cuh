@@ -79,6 +79,7 @@ struct OpTables {
 // plan has such units.
 cudaError_t build_op_tables(int p, int kernel, bool fp64, OpTables *out, cudaStream_t st);
 cudaError_t build_tc_image(int kernel, bool blocks, OpTables *t, cudaStream_t st);
+cudaError_t copy_table(void *dst, const void *src, size_t bytes, cudaStream_t st);
 // The FP64 table behind them: which = 0 M2M [c][l][k], 1 L2L [c][n][m],
 // 2 M2L [op][k][m], complex as (re, im) pairs.
 void host_op_table(int p, int kernel, int which, std::vector<double> &out);

@@ -135,7 +135,7 @@ def test_admission_counts_the_near_field_expansions():
     active = []
     for sigma in (0.1, 0.002):
         srv = _lib.Server(int(2.2 * base), max_slots=8)
-        ts = [srv.submit(x, y, g, sigma, 8, 0.01, 3, precision="mixed", levels=7) for _ in range(4)]
+        ts = [srv.submit(x, y, g, sigma, 8, 0.001, 12, precision="mixed", levels=7) for _ in range(4)]
         assert all(r["status"] == 0 for r in _wait(srv, ts))
         active.append(srv.stats()["max_active"])
         srv.close()
