@@ -1604,21 +1604,27 @@ __device__ __forceinline__ void store3(void *o, int64_t i, double v) {
 // it in direction d, own (one-sided).
 //
 // One warp evaluates a leaf pair, all of it (its reactions have one writer), so
-// a pair is left to the one-sided sums, which any number of warps share, where
-// it is more than a small part of the whole: na nb above P3_SHARE / 4096 of the
-// pairs of all leaf pairs that could be pairwise, and above P3_LEAST (a group
-// of three such pairs is no more than the six of 96 charges that two groups a
-// leaf give).
-// Measured (one GB300, whole evaluations, p = 6, us; all pairs pairwise / at this
-// limit): mixed, 5,000 clustered charges 714 / 390, 150,000 16,800 / 2,440,
-// 100,000 charges in eight leaves 342,000 / 6,900; FP64, 60,000 clustered 338,000
-// / 68,300.  Shares of 1/2048, 1/4096, 1/8192 (mixed): 600,000 clustered 27.5 /
-// 22.9 / 21.9 ms, but 1,000,000 uniform charges, 1,950 a leaf, 18.0 / 18.0 /
-// 21.8; of 1/256, 1/410, 1/512 (FP64): 150,000 clustered 135 / 110 / 104 ms,
-// 100,000 uniform, 1,560 a leaf, 99 / 99 / 126.
+// few or heavy pairs leave the GPU waiting for single warps; the one-sided sums
+// are shared by any number of them.  A pair (a leaf with itself) of na nb pairs
+// of charges is therefore summed pairwise up to a limit: the largest, in half
+// octaves, of which all pairs up to it together hold 16,384 / P3_SHARE; at least
+// up to P3_LEAST (a group of three such pairs is no more than the six of 96
+// charges that two groups a leaf give); and none where those up to the limit
+// together are fewer than P3_ENOUGH.
+// Measured (one GB300, whole evaluations, p = 6, us; every pair pairwise / at this
+// limit / every pair one-sided): mixed, clustered charges, 5,000 714 / 356 / 323,
+// 150,000 16,800 / 2,030 / 1,950, 600,000 279,000 / 18,900 / 18,800; 100,000 charges
+// in eight leaves 342,000 / 6,900 / 6,700; even trees, 8,000 329 / 297 / 277,
+// 220,000 (54 a leaf) 629 / 629 / 660, 2 M (64) 2,685 / 2,689 / 3,080; below some 48
+// a leaf one-sided is up to 15 % faster.  FP64, clustered, 20,000 39,000 / 9,900 /
+// 8,400, 150,000 296,000 / 102,000 / 90,000; even, 262,144 10,890 / 10,890 / 17,600.
+// With the limit a fixed part of the sum over all pairs, few middling ones among
+// many heavy ones still held the launch up (150,000 clustered 2,450).
 // ---------------------------------------------------------------------------
 constexpr uint32_t P3_PAIR_MIN = 24;
-constexpr uint32_t P3_SHARE = 1, P3_SHARE64 = 10, P3_LEAST = 16384;
+constexpr uint32_t P3_SHARE = 5, P3_SHARE64 = 40;  // of 16,384
+constexpr int P3_LEAST = 27;                       // half octave: below 2^14
+constexpr uint32_t P3_ENOUGH = 1u << 24, P3_ENOUGH64 = 0;
 constexpr int P3_DIRS = 13;
 // planes of one entry per charge, fwd and bwd: mixed (the leaf itself in its
 // first group) and FP64 (a group by itself in the heaviest leaves)
@@ -1646,13 +1652,15 @@ __host__ __device__ __forceinline__ int own_group3(int groups) {
 // leaf flags of the final pass: bit d: bwd[d] holds a part; bit 13: own does;
 // bit 14: fwd of the leaf's groups do
 constexpr uint32_t LF3_OWN = 1u << 13, LF3_FWD = 1u << 14;
-// counters: directed items, pair items, then per work class the pair items
-// counted and placed, then (64 bits) the pairs of all leaf pairs of at least
-// pmin charges each
+// counters: directed items, pair items, per work class the pair items counted and
+// placed, blocks of the counting launch done, the limit of a pairwise leaf pair,
+// and the leaf pairs of each half octave of their pairs of charges
 constexpr int C3_DIRECTED = 0, C3_PAIRS = 1, C3_COUNT = 2, C3_CLASSES = 64,
-              C3_PLACED = C3_COUNT + C3_CLASSES, C3_TOTAL = C3_PLACED + C3_CLASSES,
-              C3_WORDS = C3_TOTAL + 2;
-static_assert(C3_TOTAL % 2 == 0, "64-bit counter");
+              C3_PLACED = C3_COUNT + C3_CLASSES, C3_DONE = C3_PLACED + C3_CLASSES,
+              C3_LIMIT = C3_DONE + 1, C3_COST = C3_LIMIT + 1, C3_OCTAVES = 64,
+              C3_WORDS = C3_COST + C3_OCTAVES;
+
+constexpr uint32_t NO_GROUP3 = ~0u;  // an item with nothing to sum
 
 struct Near3 {
     float4 *own, *slots;  // slots[P3_SLOTS][n], or no pairs
@@ -1662,16 +1670,23 @@ struct Near3 {
     uint2 *items;         // (leaf, group)
     int64_t n;
     uint32_t pmin;        // P3_PAIR_MIN, or all ones: no pairs
-    uint32_t share;       // most3's limit, in 1/4096 of the total
+    uint32_t share, enough;  // P3_SHARE, P3_ENOUGH of the path
 };
 
+// Half octave of a leaf pair's na nb = x pairs of charges (2^e .. 1.5 2^e .. 2^(e+1)),
+// C3_OCTAVES and more: too many for any limit; the end of half octave h.
+__device__ __forceinline__ int octave3(uint64_t x) {
+    if (x >> 32) return C3_OCTAVES;
+    const int e = 31 - __clz(int(uint32_t(x) | 1u));
+    return 2 * e + int(e ? (x >> (e - 1)) & 1u : 0u);
+}
+__device__ __forceinline__ uint64_t octave_end3(int h) {
+    return h & 1 ? uint64_t(2) << (h / 2) : uint64_t(3) << (h / 2) >> 1;
+}
 // Most charges of a leaf that is summed pairwise with one of n charges (n >= 1;
 // na nb <= limit is the same for both leaves), 0: none is.
 __device__ __forceinline__ uint32_t most3(const Near3 &w, uint32_t n) {
-    if (n < w.pmin) return 0;
-    const uint64_t total = *reinterpret_cast<const unsigned long long *>(w.ctrl + C3_TOTAL);
-    const uint64_t limit = (total >> 12) * w.share;
-    return max(uint32_t(min(limit, uint64_t(0xffffffffu))), P3_LEAST) / n;
+    return n < w.pmin ? 0u : w.ctrl[C3_LIMIT] / n;
 }
 // Whether a leaf with most = most3 of its charges and a neighbour of n (or
 // itself) are summed pairwise.
@@ -1695,81 +1710,118 @@ __device__ __forceinline__ int class3(uint32_t n, uint64_t src) {
     return c >= C3_CLASSES ? 0 : C3_CLASSES - 1 - c;
 }
 
-// Calls f(class, group, pairs) for the pair items of leaf b (n charges), as if
-// every leaf pair of at least pmin charges each were summed pairwise.
-template <int MAX, typename F>
+// Calls f(class, group) for the pair items of leaf b (n charges) and pair(na nb)
+// for its leaf pairs, as if every one of at least pmin charges each were summed
+// pairwise.
+template <int MAX, typename F, typename G>
 __device__ __forceinline__ void leaf_items3(const uint32_t *__restrict__ start, int L, uint32_t b,
-                                            uint32_t n, uint32_t pmin, F &&f) {
+                                            uint32_t n, uint32_t pmin, F &&f, G &&pair) {
     const int side = 1 << L;
     const int ix = int(compact3(b)), iy = int(compact3(b >> 1)), iz = int(compact3(b >> 2));
     const int groups = groups3<MAX>(n);
     for (int g = 0; g < groups; ++g) {
-        uint64_t src = g == own_group3(groups) ? n : 0;
+        uint64_t src = 0;
+        if (g == own_group3(groups)) {
+            src = n;
+            pair(uint64_t(n) * n);
+        }
         for (int k = group_first3(g, groups); k < group_first3(g + 1, groups); ++k) {
             int dx, dy, dz;
             fwd3(k, &dx, &dy, &dz);
             const uint32_t c = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
-            if (c >= pmin) src += c;
+            if (c < pmin) continue;
+            src += c;
+            pair(uint64_t(n) * c);
         }
-        f(class3(n, src), g, uint64_t(n) * src);
+        f(class3(n, src), g);
     }
 }
 
 // Two launches over the leaves: EMIT = false counts the pair items of each
-// class, EMIT = true writes them, heaviest class first, the directed items and
+// class and finds the limit of a pairwise leaf pair (its last block), EMIT = true writes them, heaviest class first, the directed items and
 // the leaf flags.  A block counts in shared memory and takes its run of each
 // list by one atomic (the order of items changes no result).
 template <bool EMIT, int MAX>
 __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__restrict__ start,
                                                      Near3 w) {
     __shared__ uint32_t hist[C3_CLASSES], base[C3_CLASSES], ndir, dbase;
-    __shared__ unsigned long long sum;
+    __shared__ uint32_t cost[EMIT ? 1 : C3_OCTAVES];
+    __shared__ uint32_t last;
     const int64_t nleaf = int64_t(1) << (3 * L);
     const int64_t b = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (threadIdx.x < C3_CLASSES) hist[threadIdx.x] = 0;
-    if (threadIdx.x == 0) {
-        ndir = 0;
-        sum = 0;
-    }
+    if (!EMIT && threadIdx.x < C3_OCTAVES) cost[threadIdx.x] = 0;
+    if (threadIdx.x == 0) ndir = 0;
     __syncthreads();
     const uint32_t s0 = b < nleaf ? start[b] : 0u, n = b < nleaf ? start[b + 1] - s0 : 0u;
     const bool big = n >= w.pmin;
-    unsigned long long pairs = 0;
+    int run = C3_OCTAVES;  // half octave of the leaf pairs not yet counted: a leaf's
+    uint32_t pairs = 0;    // neighbours are mostly alike
+    auto flush = [&] {
+        if (!EMIT && run < C3_OCTAVES) atomicAdd(&cost[run], pairs);
+    };
     if (big)
-        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int, uint64_t q) {
-            atomicAdd(&hist[c], 1u);
-            pairs += q;
-        });
+        leaf_items3<MAX>(
+            start, L, uint32_t(b), n, w.pmin, [&](int c, int) { atomicAdd(&hist[c], 1u); },
+            [&](uint64_t q) {
+                if (EMIT) return;
+                const int h = octave3(q);
+                if (h != run) {
+                    flush();
+                    run = h;
+                    pairs = 0;
+                }
+                ++pairs;
+            });
     if (!EMIT) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) pairs += __shfl_down_sync(0xffffffffu, pairs, o);
-        if ((threadIdx.x & 31) == 0 && pairs) atomicAdd(&sum, pairs);
+        flush();
         __syncthreads();
-        if (threadIdx.x == 0 && sum)
-            atomicAdd(reinterpret_cast<unsigned long long *>(w.ctrl + C3_TOTAL), sum);
+        if (threadIdx.x < C3_OCTAVES && cost[threadIdx.x])
+            atomicAdd(w.ctrl + C3_COST + threadIdx.x, cost[threadIdx.x]);
         if (threadIdx.x < C3_CLASSES && hist[threadIdx.x]) {
             atomicAdd(w.ctrl + C3_COUNT + threadIdx.x, hist[threadIdx.x]);
             atomicAdd(w.ctrl + C3_PAIRS, hist[threadIdx.x]);
         }
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(w.ctrl + C3_DONE, 1u) + 1u == gridDim.x;
+        __syncthreads();
+        if (!last) return;
+        if (threadIdx.x < C3_OCTAVES) cost[threadIdx.x] = __ldcg(w.ctrl + C3_COST + threadIdx.x);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint64_t sum = 0, limit = 0;
+            for (int h = 0; h < C3_OCTAVES; ++h) {
+                // (a leaf pair of the half octave taken for one at its end)
+                const uint64_t end = octave_end3(h);
+                sum += cost[h] * end;
+                if (sum >= w.enough && (h <= P3_LEAST || sum * w.share >= end * 16384)) limit = end - 1;
+            }
+            w.ctrl[C3_LIMIT] = uint32_t(limit);
+        }
         return;
     }
     uint32_t mine = 0, at = 0;  // directed items and their place in the block's run
+    bool paired = false;        // some pair of the leaf's items is summed pairwise
     if (n) {
         const int side = 1 << L;
         const int ix = int(compact3(uint32_t(b))), iy = int(compact3(uint32_t(b) >> 1)),
                   iz = int(compact3(uint32_t(b) >> 2));
-        uint32_t flags = big ? LF3_FWD : 0u;
+        uint32_t flags = 0;
         const uint32_t most = most3(w, n);
-        bool directed = !pairwise3(w, most, n);
+        paired = pairwise3(w, most, n);
+        bool directed = !paired;
         for (int k = 0; big && k < P3_DIRS; ++k) {
             int dx, dy, dz;
             fwd3(k, &dx, &dy, &dz);
             const uint32_t f = leaf_count3(start, side, ix + dx, iy + dy, iz + dz);
             const uint32_t r = leaf_count3(start, side, ix - dx, iy - dy, iz - dz);
-            const bool rp = pairwise3(w, most, r);
+            const bool fp = pairwise3(w, most, f), rp = pairwise3(w, most, r);
             if (rp) flags |= 1u << k;
-            directed |= (f && !pairwise3(w, most, f)) || (r && !rp);
+            paired |= fp;
+            directed |= (f && !fp) || (r && !rp);
         }
+        if (paired) flags |= LF3_FWD;
         if (directed) {
             flags |= LF3_OWN;
             mine = (n + 31) / 32;
@@ -1791,9 +1843,13 @@ __global__ void __launch_bounds__(256) k3_near_items(int L, const uint32_t *__re
     for (uint32_t i = 0; i < mine; ++i)
         w.directed[dbase + at + i] = make_uint2(uint32_t(b), s0 + 32 * i);
     if (big)
-        leaf_items3<MAX>(start, L, uint32_t(b), n, w.pmin, [&](int c, int g, uint64_t) {
-            w.items[base[c] + atomicAdd(&hist[c], 1u)] = make_uint2(uint32_t(b), uint32_t(g));
-        });
+        leaf_items3<MAX>(
+            start, L, uint32_t(b), n, w.pmin,
+            [&](int c, int g) {
+                w.items[base[c] + atomicAdd(&hist[c], 1u)] =
+                    make_uint2(uint32_t(b), paired ? uint32_t(g) : NO_GROUP3);
+            },
+            [](uint64_t) {});
 }
 
 // 1/sqrt(x) for a normal x > 0: the PTX approximate reciprocal square root
@@ -2078,6 +2134,7 @@ __global__ void __launch_bounds__(128, 6) k3_pairs(int L, const uint32_t *__rest
     const uint32_t it = blockIdx.x * 4 + (threadIdx.x >> 5);
     if (it >= w.ctrl[C3_PAIRS]) return;
     const uint2 item = w.items[it];
+    if (item.y == NO_GROUP3) return;
     const uint32_t leaf = item.x;
     if (!PF_IN(leaf, int64_t(1) << (3 * L))) return;
     const int g = int(item.y);
@@ -2370,6 +2427,7 @@ __global__ void __launch_bounds__(PW64 * 32) k3_pairs_f64(int L, const uint32_t 
     const uint32_t it = blockIdx.x * PW64 + wid;
     if (it >= w.ctrl[C3_PAIRS]) return;
     const uint2 item = w.items[it];
+    if (item.y == NO_GROUP3) return;
     const uint32_t leaf = item.x;
     if (!PF_IN(leaf, int64_t(1) << (3 * L))) return;
     const int g = int(item.y), side = 1 << L;
@@ -3082,6 +3140,7 @@ int near3(petfmm3d_ctx *c, int64_t n, Near3 *nr, int64_t *icap) {
     nr->n = n;
     nr->pmin = ~0u;
     nr->share = mixed ? P3_SHARE : P3_SHARE64;
+    nr->enough = mixed ? P3_ENOUGH : P3_ENOUGH64;
     P3_TRY(needed3(c, n, near_buffers3));
     if (n >= 2 * int64_t(pmin) && n * parts <= c->pair_bytes && !c->no_pairs) {
         // up to 2 groups of a leaf of at least pmin, 4 above 96 charges, 14 above 384

@@ -41,9 +41,11 @@ def test_m2l_option_returns_to_its_default():
 # default's bits again afterwards.
 @pytest.mark.parametrize("precision,tol", [("fp64", 1e-12), ("mixed", 1e-5)])
 def test_pairs_from_both_sides(precision, tol):
-    # (the second one's eight leaves are so full that it has no other pairs)
-    for w, same in ((W.tiny3d(20_000, 5, L=3, p=8, clustered_frac=0.5), False),
-                    (W.tiny3d(3000, 6, L=1, p=4, clustered_frac=0.2), True)):
+    # (an even tree of enough pairs has pairwise sums; in the others it depends on
+    # their weights)
+    for w, even in ((W.tiny3d(60_000, 5, L=3, p=8), True),
+                    (W.tiny3d(20_000, 5, L=3, p=8, clustered_frac=0.5), False),
+                    (W.tiny3d(3000, 6, L=1, p=4, clustered_frac=0.2), False)):
         ctx = T._ctx(w, precision)
         first = _eval(ctx, w)
         ctx.set_option(fmm3d.PETFMM3D_OPT_PAIR_BYTES, 0)
@@ -54,7 +56,7 @@ def test_pairs_from_both_sides(precision, tol):
         with pytest.raises(Exception):
             ctx.set_option(fmm3d.PETFMM3D_OPT_PAIR_BYTES, -1)
         ctx.close()
-        assert np.array_equal(first[0], both[0]) == same
+        assert not (even and np.array_equal(first[0], both[0]))
         assert all(np.array_equal(a, b) for a, b in zip(first, again))
         assert T._rel(both[0], first[0]) <= tol and T._field_rel(both, first) <= tol
 
