@@ -129,7 +129,9 @@ __device__ __forceinline__ uint32_t work_class(uint32_t cost) {
     return 127u - (uint32_t(e) * 4u + frac);
 }
 
-// Calls emit(class, item) for every item of leaf m; the leaf's ordered pairs.
+// Calls emit(class, first item, count) for every run of alike items of leaf m (its
+// whole ones, then the rest: warps that take them together share its sources in
+// L1); the leaf's ordered pairs.
 // The class is that of the n_nd N_i^2 term of Eq. 14 (targets x sources):
 // every lane of the warp runs the source loop of its group, target slot filled
 // or not, so the cost is the sources per lane group, ceil(src / S) with S
@@ -145,12 +147,14 @@ __device__ __forceinline__ unsigned long long leaf_items(const InstDesc &d, cons
     uint32_t src = 0;  // the blobs of the leaf and its neighbours
     for (int dy = -1; dy <= 1; ++dy)
         for (int dx = -1; dx <= 1; ++dx) src += leaf_count(st, nside, ix + dx, iy + dy);
-    for (uint32_t f = 0; f < n; f += tpi) {
-        const uint32_t nt = min(n - f, tpi);
+    const uint32_t whole = n / tpi, rest = n - whole * tpi;
+    auto run = [&](uint32_t f, uint32_t nt, uint32_t count) {
         const int ns = 5 - p2p_group_log2(nt, int(tpi) / 32);  // log2 S
         emit(ordered ? work_class((src + (1u << ns) - 1) >> ns) : 0u,
-             make_uint4(inst, m, s0 + f, nt));
-    }
+             make_uint4(inst, m, s0 + f, nt), count);
+    };
+    if (whole) run(0, tpi, whole);
+    if (rest) run(whole * tpi, rest, 1);
     return (unsigned long long)n * (src - 1);
 }
 
@@ -170,7 +174,7 @@ __global__ void __launch_bounds__(256) k_item_count(const Task *__restrict__ tas
     if (m < t.count) {
         const InstDesc &d = insts[t.inst];
         pairs = leaf_items(d, start + d.soff, uint32_t(m), uint32_t(t.inst), tpi, ordered,
-                           [&](uint32_t c, const uint4 &) { atomicAdd(&hist[c], 1u); });
+                           [&](uint32_t c, const uint4 &, uint32_t k) { atomicAdd(&hist[c], k); });
     }
     // the ordered pair count, for the statistics
 #pragma unroll
@@ -203,7 +207,7 @@ __global__ void __launch_bounds__(256) k_item_emit(const Task *__restrict__ task
     __syncthreads();
     if (m < t.count)
         leaf_items(d, st, uint32_t(m), uint32_t(t.inst), tpi, ordered,
-                   [&](uint32_t c, const uint4 &) { atomicAdd(&hist[c], 1u); });
+                   [&](uint32_t c, const uint4 &, uint32_t k) { atomicAdd(&hist[c], k); });
     __syncthreads();
     // this block's run within each class
     uint32_t base = 0, n = 0;
@@ -219,9 +223,10 @@ __global__ void __launch_bounds__(256) k_item_emit(const Task *__restrict__ task
     __syncthreads();
     if (m < t.count)
         leaf_items(d, st, uint32_t(m), uint32_t(t.inst), tpi, ordered,
-                   [&](uint32_t c, const uint4 &item) {
-                       const uint32_t o = first[c] + atomicAdd(&hist[c], 1u);
-                       if (PF_IN(o, cap)) items[o] = item;
+                   [&](uint32_t c, uint4 item, uint32_t k) {
+                       const uint32_t o = first[c] + atomicAdd(&hist[c], k);
+                       for (uint32_t i = 0; i < k; ++i, item.z += tpi)
+                           if (PF_IN(o + i, cap)) items[o + i] = item;
                    });
 }
 
