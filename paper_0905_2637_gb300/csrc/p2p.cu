@@ -410,12 +410,14 @@ __global__ void __launch_bounds__(P2P_THREADS, 5) k_p2p_mixed(
     const int lane = threadIdx.x & 31;
     const uint32_t nitems = *reinterpret_cast<volatile uint32_t *>(ctrl + CTRL_NITEMS);
     const uint64_t t_begin = busy ? global_ns() : 0;
-    for (;;) {
-        uint32_t it = 0;
-        if (lane == 0) it = atomicAdd(ctrl + CTRL_QUEUE, 1u);
-        it = __shfl_sync(0xffffffffu, it, 0);
-        if (it >= nitems) break;
+    // a warp's first item by its position, block by block (few items then spread
+    // over the SMs), the others from the queue
+    const uint32_t nwarps = gridDim.x * (P2P_THREADS / 32);
+    uint32_t it = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (it < nitems) {
         directed_item<DEG, GENERAL, LAP>(items[it], insts, start, rec, own, lane);
+        if (lane == 0) it = nwarps + atomicAdd(ctrl + CTRL_QUEUE, 1u);
+        it = __shfl_sync(0xffffffffu, it, 0);
     }
     if (busy && lane == 0) {
         const uint64_t t_end = global_ns();
