@@ -3142,7 +3142,10 @@ int near3(petfmm3d_ctx *c, int64_t n, Near3 *nr, int64_t *icap) {
     nr->share = mixed ? P3_SHARE : P3_SHARE64;
     nr->enough = mixed ? P3_ENOUGH : P3_ENOUGH64;
     P3_TRY(needed3(c, n, near_buffers3));
-    if (n >= 2 * int64_t(pmin) && n * parts <= c->pair_bytes && !c->no_pairs) {
+    // (up to n^2 pairs of charges, a half octave's taken for up to 3/2 of them: too
+    // few charges for any pairwise sum need no lists of them)
+    const bool enough = uint64_t(n) * uint64_t(n) / 2 * 3 >= nr->enough;
+    if (n >= 2 * int64_t(pmin) && enough && n * parts <= c->pair_bytes && !c->no_pairs) {
         // up to 2 groups of a leaf of at least pmin, 4 above 96 charges, 14 above 384
         *icap = 2 * std::min<int64_t>(nleaf, n / pmin) + 2 * (n / 97) + 10 * (n / 385) + 1;
         int rc = ensure3(c->pitems, size_t(*icap) * sizeof(uint2), st);
